@@ -397,43 +397,6 @@ __device__ __forceinline__ void lane_codes(const uint32_t (&w)[NW], int b_lo, in
   }
 }
 
-// ---------------------------------------------------------------------------
-// Thread-per-leaf sum of byte-code leaves (codec 0): the sum (mod 2^64) of
-// the elements of the leaf at leafp with u >= 8 used bytes.  One thread walks
-// the leaf eight bytes at a time keeping the running element value val and
-// the running sum s.  Inside the eight bytes everything is 32-bit: each byte
-// adds its payload times 128^(bytes before it in its code) to acc, and acc is
-// not cleared at a terminator, so at the k-th terminator of the group acc_k
-// holds the bits of every code closed so far in the group (plus the open code
-// carried in): the element closed there is val + acc_k.  The group adds T *
-// val + sum_k acc_k to s (T terminators), val moves on by the acc of its last
-// terminator and acc keeps only the open code's bits.  With codes of at most 4
-// bytes at most 11 bytes of payload feed one group and sum_k acc_k < 9 * 2^28
-// fits in 32 bits.  Bytes after u are read as zero: each of them acts as a
-// terminator adding the last value again, which is taken off at the end.  A
-// code of more than 4 bytes overflows the 32-bit code accumulator; such a
-// leaf is summed again exactly, byte by byte.
-__device__ __forceinline__ void leaf_sum_group(uint32_t wa, uint32_t wb, uint64_t& val,
-                                               uint64_t& s, uint32_t& acc, uint32_t& pw,
-                                               uint32_t& pwor) {
-  const uint32_t pa = wa & 0x7F7F7F7Fu, pb = wb & 0x7F7F7F7Fu;
-  uint32_t ss = 0, r = 0;
-#pragma unroll
-  for (int b = 0; b < 8; b++) {
-    const uint32_t wv = b < 4 ? wa : wb, pv = b < 4 ? pa : pb;
-    acc += __byte_perm(pv, 0u, 0x4440u + (uint32_t)(b & 3)) * pw;
-    const bool term = (wv & (0x80u << (8 * (b & 3)))) == 0u;
-    pwor |= pw;
-    ss += term ? acc : 0u;
-    r = term ? acc : r;
-    pw = term ? 1u : pw << 7;
-  }
-  const uint32_t T = __popc(~wa & 0x80808080u) + __popc(~wb & 0x80808080u);
-  s += (uint64_t)T * val + ss;
-  val += r;
-  acc -= r;
-}
-
 // Bytes of w past u - p0 cleared (the leaf's zero padding, read as such).
 __device__ __forceinline__ void mask_past(uint32_t (&w)[4], uint32_t p0, uint32_t u) {
   if (p0 + 16u > u) {
@@ -443,56 +406,10 @@ __device__ __forceinline__ void mask_past(uint32_t (&w)[4], uint32_t p0, uint32_
   }
 }
 
-__device__ __forceinline__ uint64_t thread_leaf_sum(const uint8_t* __restrict__ leafp, uint32_t u) {
-  // 32 bytes (one sector) per step: both halves are loaded before either is
-  // decoded, so each sector is requested once
-  uint4 v = *reinterpret_cast<const uint4*>(leafp);
-  uint4 v2 = u > 16u ? *reinterpret_cast<const uint4*>(leafp + 16) : make_uint4(0u, 0u, 0u, 0u);
-  uint32_t w[4] = {v.x, v.y, v.z, v.w};
-  uint64_t val = (uint64_t)w[0] | ((uint64_t)w[1] << 32), s = val;
-  uint32_t acc = 0, pw = 1, pwor = 0;
-  for (uint32_t p0 = 0; p0 < u; p0 += 32) {
-    if (p0) {
-      v = *reinterpret_cast<const uint4*>(leafp + p0);
-      v2 = p0 + 16u < u ? *reinterpret_cast<const uint4*>(leafp + p0 + 16) : make_uint4(0u, 0u, 0u, 0u);
-      w[0] = v.x; w[1] = v.y; w[2] = v.z; w[3] = v.w;
-    }
-    mask_past(w, p0, u);
-    if (p0) leaf_sum_group(w[0], w[1], val, s, acc, pw, pwor);  // bytes 0-7 are the head
-    leaf_sum_group(w[2], w[3], val, s, acc, pw, pwor);
-    if (p0 + 16u < u) {
-      uint32_t w2[4] = {v2.x, v2.y, v2.z, v2.w};
-      mask_past(w2, p0 + 16u, u);
-      leaf_sum_group(w2[0], w2[1], val, s, acc, pw, pwor);
-      leaf_sum_group(w2[2], w2[3], val, s, acc, pw, pwor);
-    }
-  }
-  s -= (uint64_t)(((u + 15u) & ~15u) - u) * val;
-  if (pwor >= (1u << 28)) {  // a long code: exact 64-bit decode
-    val = *reinterpret_cast<const uint64_t*>(leafp);
-    s = val;
-    uint64_t a64 = 0;
-    uint32_t sh = 0;
-    for (uint32_t p = 8; p < u; p++) {
-      const uint32_t c = leafp[p];
-      if (sh < 64) a64 |= (uint64_t)(c & 0x7Fu) << sh;
-      if (c & 0x80u) {
-        sh += 7;
-      } else {
-        val += a64;
-        s += val;
-        a64 = 0;
-        sh = 0;
-      }
-    }
-  }
-  return s;
-}
-
 // Is x an element of the byte-code leaf at leafp (u used bytes)?  One
 // thread decodes the leaf from its head, 16 bytes at a time, until the
 // running value passes x.  The bytes are taken eight at a time as in
-// thread_leaf_sum: the element closed at a terminator is val + acc with a
+// leaf_walk.cuh: the element closed at a terminator is val + acc with a
 // 32-bit acc, so it equals x exactly when acc equals x - val (no element of
 // the group can when x - val >= 2^32, since acc stays below 9 * 2^28).
 // Zero bytes after u repeat the last value, which is an element.  A leaf
@@ -557,176 +474,52 @@ __device__ __forceinline__ bool thread_leaf_has(const uint8_t* __restrict__ leaf
   return found;
 }
 
-// Sum (mod 2^64), count and used bytes of the byte-code leaves [j0, j1), one
-// leaf per lane at a time, added to the calling lane's partials.
-__device__ __forceinline__ void thread_span_sum(const uint8_t* __restrict__ data,
-                                                const uint32_t* __restrict__ used,
-                                                const uint32_t* __restrict__ cnt, uint32_t LB,
-                                                uint64_t j0, uint64_t j1, uint64_t& s,
-                                                uint64_t& c, unsigned long long& nbytes) {
-  for (uint64_t j = j0 + lane_id(); j < j1; j += 32) {
-    const uint32_t u = min(used[j], LB);
-    if (u == 0) continue;
-    s += thread_leaf_sum(data + j * LB, u);
-    c += cnt[j];
-    nbytes += u;
-  }
-}
-
 // ---------------------------------------------------------------------------
 // Sum (mod 2^64) and count of every element of the leaves [j0, j1), added to
 // the calling lane's partials (the caller reduces them over the warp).
 //
-// Leaves are taken 32 at a time.  Their used bytes are cut into 16-byte
-// chunks and the warp takes 32 chunks per step, so no lane idles on the zero
-// padding of a leaf.  The sum of a leaf with m elements, head h and deltas
-// d_1..d_{m-1} is m*h + sum_c (m - c) d_c; a chunk holding the codes c =
-// 1+B .. B+n (B = codes earlier in its leaf, a segmented warp scan) adds
-// (m - 1 - B) * D - W with D = sum of its deltas and W = sum of lidx * delta
-// (lidx = position among the chunk's codes).  The code a chunk starts in the
-// middle of is completed with the previous chunk's partial bits (one
-// shuffle).  Chunks are summarised bit-parallel (lane_codes), valid while
-// every code is at most 4 bytes (deltas < 2^28); a window of leaves with a
-// longer code is summed again by the general decoder instead.
+// 8-byte cells (codec 1): the used 16-byte chunks of 32 leaves are numbered by
+// a prefix sum and spread over the lanes, four loads in flight per lane.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void warp_span_sum(const uint8_t* __restrict__ data,
                                               const uint32_t* __restrict__ used,
                                               const uint32_t* __restrict__ cnt, uint32_t LB,
                                               uint64_t j0, uint64_t j1, uint64_t& acc,
-                                              uint64_t& cacc, ull& nbytes, bool raw = false) {
+                                              uint64_t& cacc, ull& nbytes) {
   const unsigned lane = lane_id();
-  if (raw) {
-    // codec 1: add the cells.  The used 16-byte chunks of 32 leaves are
-    // numbered by a prefix sum and spread over the lanes, four loads in
-    // flight per lane.
-    for (uint64_t w0 = j0; w0 < j1; w0 += 32) {
-      const uint64_t jj = w0 + lane;
-      const uint32_t u_i = jj < j1 ? min(__ldg(used + jj), LB) : 0u;
-      cacc += jj < j1 ? __ldg(cnt + jj) : 0u;
-      nbytes += u_i;
-      const uint32_t nc_i = (u_i + 15u) >> 4;
-      const uint32_t cinc = warp_incl_scan(nc_i);
-      const uint32_t NC = __shfl_sync(FULL, cinc, 31);
-      for (uint32_t g0 = 0; g0 < NC; g0 += 128) {
-        ulonglong2 v[4];
-        uint32_t lim[4];
-#pragma unroll
-        for (int q = 0; q < 4; q++) {
-          const uint32_t ci = g0 + 32u * q + lane;
-          uint32_t li = 0;
-#pragma unroll
-          for (int stp = 16; stp >= 1; stp >>= 1) {
-            const uint32_t cv = __shfl_sync(FULL, cinc, li + stp - 1);
-            if (cv <= ci) li += stp;
-          }
-          const uint32_t lis = min(li, 31u);
-          const uint32_t cstart = __shfl_sync(FULL, cinc, lis) - __shfl_sync(FULL, nc_i, lis);
-          const uint32_t u = __shfl_sync(FULL, u_i, lis);
-          const uint32_t p0 = (ci - cstart) * 16u;
-          v[q] = make_ulonglong2(0ull, 0ull);
-          lim[q] = 0;
-          if (ci < NC) {
-            v[q] = __ldg(reinterpret_cast<const ulonglong2*>(data + (w0 + lis) * LB + p0));
-            lim[q] = u - p0;  // used bytes from this chunk on: 8 or at least 16
-          }
-        }
-#pragma unroll
-        for (int q = 0; q < 4; q++) acc += v[q].x * (lim[q] >= 8) + v[q].y * (lim[q] >= 16);
-      }
-    }
-    return;
-  }
   for (uint64_t w0 = j0; w0 < j1; w0 += 32) {
     const uint64_t jj = w0 + lane;
-    const bool lv = jj < j1;
-    const uint32_t u_i = lv ? min(__ldg(used + jj), LB) : 0u;
-    const uint32_t m_i = lv ? __ldg(cnt + jj) : 0u;
-    cacc += m_i;
+    const uint32_t u_i = jj < j1 ? min(__ldg(used + jj), LB) : 0u;
+    cacc += jj < j1 ? __ldg(cnt + jj) : 0u;
     nbytes += u_i;
     const uint32_t nc_i = (u_i + 15u) >> 4;
     const uint32_t cinc = warp_incl_scan(nc_i);
     const uint32_t NC = __shfl_sync(FULL, cinc, 31);
-    uint64_t wacc = 0;
-    bool bad = false;
-    uint32_t cont_li = 0xFFFFFFFFu, cont_cnt = 0, cont_val = 0, cont_sh = 0;
-    // Chunk ci of the 32 leaves: its leaf slot (the number of leaves whose
-    // chunks end at or before ci), that leaf's first chunk, used bytes and
-    // count; the 16 bytes are loaded one step ahead of their use so the load
-    // of the next step overlaps the decode of this one.
-    struct Chunk { uint32_t li, lis, cstart, u, m; uint4 v; };
-    auto locate = [&](uint32_t g0, Chunk& k) {
-      const uint32_t ci = g0 + lane;
-      uint32_t li = 0;
+    for (uint32_t g0 = 0; g0 < NC; g0 += 128) {
+      ulonglong2 v[4];
+      uint32_t lim[4];
 #pragma unroll
-      for (int stp = 16; stp >= 1; stp >>= 1) {
-        const uint32_t v = __shfl_sync(FULL, cinc, li + stp - 1);
-        if (v <= ci) li += stp;
+      for (int q = 0; q < 4; q++) {
+        const uint32_t ci = g0 + 32u * q + lane;
+        uint32_t li = 0;
+#pragma unroll
+        for (int stp = 16; stp >= 1; stp >>= 1) {
+          const uint32_t cv = __shfl_sync(FULL, cinc, li + stp - 1);
+          if (cv <= ci) li += stp;
+        }
+        const uint32_t lis = min(li, 31u);
+        const uint32_t cstart = __shfl_sync(FULL, cinc, lis) - __shfl_sync(FULL, nc_i, lis);
+        const uint32_t u = __shfl_sync(FULL, u_i, lis);
+        const uint32_t p0 = (ci - cstart) * 16u;
+        v[q] = make_ulonglong2(0ull, 0ull);
+        lim[q] = 0;
+        if (ci < NC) {
+          v[q] = __ldg(reinterpret_cast<const ulonglong2*>(data + (w0 + lis) * LB + p0));
+          lim[q] = u - p0;  // used bytes from this chunk on: 8 or at least 16
+        }
       }
-      k.li = li;
-      k.lis = min(li, 31u);
-      k.cstart = __shfl_sync(FULL, cinc, k.lis) - __shfl_sync(FULL, nc_i, k.lis);
-      k.u = __shfl_sync(FULL, u_i, k.lis);
-      k.m = __shfl_sync(FULL, m_i, k.lis);
-      k.v = make_uint4(0u, 0u, 0u, 0u);
-      if (ci < NC)
-        k.v = __ldg(reinterpret_cast<const uint4*>(data + (w0 + k.lis) * LB +
-                                                    (ci - k.cstart) * 16u));
-    };
-    Chunk cur, nxt;
-    if (NC) locate(0, cur);
-    for (uint32_t g0 = 0; g0 < NC; g0 += 32) {
-      if (g0 + 32 < NC) locate(g0 + 32, nxt);
-      const uint32_t ci = g0 + lane;
-      const bool act = ci < NC;
-      const uint32_t li = cur.li, cstart = cur.cstart, u = cur.u, m = cur.m;
-      const uint32_t cw = ci - cstart;
-      const uint32_t p0 = cw * 16u;
-      const uint32_t w[4] = {cur.v.x, cur.v.y, cur.v.z, cur.v.w};
-      const int b_lo = (cw == 0) ? 8 : 0;
-      const int b_hi = act ? (int)min(16u, u - p0) : 0;
-      LaneCodes lc;
-      lane_codes<true>(w, b_lo, b_hi, lc);
-      bad |= lc.bad;
-      // the partial code left by the previous chunk of the same leaf
-      const uint32_t prev_li = __shfl_up_sync(FULL, li, 1);
-      uint32_t pv = __shfl_up_sync(FULL, lc.tail, 1);
-      uint32_t ps = __shfl_up_sync(FULL, lc.tail_sh, 1);
-      if (lane == 0 || prev_li != li) {
-        if (lane == 0 && cont_li == li && cw > 0) { pv = cont_val; ps = cont_sh; }
-        else { pv = 0; ps = 0; }
-      }
-      const uint32_t term = lc.term;
-      uint32_t D = 0;
-      const uint32_t W = lc.W;
-      if (term) {
-        if (ps / 7u + lc.first_len > 4u) bad = true;
-        D = lc.D - lc.first_own + pv + (lc.first_own << ps);
-      }
-      // codes of this leaf in earlier chunks (segmented scan)
-      const uint32_t c = __popc(term);
-      const uint32_t incl = warp_incl_scan(c);
-      const uint32_t excl = incl - c;
-      const bool started_before = cstart < g0;
-      const uint32_t seg_lane = started_before ? 0u : cstart - g0;
-      const uint32_t B = excl - __shfl_sync(FULL, excl, seg_lane & 31u) +
-                         (started_before ? cont_cnt : 0u);
-      if (act) {
-        uint64_t contrib = (uint64_t)(m - 1u - B) * D - W;
-        if (cw == 0) contrib += (uint64_t)m * ((uint64_t)w[0] | ((uint64_t)w[1] << 32));
-        wacc += contrib;
-      }
-      cont_li = __shfl_sync(FULL, li, 31);
-      cont_cnt = __shfl_sync(FULL, B + c, 31);
-      cont_val = __shfl_sync(FULL, lc.tail, 31);
-      cont_sh = __shfl_sync(FULL, lc.tail_sh, 31);
-      cur = nxt;
-    }
-    if (__any_sync(FULL, bad)) {
-      const uint64_t je = min(w0 + 32, j1);
-      for (uint64_t q = w0; q < je; q++)
-        warp_decode(data + q * LB, min(__ldg(used + q), LB), [&](uint32_t, uint64_t val) { acc += val; });
-    } else {
-      acc += wacc;
+#pragma unroll
+      for (int q = 0; q < 4; q++) acc += v[q].x * (lim[q] >= 8) + v[q].y * (lim[q] >= 16);
     }
   }
 }

@@ -129,7 +129,8 @@ struct Scratch {
   Buf partials_q;         // scan partials of the query path, which may run
                           // on another stream while an update sorts
   Buf q_first, q_items, q_off; // range queries
-  Buf q_lo, q_hi, q_rank;       // map_range_length: rank bounds, leaf-count prefix
+  Buf q_lo, q_hi, q_rank;       // rank-space queries: rank bounds, leaf-count prefix
+  Buf q_pre, q_tiles;           // range queries: reductions before each leaf, and each tile
   Buf stage;              // padded batch of a graph-launched update
   Buf fh;                 // head fix-up: per-tile summaries
 };
@@ -288,6 +289,12 @@ int run_range_reduce(const cpma* h, const uint64_t* lo, const uint64_t* hi, uint
                      cudaStream_t st);
 int run_range_noalloc(const cpma* h, const uint64_t* lo, const uint64_t* hi, uint64_t q,
                       uint64_t* sum, uint64_t* count, cudaStream_t st);
+
+// The buffers of the range queries' prefix over the leaves, for L leaves (the
+// queries run without them when they cannot be had), and giving them back:
+// true when there was something to give (the device is then idle).
+int reserve_leaf_prefix(cpma* h, uint64_t L);
+bool release_leaf_prefix(cpma* h);
 
 int check_cuda(cudaError_t e);
 int sync_status(cpma* h, cudaStream_t st);

@@ -2,27 +2,30 @@
 //  has (Sec. 5 "Point queries"): binary search on the uncompressed heads, then
 //    one warp-cooperative pass over the leaf.
 //  range_map (Sec. 3: a search for the first element, then a scan to the end
-//    of the range) with f = (sum mod 2^64, count): every query is routed to
-//    its first and last leaf; the (query, leaf) pairs of all queries are
-//    numbered by a prefix sum and split into equal contiguous shares, one per
-//    warp of a persistent grid, so long and short ranges balance.  Leaves
-//    strictly inside a range need no filter.  A warp keeps per-lane partial
-//    sums while it stays on one query and adds them atomically when it
-//    leaves it (addition mod 2^64 is associative, so the order is free).
+//    of the range) with f = (sum mod 2^64, count).  A query covers parts of its
+//    first and last leaf and all of the leaves between them.  The parts are
+//    decoded one thread per leaf (k_range_ends).  The leaves between are
+//    either walked -- numbered over all queries by a prefix sum, one leaf per
+//    lane of equal shares -- or, when the queries together cover more leaves
+//    than the set has, every leaf is reduced once, those reductions become a
+//    prefix over the leaves, and a query takes the difference at its two ends
+//    (k_leaf_prefix, k_tile_scan, k_range_inner): each leaf is then decoded
+//    once however often the queries overlap.
 //  sum (App. A sum()): every leaf once.
 //  map_range_length (App. A: f on at most `length` elements from the first
-//    key >= start): a prefix sum of the leaves' element counts turns each
-//    query into a range of global ranks [r0, r1); the same load-balanced
-//    walk then sums whole leaves inside it and filters the two end leaves by
-//    rank instead of by key.
+//    key >= start): a prefix sum of the leaves' element counts gives the leaf
+//    of the last element; the rest is as for range_map.
 //  range_reduce (Sec. 3 range_map with other functions): min, max, xor or
 //    sum of the keys of [lo, hi) whose masked bits match a value, with the
-//    count of those keys; every covered leaf is decoded.
+//    count of those keys, as for range_map (the smallest match of a run of
+//    leaves is the first one after its start, the keys being in order).
+//  The uncompressed PMA's cells (codec 1) keep a warp per leaf.
 #include <algorithm>
 #include <mutex>
 
 #include "dev_common.cuh"
 #include "internal.h"
+#include "leaf_walk.cuh"
 
 using namespace cpmadev;
 
@@ -160,9 +163,9 @@ struct RangeArgs {
   uint64_t* count;
   ull* prof;  // profiling: leaf bytes scanned (nullable)
   const uint64_t* P = nullptr;  // rank mode: elements before each leaf (L + 1)
-  int raw = 0;                  // leaves hold 8-byte cells (codec 1)
 };
 
+// ---- the uncompressed PMA's cells (codec 1): a warp per (query, leaf) item ----
 __global__ void __launch_bounds__(kT) k_range_prep(const uint64_t* __restrict__ lo,
                                                    const uint64_t* __restrict__ hi, uint64_t q,
                                                    const uint64_t* __restrict__ heads, uint64_t L,
@@ -190,11 +193,11 @@ __global__ void __launch_bounds__(kT) k_range_prep(const uint64_t* __restrict__ 
 __device__ __forceinline__ uint64_t rank_of(uint64_t x, const uint64_t* __restrict__ heads,
                                             const uint8_t* __restrict__ data,
                                             const uint32_t* __restrict__ used, uint64_t L,
-                                            uint32_t LB, const uint64_t* __restrict__ P, int raw) {
+                                            uint32_t LB, const uint64_t* __restrict__ P) {
   const uint64_t j = route_leaf(heads, L, x);
   uint32_t below = 0;
   warp_decode(data + j * LB, min(used[j], LB), [&](uint32_t, uint64_t v) { below += v < x; },
-              raw);
+              true);
   return P[j] + warp_sum(below);
 }
 
@@ -214,15 +217,15 @@ __global__ void __launch_bounds__(kT) k_rank_prep(const uint64_t* __restrict__ A
                                                   uint64_t* __restrict__ first,
                                                   uint64_t* __restrict__ items,
                                                   uint64_t* __restrict__ sum,
-                                                  uint64_t* __restrict__ count, int raw) {
+                                                  uint64_t* __restrict__ count) {
   const unsigned lane = lane_id();
   const uint64_t gw = gtid() >> 5, nw = gstride() >> 5;
   const uint64_t n = P[L];
   for (uint64_t i = gw; i < q; i += nw) {
     const uint64_t a = A[i], b = B[i];
-    const uint64_t r0 = rank_of(a, heads, data, used, L, LB, P, raw);
+    const uint64_t r0 = rank_of(a, heads, data, used, L, LB, P);
     uint64_t r1;
-    if constexpr (KEYS) r1 = a < b ? rank_of(b, heads, data, used, L, LB, P, raw) : r0;
+    if constexpr (KEYS) r1 = a < b ? rank_of(b, heads, data, used, L, LB, P) : r0;
     else r1 = (b >= n - r0) ? n : r0 + b;
     uint64_t f = 0, it = 0;
     if (r1 > r0) {
@@ -256,7 +259,6 @@ struct ExtractArgs {
   uint32_t LB;
   uint64_t* out;
   uint64_t cap;
-  int raw;
 };
 
 __global__ void __launch_bounds__(kT) k_extract(ExtractArgs a) {
@@ -272,7 +274,7 @@ __global__ void __launch_bounds__(kT) k_extract(ExtractArgs a) {
     warp_decode(a.data + j * a.LB, min(a.used[j], a.LB), [&](uint32_t idx, uint64_t v) {
       const uint64_t r = base + idx;
       if (r >= r0 && r < r1 && o + (r - r0) < a.cap) a.out[o + (r - r0)] = v;
-    }, a.raw);
+    }, true);
   }
 }
 
@@ -296,84 +298,8 @@ __device__ __forceinline__ void op_atomic(uint64_t* p, uint64_t v) {
   else atomicXor((ull*)p, (ull)v);
 }
 
-// Thread-per-leaf reduction of a byte-code leaf: every element v with
-// (v & mask) == value is reduced into (r, c), the running value kept as in
-// thread_leaf_sum; bytes past u are no terminators here (a repeated value
-// would count twice), and a leaf with a code over 4 bytes is reduced again
-// exactly.
-template <int OP, bool FIRST>
-__device__ __forceinline__ void leaf_reduce_chunk(const uint32_t (&w)[4], uint32_t valid,
-                                                  uint64_t mask, uint64_t value, uint64_t& val,
-                                                  uint64_t& r, uint64_t& c, uint32_t& acc,
-                                                  uint32_t& pw, uint32_t& pwmax) {
-#pragma unroll
-  for (int b = FIRST ? 8 : 0; b < 16; b++) {
-    const uint32_t wb = w[b >> 2];
-    const bool in = (valid >> b) & 1u;  // bytes past u: neither codes nor terminators
-    acc += (__byte_perm(wb, 0u, 0x4440u + (uint32_t)(b & 3)) & 0x7Fu) * pw;
-    const bool term = in && (wb & (0x80u << (8 * (b & 3)))) == 0u;
-    pwmax = (in && pw > pwmax) ? pw : pwmax;
-    val += term ? (uint64_t)acc : 0ull;
-    const bool hit = term && (val & mask) == value;
-    r = hit ? op_apply<OP>(r, val) : r;
-    c += hit ? 1u : 0u;
-    acc = (term || !in) ? 0u : acc;
-    pw = (term || !in) ? 1u : pw << 7;
-  }
-}
-
-template <int OP>
-__device__ __forceinline__ void thread_leaf_reduce(const uint8_t* __restrict__ leafp, uint32_t u,
-                                                   uint64_t mask, uint64_t value, uint64_t& r,
-                                                   uint64_t& c) {
-  uint4 v = *reinterpret_cast<const uint4*>(leafp);
-  uint4 v2 = u > 16u ? *reinterpret_cast<const uint4*>(leafp + 16) : make_uint4(0u, 0u, 0u, 0u);
-  uint64_t val = (uint64_t)v.x | ((uint64_t)v.y << 32);
-  uint64_t lr = op_identity<OP>(), lc = 0;
-  if ((val & mask) == value) { lr = op_apply<OP>(lr, val); lc++; }
-  uint32_t acc = 0, pw = 1, pwmax = 0;
-  for (uint32_t p0 = 0; p0 < u; p0 += 32) {
-    if (p0) {
-      v = *reinterpret_cast<const uint4*>(leafp + p0);
-      v2 = p0 + 16u < u ? *reinterpret_cast<const uint4*>(leafp + p0 + 16) : make_uint4(0u, 0u, 0u, 0u);
-    }
-    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-    const uint32_t va = p0 + 16u <= u ? 0xFFFFu : (1u << (u - p0)) - 1u;
-    if (p0) leaf_reduce_chunk<OP, false>(w, va, mask, value, val, lr, lc, acc, pw, pwmax);
-    else leaf_reduce_chunk<OP, true>(w, va, mask, value, val, lr, lc, acc, pw, pwmax);
-    if (p0 + 16u < u) {
-      const uint32_t w2[4] = {v2.x, v2.y, v2.z, v2.w};
-      const uint32_t vb = p0 + 32u <= u ? 0xFFFFu : (1u << (u - p0 - 16u)) - 1u;
-      leaf_reduce_chunk<OP, false>(w2, vb, mask, value, val, lr, lc, acc, pw, pwmax);
-    }
-  }
-  if (pwmax >= (1u << 28)) {  // a long code: exact 64-bit decode
-    val = *reinterpret_cast<const uint64_t*>(leafp);
-    lr = op_identity<OP>();
-    lc = 0;
-    if ((val & mask) == value) { lr = op_apply<OP>(lr, val); lc++; }
-    uint64_t a64 = 0;
-    uint32_t sh = 0;
-    for (uint32_t p = 8; p < u; p++) {
-      const uint32_t b = leafp[p];
-      if (sh < 64) a64 |= (uint64_t)(b & 0x7Fu) << sh;
-      if (b & 0x80u) {
-        sh += 7;
-      } else {
-        val += a64;
-        if ((val & mask) == value) { lr = op_apply<OP>(lr, val); lc++; }
-        a64 = 0;
-        sh = 0;
-      }
-    }
-  }
-  r = op_apply<OP>(r, lr);
-  c += lc;
-}
-
-// Same load-balanced (query, leaf) walk as k_range: the end leaves of a
-// query are decoded by the warp and filtered by range and mask, the leaves
-// strictly inside are reduced one per thread (byte codes).
+// Same load-balanced (query, leaf) walk as k_range: every leaf is read by the
+// warp and filtered by range and mask.
 template <int OP>
 __global__ void __launch_bounds__(kT) k_range_reduce(RangeArgs a, uint64_t mask,
                                                      uint64_t value) {
@@ -401,21 +327,10 @@ __global__ void __launch_bounds__(kT) k_range_reduce(RangeArgs a, uint64_t mask,
       qend = a.off[qi + 1];
       lo = a.lo[qi]; hi = a.hi[qi]; fl = a.first[qi]; qoff = a.off[qi];
     }
-    const uint64_t li = g - qoff, n = qend - qoff;
-    if (!a.raw && li > 0 && li + 1 < n) {
-      // leaves strictly inside the range (byte codes): one leaf per lane
-      const uint64_t stop = min(g1, qend - 1);
-      for (uint64_t j = fl + li + lane; j < fl + (stop - qoff); j += 32) {
-        const uint32_t u = min(a.used[j], a.LB);
-        if (u) thread_leaf_reduce<OP>(a.data + j * a.LB, u, mask, value, r, c);
-      }
-      g = stop;
-      continue;
-    }
-    const uint64_t j = fl + li;
+    const uint64_t j = fl + (g - qoff);
     warp_decode(a.data + j * a.LB, min(a.used[j], a.LB), [&](uint32_t, uint64_t v) {
       if (v >= lo && v < hi && (v & mask) == value) { r = op_apply<OP>(r, v); c++; }
-    }, a.raw);
+    }, true);
     g++;
   }
 #pragma unroll
@@ -462,11 +377,7 @@ __global__ void __launch_bounds__(kT) k_range(RangeArgs a) {
       // leaves strictly inside the range: no filter, chunked span sum
       const uint64_t stop = min(g1, qend - 1);  // exclusive, global item index
       uint64_t cc = 0;
-      if (a.raw)
-        warp_span_sum(a.data, a.used, a.cnt, a.LB, fl + li, fl + (stop - qoff), s, cc, nbytes,
-                      a.raw);
-      else  // byte codes: one leaf per lane
-        thread_span_sum(a.data, a.used, a.cnt, a.LB, fl + li, fl + (stop - qoff), s, cc, nbytes);
+      warp_span_sum(a.data, a.used, a.cnt, a.LB, fl + li, fl + (stop - qoff), s, cc, nbytes);
       if (lane == 0) c += warp_sum(cc); else warp_sum(cc);
       g = stop;
       continue;
@@ -478,11 +389,11 @@ __global__ void __launch_bounds__(kT) k_range(RangeArgs a) {
       const uint64_t r = a.P[j];
       warp_decode(a.data + j * a.LB, u, [&](uint32_t idx, uint64_t v) {
         if (r + idx >= lo && r + idx < hi) { s += v; c++; }
-      }, a.raw);
+      }, true);
     } else {
       warp_decode(a.data + j * a.LB, u, [&](uint32_t, uint64_t v) {
         if (v >= lo && v < hi) { s += v; c++; }
-      }, a.raw);
+      }, true);
     }
     g++;
   }
@@ -496,8 +407,525 @@ __global__ void __launch_bounds__(kT) k_range(RangeArgs a) {
   if (a.prof && lane == 0 && nbytes) atomicAdd(a.prof, nbytes);
 }
 
+// ---- byte codes (codec 0): a thread per leaf ----
+
+// The leaf arrays of one set.
+struct Leaves {
+  const uint8_t* data;
+  const uint32_t* used;
+  const uint32_t* cnt;
+  const uint64_t* heads;
+  uint64_t L;
+  uint32_t LB;
+};
+
+// Last index i in [a, n) with p[i] <= x, p sorted; a when p[a] > x too.  The
+// next few entries are tried first: most ranges end in their first leaf or
+// the one after it.
+__device__ __forceinline__ uint64_t last_from(const uint64_t* __restrict__ p, uint64_t a, uint64_t n,
+                                              uint64_t x) {
+  uint64_t step = 1;
+#pragma unroll 1
+  for (int i = 0; i < 3; i++) {
+    if (a + step >= n) break;
+    if (__ldg(p + a + step) > x) {
+      n = a + step;
+      break;
+    }
+    a += step;
+    step <<= 1;
+  }
+  if (n - a <= 1) return a;
+  const uint64_t c = upper_count(p + a, n - a, x);
+  return c ? a + c - 1 : a;
+}
+
+// What a range query reduces: PLAIN is (sum, count) without a filter, whose
+// whole groups and leaf counts need no look at single elements.
+template <int OP, bool PLAIN>
+struct Reduce {
+  uint64_t mask, value;
+  __device__ __forceinline__ void leaf(const uint8_t* leafp, uint32_t u, const uint32_t* cnt,
+                                       uint64_t& r, uint64_t& c) const {
+    if constexpr (PLAIN) {
+      const uint32_t m = *cnt;
+      r += leafwalk::leaf_sum(leafp, u, m);
+      c += m;
+    } else {
+      leafwalk::leaf_visit(leafp, u, [&](uint64_t v) {
+        if ((v & mask) == value) { r = op_apply<OP>(r, v); c++; }
+      });
+    }
+  }
+  __device__ __forceinline__ void part(const uint8_t* leafp, uint32_t u, uint64_t lo, uint64_t hi,
+                                       uint64_t& r, uint64_t& c) const {
+    if constexpr (PLAIN) {
+      leafwalk::leaf_range_sum(leafp, u, lo, hi, r, c);
+    } else {
+      leafwalk::leaf_visit(leafp, u, [&](uint64_t v) {
+        if (v >= lo && v < hi && (v & mask) == value) { r = op_apply<OP>(r, v); c++; }
+      });
+    }
+  }
+};
+
+// A range query's first and last leaf: thread i routes query i and reduces
+// its part of the first leaf; the queries that reach another leaf put their
+// last one on the block's list, which the first threads then take, so a warp
+// runs the second decode only when 32 of them have one.  Writes the ends'
+// reduction and count and the leaves strictly between (first, items).
+template <int OP, bool PLAIN>
+__global__ void __launch_bounds__(kT) k_range_ends(const uint64_t* __restrict__ lo,
+                                                   const uint64_t* __restrict__ hi, uint64_t q,
+                                                   Leaves t, Reduce<OP, PLAIN> f,
+                                                   uint64_t* __restrict__ first,
+                                                   uint64_t* __restrict__ items,
+                                                   uint64_t* __restrict__ out,
+                                                   uint64_t* __restrict__ count, ull* prof) {
+  __shared__ uint64_t s_hi[kT], s_r[kT], s_c[kT];
+  __shared__ uint32_t s_leaf[kT], s_q[kT];
+  __shared__ uint32_t s_n;
+  ull nbytes = 0;
+  const uint64_t T = blockDim.x;
+  for (uint64_t base = blockIdx.x * T; base < q; base += gridDim.x * T) {
+    const uint64_t i = base + threadIdx.x;
+    if (threadIdx.x == 0) s_n = 0;
+    __syncthreads();
+    uint64_t r = op_identity<OP>(), c = 0, fl = 0, ll = 0, a = 0, b = 0;
+    if (i < q) { a = lo[i]; b = hi[i]; }
+    if (a < b) {
+      fl = route_leaf(t.heads, t.L, a);
+      ll = last_from(t.heads, fl, t.L, b - 1);
+    }
+    s_c[threadIdx.x] = 0;
+    if (ll > fl) {
+      const uint32_t slot = atomicAdd(&s_n, 1u);
+      s_q[slot] = threadIdx.x;
+      s_leaf[threadIdx.x] = (uint32_t)ll;
+      s_hi[threadIdx.x] = b;
+    }
+    if (a < b) {
+      const uint32_t u = min(t.used[fl], t.LB);
+      nbytes += u;
+      if (u) f.part(t.data + fl * t.LB, u, a, b, r, c);
+    }
+    __syncthreads();
+    if (threadIdx.x < s_n) {
+      const uint32_t w = s_q[threadIdx.x], j = s_leaf[w];
+      const uint32_t u = min(t.used[j], t.LB);
+      uint64_t r2 = op_identity<OP>(), c2 = 0;
+      nbytes += u;
+      if (u) f.part(t.data + (uint64_t)j * t.LB, u, 0, s_hi[w], r2, c2);
+      s_r[w] = r2;
+      s_c[w] = c2;
+    }
+    __syncthreads();
+    if (s_c[threadIdx.x]) {
+      r = op_apply<OP>(r, s_r[threadIdx.x]);
+      c += s_c[threadIdx.x];
+    }
+    if (i < q) {
+      first[i] = fl + 1;
+      items[i] = ll > fl ? ll - fl - 1 : 0;
+      out[i] = r;
+      count[i] = c;
+    }
+    __syncthreads();
+  }
+  nbytes = warp_sum(nbytes);
+  if (prof && lane_id() == 0 && nbytes) atomicAdd(prof, nbytes);
+}
+
+// The same for map_range_length: thread i takes the first length[i] elements
+// from start[i] on as far as its first leaf holds them; P (elements before
+// each leaf) then names the leaf of the last one and how many it gives.
+__global__ void __launch_bounds__(kT) k_length_ends(const uint64_t* __restrict__ start,
+                                                    const uint64_t* __restrict__ length, uint64_t q,
+                                                    Leaves t, const uint64_t* __restrict__ P,
+                                                    uint64_t* __restrict__ first,
+                                                    uint64_t* __restrict__ items,
+                                                    uint64_t* __restrict__ sum,
+                                                    uint64_t* __restrict__ count, ull* prof) {
+  pdl_wait();
+  pdl_launch();
+  __shared__ uint64_t s_s[kT];
+  __shared__ uint32_t s_leaf[kT], s_q[kT], s_k[kT];
+  __shared__ uint32_t s_n;
+  ull nbytes = 0;
+  const uint64_t n = P[t.L];
+  const uint64_t T = blockDim.x;
+  for (uint64_t base = blockIdx.x * T; base < q; base += gridDim.x * T) {
+    const uint64_t i = base + threadIdx.x;
+    if (threadIdx.x == 0) s_n = 0;
+    __syncthreads();
+    uint64_t s = 0, c = 0, fl = 0, ll = 0, len = 0;
+    if (i < q) len = length[i];
+    s_s[threadIdx.x] = 0;
+    if (len) {
+      const uint64_t x = start[i];
+      fl = ll = route_leaf(t.heads, t.L, x);
+      const uint32_t u = min(t.used[fl], t.LB);
+      nbytes += u;
+      uint32_t below = 0, taken = 0;
+      if (u) leafwalk::leaf_take_sum(t.data + fl * t.LB, u, x, len, below, taken, s);
+      c = taken;
+      const uint64_t r0 = P[fl] + below;              // rank of the first key >= x
+      const uint64_t r1 = len >= n - r0 ? n : r0 + len;
+      if (r1 > r0 + taken) {                          // more in later leaves
+        ll = last_from(P, fl, t.L + 1, r1 - 1);
+        const uint32_t k = (uint32_t)(r1 - P[ll]);
+        const uint32_t slot = atomicAdd(&s_n, 1u);
+        s_q[slot] = threadIdx.x;
+        s_leaf[threadIdx.x] = (uint32_t)ll;
+        s_k[threadIdx.x] = k;
+        c += k;
+      }
+    }
+    __syncthreads();
+    if (threadIdx.x < s_n) {
+      const uint32_t w = s_q[threadIdx.x], j = s_leaf[w];
+      const uint32_t u = min(t.used[j], t.LB);
+      uint32_t below, taken;
+      uint64_t s2 = 0;
+      nbytes += u;
+      if (u) leafwalk::leaf_take_sum(t.data + (uint64_t)j * t.LB, u, 0, s_k[w], below, taken, s2);
+      s_s[w] = s2;
+    }
+    __syncthreads();
+    if (i < q) {
+      first[i] = fl + 1;
+      items[i] = ll > fl ? ll - fl - 1 : 0;
+      sum[i] = s + s_s[threadIdx.x];
+      count[i] = c;
+    }
+    __syncthreads();
+  }
+  nbytes = warp_sum(nbytes);
+  if (prof && lane_id() == 0 && nbytes) atomicAdd(prof, nbytes);
+}
+
+// Reductions before (min: from) each leaf, in two levels: val / cnt inside
+// the tile of kT leaves, tval / tcnt over the tiles.  Unused (null) when its
+// memory cannot be had; taken when the queries' inner leaves number more than
+// `most`.
+struct LeafPrefix {
+  uint64_t* val = nullptr;   // per leaf
+  uint32_t* cnt = nullptr;   // per leaf: matches before it in its tile
+  uint64_t* tval = nullptr;  // per tile
+  uint64_t* tcnt = nullptr;
+  uint64_t most = ~0ull;
+};
+
+// Scan of one value per thread of a block of kT by op: exclusive from the
+// front (REV false) or inclusive from the back; total = all of them.
+template <int OP, bool REV>
+__device__ __forceinline__ uint64_t block_scan_op(uint64_t v, uint64_t* ws, uint64_t* total) {
+  const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
+  uint64_t x = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint64_t y = REV ? __shfl_down_sync(FULL, x, o) : __shfl_up_sync(FULL, x, o);
+    if (REV ? lane + o < 32u : lane >= (unsigned)o) x = op_apply<OP>(x, y);
+  }
+  if (lane == (REV ? 0u : 31u)) ws[warp] = x;
+  __syncthreads();
+  uint64_t carry = op_identity<OP>(), all = op_identity<OP>();
+#pragma unroll
+  for (unsigned w = 0; w < kT / 32; w++) {
+    const uint64_t y = ws[w];
+    all = op_apply<OP>(all, y);
+    if (REV ? w > warp : w < warp) carry = op_apply<OP>(carry, y);
+  }
+  *total = all;
+  __syncthreads();  // ws is reused
+  if (REV) return op_apply<OP>(carry, x);
+  uint64_t e = __shfl_up_sync(FULL, x, 1);
+  if (lane == 0) e = op_identity<OP>();
+  return op_apply<OP>(carry, e);
+}
+
 constexpr uint32_t kSumShift = 4;      // sort key of a leaf: used bytes / 16
 constexpr uint32_t kSumBuckets = 128;  // enough for 2048-byte leaves (a multiple of 32)
+
+// Order of the nt <= kT leaves of a tile by used bytes (a counting sort in
+// shared memory), so the 32 leaves a warp decodes side by side take about the
+// same number of steps: order[i] = the tile's leaf that thread i takes.
+__device__ __forceinline__ void order_tile(uint32_t u, uint32_t nt, uint32_t* hist,
+                                           uint32_t* order) {
+  for (uint32_t i = threadIdx.x; i < kSumBuckets; i += kT) hist[i] = 0;
+  __syncthreads();
+  const uint32_t bkt = min(u >> kSumShift, kSumBuckets - 1);
+  const uint32_t slot = threadIdx.x < nt ? atomicAdd(&hist[bkt], 1u) : 0u;
+  __syncthreads();
+  if (threadIdx.x < 32) {  // exclusive scan of the bucket counts
+    uint32_t run = 0;
+    for (uint32_t b = 0; b < kSumBuckets; b += 32) {
+      const uint32_t v = hist[b + threadIdx.x];
+      const uint32_t inc = warp_incl_scan(v);
+      hist[b + threadIdx.x] = run + inc - v;
+      run += __shfl_sync(FULL, inc, 31);
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < nt) order[hist[bkt] + slot] = threadIdx.x;
+  __syncthreads();
+}
+
+// Every leaf reduced once, scanned inside tiles of kT leaves (when the
+// queries cover more than p.most leaves; otherwise nothing).
+template <int OP, bool PLAIN>
+__global__ void __launch_bounds__(kT) k_leaf_prefix(Leaves t, Reduce<OP, PLAIN> f,
+                                                    const uint64_t* __restrict__ total,
+                                                    LeafPrefix p, ull* prof) {
+  __shared__ uint32_t s_hist[kSumBuckets], s_order[kT];
+  __shared__ uint64_t s_r[kT], s_ws[kT / 32];
+  __shared__ uint32_t s_c[kT];
+  pdl_wait();
+  pdl_launch();
+  if (*total <= p.most) return;
+  ull nbytes = 0;
+  const uint64_t nt = (t.L + kT - 1) / kT;
+  for (uint64_t tile = blockIdx.x; tile < nt; tile += gridDim.x) {
+    const uint64_t j0 = tile * kT, j = j0 + threadIdx.x;
+    const uint32_t n = (uint32_t)min((uint64_t)kT, t.L - j0);
+    order_tile(threadIdx.x < n ? min(t.used[j], t.LB) : 0u, n, s_hist, s_order);
+    s_r[threadIdx.x] = op_identity<OP>();
+    s_c[threadIdx.x] = 0;
+    __syncthreads();
+    if (threadIdx.x < n) {
+      const uint32_t o = s_order[threadIdx.x];
+      const uint32_t u = min(t.used[j0 + o], t.LB);
+      uint64_t r = op_identity<OP>(), c = 0;
+      if (u) {
+        f.leaf(t.data + (j0 + o) * t.LB, u, t.cnt + j0 + o, r, c);
+        nbytes += u;
+      }
+      s_r[o] = r;
+      s_c[o] = (uint32_t)c;
+    }
+    __syncthreads();
+    uint64_t all, call;
+    const uint64_t x = block_scan_op<OP, OP == CPMA_OP_MIN>(s_r[threadIdx.x], s_ws, &all);
+    const uint64_t c = block_scan_op<CPMA_OP_SUM, false>((uint64_t)s_c[threadIdx.x], s_ws, &call);
+    if (threadIdx.x < n) {
+      p.val[j] = x;
+      p.cnt[j] = (uint32_t)c;
+    }
+    if (threadIdx.x == 0) {
+      p.tval[tile] = all;
+      p.tcnt[tile] = call;
+    }
+  }
+  nbytes = warp_sum(nbytes);
+  if (prof && lane_id() == 0 && nbytes) atomicAdd(prof, nbytes);
+}
+
+// The tiles' reductions scanned in place by one block: exclusive from the
+// front (min: from the back).
+template <int OP>
+__global__ void __launch_bounds__(kT) k_tile_scan(const uint64_t* __restrict__ total, LeafPrefix p,
+                                                  uint64_t nt) {
+  __shared__ uint64_t s_ws[kT / 32];
+  pdl_wait();
+  pdl_launch();
+  if (*total <= p.most) return;
+  constexpr bool REV = OP == CPMA_OP_MIN;
+  // a contiguous run of tiles per thread: reduced, scanned over the block,
+  // rescanned
+  const uint64_t per = (nt + kT - 1) / kT;
+  const uint64_t b0 = min(nt, threadIdx.x * per), b1 = min(nt, b0 + per);
+  uint64_t r = op_identity<OP>(), c = 0;
+  for (uint64_t b = b0; b < b1; b++) {
+    r = op_apply<OP>(r, p.tval[b]);
+    c += p.tcnt[b];
+  }
+  uint64_t all;
+  uint64_t x;
+  if (REV) {  // exclusive from the back: the inclusive one of the next thread
+    const uint64_t inc = block_scan_op<OP, true>(r, s_ws, &all);
+    __shared__ uint64_t s_inc[kT + 1];
+    s_inc[threadIdx.x] = inc;
+    if (threadIdx.x == 0) s_inc[kT] = op_identity<OP>();
+    __syncthreads();
+    x = s_inc[threadIdx.x + 1];
+  } else {
+    x = block_scan_op<OP, false>(r, s_ws, &all);
+  }
+  uint64_t y = block_scan_op<CPMA_OP_SUM, false>(c, s_ws, &all);
+  for (uint64_t b = b0; b < b1; b++) {
+    const uint64_t v = p.tcnt[b];
+    p.tcnt[b] = y;
+    y += v;
+  }
+  if (REV) {
+    for (uint64_t b = b1; b-- > b0;) {
+      const uint64_t v = p.tval[b];
+      p.tval[b] = x;
+      x = op_apply<OP>(x, v);
+    }
+  } else {
+    for (uint64_t b = b0; b < b1; b++) {
+      const uint64_t v = p.tval[b];
+      p.tval[b] = x;
+      x = op_apply<OP>(x, v);
+    }
+  }
+}
+
+// The leaves strictly inside the ranges.  From the prefix: a thread per
+// query.  Otherwise the (query, leaf) items in equal contiguous shares per
+// warp, one leaf per lane: a lane keeps its partial while it stays on one
+// query and adds it atomically when it leaves it (the functions commute); a
+// warp whose lanes end on one query adds once.
+template <int OP, bool PLAIN>
+__global__ void __launch_bounds__(kT) k_range_inner(Leaves t, Reduce<OP, PLAIN> f, uint64_t q,
+                                                    const uint64_t* __restrict__ first,
+                                                    const uint64_t* __restrict__ off, LeafPrefix p,
+                                                    uint64_t* __restrict__ out,
+                                                    uint64_t* __restrict__ count, ull* prof) {
+  pdl_wait();
+  const uint64_t N = off[q];
+  if (N > p.most) {
+    for (uint64_t i = gtid(); i < q; i += gstride()) {
+      const uint64_t n = off[i + 1] - off[i];
+      if (!n) continue;
+      const uint64_t a = first[i], b = a + n;  // b: the query's last leaf
+      const uint64_t ca = p.tcnt[a / kT] + p.cnt[a], cb = p.tcnt[b / kT] + p.cnt[b];
+      if (ca == cb) continue;
+      uint64_t r;
+      if constexpr (OP == CPMA_OP_MIN) r = min(p.val[a], p.tval[a / kT]);
+      else if constexpr (OP == CPMA_OP_MAX) r = max(p.val[b], p.tval[b / kT]);
+      else if constexpr (OP == CPMA_OP_XOR)
+        r = (p.val[b] ^ p.tval[b / kT]) ^ (p.val[a] ^ p.tval[a / kT]);
+      else r = (p.val[b] + p.tval[b / kT]) - (p.val[a] + p.tval[a / kT]);
+      out[i] = op_apply<OP>(out[i], r);
+      count[i] += cb - ca;
+    }
+    return;
+  }
+  const unsigned lane = lane_id();
+  const uint64_t gw = gtid() >> 5, nw = gstride() >> 5;
+  const uint64_t g0 = N * gw / nw, g1 = N * (gw + 1) / nw;
+  if (g0 >= g1) return;
+  uint64_t qi = 0, qend = 0, qoff = 0, fl = 0;
+  uint64_t r = op_identity<OP>(), c = 0;
+  ull nbytes = 0;
+  auto flush = [&] {
+    if (c) {
+      op_atomic<OP>(&out[qi], r);
+      atomicAdd((ull*)&count[qi], (ull)c);
+    }
+    r = op_identity<OP>();
+    c = 0;
+  };
+  for (uint64_t g = g0 + lane; g < g1; g += 32) {
+    if (g >= qend) {
+      flush();
+      qi += upper_count(off + qi, q + 1 - qi, g) - 1;
+      qoff = off[qi];
+      qend = off[qi + 1];
+      fl = first[qi];
+    }
+    const uint64_t j = fl + (g - qoff);
+    const uint32_t u = min(t.used[j], t.LB);
+    nbytes += u;
+    if (u) f.leaf(t.data + j * t.LB, u, t.cnt + j, r, c);
+  }
+  const uint64_t q0 = __shfl_sync(FULL, qi, 0);
+  if (__all_sync(FULL, qi == q0 || c == 0)) {
+#pragma unroll
+    for (int o = 16; o; o >>= 1) r = op_apply<OP>(r, __shfl_xor_sync(FULL, r, o));
+    c = warp_sum(c);
+    if (lane == 0) flush();
+  } else {
+    flush();
+  }
+  nbytes = warp_sum(nbytes);
+  if (prof && lane == 0 && nbytes) atomicAdd(prof, nbytes);
+}
+
+// Ranks of both ends of the key ranges [A, B): two lanes per query, one end
+// each.  The leaves that hold the ranks come from P (elements before each
+// leaf), searched from the end's own leaf on.
+__global__ void __launch_bounds__(kT) k_rank_ends(const uint64_t* __restrict__ A,
+                                                  const uint64_t* __restrict__ B, uint64_t q,
+                                                  Leaves t, const uint64_t* __restrict__ P,
+                                                  uint64_t* __restrict__ r0o,
+                                                  uint64_t* __restrict__ r1o,
+                                                  uint64_t* __restrict__ first,
+                                                  uint64_t* __restrict__ items,
+                                                  uint64_t* __restrict__ count) {
+  pdl_wait();
+  pdl_launch();
+  // whole warps stay in the loop: both lanes of a query take part in it
+  for (uint64_t g = gtid() & ~31ull; g < 2 * q; g += gstride()) {
+    const uint64_t e = g + lane_id(), i = e >> 1;
+    uint64_t r = 0, j = 0;
+    if (i < q) {
+      const uint64_t x = (e & 1) ? B[i] : A[i];
+      j = route_leaf(t.heads, t.L, x);
+      const uint32_t u = min(t.used[j], t.LB);
+      r = P[j] + (u ? leafwalk::leaf_below(t.data + j * t.LB, u, x) : 0u);
+    }
+    const uint64_t r1 = __shfl_down_sync(FULL, r, 1);
+    if (i < q && !(e & 1)) {
+      uint64_t hi = A[i] < B[i] ? r1 : r, fl = 0, it = 0;
+      if (hi > r) {
+        fl = last_from(P, j, t.L + 1, r);
+        it = last_from(P, fl, t.L + 1, hi - 1) - fl + 1;
+      } else {
+        hi = r;
+      }
+      r0o[i] = r;
+      r1o[i] = hi;
+      first[i] = fl;
+      items[i] = it;
+      count[i] = hi - r;
+    }
+  }
+}
+
+// The keys of ranks [r0, r1) of every query, one (query, leaf) item per lane:
+// out[off + r - r0] = key of rank r (entries at or past cap are dropped).  A
+// lane stores its leaf's keys one after another; the eight bytes of
+// neighbouring keys meet in the L2's lines.
+__global__ void __launch_bounds__(kT) k_extract_leaf(ExtractArgs a) {
+  pdl_wait();
+  const uint64_t gw = gtid() >> 5, nw = gstride() >> 5;
+  const uint64_t N = a.item_off[a.q];
+  const uint64_t g0 = N * gw / nw, g1 = N * (gw + 1) / nw;
+  uint64_t qi = 0, qend = 0;
+  for (uint64_t g = g0 + lane_id(); g < g1; g += 32) {
+    if (g >= qend) {
+      qi += upper_count(a.item_off + qi, a.q + 1 - qi, g) - 1;
+      qend = a.item_off[qi + 1];
+    }
+    const uint64_t j = a.first[qi] + (g - a.item_off[qi]);
+    const uint64_t r0 = a.r0[qi], r1 = a.r1[qi], base = a.P[j], o = a.out_off[qi];
+    const uint32_t u = min(a.used[j], a.LB);
+    if (!u) continue;
+    if (a.cap <= o) continue;
+    // element idx of the leaf goes to dst[idx] for skip <= idx < stop
+    const uint64_t room = a.cap - o;
+    uint64_t stop = r1 - base;
+    uint32_t skip = 0;
+    if (r0 >= base) {
+      skip = (uint32_t)(r0 - base);
+      if (stop - skip > room) stop = skip + room;
+    } else {
+      const uint64_t before = base - r0;  // the query's keys in earlier leaves
+      if (room <= before) continue;
+      stop = min(stop, room - before);
+    }
+    uint64_t* dst = a.out + (int64_t)(o + base - r0);
+    uint32_t idx = 0;
+    const uint32_t st = (uint32_t)min(stop, (uint64_t)0xFFFFFFFFu);
+    leafwalk::leaf_visit(a.data + j * a.LB, u, [&](uint64_t v) {
+      if (idx >= skip && idx < st) dst[idx] = v;
+      idx++;
+    });
+  }
+}
 
 __global__ void __launch_bounds__(kT) k_sum(const uint8_t* __restrict__ data,
                                             const uint32_t* __restrict__ used,
@@ -510,42 +938,23 @@ __global__ void __launch_bounds__(kT) k_sum(const uint8_t* __restrict__ data,
   uint64_t s = 0, c = 0;
   ull nbytes = 0;
   if (raw) {
-    warp_span_sum(data, used, cnt, LB, j0, j1, s, c, nbytes, raw);
+    warp_span_sum(data, used, cnt, LB, j0, j1, s, c, nbytes);
   } else {
-    // The block's leaves in tiles of kT, each ordered by used bytes (a
-    // counting sort in shared memory), so the 32 leaves a warp decodes side
-    // by side take about the same number of steps.
+    // the block's leaves in tiles of kT, each ordered by used bytes
     __shared__ uint32_t s_hist[kSumBuckets];
     __shared__ uint32_t s_order[kT];
     const uint64_t b0 = L * blockIdx.x / gridDim.x, b1 = L * (blockIdx.x + 1) / gridDim.x;
     for (uint64_t t0 = b0; t0 < b1; t0 += kT) {
-      for (uint32_t i = threadIdx.x; i < kSumBuckets; i += kT) s_hist[i] = 0;
-      __syncthreads();
-      const uint64_t j = t0 + threadIdx.x;
-      const uint32_t u = j < b1 ? min(used[j], LB) : 0u;
-      const uint32_t bkt = min(u >> kSumShift, kSumBuckets - 1);
-      const uint32_t slot = j < b1 ? atomicAdd(&s_hist[bkt], 1u) : 0u;
-      __syncthreads();
-      if (threadIdx.x < 32) {  // exclusive scan of the bucket counts
-        uint32_t run = 0;
-        for (uint32_t b = 0; b < kSumBuckets; b += 32) {
-          const uint32_t v = s_hist[b + lane];
-          const uint32_t inc = warp_incl_scan(v);
-          s_hist[b + lane] = run + inc - v;
-          run += __shfl_sync(FULL, inc, 31);
-        }
-      }
-      __syncthreads();
-      if (j < b1) s_order[s_hist[bkt] + slot] = threadIdx.x;
-      __syncthreads();
       const uint32_t nt = (uint32_t)min((uint64_t)kT, b1 - t0);
+      order_tile(threadIdx.x < nt ? min(used[t0 + threadIdx.x], LB) : 0u, nt, s_hist, s_order);
       if (threadIdx.x < nt) {
         const uint64_t jj = t0 + s_order[threadIdx.x];
         const uint32_t uu = min(used[jj], LB);
         nbytes += 8;  // its used and element counts
         if (uu) {
-          s += thread_leaf_sum(data + jj * LB, uu);
-          c += cnt[jj];
+          const uint32_t m = cnt[jj];
+          s += leafwalk::leaf_sum(data + jj * LB, uu, m);
+          c += m;
           nbytes += uu;
         }
       }
@@ -612,43 +1021,189 @@ int run_has(const cpma* h, const uint64_t* d_keys, uint64_t q, uint8_t* d_out, c
   return check_cuda(cudaGetLastError());
 }
 
-int run_range(const cpma* h, const uint64_t* lo, const uint64_t* hi, uint64_t q, uint64_t* sum,
-              uint64_t* count, cudaStream_t st) {
-  if (q == 0) return CPMA_OK;
-  cpma* hm = const_cast<cpma*>(h);
-  CPMA_TRY(ensure(hm, hm->s.q_first, q * 8));
-  CPMA_TRY(ensure(hm, hm->s.q_items, q * 8));
-  CPMA_TRY(ensure(hm, hm->s.q_off, (q + 1) * 8));
-  uint64_t* first = (uint64_t*)hm->s.q_first.p;
-  uint64_t* items = (uint64_t*)hm->s.q_items.p;
-  uint64_t* off = (uint64_t*)hm->s.q_off.p;
-  const int g1 = (int)std::max<uint64_t>(
-      1, std::min<uint64_t>((q + kT - 1) / kT, (uint64_t)h->num_sms * 8));
-  prof_begin(h, PH_RANGE_PREP, st);
-  prof_add_bytes(h, PH_RANGE_PREP, 72ull * q);  // lo, hi in; first, items, sums out; scan
-  k_range_prep<<<g1, kT, 0, st>>>(lo, hi, q, h->heads, h->L, first, items, sum, count);
+namespace {
+
+Leaves leaves_of(const cpma* h) {
+  return Leaves{h->data, h->used, h->cnt, h->heads, h->L, h->cfg.leaf_bytes};
+}
+
+// Blocks of a grid of one thread per query: small batches spread over more
+// SMs in blocks of two warps.
+int query_block(const cpma* h, uint64_t q) { return q < (uint64_t)h->num_sms * kT ? 64 : kT; }
+int query_grid(const cpma* h, uint64_t q, int block, uint64_t per_sm) {
+  return (int)std::max<uint64_t>(
+      1, std::min<uint64_t>((q + block - 1) / block, (uint64_t)h->num_sms * per_sm));
+}
+
+// Grows a query buffer; the leaf prefix, which the queries can do without, is
+// given back when there is no room for it.
+int ensure_query(cpma* h, Buf& b, size_t bytes) {
+  int rc = ensure(h, b, bytes);
+  if (rc == CPMA_ENOMEM && release_leaf_prefix(h)) rc = ensure(h, b, bytes);
+  return rc;
+}
+
+// The leaf prefix's buffers for this call, or none (the inner leaves are then
+// walked): one query covers no leaf twice, a set without room for them under
+// its memory budget does without, and so does a stream that is being captured
+// while they would have to grow.
+//
+// The rule of the kernels: the prefix is taken when the inner leaves of all
+// queries number more than the set's leaves.  Both forms decode a leaf in the
+// same time, so that is where the walk starts to cost more than one pass over
+// the set.  Measured at 1e8 keys (0.9e6 leaves), 1e5 ranges of 10 to 1e6
+// elements (8e7 inner leaves): 9.5 ms walked, 0.19 ms with the prefix.
+LeafPrefix leaf_prefix(cpma* h, uint64_t q, cudaStream_t st) {
+  LeafPrefix p;
+  if (q < 2) return p;
+  Scratch& s = h->s;
+  const uint64_t nt = (h->L + kT - 1) / kT;
+  if (s.q_pre.cap < h->L * 12 + 16 || s.q_tiles.cap < nt * 16) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+      cudaGetLastError();
+      return p;
+    }
+    if (reserve_leaf_prefix(h, h->L) != CPMA_OK) return p;
+  }
+  p.val = (uint64_t*)s.q_pre.p;
+  p.cnt = (uint32_t*)(p.val + h->L);
+  p.tval = (uint64_t*)s.q_tiles.p;
+  p.tcnt = p.tval + nt;
+  p.most = h->L;
+  return p;
+}
+
+// What a batch of range queries keeps between its kernels.
+struct RangeScratch {
+  uint64_t *first, *items, *off;   // q, q, q + 1 entries
+  uint64_t* partials = nullptr;    // given partials of the offset scan (else the handle's)
+  uint64_t partials_cap = 0;
+};
+
+int range_scratch(cpma* h, uint64_t q, RangeScratch* r) {
+  Scratch& s = h->s;
+  CPMA_TRY(ensure_query(h, s.q_first, q * 8));
+  CPMA_TRY(ensure_query(h, s.q_items, (q + 1) * 8));
+  CPMA_TRY(ensure_query(h, s.q_off, (q + 1) * 8));
+  CPMA_TRY(ensure_query(h, s.partials_q, (size_t)(2 * h->num_sms + 2) * 8));
+  r->first = (uint64_t*)s.q_first.p;
+  r->items = (uint64_t*)s.q_items.p;
+  r->off = (uint64_t*)s.q_off.p;
+  return CPMA_OK;
+}
+
+int scan_items(cpma* h, const RangeScratch& r, uint64_t q, cudaStream_t st) {
+  if (r.partials)
+    return scan_u64_given_partials(h, r.items, r.off, q, r.partials, r.partials_cap, st);
+  return scan_u64_query(h, r.items, r.off, q, st);
+}
+
+// After the ends: the inner leaves of every query, added to out and count.
+template <int OP, bool PLAIN>
+int range_inner(cpma* h, Reduce<OP, PLAIN> f, uint64_t q, uint64_t* out, uint64_t* count,
+                const RangeScratch& r, const LeafPrefix& p, cudaStream_t st, ull* prof) {
+  const Leaves t = leaves_of(h);
+  CPMA_TRY(scan_items(h, r, q, st));
+  const uint64_t nt = (t.L + kT - 1) / kT;
+  if (p.val) {
+    const unsigned g = (unsigned)std::min<uint64_t>(nt, (uint64_t)persistent_grid(h));
+    const uint64_t* total = r.off + q;
+    CPMA_CUDA(launch_pdl(k_leaf_prefix<OP, PLAIN>, g, kT, 0, st, t, f, total, p, prof));
+    CPMA_CUDA(launch_pdl(k_tile_scan<OP>, 1, kT, 0, st, total, p, nt));
+    h->launches += 2;
+  }
+  CPMA_CUDA(launch_pdl(k_range_inner<OP, PLAIN>, (unsigned)persistent_grid(h), kT, 0, st, t, f, q,
+                       r.first, r.off, p, out, count, prof));
   CPMA_LAUNCHED(h);
-  CPMA_TRY(scan_u64_query(hm, items, off, q, st));
-  prof_end(h, st);
+  return check_cuda(cudaGetLastError());
+}
+
+template <int OP, bool PLAIN>
+int range_leaves(cpma* h, const uint64_t* lo, const uint64_t* hi, uint64_t q, uint64_t mask,
+                 uint64_t value, uint64_t* out, uint64_t* count, const RangeScratch& r,
+                 const LeafPrefix& p, cudaStream_t st, ull* prof) {
+  const Reduce<OP, PLAIN> f{mask, value};
+  const int b = query_block(h, q);
+  k_range_ends<OP, PLAIN><<<query_grid(h, q, b, 8), b, 0, st>>>(lo, hi, q, leaves_of(h), f, r.first,
+                                                                r.items, out, count, prof);
+  CPMA_LAUNCHED(h);
+  CPMA_CUDA(cudaGetLastError());
+  return range_inner<OP, PLAIN>(h, f, q, out, count, r, p, st, prof);
+}
+
+RangeArgs raw_args(const cpma* h, const uint64_t* lo, const uint64_t* hi, uint64_t q,
+                   const RangeScratch& r, uint64_t* out, uint64_t* count) {
   RangeArgs a;
   a.lo = lo;
   a.hi = hi;
   a.q = q;
-  a.first = first;
-  a.off = off;
+  a.first = r.first;
+  a.off = r.off;
   a.data = h->data;
   a.used = h->used;
   a.cnt = h->cnt;
   a.LB = h->cfg.leaf_bytes;
-  a.sum = sum;
+  a.sum = out;
   a.count = count;
-  a.prof = prof_bytes(h, PH_RANGE);
-  a.raw = (int)h->cfg.codec;
-  prof_begin(h, PH_RANGE, st);
-  k_range<false><<<persistent_grid(h), kT, 0, st>>>(a);
+  a.prof = nullptr;
+  return a;
+}
+
+// Cells (codec 1): route, number the items, init the outputs.
+int raw_prep(cpma* h, const uint64_t* lo, const uint64_t* hi, uint64_t q, uint64_t* out,
+             uint64_t* count, uint64_t init, const RangeScratch& r, cudaStream_t st) {
+  k_range_prep<<<query_grid(h, q, kT, 8), kT, 0, st>>>(lo, hi, q, h->heads, h->L, r.first, r.items,
+                                                       out, count, init);
   CPMA_LAUNCHED(h);
+  CPMA_CUDA(cudaGetLastError());
+  return scan_items(h, r, q, st);
+}
+
+}  // namespace
+
+bool release_leaf_prefix(cpma* h) {
+  if (!h->s.q_pre.p && !h->s.q_tiles.p) return false;
+  if (cudaDeviceSynchronize() != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  release(h, h->s.q_pre);
+  release(h, h->s.q_tiles);
+  return true;
+}
+
+int reserve_leaf_prefix(cpma* h, uint64_t L) {
+  CPMA_TRY(ensure(h, h->s.q_pre, L * 12 + 16));
+  return ensure(h, h->s.q_tiles, (L + kT - 1) / kT * 16);
+}
+
+int run_range(const cpma* h, const uint64_t* lo, const uint64_t* hi, uint64_t q, uint64_t* sum,
+              uint64_t* count, cudaStream_t st) {
+  if (q == 0) return CPMA_OK;
+  cpma* hm = const_cast<cpma*>(h);
+  RangeScratch r;
+  CPMA_TRY(range_scratch(hm, q, &r));
+  int rc;
+  if (h->cfg.codec) {
+    prof_begin(h, PH_RANGE_PREP, st);
+    prof_add_bytes(h, PH_RANGE_PREP, 72ull * q);  // lo, hi in; first, items, sums out; scan
+    CPMA_TRY(raw_prep(hm, lo, hi, q, sum, count, 0, r, st));
+    prof_end(h, st);
+    RangeArgs a = raw_args(h, lo, hi, q, r, sum, count);
+    a.prof = prof_bytes(h, PH_RANGE);
+    prof_begin(h, PH_RANGE, st);
+    k_range<false><<<persistent_grid(h), kT, 0, st>>>(a);
+    CPMA_LAUNCHED(h);
+    rc = check_cuda(cudaGetLastError());
+  } else {
+    const LeafPrefix p = leaf_prefix(hm, q, st);
+    prof_begin(h, PH_RANGE, st);
+    rc = range_leaves<CPMA_OP_SUM, true>(hm, lo, hi, q, 0, 0, sum, count, r, p, st,
+                                         prof_bytes(h, PH_RANGE));
+  }
   prof_end(h, st);
-  return check_cuda(cudaGetLastError());
+  return rc;
 }
 
 int run_range_length(const cpma* h, const uint64_t* start, const uint64_t* length, uint64_t q,
@@ -656,44 +1211,42 @@ int run_range_length(const cpma* h, const uint64_t* start, const uint64_t* lengt
   if (q == 0) return CPMA_OK;
   cpma* hm = const_cast<cpma*>(h);
   Scratch& s = hm->s;
-  CPMA_TRY(ensure(hm, s.q_first, q * 8));
-  CPMA_TRY(ensure(hm, s.q_items, q * 8));
-  CPMA_TRY(ensure(hm, s.q_off, (q + 1) * 8));
-  CPMA_TRY(ensure(hm, s.q_lo, q * 8));
-  CPMA_TRY(ensure(hm, s.q_hi, q * 8));
-  CPMA_TRY(ensure(hm, s.q_rank, (h->L + 1) * 8));
+  RangeScratch r;
+  CPMA_TRY(range_scratch(hm, q, &r));
+  if (h->cfg.codec) {
+    CPMA_TRY(ensure_query(hm, s.q_lo, q * 8));
+    CPMA_TRY(ensure_query(hm, s.q_hi, q * 8));
+  }
+  CPMA_TRY(ensure_query(hm, s.q_rank, (h->L + 1) * 8));
   uint64_t* P = (uint64_t*)s.q_rank.p;
-  uint64_t* r0 = (uint64_t*)s.q_lo.p;
-  uint64_t* r1 = (uint64_t*)s.q_hi.p;
-  uint64_t* first = (uint64_t*)s.q_first.p;
-  uint64_t* items = (uint64_t*)s.q_items.p;
-  uint64_t* off = (uint64_t*)s.q_off.p;
   prof_begin(h, PH_RANGE_PREP, st);
   prof_add_bytes(h, PH_RANGE_PREP, 12ull * h->L + 88ull * q);
   CPMA_TRY(scan_u32_query(hm, h->cnt, P, h->L, st));
-  const int g1 = (int)std::max<uint64_t>(
-      1, std::min<uint64_t>((q * 32 + kT - 1) / kT, (uint64_t)h->num_sms * 16));
-  k_rank_prep<false><<<g1, kT, 0, st>>>(start, length, q, h->heads, h->data, h->used, h->L,
-                                        h->cfg.leaf_bytes, P, r0, r1, first, items, sum, count,
-                                        (int)h->cfg.codec);
+  if (!h->cfg.codec) {
+    prof_end(h, st);
+    const LeafPrefix p = leaf_prefix(hm, q, st);
+    ull* prof = prof_bytes(h, PH_RANGE);
+    prof_begin(h, PH_RANGE, st);
+    const int b = query_block(h, q);
+    CPMA_CUDA(launch_pdl(k_length_ends, (unsigned)query_grid(h, q, b, 8), (unsigned)b, 0, st, start,
+                         length, q, leaves_of(h), P, r.first, r.items, sum, count, prof));
+    CPMA_LAUNCHED(h);
+    const int rc = range_inner<CPMA_OP_SUM, true>(hm, Reduce<CPMA_OP_SUM, true>{0, 0}, q, sum,
+                                                  count, r, p, st, prof);
+    prof_end(h, st);
+    return rc;
+  }
+  uint64_t* r0 = (uint64_t*)s.q_lo.p;
+  uint64_t* r1 = (uint64_t*)s.q_hi.p;
+  k_rank_prep<false><<<query_grid(h, q * 32, kT, 16), kT, 0, st>>>(
+      start, length, q, h->heads, h->data, h->used, h->L, h->cfg.leaf_bytes, P, r0, r1, r.first,
+      r.items, sum, count);
   CPMA_LAUNCHED(h);
-  CPMA_TRY(scan_u64_query(hm, items, off, q, st));
+  CPMA_TRY(scan_items(hm, r, q, st));
   prof_end(h, st);
-  RangeArgs a;
-  a.lo = r0;
-  a.hi = r1;
-  a.q = q;
-  a.first = first;
-  a.off = off;
-  a.data = h->data;
-  a.used = h->used;
-  a.cnt = h->cnt;
-  a.LB = h->cfg.leaf_bytes;
-  a.sum = sum;
-  a.count = count;
+  RangeArgs a = raw_args(h, r0, r1, q, r, sum, count);
   a.prof = prof_bytes(h, PH_RANGE);
   a.P = P;
-  a.raw = (int)h->cfg.codec;
   prof_begin(h, PH_RANGE, st);
   k_range<true><<<persistent_grid(h), kT, 0, st>>>(a);
   CPMA_LAUNCHED(h);
@@ -706,37 +1259,37 @@ int run_range_extract(const cpma* h, const uint64_t* lo, const uint64_t* hi, uin
   if (q == 0) return check_cuda(cudaMemsetAsync(offsets, 0, 8, st));
   cpma* hm = const_cast<cpma*>(h);
   Scratch& s = hm->s;
-  CPMA_TRY(ensure(hm, s.q_first, q * 8));
-  CPMA_TRY(ensure(hm, s.q_items, (q + 1) * 8));
-  CPMA_TRY(ensure(hm, s.q_off, (q + 1) * 8));
-  CPMA_TRY(ensure(hm, s.q_lo, q * 8));
-  CPMA_TRY(ensure(hm, s.q_hi, q * 8));
-  CPMA_TRY(ensure(hm, s.q_rank, (h->L + 1) * 8));
+  RangeScratch r;
+  CPMA_TRY(range_scratch(hm, q, &r));
+  CPMA_TRY(ensure_query(hm, s.q_lo, q * 8));
+  CPMA_TRY(ensure_query(hm, s.q_hi, q * 8));
+  CPMA_TRY(ensure_query(hm, s.q_rank, (h->L + 1) * 8));
   uint64_t* P = (uint64_t*)s.q_rank.p;
   uint64_t* r0 = (uint64_t*)s.q_lo.p;
   uint64_t* r1 = (uint64_t*)s.q_hi.p;
-  uint64_t* first = (uint64_t*)s.q_first.p;
-  uint64_t* items = (uint64_t*)s.q_items.p;
-  uint64_t* off = (uint64_t*)s.q_off.p;
   prof_begin(h, PH_RANGE_PREP, st);
   CPMA_TRY(scan_u32_query(hm, h->cnt, P, h->L, st));
-  const int g1 = (int)std::max<uint64_t>(
-      1, std::min<uint64_t>((q * 32 + kT - 1) / kT, (uint64_t)h->num_sms * 16));
-  // counts (r1 - r0) go into `items` of a second pass: first the ranks
-  k_rank_prep<true><<<g1, kT, 0, st>>>(lo, hi, q, h->heads, h->data, h->used, h->L,
-                                       h->cfg.leaf_bytes, P, r0, r1, first, items, nullptr,
-                                       offsets, (int)h->cfg.codec);
+  // the counts (r1 - r0) go to `offsets` first
+  if (h->cfg.codec) {
+    k_rank_prep<true><<<query_grid(h, q * 32, kT, 16), kT, 0, st>>>(
+        lo, hi, q, h->heads, h->data, h->used, h->L, h->cfg.leaf_bytes, P, r0, r1, r.first, r.items,
+        nullptr, offsets);
+  } else {
+    CPMA_CUDA(launch_pdl(k_rank_ends, (unsigned)query_grid(h, 2 * q, kT, 8), kT, 0, st, lo, hi, q,
+                         leaves_of(h), P, r0, r1, r.first, r.items, offsets));
+  }
   CPMA_LAUNCHED(h);
   CPMA_TRY(scan_u64_query(hm, offsets, offsets, q, st));
-  CPMA_TRY(scan_u64_query(hm, items, off, q, st));
+  const bool emit = out && cap;
+  if (emit) CPMA_TRY(scan_items(hm, r, q, st));
   prof_end(h, st);
-  if (!out || cap == 0) return check_cuda(cudaGetLastError());
+  if (!emit) return check_cuda(cudaGetLastError());
   ExtractArgs a;
   a.r0 = r0;
   a.r1 = r1;
   a.q = q;
-  a.first = first;
-  a.item_off = off;
+  a.first = r.first;
+  a.item_off = r.off;
   a.out_off = offsets;
   a.P = P;
   a.data = h->data;
@@ -744,9 +1297,9 @@ int run_range_extract(const cpma* h, const uint64_t* lo, const uint64_t* hi, uin
   a.LB = h->cfg.leaf_bytes;
   a.out = out;
   a.cap = cap;
-  a.raw = (int)h->cfg.codec;
   prof_begin(h, PH_RANGE, st);
-  k_extract<<<persistent_grid(h), kT, 0, st>>>(a);
+  if (h->cfg.codec) k_extract<<<persistent_grid(h), kT, 0, st>>>(a);
+  else CPMA_CUDA(launch_pdl(k_extract_leaf, (unsigned)persistent_grid(h), kT, 0, st, a));
   CPMA_LAUNCHED(h);
   prof_end(h, st);
   return check_cuda(cudaGetLastError());
@@ -759,14 +1312,34 @@ int run_range_reduce(const cpma* h, const uint64_t* lo, const uint64_t* hi, uint
     return run_range(h, lo, hi, q, out, count, st);
   if (q == 0) return CPMA_OK;
   cpma* hm = const_cast<cpma*>(h);
-  CPMA_TRY(ensure(hm, hm->s.q_first, q * 8));
-  CPMA_TRY(ensure(hm, hm->s.q_items, q * 8));
-  CPMA_TRY(ensure(hm, hm->s.q_off, (q + 1) * 8));
-  uint64_t* first = (uint64_t*)hm->s.q_first.p;
-  uint64_t* items = (uint64_t*)hm->s.q_items.p;
-  uint64_t* off = (uint64_t*)hm->s.q_off.p;
-  const int g1 = (int)std::max<uint64_t>(
-      1, std::min<uint64_t>((q + kT - 1) / kT, (uint64_t)h->num_sms * 8));
+  RangeScratch r;
+  CPMA_TRY(range_scratch(hm, q, &r));
+  if (!h->cfg.codec) {
+    const LeafPrefix p = leaf_prefix(hm, q, st);
+    prof_begin(h, PH_RANGE, st);
+    int rc;
+    switch (op) {
+      case CPMA_OP_SUM:
+        rc = range_leaves<CPMA_OP_SUM, false>(hm, lo, hi, q, mask, value, out, count, r, p, st,
+                                              nullptr);
+        break;
+      case CPMA_OP_MIN:
+        rc = range_leaves<CPMA_OP_MIN, false>(hm, lo, hi, q, mask, value, out, count, r, p, st,
+                                              nullptr);
+        break;
+      case CPMA_OP_MAX:
+        rc = range_leaves<CPMA_OP_MAX, false>(hm, lo, hi, q, mask, value, out, count, r, p, st,
+                                              nullptr);
+        break;
+      case CPMA_OP_XOR:
+        rc = range_leaves<CPMA_OP_XOR, false>(hm, lo, hi, q, mask, value, out, count, r, p, st,
+                                              nullptr);
+        break;
+      default: rc = CPMA_EINVAL;
+    }
+    prof_end(h, st);
+    return rc;
+  }
   uint64_t init = 0;
   switch (op) {
     case CPMA_OP_SUM: init = op_identity<CPMA_OP_SUM>(); break;
@@ -776,24 +1349,9 @@ int run_range_reduce(const cpma* h, const uint64_t* lo, const uint64_t* hi, uint
     default: return CPMA_EINVAL;
   }
   prof_begin(h, PH_RANGE_PREP, st);
-  k_range_prep<<<g1, kT, 0, st>>>(lo, hi, q, h->heads, h->L, first, items, out, count, init);
-  CPMA_LAUNCHED(h);
-  CPMA_TRY(scan_u64_query(hm, items, off, q, st));
+  CPMA_TRY(raw_prep(hm, lo, hi, q, out, count, init, r, st));
   prof_end(h, st);
-  RangeArgs a;
-  a.lo = lo;
-  a.hi = hi;
-  a.q = q;
-  a.first = first;
-  a.off = off;
-  a.data = h->data;
-  a.used = h->used;
-  a.cnt = h->cnt;
-  a.LB = h->cfg.leaf_bytes;
-  a.sum = out;
-  a.count = count;
-  a.prof = nullptr;
-  a.raw = (int)h->cfg.codec;
+  const RangeArgs a = raw_args(h, lo, hi, q, r, out, count);
   prof_begin(h, PH_RANGE, st);
   const int G = persistent_grid(h);
   switch (op) {
@@ -816,37 +1374,23 @@ int run_range_noalloc(const cpma* h, const uint64_t* lo, const uint64_t* hi, uin
   if (dev != h->device) return CPMA_EINVAL;
   uint8_t* base = nullptr;
   CPMA_TRY(scratch_address(dev, &base));
-  uint64_t* first = reinterpret_cast<uint64_t*>(base);
-  uint64_t* items = first + kNoAllocMaxQueries;
-  uint64_t* off = items + kNoAllocMaxQueries;            // q + 1 entries
-  uint64_t* partials = off + kNoAllocMaxQueries + 1;     // kNoAllocPartials entries
+  RangeScratch r;
+  r.first = reinterpret_cast<uint64_t*>(base);
+  r.items = r.first + kNoAllocMaxQueries;
+  r.off = r.items + kNoAllocMaxQueries;                  // q + 1 entries
+  r.partials = r.off + kNoAllocMaxQueries + 1;           // kNoAllocPartials entries
+  r.partials_cap = kNoAllocPartials;
   // the offset scan needs at most 2 * SMs + 1 partials: checked before any
   // launch, so a rejected call leaves the outputs untouched
   if ((uint64_t)2 * h->num_sms + 1 > kNoAllocPartials) return CPMA_EINVAL;
-  const int g1 = (int)std::max<uint64_t>(
-      1, std::min<uint64_t>((q + kT - 1) / kT, (uint64_t)h->num_sms * 8));
   // every scratch entry read below is written first on this stream: nothing
   // carries over from an earlier call
-  k_range_prep<<<g1, kT, 0, st>>>(lo, hi, q, h->heads, h->L, first, items, sum, count);
-  CPMA_LAUNCHED(h);
-  CPMA_CUDA(cudaGetLastError());
-  CPMA_TRY(scan_u64_given_partials(const_cast<cpma*>(h), items, off, q, partials,
-                                   kNoAllocPartials, st));
-  RangeArgs a;
-  a.lo = lo;
-  a.hi = hi;
-  a.q = q;
-  a.first = first;
-  a.off = off;
-  a.data = h->data;
-  a.used = h->used;
-  a.cnt = h->cnt;
-  a.LB = h->cfg.leaf_bytes;
-  a.sum = sum;
-  a.count = count;
-  a.prof = nullptr;
-  a.raw = (int)h->cfg.codec;
-  k_range<false><<<persistent_grid(h), kT, 0, st>>>(a);
+  cpma* hm = const_cast<cpma*>(h);
+  if (!h->cfg.codec)
+    return range_leaves<CPMA_OP_SUM, true>(hm, lo, hi, q, 0, 0, sum, count, r, LeafPrefix(), st,
+                                           nullptr);
+  CPMA_TRY(raw_prep(hm, lo, hi, q, sum, count, 0, r, st));
+  k_range<false><<<persistent_grid(h), kT, 0, st>>>(raw_args(h, lo, hi, q, r, sum, count));
   CPMA_LAUNCHED(h);
   return check_cuda(cudaGetLastError());
 }

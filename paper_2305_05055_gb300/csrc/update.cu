@@ -3381,7 +3381,9 @@ int reserve(cpma* h, uint64_t max_batch, int tagged, cudaStream_t st) {
   if (max_batch >= (1ull << 31)) return CPMA_EINVAL;
   if (max_batch == 0) return CPMA_OK;
   // everything an insert of max_batch keys reserves, a growing resize included
-  CPMA_TRY(reserve_update(h, max_batch, 0, st, true));
+  int rc = reserve_update(h, max_batch, 0, st, true);
+  if (rc == CPMA_ENOMEM && release_leaf_prefix(h)) rc = reserve_update(h, max_batch, 0, st, true);
+  CPMA_TRY(rc);
   CPMA_TRY(front_scratch(h, max_batch, tagged != 0, st));
   if (!tagged && h->point_max) CPMA_TRY(point_scratch(h, std::min(max_batch, h->point_max), st));
   if (h->graph_max_batch && !tagged) {
@@ -3511,13 +3513,19 @@ int run_update(cpma* h, const uint64_t* d_keys, uint64_t k, int sorted, int is_d
     return run_rebuild(h, d_keys, k, sorted, is_delete, d_delta, st);
   Scratch& s = h->s;
   const bool graph = k <= h->graph_max_batch && !tags && graph_bucket(k) < (1ull << 31);
-  int rc = reserve_update(h, k, is_delete, st, false);
-  if (rc == CPMA_OK && graph) {
-    rc = ensure(h, s.stage, graph_bucket(k) * 8, st);
-    if (rc == CPMA_OK) rc = front_scratch(h, graph_bucket(k), false, st);
-  } else if (rc == CPMA_OK) {
-    rc = front_scratch(h, k, tags != nullptr, st);
-  }
+  auto take = [&] {
+    int e = reserve_update(h, k, is_delete, st, false);
+    if (e == CPMA_OK && graph) {
+      e = ensure(h, s.stage, graph_bucket(k) * 8, st);
+      if (e == CPMA_OK) e = front_scratch(h, graph_bucket(k), false, st);
+    } else if (e == CPMA_OK) {
+      e = front_scratch(h, k, tags != nullptr, st);
+    }
+    return e;
+  };
+  int rc = take();
+  // the range queries' prefix makes room first: they run without it
+  if (rc == CPMA_ENOMEM && release_leaf_prefix(h)) rc = take();
   if (rc == CPMA_ENOMEM) {
     // refused before any change; give back the scratch grown so far, so
     // that a smaller batch after this one starts from the structure alone

@@ -1,0 +1,32 @@
+// Host build of a thread's walk over a leaf (leaf_walk.cuh) for the CPU tests.
+#include "../paper_2305_05055_gb300/csrc/leaf_walk.cuh"
+
+extern "C" uint64_t lw_sum(const uint8_t* leaf, uint32_t u, uint32_t m, int form) {
+  uint64_t s = 0;
+  if (form == 0) return leafwalk::leaf_sum(leaf, u, m);
+  if (form == 1) return leafwalk::sum_walked(leaf, u);
+  return (form == 2 ? leafwalk::sum_few(leaf, u, m, s) : leafwalk::sum_many(leaf, u, m, s)) ? s : ~0ull;
+}
+
+extern "C" uint32_t lw_visit(const uint8_t* leaf, uint32_t u, uint64_t* out) {
+  uint32_t n = 0;
+  leafwalk::leaf_visit(leaf, u, [&](uint64_t v) { out[n++] = v; });
+  return n;
+}
+
+extern "C" void lw_range(const uint8_t* leaf, uint32_t u, uint64_t lo, uint64_t hi, uint64_t* out) {
+  out[0] = out[1] = 0;
+  leafwalk::leaf_range_sum(leaf, u, lo, hi, out[0], out[1]);
+}
+
+extern "C" void lw_take(const uint8_t* leaf, uint32_t u, uint64_t lo, uint64_t most,
+                        uint64_t* out) {
+  uint32_t below, taken;
+  leafwalk::leaf_take_sum(leaf, u, lo, most, below, taken, out[2]);
+  out[0] = below;
+  out[1] = taken;
+}
+
+extern "C" uint32_t lw_below(const uint8_t* leaf, uint32_t u, uint64_t x) {
+  return leafwalk::leaf_below(leaf, u, x);
+}
