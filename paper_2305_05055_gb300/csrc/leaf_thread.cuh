@@ -428,13 +428,6 @@ LT_HD uint32_t plan_leaf(uint8_t* leafp, uint32_t LB, uint32_t uold, uint32_t m,
   return kWritten;
 }
 
-// The segment after the last edit: old bytes [oe, uold) land at [dlo, nb)
-// shifted by sa (nb = the new used bytes).
-LT_HD void tail_segment(const Scratch& S, uint32_t E, uint32_t uold, int32_t& dlo, int32_t& nb,
-                        int32_t& sa) {
-  seg_bounds(S, E, uold, S.epos[0] & 0xFFFu, (int)E - 1, dlo, nb, sa);
-}
-
 // The 16 bytes at leaf[src, src + 16) (0 <= src, src + 16 <= the old used
 // bytes): the aligned chunk below src and, unless src is aligned, the one
 // after it, shifted together.  A destination chunk wholly inside the
@@ -481,28 +474,36 @@ LT_HD void chunk_tail(const uint8_t* leafp, int32_t src, uint32_t (&r)[4]) {
 }
 
 // Pass B by one thread: the chunks R.wlo .. R.whi of the leaf from the end
-// backwards, each gathered from the segments that land in it and stored
-// whole (the edits' own bytes are left zero: write_edits fills them).
+// backwards, each built from the segments that land in it and stored whole
+// (the edits' own bytes are left zero: write_edits fills them).  A run of
+// chunks inside one segment is one shift each; the chunk below it, where an
+// edit falls, is gathered segment by segment.  Runs of every segment, not only
+// of the last, take the short way: with one or two keys in most leaves, some
+// lane of every warp has chunks between two edits, and gathering those too
+// kept its whole warp (1e6 keys into 1e8: 314 us a launch, RW_NEW us so).
 LT_HD void rewrite_leaf(uint8_t* leafp, uint32_t LB, uint32_t uold, const Scratch& S,
                         const Result& R) {
   const uint32_t E = R.E;
   const uint32_t os0 = S.epos[0] & 0xFFFu;
-  const uint32_t olo = R.wlo, ohi = R.whi;
-  int32_t tlo, tnb, tsa;
-  tail_segment(S, E, uold, tlo, tnb, tsa);
-  int cur = (int)E - 1;
-  for (int32_t o = (int32_t)ohi - 16; o >= (int32_t)olo; o -= 16) {
-    if (o >= tlo && o + 16 <= tnb) {  // wholly inside the last segment
+  const int32_t olo = (int32_t)R.wlo;
+  int cur = (int)E - 1;  // the highest segment not wholly above chunk o
+  int32_t slo, shi, ssa;
+  seg_bounds(S, E, uold, os0, cur, slo, shi, ssa);
+  for (int32_t o = (int32_t)R.whi - 16; o >= olo; o -= 16) {
+    while (o >= olo && o >= slo && o + 16 <= shi) {
       uint32_t r[4];
-      chunk_tail(leafp, o - tsa, r);
+      chunk_tail(leafp, o - ssa, r);
       st16(leafp + o, r);
-      continue;
+      o -= 16;
     }
-    for (;;) {  // the highest segment not wholly above chunk o
-      int32_t dlo, dhi, sa;
-      seg_bounds(S, E, uold, os0, cur, dlo, dhi, sa);
-      if (cur < 0 || dlo < o + 16) break;
+    if (o < olo) break;
+    while (cur >= 0 && slo >= o + 16) {
       cur--;
+      seg_bounds(S, E, uold, os0, cur, slo, shi, ssa);
+    }
+    if (o >= slo && o + 16 <= shi) {  // the next segment's run starts here
+      o += 16;
+      continue;
     }
     uint32_t r[4] = {0u, 0u, 0u, 0u};
     for (int e = cur; e >= -1; e--) {
@@ -643,27 +644,32 @@ LT_HD uint32_t plan_delete(uint8_t* leafp, uint32_t LB, uint32_t uold, uint32_t 
 }
 
 // Pass B of a delete by one thread: the chunks R.wlo .. R.whi from the front,
-// each gathered from the segments that land in it (every shift is <= 0, so a
-// chunk's sources lie at or above it: not yet written).
+// each built from the segments that land in it (every shift is <= 0, so a
+// chunk's sources lie at or above it: not yet written), runs inside one
+// segment by one shift each as in rewrite_leaf.
 LT_HD void rewrite_forward(uint8_t* leafp, uint32_t LB, uint32_t uold, const Scratch& S,
                            const Result& R) {
   const uint32_t E = R.E;
   const uint32_t os0 = S.epos[0] & 0xFFFu;
-  int32_t tlo, tnb, tsa;
-  tail_segment(S, E, uold, tlo, tnb, tsa);
-  int cur = -1;
-  for (int32_t o = (int32_t)R.wlo; o < (int32_t)R.whi; o += 16) {
-    if (o >= tlo && o + 16 <= tnb) {  // wholly inside the last segment
+  const int32_t ohi = (int32_t)R.whi;
+  int cur = -1;  // the lowest segment not wholly below chunk o
+  int32_t slo, shi, ssa;
+  seg_bounds(S, E, uold, os0, cur, slo, shi, ssa);
+  for (int32_t o = (int32_t)R.wlo; o < ohi; o += 16) {
+    while (o < ohi && o >= slo && o + 16 <= shi) {
       uint32_t r[4];
-      chunk_tail(leafp, o - tsa, r);
+      chunk_tail(leafp, o - ssa, r);
       st16(leafp + o, r);
-      continue;
+      o += 16;
     }
-    for (;;) {  // the lowest segment not wholly below chunk o
-      int32_t dlo, dhi, sa;
-      seg_bounds(S, E, uold, os0, cur, dlo, dhi, sa);
-      if (cur + 1 >= (int)E || dhi > o) break;
+    if (o >= ohi) break;
+    while (cur + 1 < (int)E && shi <= o) {
       cur++;
+      seg_bounds(S, E, uold, os0, cur, slo, shi, ssa);
+    }
+    if (o >= slo && o + 16 <= shi) {  // the next segment's run starts here
+      o -= 16;
+      continue;
     }
     uint32_t r[4] = {0u, 0u, 0u, 0u};
     for (int e = cur; e < (int)E; e++) {
