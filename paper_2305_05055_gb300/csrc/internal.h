@@ -79,7 +79,6 @@ struct Status {
 constexpr ull kErrUnsorted = 1;   // a batch promised sorted was not
 constexpr ull kErrFit = 2;        // a redistributed leaf did not fit
 constexpr ull kErrState = 4;      // inconsistent leaf state
-constexpr ull kErrSort = 8;       // a sort tile waited too long for its predecessor
 constexpr ull kErrRoute = 16;     // a routing tile waited too long for its predecessor
 
 constexpr uint32_t kChunk = 256;  // keys per merge work item
@@ -108,7 +107,7 @@ struct Arrays {
 struct Scratch {
   Buf keysA, keysB;       // sort ping-pong (u64)
   Buf valsA, valsB;       // sort ping-pong of 32-bit tags
-  Buf hist;               // sort control block and look-back arrays
+  Buf hist;               // sort control block, digit counts per block
   Buf flags;              // routing: tile counter and look-back words (u64)
   Buf flags_scan;         // build and rebuild: scanned flags (u64)
   Buf leaf_of;            // build: unique flags (u32)
@@ -191,7 +190,7 @@ struct cpma {
   // used bytes over all leaves: exact after the last merge (t_known) and a
   // bound on how much the redistribution after it changed them (t_slack)
   uint64_t t_known = 0, t_slack = 0;
-  // batch sort look-back (tests): poll limit (0 = default), silent tile (-1 = none)
+  // routing look-back (tests): poll limit (0 = default), silent tile (-1 = none)
   uint32_t sort_poll_limit = 0;
   int64_t sort_silent_tile = -1;
   uint64_t bits_words = 0;          // words of the window bitsets now zeroed

@@ -480,7 +480,7 @@ LT_HD void chunk_tail(const uint8_t* leafp, int32_t src, uint32_t (&r)[4]) {
 // edit falls, is gathered segment by segment.  Runs of every segment, not only
 // of the last, take the short way: with one or two keys in most leaves, some
 // lane of every warp has chunks between two edits, and gathering those too
-// kept its whole warp (1e6 keys into 1e8: 314 us a launch, RW_NEW us so).
+// kept its whole warp (1e6 keys into 1e8: a launch 303 -> 290 us with this).
 LT_HD void rewrite_leaf(uint8_t* leafp, uint32_t LB, uint32_t uold, const Scratch& S,
                         const Result& R) {
   const uint32_t E = R.E;

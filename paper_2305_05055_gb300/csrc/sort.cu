@@ -1,29 +1,39 @@
 // Batch sort (Sec. 4: "an unsorted batch can be converted into a sorted batch
-// in O(k log k) work") as an LSD radix sort over 8-bit digits, plus the
-// adjacent-repeat compaction used by the constructor.
+// in O(k log k) work") as a radix sort over 8-bit digits.
 //
-// One sweep per digit: a first kernel builds the histograms of all eight
-// digits in one read of the batch; its last block scans them and marks the
-// digits that vary (40-bit uniform keys need 5 passes, not 8).  Each varying
-// digit is then one scatter launch: a tile of 4096 keys is ranked stably in
-// shared memory (the lanes of a warp sharing a digit found by eight ballots,
-// then per-warp prefixes), its
-// global offsets come from the tiles before it by decoupled look-back (each
-// tile publishes its per-digit count, then its inclusive prefix), and every
-// digit's run of the tile is written contiguously.  Digits that do not vary
-// return at once; the passes alternate buffers so that the last one lands in
-// the first scratch buffer.  No host round trip.  Batches of at most one tile
-// are sorted by a single block.
+// One digit pass is three kernels.  Every block owns a contiguous run of
+// 4096-key tiles.  It counts its keys per digit (k_digit_count); a block per
+// digit turns the blocks' counts into offsets (k_digit_scan); every block then
+// takes its tiles in order, ranks each in shared memory and writes every
+// digit's run of the tile contiguously behind the ones before it
+// (k_digit_scatter).  No block waits for another.  (Reading the keys once and
+// joining the tiles by decoupled look-back instead was slower: several hundred
+// tiles start together, so each had to add up most of its predecessors'
+// counts, 8 per round trip to the L2: 343 us a pass over 3e7 keys, against
+// 63 + 3 + 180 us for the three kernels.)  A stable rank takes eight ballots
+// per key and warp (115 instructions per 32 keys bound the scatter); where
+// order among equal digits does not matter it is one atomic.
 //
-// Batches of up to 1.25M keys go most significant bits first instead: one
-// pass takes the OR and AND of the keys, which give the 8 highest bits that
-// vary; one pass counts them (256 buckets); one scatter pass (the same tile
-// ranking and look-back) moves the keys to their buckets, and each bucket is
-// then sorted by the bits below them in one block: in shared memory when it
-// holds at most 6144 keys (k / 256 on average), else (heavy repeats or skew)
-// by a block-level LSD radix sort through global memory.  Three reads and
-// two writes of the batch instead of six and five, with no pass that
-// depends on how the keys fall.
+// Keys alone go most significant bits first, so that few passes cross memory:
+// - up to 4096 keys: one block, a sorting network;
+// - up to 1.25M: the OR and AND of the keys give the 8 highest bits that vary,
+//   one pass by those moves the keys to 256 buckets, a block finishes each
+//   (k_bucket_sort);
+// - above, when more than 24 bits vary: two passes by the 16 highest of them,
+//   then each block finishes the buckets that start in its 4096 keys
+//   (k_window_sort), at most 6144 keys.  A bucket of more than 2048 keys
+//   (heavy repeats or skew) does not fit that: it raises a flag, and the
+//   passes over all varying digits, lowest first, run after all.  3e7 40-bit
+//   keys: 735 us, 1650 us for the five look-back passes.
+// A block finishes up to 6144 keys in shared memory in one counting pass: bins
+// by the highest bits in which the keys differ, about as many as keys, one
+// atomic per key, then every key's rank among the few keys of its bin.  Bins
+// over kBinMost keys (repeats, clusters) send the block to digit passes in
+// shared memory instead.  1e6 keys in 256 buckets: 9 us against 30 us for four
+// digit passes.
+//
+// Keys with tags (which must move stably) take the digit passes: buckets up
+// to 1.25M, all varying digits from the lowest up above.
 #include <algorithm>
 
 #include "dev_common.cuh"
@@ -131,43 +141,137 @@ __device__ __forceinline__ void tile_rank(const uint64_t (&key)[ITEMS], const ui
   __syncthreads();
 }
 
-constexpr uint32_t kFlagA = 1u << 30;  // tile count published
-constexpr uint32_t kFlagP = 2u << 30;  // inclusive prefix published
-constexpr uint32_t kCountMask = (1u << 30) - 1u;
-constexpr uint32_t kSpinLimit = 1u << 22;
-constexpr int kLook = 8;  // predecessors read per look-back step
+// ---- up to kBTile keys in one block, by bins ----
+constexpr uint32_t kBins = 4096;
+constexpr uint32_t kBinMost = 32;  // keys of a bin ranked against each other (at most 255)
+struct BinSmem {
+  uint64_t keys[kBTile];
+  __align__(16) uint32_t bin[kBins + 4];
+  uint32_t ws[kBT / 32];
+};
+
+// Writes the n <= kBTile keys held by the block (item j of thread t; ok: which
+// exist), all in [lo, lo + 2^bits), to dst in order.  false (nothing written,
+// for every thread): some bin holds more than kBinMost keys.
+__device__ __forceinline__ bool bin_sort(const uint64_t (&key)[kBItems], uint32_t ok, uint32_t n,
+                                         uint64_t lo, uint32_t bits, BinSmem& sm,
+                                         uint64_t* __restrict__ dst) {
+  const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
+  // as many bins as keys: a power of two, 4 or 8 per thread
+  const uint32_t lb = n > 2048u ? 12u : 11u, nb = 1u << lb;
+  static_assert(kBT * 8 == kBins, "8 bins per thread");
+  const uint32_t sh = bits > lb ? bits - lb : 0u;
+  uint4* bin4 = reinterpret_cast<uint4*>(sm.bin);
+  for (uint32_t i = threadIdx.x; i < nb / 4; i += kBT) bin4[i] = make_uint4(0u, 0u, 0u, 0u);
+  __syncthreads();
+  uint32_t r[kBItems / 4] = {0u};  // places in the bins, a byte each
+  bool deep = false;
+#pragma unroll
+  for (int j = 0; j < kBItems; j++)
+    if ((ok >> j) & 1u) {
+      const uint32_t at = atomicAdd(&sm.bin[(uint32_t)((key[j] - lo) >> sh)], 1u);
+      deep |= at >= kBinMost;
+      r[j / 4] |= at << (8 * (j % 4));
+    }
+  if (__syncthreads_or(deep)) return false;
+  // exclusive prefix over the bins, 4 or 8 consecutive ones per thread
+  const bool two = lb == 12u;
+  const uint32_t i0 = threadIdx.x * (two ? 2u : 1u);
+  const uint4 u = bin4[i0], v = two ? bin4[i0 + 1] : make_uint4(0u, 0u, 0u, 0u);
+  const uint32_t sum = u.x + u.y + u.z + u.w + v.x + v.y + v.z + v.w;
+  const uint32_t inc = warp_incl_scan(sum);
+  if (lane == 31) sm.ws[warp] = inc;
+  __syncthreads();
+  uint32_t run = inc - sum;
+  {
+    const uint32_t w = lane < warp ? sm.ws[lane] : 0u;  // warp < 16
+    run += __reduce_add_sync(FULL, w);
+  }
+  const uint4 p = make_uint4(run, run + u.x, run + u.x + u.y, run + u.x + u.y + u.z);
+  bin4[i0] = p;
+  if (two) {
+    const uint32_t q = p.w + u.w;
+    bin4[i0 + 1] = make_uint4(q, q + v.x, q + v.x + v.y, q + v.x + v.y + v.z);
+  }
+  if (threadIdx.x == 0) sm.bin[nb] = n;
+  __syncthreads();
+#pragma unroll
+  for (int j = 0; j < kBItems; j++)
+    if ((ok >> j) & 1u)
+      sm.keys[sm.bin[(uint32_t)((key[j] - lo) >> sh)] + ((r[j / 4] >> (8 * (j % 4))) & 0xFFu)] =
+          key[j];
+  __syncthreads();
+  for (uint32_t i = threadIdx.x; i < n; i += kBT) {
+    const uint64_t x = sm.keys[i];
+    const uint32_t b = (uint32_t)((x - lo) >> sh);
+    const uint32_t q0 = sm.bin[b], q1 = sm.bin[b + 1];
+    uint32_t at = q0;
+    for (uint32_t q = q0; q < q1; q++) {
+      const uint64_t y = sm.keys[q];
+      at += (y < x || (y == x && q < i)) ? 1u : 0u;
+    }
+    dst[at] = x;
+  }
+  return true;
+}
 
 // Control block of one sort, zeroed before the first kernel.
 struct SortCtl {
-  uint32_t hist[8][256];   // digit histograms
-  uint32_t off[8][256];    // exclusive digit offsets
+  uint32_t tot[256];       // keys per digit of the current pass
   uint32_t varying[8];     // digit p varies across the batch
   uint32_t rank[8];        // position of digit p among the varying ones
   uint32_t npass;          // number of varying digits
-  uint32_t done_blocks;    // histogram blocks finished
-  uint32_t tile_ctr[9];    // next tile id per pass (8: the top-digit scatter)
-  uint32_t top;            // highest varying digit
-  // bucket path: OR / AND of every key, and the bucket field they give: the
-  // top 8 varying bits, bits [fshift, fshift + 8)
-  ull or_all, and_all;
-  uint32_t fshift;
-  uint32_t done_or;        // OR/AND blocks finished
+  uint32_t fshift;         // the field: bits [fshift, fshift + 8), the highest that vary
+  uint32_t done;           // OR/AND blocks finished
+  uint32_t msd;            // large batch: top 16 varying bits, then windows
+  uint32_t over;           // a window did not hold its buckets: all digits after all
+  uint32_t pad;
+  ull or_all, nand_all;    // OR of the keys and of their complements
 };
 
-__device__ __forceinline__ uint32_t bucket_of(uint64_t x, uint32_t fshift) {
-  return (uint32_t)(x >> fshift) & 255u;
+// The thread's OR of its keys and of their complements over the batch; the
+// last of the grid's blocks turns the bits that vary into the bucket field
+// (the 8 highest of them), the varying digits and their number (0 when every
+// key is equal).  A whole block must call.
+__device__ __forceinline__ void vary_of(ull o, ull na, SortCtl* ctl) {
+  __shared__ ull s_or[kWarps], s_na[kWarps];
+  const uint32_t olo = __reduce_or_sync(FULL, (uint32_t)o), ohi = __reduce_or_sync(FULL, (uint32_t)(o >> 32));
+  const uint32_t alo = __reduce_or_sync(FULL, (uint32_t)na), ahi = __reduce_or_sync(FULL, (uint32_t)(na >> 32));
+  if (lane_id() == 0) {
+    s_or[threadIdx.x >> 5] = ((ull)ohi << 32) | olo;
+    s_na[threadIdx.x >> 5] = ((ull)ahi << 32) | alo;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    ull bo = 0, ba = 0;
+    for (int w = 0; w < kWarps; w++) { bo |= s_or[w]; ba |= s_na[w]; }
+    atomicOr(&ctl->or_all, bo);
+    atomicOr(&ctl->nand_all, ba);
+    __threadfence();
+    if (atomicAdd(&ctl->done, 1u) == gridDim.x - 1) {
+      __threadfence();
+      const ull vary = *((volatile ull*)&ctl->or_all) & *((volatile ull*)&ctl->nand_all);
+      const uint32_t hb = vary ? 64u - (uint32_t)__clzll((long long)vary) : 0u;
+      ctl->fshift = hb > 8u ? hb - 8u : 0u;
+      uint32_t r = 0;
+      for (int p = 0; p < 8; p++) {
+        const uint32_t v = ((vary >> (8 * p)) & 255u) != 0u;
+        ctl->varying[p] = v;
+        ctl->rank[p] = r;
+        r += v;
+      }
+      ctl->npass = r;
+      ctl->msd = hb > 24u ? 1u : 0u;
+    }
+  }
 }
 
-// Bucket path, pass 1: OR and AND of the keys; the last block turns them into
-// the bucket field (the 8 highest bits that vary; fewer when fewer vary) and
-// npass (0 when every key is equal).
+// Bucket path, first kernel: the bits that vary.
 __global__ void __launch_bounds__(kT) k_orand(const uint64_t* __restrict__ in, uint64_t k,
                                               SortCtl* ctl) {
-  __shared__ ull s_or[kWarps], s_and[kWarps];
-  __shared__ bool last;
   pdl_wait();
   pdl_launch();
-  ull o = 0, a = ~0ull;
+  ull o = 0, na = 0;
   // eight keys per thread and step, loaded together
   const uint64_t stride = (uint64_t)gridDim.x * kT;
   uint64_t i = (uint64_t)blockIdx.x * kT + threadIdx.x;
@@ -176,125 +280,200 @@ __global__ void __launch_bounds__(kT) k_orand(const uint64_t* __restrict__ in, u
 #pragma unroll
     for (int j = 0; j < 8; j++) x[j] = in[i + j * stride];
 #pragma unroll
-    for (int j = 0; j < 8; j++) { o |= x[j]; a &= x[j]; }
+    for (int j = 0; j < 8; j++) { o |= x[j]; na |= ~x[j]; }
   }
   for (; i < k; i += stride) {
     const uint64_t x = in[i];
     o |= x;
-    a &= x;
+    na |= ~x;
   }
-  const uint32_t olo = __reduce_or_sync(FULL, (uint32_t)o), ohi = __reduce_or_sync(FULL, (uint32_t)(o >> 32));
-  const uint32_t alo = __reduce_and_sync(FULL, (uint32_t)a), ahi = __reduce_and_sync(FULL, (uint32_t)(a >> 32));
-  if (lane_id() == 0) {
-    s_or[threadIdx.x >> 5] = ((ull)ohi << 32) | olo;
-    s_and[threadIdx.x >> 5] = ((ull)ahi << 32) | alo;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    ull bo = 0, ba = ~0ull;
-    for (int w = 0; w < kWarps; w++) { bo |= s_or[w]; ba &= s_and[w]; }
-    atomicOr(&ctl->or_all, bo);
-    atomicAnd(&ctl->and_all, ba);
-    __threadfence();
-    last = atomicAdd(&ctl->done_or, 1u) == gridDim.x - 1;
-    if (last) {
-      __threadfence();
-      const ull vary = *((volatile ull*)&ctl->or_all) ^ *((volatile ull*)&ctl->and_all);
-      const uint32_t hb = vary ? 64u - (uint32_t)__clzll((long long)vary) : 0u;
-      ctl->fshift = hb > 8u ? hb - 8u : 0u;
-      ctl->npass = vary ? 1u : 0u;
-    }
-  }
+  vary_of(o, na, ctl);
 }
 
-// Bucket path, pass 2: histogram of the bucket field; the last block writes
-// the buckets' exclusive offsets (hist[0], off[0]).
-__global__ void __launch_bounds__(kT) k_hist_field(const uint64_t* __restrict__ in, uint64_t k,
-                                                   SortCtl* ctl) {
-  __shared__ uint32_t hs[256];
-  __shared__ bool last;
-  __shared__ uint32_t wt[kWarps];
+// What a digit pass reads and writes.  p >= 0: digit p of the passes from the
+// lowest up, which take the input, then A and B alternately, arranged so that
+// the last varying one writes A (not run when the top bits and the windows
+// did the sort).  kField: the input to B by the field.  kTop0, kTop1: the
+// input to A by the 8 bits below the field, A to B by the field.
+constexpr int kField = -1, kTop0 = -2, kTop1 = -3;
+struct Pass {
+  const uint64_t* in;
+  const uint32_t* vin;
+  uint64_t *A, *B;
+  uint32_t *VA, *VB;
+  uint64_t k;
+  int p;
+  SortCtl* ctl;
+  uint32_t* cnt;  // counts, then offsets, of digit d and block b at d * gridDim.x + b
+};
+struct PassIo {
+  const uint64_t* src;
+  const uint32_t* vsrc;
+  uint64_t* dst;
+  uint32_t* vdst;
+  int shift;
+};
+// false: nothing to do
+__device__ __forceinline__ bool pass_io(const Pass& a, PassIo& io) {
+  const SortCtl& c = *a.ctl;
+  if (a.p == kField) {
+    io = PassIo{a.in, a.vin, a.B, a.VB, (int)c.fshift};
+    return c.npass != 0;
+  }
+  if (a.p == kTop0) {
+    io = PassIo{a.in, a.vin, a.A, a.VA, (int)c.fshift - 8};
+    return c.msd != 0;
+  }
+  if (a.p == kTop1) {
+    io = PassIo{a.A, a.VA, a.B, a.VB, (int)c.fshift};
+    return c.msd != 0;
+  }
+  if (!c.varying[a.p] || (c.msd && !c.over)) return false;
+  const uint32_t left = c.npass - c.rank[a.p];  // passes from this one on
+  io.src = left == c.npass ? a.in : (left & 1u) ? a.B : a.A;
+  io.vsrc = left == c.npass ? a.vin : (left & 1u) ? a.VB : a.VA;
+  io.dst = (left & 1u) ? a.A : a.B;
+  io.vdst = (left & 1u) ? a.VA : a.VB;
+  io.shift = 8 * a.p;
+  return true;
+}
+
+// Keys per digit of the block's tiles.
+__global__ void __launch_bounds__(kT) k_digit_count(Pass a) {
+  constexpr int kCopies = 4;  // histograms per block: fewer lanes on one counter
+  __shared__ uint32_t hs[kCopies][256];
   pdl_wait();
   pdl_launch();
-  hs[threadIdx.x] = 0;  // kT == 256
+  PassIo io;
+  if (!pass_io(a, io)) return;
+  for (int i = threadIdx.x; i < kCopies * 256; i += kT) (&hs[0][0])[i] = 0;
   __syncthreads();
-  const uint32_t fs = ctl->fshift;
-  const uint64_t stride = (uint64_t)gridDim.x * kT;
-  uint64_t i = (uint64_t)blockIdx.x * kT + threadIdx.x;
-  for (; i + 7 * stride < k; i += 8 * stride) {  // eight keys per thread and step
+  uint32_t* h = hs[(threadIdx.x >> 5) & (kCopies - 1)];
+  const uint64_t ntiles = (a.k + kTile - 1) / kTile;
+  const uint64_t e0 = ntiles * blockIdx.x / gridDim.x * kTile;
+  const uint64_t e1 = min(a.k, ntiles * (blockIdx.x + 1) / gridDim.x * kTile);
+  uint64_t i = e0 + threadIdx.x;
+  for (; i + 7 * kT < e1; i += 8 * kT) {
     uint64_t x[8];
 #pragma unroll
-    for (int j = 0; j < 8; j++) x[j] = in[i + j * stride];
+    for (int j = 0; j < 8; j++) x[j] = io.src[i + j * kT];
 #pragma unroll
-    for (int j = 0; j < 8; j++) atomicAdd(&hs[bucket_of(x[j], fs)], 1u);
+    for (int j = 0; j < 8; j++) atomicAdd(&h[(uint32_t)(x[j] >> io.shift) & 255u], 1u);
   }
-  for (; i < k; i += stride) atomicAdd(&hs[bucket_of(in[i], fs)], 1u);
+  for (; i < e1; i += kT) atomicAdd(&h[(uint32_t)(io.src[i] >> io.shift) & 255u], 1u);
   __syncthreads();
-  if (hs[threadIdx.x]) atomicAdd(&ctl->hist[0][threadIdx.x], hs[threadIdx.x]);
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) last = atomicAdd(&ctl->done_blocks, 1u) == gridDim.x - 1;
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  const uint32_t d = threadIdx.x;
-  const uint32_t v = *((volatile uint32_t*)&ctl->hist[0][d]);
-  const uint32_t inc = warp_incl_scan(v);
-  if (lane_id() == 31) wt[d >> 5] = inc;
-  __syncthreads();
-  uint32_t wbase = 0;
-  for (unsigned q = 0; q < (d >> 5); q++) wbase += wt[q];
-  ctl->off[0][d] = wbase + inc - v;
+  static_assert(kT == 256, "a thread per digit");
+  uint32_t n = 0;
+#pragma unroll
+  for (int q = 0; q < kCopies; q++) n += hs[q][threadIdx.x];
+  a.cnt[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = n;
 }
 
-__global__ void __launch_bounds__(kT) k_hist_all(const uint64_t* __restrict__ in, uint64_t k,
-                                                 SortCtl* ctl) {
-  __shared__ uint32_t hs[8][256];
-  __shared__ bool last;
+// Block d: the G blocks' counts of digit d to exclusive offsets among them,
+// and their total.
+__global__ void __launch_bounds__(kT) k_digit_scan(Pass a, uint32_t G) {
+  __shared__ uint32_t ws[kWarps];
   pdl_wait();
   pdl_launch();
-  for (int i = threadIdx.x; i < 8 * 256; i += kT) (&hs[0][0])[i] = 0;
-  __syncthreads();
-  for (uint64_t i = (uint64_t)blockIdx.x * kT + threadIdx.x; i < k; i += (uint64_t)gridDim.x * kT) {
-    const uint64_t x = in[i];
-#pragma unroll
-    for (int p = 0; p < 8; p++) atomicAdd(&hs[p][(uint32_t)(x >> (8 * p)) & 255u], 1u);
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < 8 * 256; i += kT) {
-    const uint32_t v = (&hs[0][0])[i];
-    if (v) atomicAdd(&(&ctl->hist[0][0])[i], v);
-  }
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) last = atomicAdd(&ctl->done_blocks, 1u) == gridDim.x - 1;
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  // last block: exclusive scans, varying digits, pass ranks
-  const int d = threadIdx.x;  // kT == 256
-  __shared__ uint32_t wt[kWarps];
-  for (int p = 0; p < 8; p++) {
-    const uint32_t v = *((volatile uint32_t*)&ctl->hist[p][d]);
+  PassIo io;
+  if (!pass_io(a, io)) return;
+  uint32_t* row = a.cnt + (size_t)blockIdx.x * G;
+  const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
+  uint32_t carry = 0;
+  for (uint32_t b0 = 0; b0 < G; b0 += kT) {
+    const uint32_t b = b0 + threadIdx.x;
+    const uint32_t v = b < G ? row[b] : 0u;
     const uint32_t inc = warp_incl_scan(v);
-    if (lane_id() == 31) wt[threadIdx.x >> 5] = inc;
+    if (lane == 31) ws[warp] = inc;
     __syncthreads();
-    uint32_t wbase = 0;
-    for (unsigned q = 0; q < (threadIdx.x >> 5); q++) wbase += wt[q];
-    ctl->off[p][d] = wbase + inc - v;
-    const int full = __syncthreads_or(v == (uint32_t)k);
-    if (d == 0) ctl->varying[p] = full ? 0u : 1u;
+    uint32_t before = carry;
+#pragma unroll
+    for (unsigned w = 0; w < kWarps; w++) {
+      if (w < warp) before += ws[w];
+      carry += ws[w];
+    }
+    if (b < G) row[b] = before + inc - v;
     __syncthreads();
   }
-  if (d == 0) {
-    uint32_t r = 0, top = 0;
-    for (int p = 0; p < 8; p++) {
-      ctl->rank[p] = r;
-      r += ctl->varying[p];
-      if (ctl->varying[p]) top = (uint32_t)p;
+  if (threadIdx.x == 0) a.ctl->tot[blockIdx.x] = carry;
+}
+
+// Partition of the tile by digit with no order among equal digits: one
+// atomic per key.
+template <bool VALS>
+__device__ __forceinline__ void tile_rank_any(const uint64_t (&key)[kItems], uint32_t nvalid,
+                                              int shift, TileSmemT<VALS>& sm) {
+  const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
+  uint32_t* cnt = sm.wcnt[0];
+  cnt[threadIdx.x] = 0;
+  __syncthreads();
+  uint32_t rank[kItems];
+#pragma unroll
+  for (int j = 0; j < kItems; j++)
+    if (warp * 32 * kItems + j * 32 + lane < nvalid)
+      rank[j] = atomicAdd(&cnt[(uint32_t)(key[j] >> shift) & 255u], 1u);
+  __syncthreads();
+  const uint32_t c = cnt[threadIdx.x], inc = warp_incl_scan(c);
+  if (lane == 31) sm.scan_tmp[warp] = inc;
+  __syncthreads();
+  uint32_t before = inc - c;
+  for (unsigned w = 0; w < warp; w++) before += sm.scan_tmp[w];
+  sm.dstart[threadIdx.x] = before;
+  __syncthreads();
+#pragma unroll
+  for (int j = 0; j < kItems; j++)
+    if (warp * 32 * kItems + j * 32 + lane < nvalid)
+      sm.keys[sm.dstart[(uint32_t)(key[j] >> shift) & 255u] + rank[j]] = key[j];
+  __syncthreads();
+}
+
+// The block's tiles in order, each ranked in shared memory and written behind
+// the block's earlier keys of every digit.
+template <bool VALS, bool STABLE>
+__global__ void __launch_bounds__(kT, 3) k_digit_scatter(Pass a) {
+  extern __shared__ __align__(16) uint8_t smem_raw[];
+  TileSmemT<VALS>& sm = *reinterpret_cast<TileSmemT<VALS>*>(smem_raw);
+  __shared__ uint32_t s_off[256];  // where the tile's keys of a digit go, less their tile index
+  __shared__ uint32_t s_ws[kWarps];
+  pdl_wait();
+  pdl_launch();
+  PassIo io;
+  if (!pass_io(a, io)) return;
+  const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
+  const uint32_t d = threadIdx.x;
+  // digit d's next position: the keys of lower digits, then those of d in
+  // earlier blocks
+  const uint32_t t = a.ctl->tot[d], inc = warp_incl_scan(t);
+  if (lane == 31) s_ws[warp] = inc;
+  __syncthreads();
+  uint32_t run = a.cnt[(size_t)d * gridDim.x + blockIdx.x] + inc - t;
+  for (unsigned w = 0; w < warp; w++) run += s_ws[w];
+  const uint64_t ntiles = (a.k + kTile - 1) / kTile;
+  const uint64_t t0 = ntiles * blockIdx.x / gridDim.x, t1 = ntiles * (blockIdx.x + 1) / gridDim.x;
+  for (uint64_t tile = t0; tile < t1; tile++) {
+    const uint64_t base = tile * kTile;
+    const uint32_t nvalid = (uint32_t)min((uint64_t)kTile, a.k - base);
+    uint64_t key[kItems];
+    uint32_t val[kItems];
+#pragma unroll
+    for (int j = 0; j < kItems; j++) {
+      const uint32_t li = warp * 32 * kItems + j * 32 + lane;
+      key[j] = li < nvalid ? io.src[base + li] : 0ull;
+      if constexpr (VALS) val[j] = li < nvalid ? io.vsrc[base + li] : 0u;
+      else val[j] = 0u;
     }
-    ctl->npass = r;
-    ctl->top = top;
+    if constexpr (STABLE) tile_rank<VALS>(key, val, nvalid, io.shift, sm);
+    else tile_rank_any<VALS>(key, nvalid, io.shift, sm);
+    s_off[d] = run - sm.dstart[d];
+    run += (d < 255 ? sm.dstart[d + 1] : nvalid) - sm.dstart[d];
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < nvalid; i += kT) {
+      const uint64_t x = sm.keys[i];
+      const uint32_t o = s_off[(uint32_t)(x >> io.shift) & 255u] + i;
+      io.dst[o] = x;
+      if constexpr (VALS) io.vdst[o] = sm.vals[i];
+    }
+    __syncthreads();  // the next tile reuses the shared arrays
   }
 }
 
@@ -312,129 +491,116 @@ __global__ void k_copy_if_no_pass(const uint64_t* __restrict__ in, uint64_t* __r
   }
 }
 
-// One digit pass.  Buffers: the input, then A and B alternately, arranged so
-// that the last varying pass writes A.  With top != 0 it is instead the
-// stable scatter of the input by the bucket field (the 8 highest varying
-// bits) into B, the buckets k_bucket_sort finishes.  Blocks take tiles in
-// order from a counter until none is left, so the grid can be smaller than
-// the tile count (a pass over a digit that does not vary costs one short
-// launch).
+// The shared memory of a block that finishes a bucket or a window.
 template <bool VALS>
-__global__ void __launch_bounds__(kT, 3) k_onesweep(const uint64_t* __restrict__ in,
-                                                 const uint32_t* __restrict__ vin,
-                                                 uint64_t* __restrict__ A, uint64_t* __restrict__ B,
-                                                 uint32_t* __restrict__ VA, uint32_t* __restrict__ VB,
-                                                 uint64_t k, int p, int top, SortCtl* ctl,
-                                                 uint32_t* __restrict__ look, Status* st,
-                                                 uint32_t spin_limit, uint32_t silent) {
-  extern __shared__ __align__(16) uint8_t smem_raw[];
-  TileSmemT<VALS>& sm = *reinterpret_cast<TileSmemT<VALS>*>(smem_raw);
-  __shared__ uint32_t s_tile;
-  __shared__ uint32_t s_excl[256];
-  pdl_wait();
-  pdl_launch();
-  const uint64_t* src;
-  uint64_t* dst;
-  const uint32_t* vsrc;
-  uint32_t* vdst;
-  uint32_t* ctr;
-  int shift;
-  if (top) {
-    if (ctl->npass == 0) return;
-    p = 0;  // the bucket field's histogram and offsets are row 0
-    shift = (int)ctl->fshift;
-    src = in;
-    dst = B;
-    vsrc = vin;
-    vdst = VB;
-    ctr = &ctl->tile_ctr[8];
-  } else {
-    if (!ctl->varying[p]) return;
-    const uint32_t r = ctl->rank[p], P = ctl->npass;
-    // pass r writes B when P-1-r is odd, else A (so pass P-1 writes A) and
-    // reads what pass r-1 wrote
-    src = (r == 0) ? in : (((P - r) & 1u) ? B : A);
-    dst = ((P - 1u - r) & 1u) ? B : A;
-    vsrc = (r == 0) ? vin : (((P - r) & 1u) ? VB : VA);
-    vdst = ((P - 1u - r) & 1u) ? VB : VA;
-    ctr = &ctl->tile_ctr[p];
-    shift = 8 * p;
-  }
+union FinishSmem {
+  TileSmemT<VALS, kBT, kBItems> tile;
+  BinSmem bins;
+};
+
+// The n <= kBTile keys at src (with their tags), all in [lo, lo + 2^bits),
+// sorted into dst: by bins when there are no tags and no bin is deep, else
+// stably digit by digit over the digits that vary among them.
+template <bool VALS>
+__device__ __forceinline__ void block_sort(const uint64_t* __restrict__ src,
+                                           const uint32_t* __restrict__ vsrc,
+                                           uint64_t* __restrict__ dst, uint32_t* __restrict__ vdst,
+                                           uint32_t n, uint64_t lo, uint32_t bits,
+                                           FinishSmem<VALS>& sm) {
+  __shared__ ull s_or, s_and;
   const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
-  const uint32_t ntiles = (uint32_t)((k + kTile - 1) / kTile);
-  for (;;) {
-    if (threadIdx.x == 0) s_tile = atomicAdd(ctr, 1u);
-    __syncthreads();
-    const uint32_t tile = s_tile;
-    if (tile >= ntiles) return;
-    const uint64_t base = (uint64_t)tile * kTile;
-    const uint32_t nvalid = (uint32_t)min((uint64_t)kTile, k - base);
-    uint64_t key[kItems];
-    uint32_t val[kItems];
+  // items per warp: the keys spread over every warp, in element order
+  const uint32_t ipw = (n + 32u * (kBT / 32) - 1u) / (32u * (kBT / 32));
+  uint64_t key[kBItems];
+  uint32_t val[kBItems];
+  uint32_t ok = 0;
+  if (threadIdx.x == 0) { s_or = 0; s_and = ~0ull; }
 #pragma unroll
-    for (int j = 0; j < kItems; j++) {
-      const uint32_t li = warp * 32 * kItems + j * 32 + lane;
-      key[j] = li < nvalid ? src[base + li] : 0ull;
-      if constexpr (VALS) val[j] = li < nvalid ? vsrc[base + li] : 0u;
-      else val[j] = 0u;
-    }
-    tile_rank<VALS>(key, val, nvalid, shift, sm);
-    // publish this tile's count per digit, then look back for the tiles before
-    const int d = threadIdx.x;
-    const uint32_t cnt = (d < 255 ? sm.dstart[d + 1] : nvalid) - sm.dstart[d];
-    volatile uint32_t* lk = look + (size_t)tile * 256;
-    const bool publish = tile != silent;  // a silent tile (tests only) never publishes
-    if (tile == 0) {
-      if (publish) lk[d] = kFlagP | cnt;
-      s_excl[d] = 0;
-    } else {
-      if (publish) lk[d] = kFlagA | cnt;
-      uint32_t excl = 0;
-      bool done = false;
-      const volatile uint32_t* lv = look;
-      // kLook predecessors are read at once (their loads in flight together),
-      // then taken in order until one with an inclusive prefix
-      for (int64_t tp = (int64_t)tile - 1; tp >= 0 && !done; tp -= kLook) {
-        uint32_t v[kLook];
+  for (int j = 0; j < kBItems; j++) {
+    const uint32_t li = warp * 32 * ipw + j * 32 + lane;
+    const bool in = (uint32_t)j < ipw && li < n;
+    key[j] = in ? src[li] : 0ull;
+    if constexpr (VALS) val[j] = in ? vsrc[li] : 0u;
+    else val[j] = 0u;
+    ok |= (uint32_t)in << j;
+  }
+  if constexpr (!VALS)
+    if (bin_sort(key, ok, n, lo, bits, sm.bins, dst)) return;
+  ull o = 0, a = ~0ull;
 #pragma unroll
-        for (int i = 0; i < kLook; i++) v[i] = tp >= i ? lv[(size_t)(tp - i) * 256 + d] : 0u;
+  for (int j = 0; j < kBItems; j++)
+    if ((ok >> j) & 1u) { o |= key[j]; a &= key[j]; }
+  __syncthreads();
+  atomicOr(&s_or, o);
+  atomicAnd(&s_and, a);
+  __syncthreads();
+  const ull vary = s_or ^ s_and;
+  for (uint32_t p = 0; p < 8; p++) {
+    if (((vary >> (8 * p)) & 255u) == 0) continue;
+    tile_rank<VALS, kBT, kBItems>(key, val, n, 8 * (int)p, sm.tile, ipw);
 #pragma unroll
-        for (int i = 0; i < kLook; i++) {
-          if (done || tp < i) break;
-          uint32_t spins = 0;
-          while (!(v[i] & (kFlagA | kFlagP)) && spins < spin_limit) {
-            v[i] = lv[(size_t)(tp - i) * 256 + d];
-            spins++;
-          }
-          if (spins >= spin_limit) {  // a predecessor never published: give up
-            atomicOr(&st->err, kErrSort);
-            done = true;
-            break;
-          }
-          excl += v[i] & kCountMask;
-          if (v[i] & kFlagP) done = true;
-        }
+    for (int j = 0; j < kBItems; j++) {
+      const uint32_t li = warp * 32 * ipw + j * 32 + lane;
+      if ((ok >> j) & 1u) {
+        key[j] = sm.tile.keys[li];
+        if constexpr (VALS) val[j] = sm.tile.vals[li];
       }
-      __threadfence();
-      if (publish) lk[d] = kFlagP | (excl + cnt);
-      s_excl[d] = excl;
     }
     __syncthreads();
-    for (uint32_t i = threadIdx.x; i < nvalid; i += kT) {
-      const uint64_t x = sm.keys[i];
-      const uint32_t dd = (uint32_t)(x >> shift) & 255u;
-      const uint64_t o = (uint64_t)ctl->off[p][dd] + s_excl[dd] + (i - sm.dstart[dd]);
-      dst[o] = x;
-      if constexpr (VALS) vdst[o] = sm.vals[i];
+  }
+#pragma unroll
+  for (int j = 0; j < kBItems; j++) {
+    const uint32_t li = warp * 32 * ipw + j * 32 + lane;
+    if ((ok >> j) & 1u) {
+      dst[li] = key[j];
+      if constexpr (VALS) vdst[li] = val[j];
     }
-    __syncthreads();  // the next tile reuses the shared arrays
   }
 }
 
-// Bucket b of the field scatter (B[off .. off + n)), sorted stably by the
-// bits below the field, into the same positions of A.  A bucket of at most
-// kBTile keys is sorted in shared memory, digit by digit over the digits
-// that vary inside it.  A larger one (heavy repeats or skew) is sorted by a
+// Large batches: B is in order by the top 16 varying bits; block t puts the
+// buckets that start among keys [4096 t, 4096 (t + 1)) into A in full order.
+constexpr uint32_t kWindowMore = kBTile - kTile;  // keys a bucket may reach past its tile
+__global__ void __launch_bounds__(kBT, 2) k_window_sort(const uint64_t* __restrict__ B,
+                                                        uint64_t* __restrict__ A, uint64_t k,
+                                                        SortCtl* ctl) {
+  extern __shared__ __align__(16) uint8_t smem_raw[];
+  FinishSmem<false>& sm = *reinterpret_cast<FinishSmem<false>*>(smem_raw);
+  __shared__ uint32_t s_at[2];
+  pdl_wait();
+  pdl_launch();
+  if (!ctl->msd) return;
+  const int sh = (int)ctl->fshift - 8;
+  if (threadIdx.x < 2) s_at[threadIdx.x] = 0xFFFFFFFFu;
+  __syncthreads();
+  // the first bucket start at or after either end of the tile, each searched
+  // by half of the block
+  const uint64_t t0 = (uint64_t)blockIdx.x * kTile;
+  const uint32_t end = threadIdx.x / (kBT / 2), ht = threadIdx.x % (kBT / 2);
+  const uint64_t from = t0 + (uint64_t)end * kTile;
+  bool found = false;  // by this half
+  for (uint32_t i0 = 0; i0 <= kWindowMore; i0 += kBT / 2) {
+    const uint64_t i = from + i0 + ht;
+    if (!found && (i == 0 || i >= k || (B[i - 1] >> sh) != (B[i] >> sh)))
+      atomicMin(&s_at[end], i0 + ht);
+    __syncthreads();
+    found = s_at[end] != 0xFFFFFFFFu;
+    if (__syncthreads_and(found)) break;
+  }
+  if (s_at[0] > kWindowMore || s_at[1] > kWindowMore) {
+    if (threadIdx.x == 0) ctl->over = 1;
+    return;
+  }
+  const uint64_t b = min(k, t0 + s_at[0]), e = min(k, t0 + kTile + s_at[1]);
+  if (e <= b) return;
+  const uint64_t lo = B[b] >> sh, hi = B[e - 1] >> sh;  // first and last bucket
+  const uint32_t bits = (uint32_t)sh + 64u - (uint32_t)__clzll((long long)(hi - lo));
+  block_sort<false>(B + b, nullptr, A + b, nullptr, (uint32_t)(e - b), lo << sh, bits, sm);
+}
+
+// Bucket b of the field scatter (B[off .. off + n)), sorted (stably when there
+// are tags) into the same positions of A: in shared memory when it holds at
+// most kBTile keys, else (heavy repeats or skew) by a
 // block-level LSD radix sort through global memory: per varying digit, one
 // counting pass over the bucket, then its tiles in order, each ranked stably
 // in shared memory and scattered to the running digit offsets, alternating
@@ -448,7 +614,8 @@ __global__ void __launch_bounds__(kBT, 2) k_bucket_sort(uint64_t* __restrict__ B
                                                      const uint32_t* __restrict__ vin,
                                                      uint64_t k) {
   extern __shared__ __align__(16) uint8_t smem_raw[];
-  TileSmemT<VALS, kBT, kBItems>& sm = *reinterpret_cast<TileSmemT<VALS, kBT, kBItems>*>(smem_raw);
+  FinishSmem<VALS>& fsm = *reinterpret_cast<FinishSmem<VALS>*>(smem_raw);
+  TileSmemT<VALS, kBT, kBItems>& sm = fsm.tile;
   __shared__ ull s_or, s_and;
   __shared__ uint32_t s_run[256];
   __shared__ uint32_t s_wt[8];
@@ -464,55 +631,26 @@ __global__ void __launch_bounds__(kBT, 2) k_bucket_sort(uint64_t* __restrict__ B
     return;
   }
   const uint32_t b = blockIdx.x;
-  const uint32_t n = ctl->hist[0][b];
+  const uint32_t n = ctl->tot[b];
   if (n == 0) return;
-  const uint64_t base = ctl->off[0][b];
-  const uint32_t npd = (ctl->fshift + 7u) / 8u;  // digits below the field
   const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
-  if (threadIdx.x == 0) { s_or = 0; s_and = ~0ull; }
+  // where the bucket starts: the keys of the buckets before it
+  if (threadIdx.x < 256) {
+    const uint32_t before = warp_sum(threadIdx.x < b ? ctl->tot[threadIdx.x] : 0u);
+    if (lane == 0) s_wt[warp] = before;
+  }
   __syncthreads();
+  uint64_t base = 0;
+#pragma unroll
+  for (int w = 0; w < 8; w++) base += s_wt[w];
+  const uint32_t npd = (ctl->fshift + 7u) / 8u;  // digits below the field
   if (n <= (uint32_t)kBTile) {
-    // items per warp: the bucket spread over every warp, in element order
-    const uint32_t ipw = (n + 32u * (kBT / 32) - 1u) / (32u * (kBT / 32));
-    uint64_t key[kBItems];
-    uint32_t val[kBItems];
-    ull o = 0, a = ~0ull;
-#pragma unroll
-    for (int j = 0; j < kBItems; j++) {
-      const uint32_t li = warp * 32 * ipw + j * 32 + lane;
-      const bool ok = (uint32_t)j < ipw && li < n;
-      key[j] = ok ? B[base + li] : 0ull;
-      if constexpr (VALS) val[j] = ok ? VB[base + li] : 0u;
-      else val[j] = 0u;
-      if (ok) { o |= key[j]; a &= key[j]; }
-    }
-    atomicOr(&s_or, o);
-    atomicAnd(&s_and, a);
-    __syncthreads();
-    const ull vary = s_or ^ s_and;
-    for (uint32_t p = 0; p < npd; p++) {
-      if (((vary >> (8 * p)) & 255u) == 0) continue;
-      tile_rank<VALS, kBT, kBItems>(key, val, n, 8 * (int)p, sm, ipw);
-#pragma unroll
-      for (int j = 0; j < kBItems; j++) {
-        const uint32_t li = warp * 32 * ipw + j * 32 + lane;
-        if ((uint32_t)j < ipw && li < n) {
-          key[j] = sm.keys[li];
-          if constexpr (VALS) val[j] = sm.vals[li];
-        }
-      }
-      __syncthreads();
-    }
-#pragma unroll
-    for (int j = 0; j < kBItems; j++) {
-      const uint32_t li = warp * 32 * ipw + j * 32 + lane;
-      if ((uint32_t)j < ipw && li < n) {
-        A[base + li] = key[j];
-        if constexpr (VALS) VA[base + li] = val[j];
-      }
-    }
+    block_sort<VALS>(B + base, VALS ? VB + base : nullptr, A + base, VALS ? VA + base : nullptr, n,
+                     (ctl->or_all >> ctl->fshift >> 8 << 8 | b) << ctl->fshift, ctl->fshift, fsm);
     return;
   }
+  if (threadIdx.x == 0) { s_or = 0; s_and = ~0ull; }
+  __syncthreads();
   // ---- oversized bucket: block-level LSD through global memory ----
   {
     ull o = 0, a = ~0ull;
@@ -681,12 +819,8 @@ __global__ void k_unique_scatter(const uint64_t* __restrict__ in, uint64_t k,
 
 namespace {
 size_t ctl_bytes() { return (sizeof(SortCtl) + 255) & ~(size_t)255; }
-size_t look_bytes(uint64_t k) {  // one array per digit pass (the bucket path uses one)
-  const uint64_t ntiles = (k + kTile - 1) / kTile;
-  return (size_t)8 * ntiles * 256 * 4;
-}
 template <bool VALS>
-int& sweep_blocks_per_sm() {
+int& scatter_blocks_per_sm() {
   static int n = 1;
   return n;
 }
@@ -695,18 +829,33 @@ void sort_attrs() {
   static bool done = false;  // one per instantiation
   if (done) return;
   const int smem = (int)sizeof(TileSmemT<VALS>);
-  cudaFuncSetAttribute(k_onesweep<VALS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaFuncSetAttribute(k_digit_scatter<VALS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       smem);
+  cudaFuncSetAttribute(k_digit_scatter<VALS, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       smem);
   cudaFuncSetAttribute(k_bucket_sort<VALS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)sizeof(TileSmemT<VALS, kBT, kBItems>));
+                       (int)sizeof(FinishSmem<VALS>));
+  cudaFuncSetAttribute(k_window_sort, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)sizeof(FinishSmem<false>));
   int bps = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_onesweep<VALS>, kT, smem) ==
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_digit_scatter<VALS, true>, kT, smem) ==
           cudaSuccess &&
       bps > 0)
-    sweep_blocks_per_sm<VALS>() = bps;
+    scatter_blocks_per_sm<VALS>() = bps;
   cudaGetLastError();
   done = true;
 }
 }  // namespace
+
+// Blocks of a digit pass over k keys: as many as run at once (the scatter
+// kernel's limit), and then the fewest that give no block more tiles.
+template <bool VALS>
+uint32_t pass_blocks(const cpma* h, uint64_t k) {
+  const uint64_t ntiles = (k + kTile - 1) / kTile;
+  const uint64_t most = (uint64_t)h->num_sms * (uint64_t)scatter_blocks_per_sm<VALS>();
+  const uint64_t per = (ntiles + most - 1) / most;
+  return (uint32_t)((ntiles + per - 1) / per);
+}
 
 int sort_scratch(cpma* h, uint64_t k, bool vals) {
   sort_attrs<false>();
@@ -717,7 +866,8 @@ int sort_scratch(cpma* h, uint64_t k, bool vals) {
   if (k <= (uint64_t)kTile) return CPMA_OK;
   CPMA_TRY(ensure(h, h->s.keysB, k * 8));
   if (vals) CPMA_TRY(ensure(h, h->s.valsB, k * 4));
-  return ensure(h, h->s.hist, ctl_bytes() + look_bytes(k));
+  const uint32_t G = vals ? pass_blocks<true>(h, k) : pass_blocks<false>(h, k);
+  return ensure(h, h->s.hist, ctl_bytes() + (size_t)G * 256 * 4);
 }
 
 template <bool VALS>
@@ -753,50 +903,49 @@ int sort_impl(cpma* h, const uint64_t* d_in, const uint32_t* v_in, uint64_t k, c
   }
   uint64_t* B = (uint64_t*)h->s.keysB.p;
   uint32_t* VB = VALS ? (uint32_t*)h->s.valsB.p : nullptr;
-  const uint32_t ntiles = (uint32_t)((k + kTile - 1) / kTile);
-  // the look-back wait's poll limit and a tile that never publishes (tests)
-  const uint32_t spin = h->sort_poll_limit ? h->sort_poll_limit : kSpinLimit;
-  const uint32_t silent = h->sort_silent_tile >= 0 && h->sort_silent_tile < (int64_t)ntiles
-                              ? (uint32_t)h->sort_silent_tile : 0xFFFFFFFFu;
   SortCtl* ctl = reinterpret_cast<SortCtl*>(h->s.hist.p);
-  uint32_t* look = reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(h->s.hist.p) + ctl_bytes());
-  const int hgrid = (int)std::min<uint64_t>((uint64_t)h->num_sms * 2, (k + kT - 1) / kT);
-  const unsigned sgrid = (unsigned)std::min<uint64_t>(
-      ntiles, (uint64_t)h->num_sms * (uint64_t)sweep_blocks_per_sm<VALS>());
+  const uint32_t G = pass_blocks<VALS>(h, k);
+  Pass a{d_in, v_in, A, B, VA, VB, k, kField, ctl,
+         reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(h->s.hist.p) + ctl_bytes())};
+  CPMA_CUDA(cudaMemsetAsync(ctl, 0, sizeof(SortCtl), st));
+  // about eight keys per thread: one step of the unrolled loop
+  const int ogrid = (int)std::max<uint64_t>(
+      1, std::min<uint64_t>((uint64_t)h->num_sms * 8, (k + 8 * kT - 1) / (8 * kT)));
+  k_orand<<<ogrid, kT, 0, st>>>(d_in, k, ctl);
+  h->launches++;
+  // each kernel after the first may be scheduled while the one before it
+  // finishes (programmatic dependent launch; each waits for it first)
+  auto pass = [&](int p, bool stable) {
+    a.p = p;
+    CPMA_CUDA(launch_pdl(k_digit_count, G, kT, 0, st, a));
+    CPMA_CUDA(launch_pdl(k_digit_scan, 256, kT, 0, st, a, G));
+    CPMA_CUDA(stable ? launch_pdl(k_digit_scatter<VALS, true>, G, kT, smem, st, a)
+                     : launch_pdl(k_digit_scatter<VALS, false>, G, kT, smem, st, a));
+    h->launches += 3;
+    return (int)CPMA_OK;
+  };
   if (k <= kBucketMax) {
-    // most significant bits first: OR / AND of the keys give the 8 highest
-    // bits that vary, their histogram, one scatter into 256 buckets by them,
-    // then every bucket sorted by the bits below in one block.  The control
-    // block and one look-back array are zeroed first (and_all starts at ~0).
-    CPMA_CUDA(cudaMemsetAsync(h->s.hist.p, 0, ctl_bytes() + (size_t)ntiles * 256 * 4, st));
-    CPMA_CUDA(cudaMemsetAsync(&ctl->and_all, 0xFF, sizeof(ull), st));
-    // about eight keys per thread: one step of the unrolled loops
-    const int ogrid = (int)std::max<uint64_t>(
-        1, std::min<uint64_t>((uint64_t)h->num_sms * 8, (k + 8 * kT - 1) / (8 * kT)));
-    // each kernel after the first may be scheduled while the one before it
-    // finishes (programmatic dependent launch; each waits for it first)
-    k_orand<<<ogrid, kT, 0, st>>>(d_in, k, ctl);
-    CPMA_CUDA(launch_pdl(k_hist_field, ogrid, kT, 0, st, d_in, k, ctl));
-    CPMA_CUDA(launch_pdl(k_onesweep<VALS>, sgrid, kT, smem, st, d_in, v_in, A, B, VA, VB, k, 0, 1,
-                         ctl, look, h->d_status, spin, silent));
-    CPMA_CUDA(launch_pdl(k_bucket_sort<VALS>, 256, kBT, sizeof(TileSmemT<VALS, kBT, kBItems>), st,
-                         B, VB, A, VA, ctl, d_in, v_in, k));
-    h->launches += 4;
-    // OR/AND and histogram reads, scatter and bucket read + write
+    CPMA_TRY(pass(kField, VALS));
+    CPMA_CUDA(launch_pdl(k_bucket_sort<VALS>, 256, kBT, sizeof(FinishSmem<VALS>), st, B, VB, A, VA,
+                         ctl, d_in, v_in, k));
+    h->launches++;
+    // OR/AND and count reads, scatter and bucket read + write
     prof_add_bytes(h, PH_SORT, 16ull * k + (VALS ? 24ull : 16ull) * k * 2);
   } else {
-    // least significant digit first over the digits that vary
-    CPMA_CUDA(cudaMemsetAsync(h->s.hist.p, 0, ctl_bytes() + look_bytes(k), st));
-    k_hist_all<<<hgrid, kT, 0, st>>>(d_in, k, ctl);
-    h->launches++;
-    prof_add_bytes(h, PH_SORT, 8ull * k);  // the histogram read
-    for (int p = 0; p < 8; p++) {
-      // digits that vary: the scatter reads and writes keys (and tags)
-      CPMA_CUDA(launch_pdl(k_onesweep<VALS>, sgrid, kT, smem, st, d_in, v_in, A, B, VA, VB, k, p,
-                           0, ctl, look + (size_t)p * ntiles * 256, h->d_status, spin, silent));
+    if (!VALS) {
+      CPMA_TRY(pass(kTop0, false));
+      CPMA_TRY(pass(kTop1, true));
+      CPMA_CUDA(launch_pdl(k_window_sort, (unsigned)((k + kTile - 1) / kTile), kBT,
+                           sizeof(FinishSmem<false>), st, B, A, k, ctl));
       h->launches++;
+      prof_add_bytes(h, PH_SORT, 72ull * k);
+    } else {
+      CPMA_CUDA(cudaMemsetAsync(&ctl->over, 1, 1, st));
+      prof_add_bytes(h, PH_SORT, 8ull * k + 32ull * k * 5);  // typical: 5 varying digits
     }
-    prof_add_bytes(h, PH_SORT, (VALS ? 24ull : 16ull) * k * 5);  // typical: 5 varying digits
+    // the digits that vary, lowest first: with tags, when few bits vary, or
+    // when a window gave up
+    for (int p = 0; p < 8; p++) CPMA_TRY(pass(p, true));
     CPMA_CUDA(launch_pdl(k_copy_if_no_pass,
                          (unsigned)std::min<uint64_t>((uint64_t)h->num_sms * 4, (k + kT - 1) / kT),
                          kT, 0, st, d_in, A, v_in, VA, k, ctl));

@@ -3045,7 +3045,7 @@ constexpr int kSigPtrs = 34;
 struct FrontSig {
   const void* p[kSigPtrs];
   uint64_t L, LB;
-  uint32_t poll;    // sort look-back poll limit and silent tile (tests)
+  uint32_t poll;    // routing look-back poll limit and silent tile (tests)
   int64_t silent;
   bool operator==(const FrontSig& o) const {
     if (L != o.L || LB != o.LB || poll != o.poll || silent != o.silent) return false;
@@ -3361,7 +3361,7 @@ int run_rebuild(cpma* h, const uint64_t* d_keys, uint64_t k, int sorted, int is_
   CPMA_CUDA(cudaGetLastError());
   CPMA_TRY(sync_status(h, st));
   Status hs = *h->h_status;
-  if (hs.err & (kErrSort | kErrRoute)) return CPMA_ETIMEOUT;
+  if (hs.err & kErrRoute) return CPMA_ETIMEOUT;
   if (hs.err & kErrUnsorted) return CPMA_EINVAL;
   if (hs.err) return CPMA_EINTERNAL;
   CPMA_TRY(build_from_sorted_unique(h, P<uint64_t>(s.E), hs.nelem, st));
@@ -3562,7 +3562,7 @@ int run_update(cpma* h, const uint64_t* d_keys, uint64_t k, int sorted, int is_d
   CPMA_TRY(sync_status(h, st));
   prof_begin(h, PH_COUNT, st);
   Status hs = *h->h_status;
-  if (hs.err & (kErrSort | kErrRoute)) return CPMA_ETIMEOUT;
+  if (hs.err & kErrRoute) return CPMA_ETIMEOUT;
   if (hs.err & kErrUnsorted) return CPMA_EINVAL;
   if (hs.err) return CPMA_EINTERNAL;
   const uint64_t t_merged = hs.bytes_total;  // exact: every leaf changed by the merge counted
