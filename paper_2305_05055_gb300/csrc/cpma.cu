@@ -3,6 +3,7 @@
 #include <algorithm>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <new>
 
 #include "internal.h"
@@ -89,23 +90,31 @@ void release(cpma* h, Buf& b) {
 // reads whole 4-byte words, which may reach up to 3 bytes past the last leaf.
 constexpr uint64_t kLeafPad = 16;
 
+// One block of memory for the four arrays (an allocation costs 30 us and its
+// release as much): the leaf bytes, then the head index, the used bytes and
+// the counts, each 256-byte aligned.
+uint64_t up256(uint64_t x) { return (x + 255) & ~(uint64_t)255; }
+uint64_t arrays_bytes(uint64_t leaves, uint64_t data_bytes) {
+  return up256(data_bytes + kLeafPad) + up256((leaves + 1) * 8) + 2 * up256(leaves * 4);
+}
+
 int alloc_arrays(cpma* h, uint64_t leaves, uint64_t data_bytes, Arrays* a, cudaStream_t st) {
   *a = Arrays{};
-  int rc = dev_alloc(h, (void**)&a->data, data_bytes + kLeafPad, st);
-  if (rc == CPMA_OK) rc = dev_alloc(h, (void**)&a->used, leaves * 4, st);
-  if (rc == CPMA_OK) rc = dev_alloc(h, (void**)&a->cnt, leaves * 4, st);
-  if (rc == CPMA_OK) rc = dev_alloc(h, (void**)&a->heads, (leaves + 1) * 8, st);
+  uint8_t* p = nullptr;
+  CPMA_TRY(dev_alloc(h, (void**)&p, arrays_bytes(leaves, data_bytes), st));
+  a->data = p;
+  p += up256(data_bytes + kLeafPad);
+  a->heads = reinterpret_cast<uint64_t*>(p);
+  p += up256((leaves + 1) * 8);
+  a->used = reinterpret_cast<uint32_t*>(p);
+  a->cnt = reinterpret_cast<uint32_t*>(p + up256(leaves * 4));
   a->cap_leaves = leaves;
   a->cap_bytes = data_bytes;
-  if (rc != CPMA_OK) free_arrays(h, a);
-  return rc;
+  return CPMA_OK;
 }
 
 void free_arrays(cpma* h, Arrays* a) {
-  if (a->data) dev_free(h, a->data, a->cap_bytes + kLeafPad, nullptr);
-  dev_free(h, a->used, a->cap_leaves * 4, nullptr);
-  dev_free(h, a->cnt, a->cap_leaves * 4, nullptr);
-  dev_free(h, a->heads, (a->cap_leaves + 1) * 8, nullptr);
+  if (a->data) dev_free(h, a->data, arrays_bytes(a->cap_leaves, a->cap_bytes), nullptr);
   *a = Arrays{};
 }
 
@@ -259,6 +268,40 @@ void prof_push(const cpma* hc, const Prof::Rec* recs, int n, const unsigned long
 
 namespace {
 
+// Pinned status blocks of destroyed handles, kept for the next ones (pinning
+// and unpinning one took 250 us of a build of 3e7 keys): at most kPinned of
+// them, 256 bytes each; more go back at once.  A block belongs to no device,
+// stream or handle while it is here.
+constexpr int kPinned = 64;
+std::mutex g_pinned_mu;
+Status* g_pinned[kPinned];
+int g_npinned = 0;
+
+Status* take_pinned() {
+  {
+    std::lock_guard<std::mutex> lock(g_pinned_mu);
+    if (g_npinned) return g_pinned[--g_npinned];
+  }
+  void* p = nullptr;
+  if (cudaHostAlloc(&p, sizeof(Status), cudaHostAllocPortable) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  return static_cast<Status*>(p);
+}
+
+void give_pinned(Status* p) {
+  if (!p) return;
+  {
+    std::lock_guard<std::mutex> lock(g_pinned_mu);
+    if (g_npinned < kPinned) {
+      g_pinned[g_npinned++] = p;
+      return;
+    }
+  }
+  cudaFreeHost(p);
+}
+
 int validate(const cpma_config& c) {
   if (c.leaf_bytes < 256 || c.leaf_bytes > 2048 || c.leaf_bytes % 16) return CPMA_EINVAL;
   if (!(c.rho_leaf <= c.rho_root && c.rho_root < c.tau_root && c.tau_root <= c.tau_leaf &&
@@ -275,7 +318,7 @@ int validate(const cpma_config& c) {
 
 void release_all(cpma* h) {
   Scratch& s = h->s;
-  for (Buf* b : {&s.keysA, &s.keysB, &s.valsA, &s.valsB, &s.hist, &s.flags, &s.flags_scan, &s.leaf_of,
+  for (Buf* b : {&s.keysA, &s.keysB, &s.valsA, &s.valsB, &s.hist, &s.flags, &s.flags_scan,
                  &s.chunk_begin, &s.chunk_leaf, &s.chunk_tid, &s.chunk_cnt, &s.chunk_off,
                  &s.T_leaf, &s.T_begin, &s.T_first_chunk, &s.T_oldcnt, &s.T_oldused, &s.T_newcnt,
                  &s.T_newbytes, &s.T_state, &s.viol, &s.list_lane, &s.list_v1, &s.list_gen, &s.list_pend, &s.point_stage, &s.point_rec, &s.cand,
@@ -296,7 +339,7 @@ void release_all(cpma* h) {
   free_arrays(h, &cur);
   free_arrays(h, &h->spare);
   dev_free(h, h->d_status, sizeof(Status), nullptr);
-  if (h->h_status) cudaFreeHost(h->h_status);
+  give_pinned(h->h_status);
   prof_resolve(h);
   for (int i = 0; i < h->prof.npool; i++) cudaEventDestroy(h->prof.pool[i]);
   delete[] h->prof.pool;
@@ -339,8 +382,8 @@ int new_handle(const cpma_config* cfg, cpma** out) {
     delete h;
     return rc;
   }
-  if (cudaMallocHost(&h->h_status, sizeof(Status)) != cudaSuccess) {
-    cudaGetLastError();
+  h->h_status = take_pinned();
+  if (!h->h_status) {
     release_all(h);
     delete h;
     return CPMA_ENOMEM;
@@ -386,20 +429,19 @@ int cpma_create(cpma_t** out, const cpma_config* cfg, const uint64_t* d_keys, ui
   cudaStream_t st = (cudaStream_t)stream;
   int rc = CPMA_OK;
   do {
-    rc = ensure(h, h->s.E, (n + 1) * 8);
+    const uint64_t* sorted = d_keys;
+    const uint32_t* over = nullptr;
+    rc = sort_keys_most(h, d_keys, n, &sorted, &over, st);
     if (rc) break;
-    uint64_t nu = 0;
-    if (n) {
-      const uint64_t* sorted = nullptr;
-      rc = sort_keys(h, d_keys, n, &sorted, st);
+    rc = build_measure(h, sorted, n, over, st);
+    if (rc) break;
+    if (h->h_status->sort_over) {
+      rc = sort_keys_rest(h, d_keys, n, st);
       if (rc) break;
-      rc = unique_keys(h, sorted, n, (uint64_t*)h->s.E.p, st);
+      rc = build_measure(h, sorted, n, nullptr, st);
       if (rc) break;
-      rc = sync_status(h, st);
-      if (rc) break;
-      nu = h->h_status->nunique;
     }
-    rc = build_from_sorted_unique(h, (const uint64_t*)h->s.E.p, nu, st);
+    rc = build_from_sorted(h, sorted, n, st);
   } while (0);
   if (rc != CPMA_OK) {
     cudaStreamSynchronize(st);

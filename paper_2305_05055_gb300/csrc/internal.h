@@ -61,7 +61,7 @@ struct Status {
   ull mask_or;     // OR / AND of the batch keys (radix pass selection)
   ull mask_and;
   ull nelem;       // elements moved by the current redistribution
-  ull nunique;     // distinct keys after sort+dedup (create)
+  ull nunique;     // distinct keys (create)
   ull stream_bytes;// bytes of the build stream (create)
   ull n_lane;      // touched leaves for the lane-granular insert
   ull n_v1;        // touched leaves for the element-array splice
@@ -69,7 +69,8 @@ struct Status {
   ull n_pendl;     // pending leaves left by the thread- and lane-granular inserts
   ull point_fb;    // point path: touched leaves that need the batch algorithm
   ull point_done;  // point path: blocks finished (the last one finishes the pass)
-  ull pad[7];
+  ull sort_over;   // create: the windows of the batch sort did not hold its buckets
+  ull pad[6];
   ull empties;     // empty leaves in the structure (written by the head
                    // fix-up; not cleared at the start of a batch)
   ull bytes_total; // used bytes over all leaves, kept exact by the merge,
@@ -109,8 +110,7 @@ struct Scratch {
   Buf valsA, valsB;       // sort ping-pong of 32-bit tags
   Buf hist;               // sort control block, digit counts per block
   Buf flags;              // routing: tile counter and look-back words (u64)
-  Buf flags_scan;         // build and rebuild: scanned flags (u64)
-  Buf leaf_of;            // build: unique flags (u32)
+  Buf flags_scan;         // rebuild: scanned flags (u64)
   Buf chunk_begin, chunk_leaf, chunk_tid, chunk_cnt, chunk_off;
   Buf T_leaf, T_begin, T_first_chunk, T_oldcnt, T_oldused, T_newcnt, T_newbytes, T_state;
   Buf viol, cand, wins;   // violating leaves, window candidates, windows
@@ -262,8 +262,13 @@ int sort_keys(cpma* h, const uint64_t* d_in, uint64_t k, const uint64_t** out,
 // the same, moving a 32-bit payload with every key (stable)
 int sort_pairs(cpma* h, const uint64_t* d_in, const uint32_t* v_in, uint64_t k,
                const uint64_t** out, const uint32_t** vout, cudaStream_t st);
-// sort.cu: drop adjacent repeats of sorted keys; result count into status->nunique.
-int unique_keys(cpma* h, const uint64_t* in, uint64_t k, uint64_t* out, cudaStream_t st);
+// sort.cu: sort_keys without the passes that a large batch needs only when a
+// window did not hold its buckets: *over (device; null when there is nothing
+// to decide) is then not zero once the work queued here is done, and
+// sort_keys_rest must follow.
+int sort_keys_most(cpma* h, const uint64_t* d_in, uint64_t k, const uint64_t** out,
+                   const uint32_t** over, cudaStream_t st);
+int sort_keys_rest(cpma* h, const uint64_t* d_in, uint64_t k, cudaStream_t st);
 
 // update.cu
 // tags / tag_counts (nullable): per key a request tag; every key that the
@@ -272,7 +277,8 @@ int unique_keys(cpma* h, const uint64_t* in, uint64_t k, uint64_t* out, cudaStre
 int run_update(cpma* h, const uint64_t* d_keys, uint64_t k, int sorted, int is_delete,
                uint64_t* d_delta, cudaStream_t st, const uint32_t* tags = nullptr,
                uint64_t* tag_counts = nullptr, uint64_t ntags = 0);
-int build_from_sorted_unique(cpma* h, const uint64_t* E, uint64_t n, cudaStream_t st);
+int build_measure(cpma* h, const uint64_t* x, uint64_t n, const uint32_t* over, cudaStream_t st);
+int build_from_sorted(cpma* h, const uint64_t* x, uint64_t n, cudaStream_t st);
 
 // query.cu
 int run_has(const cpma* h, const uint64_t* d_keys, uint64_t q, uint8_t* d_out, cudaStream_t st);

@@ -224,7 +224,8 @@ struct SortCtl {
   uint32_t fshift;         // the field: bits [fshift, fshift + 8), the highest that vary
   uint32_t done;           // OR/AND blocks finished
   uint32_t msd;            // large batch: top 16 varying bits, then windows
-  uint32_t over;           // a window did not hold its buckets: all digits after all
+  uint32_t rest;           // the passes over all digits are needed: few bits vary, or a
+                           // window did not hold its buckets
   uint32_t pad;
   ull or_all, nand_all;    // OR of the keys and of their complements
 };
@@ -232,8 +233,9 @@ struct SortCtl {
 // The thread's OR of its keys and of their complements over the batch; the
 // last of the grid's blocks turns the bits that vary into the bucket field
 // (the 8 highest of them), the varying digits and their number (0 when every
-// key is equal).  A whole block must call.
-__device__ __forceinline__ void vary_of(ull o, ull na, SortCtl* ctl) {
+// key is equal); `digits`: by the digit passes whatever varies (tags).  A whole
+// block must call.
+__device__ __forceinline__ void vary_of(ull o, ull na, SortCtl* ctl, bool digits) {
   __shared__ ull s_or[kWarps], s_na[kWarps];
   const uint32_t olo = __reduce_or_sync(FULL, (uint32_t)o), ohi = __reduce_or_sync(FULL, (uint32_t)(o >> 32));
   const uint32_t alo = __reduce_or_sync(FULL, (uint32_t)na), ahi = __reduce_or_sync(FULL, (uint32_t)(na >> 32));
@@ -261,14 +263,16 @@ __device__ __forceinline__ void vary_of(ull o, ull na, SortCtl* ctl) {
         r += v;
       }
       ctl->npass = r;
-      ctl->msd = hb > 24u ? 1u : 0u;
+      const bool msd = hb > 24u && !digits;
+      ctl->msd = msd ? 1u : 0u;
+      ctl->rest = msd ? 0u : 1u;
     }
   }
 }
 
 // Bucket path, first kernel: the bits that vary.
 __global__ void __launch_bounds__(kT) k_orand(const uint64_t* __restrict__ in, uint64_t k,
-                                              SortCtl* ctl) {
+                                              SortCtl* ctl, bool digits) {
   pdl_wait();
   pdl_launch();
   ull o = 0, na = 0;
@@ -287,7 +291,7 @@ __global__ void __launch_bounds__(kT) k_orand(const uint64_t* __restrict__ in, u
     o |= x;
     na |= ~x;
   }
-  vary_of(o, na, ctl);
+  vary_of(o, na, ctl, digits);
 }
 
 // What a digit pass reads and writes.  p >= 0: digit p of the passes from the
@@ -328,7 +332,7 @@ __device__ __forceinline__ bool pass_io(const Pass& a, PassIo& io) {
     io = PassIo{a.A, a.VA, a.B, a.VB, (int)c.fshift};
     return c.msd != 0;
   }
-  if (!c.varying[a.p] || (c.msd && !c.over)) return false;
+  if (!c.varying[a.p] || !c.rest) return false;
   const uint32_t left = c.npass - c.rank[a.p];  // passes from this one on
   io.src = left == c.npass ? a.in : (left & 1u) ? a.B : a.A;
   io.vsrc = left == c.npass ? a.vin : (left & 1u) ? a.VB : a.VA;
@@ -588,7 +592,7 @@ __global__ void __launch_bounds__(kBT, 2) k_window_sort(const uint64_t* __restri
     if (__syncthreads_and(found)) break;
   }
   if (s_at[0] > kWindowMore || s_at[1] > kWindowMore) {
-    if (threadIdx.x == 0) ctl->over = 1;
+    if (threadIdx.x == 0) ctl->rest = 1;
     return;
   }
   const uint64_t b = min(k, t0 + s_at[0]), e = min(k, t0 + kTile + s_at[1]);
@@ -797,24 +801,6 @@ __global__ void __launch_bounds__(kRankT) k_sort_rank(const uint64_t* __restrict
   }
 }
 
-__global__ void k_unique_flags(const uint64_t* __restrict__ in, uint64_t k,
-                               uint32_t* __restrict__ flags) {
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < k;
-       i += (uint64_t)gridDim.x * blockDim.x)
-    flags[i] = (i == 0 || in[i] != in[i - 1]) ? 1u : 0u;
-}
-
-__global__ void k_unique_scatter(const uint64_t* __restrict__ in, uint64_t k,
-                                 const uint32_t* __restrict__ flags,
-                                 const uint64_t* __restrict__ pos, uint64_t* __restrict__ out,
-                                 Status* st) {
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < k;
-       i += (uint64_t)gridDim.x * blockDim.x) {
-    if (flags[i]) out[pos[i]] = in[i];
-    if (i == k - 1) st->nunique = pos[k];
-  }
-}
-
 }  // namespace
 
 namespace {
@@ -871,15 +857,52 @@ int sort_scratch(cpma* h, uint64_t k, bool vals) {
 }
 
 template <bool VALS>
+Pass pass_of(cpma* h, const uint64_t* d_in, const uint32_t* v_in, uint64_t k) {
+  Scratch& s = h->s;
+  uint8_t* ctl = reinterpret_cast<uint8_t*>(s.hist.p);
+  return Pass{d_in, v_in, (uint64_t*)s.keysA.p, (uint64_t*)s.keysB.p,
+              VALS ? (uint32_t*)s.valsA.p : nullptr, VALS ? (uint32_t*)s.valsB.p : nullptr, k, 0,
+              reinterpret_cast<SortCtl*>(ctl), reinterpret_cast<uint32_t*>(ctl + ctl_bytes())};
+}
+
+// The three kernels of a digit pass, each scheduled while the one before it
+// finishes (programmatic dependent launch; each waits for it first).
+template <bool VALS>
+int digit_pass(cpma* h, Pass a, uint32_t G, int p, bool stable, cudaStream_t st) {
+  const size_t smem = sizeof(TileSmemT<VALS>);
+  a.p = p;
+  CPMA_CUDA(launch_pdl(k_digit_count, G, kT, 0, st, a));
+  CPMA_CUDA(launch_pdl(k_digit_scan, 256, kT, 0, st, a, G));
+  CPMA_CUDA(stable ? launch_pdl(k_digit_scatter<VALS, true>, G, kT, smem, st, a)
+                   : launch_pdl(k_digit_scatter<VALS, false>, G, kT, smem, st, a));
+  h->launches += 3;
+  return CPMA_OK;
+}
+
+// A large batch by the digits that vary, lowest first: with tags, when few
+// bits vary, or when a window gave up (the kernels return at once otherwise).
+template <bool VALS>
+int sort_digits(cpma* h, const uint64_t* d_in, const uint32_t* v_in, uint64_t k, cudaStream_t st) {
+  const Pass a = pass_of<VALS>(h, d_in, v_in, k);
+  const uint32_t G = pass_blocks<VALS>(h, k);
+  for (int p = 0; p < 8; p++) CPMA_TRY(digit_pass<VALS>(h, a, G, p, true, st));
+  CPMA_CUDA(launch_pdl(k_copy_if_no_pass,
+                       (unsigned)std::min<uint64_t>((uint64_t)h->num_sms * 4, (k + kT - 1) / kT),
+                       kT, 0, st, d_in, a.A, v_in, a.VA, k, a.ctl));
+  h->launches++;
+  return CPMA_OK;
+}
+
+// most: a large batch without sort_digits (the caller looks at ctl->rest)
+template <bool VALS>
 int sort_impl(cpma* h, const uint64_t* d_in, const uint32_t* v_in, uint64_t k, const uint64_t** out,
-              const uint32_t** vout, cudaStream_t st) {
+              const uint32_t** vout, cudaStream_t st, bool most = false) {
   *out = d_in;
   if (vout) *vout = v_in;
   if (k <= 1) return CPMA_OK;
   CPMA_TRY(sort_scratch(h, k, VALS));
   uint64_t* A = (uint64_t*)h->s.keysA.p;
   uint32_t* VA = VALS ? (uint32_t*)h->s.valsA.p : nullptr;
-  const size_t smem = sizeof(TileSmemT<VALS>);
   if (!VALS && k <= (uint64_t)kTile) {
     prof_add_bytes(h, PH_SORT, 16ull * k);
     uint32_t n = 2;
@@ -905,27 +928,15 @@ int sort_impl(cpma* h, const uint64_t* d_in, const uint32_t* v_in, uint64_t k, c
   uint32_t* VB = VALS ? (uint32_t*)h->s.valsB.p : nullptr;
   SortCtl* ctl = reinterpret_cast<SortCtl*>(h->s.hist.p);
   const uint32_t G = pass_blocks<VALS>(h, k);
-  Pass a{d_in, v_in, A, B, VA, VB, k, kField, ctl,
-         reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(h->s.hist.p) + ctl_bytes())};
+  const Pass a = pass_of<VALS>(h, d_in, v_in, k);
   CPMA_CUDA(cudaMemsetAsync(ctl, 0, sizeof(SortCtl), st));
   // about eight keys per thread: one step of the unrolled loop
   const int ogrid = (int)std::max<uint64_t>(
       1, std::min<uint64_t>((uint64_t)h->num_sms * 8, (k + 8 * kT - 1) / (8 * kT)));
-  k_orand<<<ogrid, kT, 0, st>>>(d_in, k, ctl);
+  k_orand<<<ogrid, kT, 0, st>>>(d_in, k, ctl, VALS);
   h->launches++;
-  // each kernel after the first may be scheduled while the one before it
-  // finishes (programmatic dependent launch; each waits for it first)
-  auto pass = [&](int p, bool stable) {
-    a.p = p;
-    CPMA_CUDA(launch_pdl(k_digit_count, G, kT, 0, st, a));
-    CPMA_CUDA(launch_pdl(k_digit_scan, 256, kT, 0, st, a, G));
-    CPMA_CUDA(stable ? launch_pdl(k_digit_scatter<VALS, true>, G, kT, smem, st, a)
-                     : launch_pdl(k_digit_scatter<VALS, false>, G, kT, smem, st, a));
-    h->launches += 3;
-    return (int)CPMA_OK;
-  };
   if (k <= kBucketMax) {
-    CPMA_TRY(pass(kField, VALS));
+    CPMA_TRY(digit_pass<VALS>(h, a, G, kField, VALS, st));
     CPMA_CUDA(launch_pdl(k_bucket_sort<VALS>, 256, kBT, sizeof(FinishSmem<VALS>), st, B, VB, A, VA,
                          ctl, d_in, v_in, k));
     h->launches++;
@@ -933,23 +944,16 @@ int sort_impl(cpma* h, const uint64_t* d_in, const uint32_t* v_in, uint64_t k, c
     prof_add_bytes(h, PH_SORT, 16ull * k + (VALS ? 24ull : 16ull) * k * 2);
   } else {
     if (!VALS) {
-      CPMA_TRY(pass(kTop0, false));
-      CPMA_TRY(pass(kTop1, true));
+      CPMA_TRY(digit_pass<VALS>(h, a, G, kTop0, false, st));
+      CPMA_TRY(digit_pass<VALS>(h, a, G, kTop1, true, st));
       CPMA_CUDA(launch_pdl(k_window_sort, (unsigned)((k + kTile - 1) / kTile), kBT,
                            sizeof(FinishSmem<false>), st, B, A, k, ctl));
       h->launches++;
       prof_add_bytes(h, PH_SORT, 72ull * k);
     } else {
-      CPMA_CUDA(cudaMemsetAsync(&ctl->over, 1, 1, st));
       prof_add_bytes(h, PH_SORT, 8ull * k + 32ull * k * 5);  // typical: 5 varying digits
     }
-    // the digits that vary, lowest first: with tags, when few bits vary, or
-    // when a window gave up
-    for (int p = 0; p < 8; p++) CPMA_TRY(pass(p, true));
-    CPMA_CUDA(launch_pdl(k_copy_if_no_pass,
-                         (unsigned)std::min<uint64_t>((uint64_t)h->num_sms * 4, (k + kT - 1) / kT),
-                         kT, 0, st, d_in, A, v_in, VA, k, ctl));
-    h->launches++;
+    if (!most) CPMA_TRY(sort_digits<VALS>(h, d_in, v_in, k, st));
   }
   CPMA_CUDA(cudaGetLastError());
   const uint64_t* src = A;
@@ -969,22 +973,16 @@ int sort_pairs(cpma* h, const uint64_t* d_in, const uint32_t* v_in, uint64_t k,
   return sort_impl<true>(h, d_in, v_in, k, out, vout, st);
 }
 
-int unique_keys(cpma* h, const uint64_t* in, uint64_t k, uint64_t* out, cudaStream_t st) {
-  if (k == 0) {
-    CPMA_CUDA(cudaMemsetAsync(&h->d_status->nunique, 0, 8, st));
-    return CPMA_OK;
-  }
-  CPMA_TRY(ensure(h, h->s.leaf_of, k * 4));
-  CPMA_TRY(ensure(h, h->s.flags_scan, (k + 1) * 8));
-  uint32_t* flags = (uint32_t*)h->s.leaf_of.p;
-  uint64_t* pos = (uint64_t*)h->s.flags_scan.p;
-  const int grid = (int)std::min<uint64_t>((uint64_t)h->num_sms * 8, (k + 255) / 256);
-  k_unique_flags<<<grid, 256, 0, st>>>(in, k, flags);
-  h->launches++;
-  CPMA_TRY(scan_u32_to_u64(h, flags, pos, k, nullptr, st));
-  k_unique_scatter<<<grid, 256, 0, st>>>(in, k, flags, pos, out, h->d_status);
-  h->launches++;
-  return check_cuda(cudaGetLastError());
+int sort_keys_most(cpma* h, const uint64_t* d_in, uint64_t k, const uint64_t** out,
+                   const uint32_t** over, cudaStream_t st) {
+  *over = nullptr;
+  CPMA_TRY(sort_impl<false>(h, d_in, nullptr, k, out, nullptr, st, true));
+  if (k > kBucketMax) *over = &reinterpret_cast<SortCtl*>(h->s.hist.p)->rest;
+  return CPMA_OK;
+}
+
+int sort_keys_rest(cpma* h, const uint64_t* d_in, uint64_t k, cudaStream_t st) {
+  return sort_digits<false>(h, d_in, nullptr, k, st);
 }
 
 }  // namespace cpmaimpl

@@ -2733,6 +2733,287 @@ __global__ void __launch_bounds__(kT) k_rebuild_scatter(const uint64_t* __restri
   }
 }
 
+// ---- the constructor ----
+//
+// From sorted keys (repeats allowed) straight to leaves, without a compacted
+// copy, element costs or their prefix in memory: one pass adds up the distinct
+// keys and the bytes of their stream per block (k_build_sum), which give the
+// leaf count; a second one prefixes the bytes again tile by tile and finds the
+// key each leaf starts at (k_build_cuts); a warp per leaf then writes it
+// (k_build_encode).  A repeat costs no bytes and is skipped wherever it falls.
+// Two reads of the keys and one of them with the leaves' bytes out; flags,
+// their scan, a compaction, costs, their scan and a search per leaf took 820
+// us of 3e7 keys, these three 320 us.
+constexpr int kBuildItems = 8;
+constexpr uint32_t kBuildTile = kT * kBuildItems;  // keys per block step
+
+struct BuildArgs {
+  const uint64_t* x;  // sorted keys
+  uint64_t n;
+  uint64_t* part;     // per block: distinct keys before it, bytes before it (2 x (G + 1))
+  uint64_t L, S;      // leaves, bytes of the stream
+  uint64_t* dstart;   // per leaf: its first key
+  int raw;
+};
+
+// Bytes of the thread's kBuildItems consecutive keys from i0 on in the stream
+// (8 for the first key of all and for every cell, 0 for a repeat and past the
+// end); returns their distinct ones.  prev: the key before i0.
+__device__ __forceinline__ uint32_t build_costs(const BuildArgs& a, uint64_t i0,
+                                                const uint64_t (&x)[kBuildItems], uint64_t prev,
+                                                uint32_t (&c)[kBuildItems]) {
+  uint32_t n = 0;
+#pragma unroll
+  for (int q = 0; q < kBuildItems; q++) {
+    const uint64_t i = i0 + q;
+    const uint64_t p = q ? x[q - 1] : prev;
+    const bool keep = i < a.n && (i == 0 || x[q] != p);
+    c[q] = !keep ? 0u : (i == 0 || a.raw) ? 8u : leb_len(x[q] - p);
+    n += keep;
+  }
+  return n;
+}
+
+// The thread's keys of the tile at t0, and the one before them.
+__device__ __forceinline__ void build_load(const BuildArgs& a, uint64_t t0,
+                                           uint64_t (&x)[kBuildItems], uint64_t& prev) {
+  const uint64_t i0 = t0 + (uint64_t)threadIdx.x * kBuildItems;
+  if (i0 + kBuildItems <= a.n && (reinterpret_cast<uintptr_t>(a.x) & 15u) == 0) {
+#pragma unroll
+    for (int q = 0; q < kBuildItems; q += 2) {
+      const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(a.x + i0 + q);
+      x[q] = v.x;
+      x[q + 1] = v.y;
+    }
+  } else {
+#pragma unroll
+    for (int q = 0; q < kBuildItems; q++) x[q] = i0 + q < a.n ? a.x[i0 + q] : 0ull;
+  }
+  prev = __shfl_up_sync(FULL, x[kBuildItems - 1], 1);
+  if (lane_id() == 0) prev = i0 && i0 < a.n ? a.x[i0 - 1] : 0ull;
+}
+
+// Tiles [t0, t1) of this block.
+__device__ __forceinline__ void build_tiles(const BuildArgs& a, uint64_t& t0, uint64_t& t1) {
+  const uint64_t nt = (a.n + kBuildTile - 1) / kBuildTile;
+  t0 = nt * blockIdx.x / gridDim.x;
+  t1 = nt * (blockIdx.x + 1) / gridDim.x;
+}
+
+__global__ void __launch_bounds__(kT) k_build_sum(BuildArgs a) {
+  __shared__ uint64_t s_n[kT / 32], s_b[kT / 32];
+  pdl_wait();
+  pdl_launch();
+  uint64_t t0, t1;
+  build_tiles(a, t0, t1);
+  uint64_t n = 0, b = 0;
+  for (uint64_t t = t0; t < t1; t++) {
+    uint64_t x[kBuildItems], prev;
+    uint32_t c[kBuildItems];
+    build_load(a, t * kBuildTile, x, prev);
+    n += build_costs(a, t * kBuildTile + (uint64_t)threadIdx.x * kBuildItems, x, prev, c);
+#pragma unroll
+    for (int q = 0; q < kBuildItems; q++) b += c[q];
+  }
+  n = warp_sum(n);
+  b = warp_sum(b);
+  if (lane_id() == 0) {
+    s_n[threadIdx.x >> 5] = n;
+    s_b[threadIdx.x >> 5] = b;
+  }
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    n = warp_sum(threadIdx.x < kT / 32 ? s_n[threadIdx.x] : 0ull);
+    b = warp_sum(threadIdx.x < kT / 32 ? s_b[threadIdx.x] : 0ull);
+    if (threadIdx.x == 0) {
+      a.part[2 * blockIdx.x] = n;
+      a.part[2 * blockIdx.x + 1] = b;
+    }
+  }
+}
+
+// One warp: the blocks' sums to exclusive prefixes, the totals to the status.
+__global__ void k_build_totals(BuildArgs a, uint32_t G, const uint32_t* over, Status* st) {
+  pdl_wait();
+  pdl_launch();
+  uint64_t n = 0, b = 0;
+  for (uint32_t g0 = 0; g0 < G; g0 += 32) {
+    const uint32_t g = g0 + threadIdx.x;
+    const uint64_t vn = g < G ? a.part[2 * g] : 0, vb = g < G ? a.part[2 * g + 1] : 0;
+    const uint64_t in = warp_incl_scan(vn), ib = warp_incl_scan(vb);
+    if (g < G) {
+      a.part[2 * g] = n + in - vn;
+      a.part[2 * g + 1] = b + ib - vb;
+    }
+    n += __shfl_sync(FULL, in, 31);
+    b += __shfl_sync(FULL, ib, 31);
+  }
+  if (threadIdx.x == 0) {
+    st->nunique = n;
+    st->stream_bytes = b;
+    st->sort_over = over ? *over : 0;
+  }
+}
+
+// Leaf w starts at the first key whose bytes before it reach floor(w S / L)
+// (the byte-balanced cut points of R8).  A tile finds the leaves whose target
+// lies in (bytes before the tile, bytes through it]: their number from one
+// division each end, then one thread per leaf searches the tile's prefix.
+__global__ void __launch_bounds__(kT) k_build_cuts(BuildArgs a) {
+  typedef unsigned __int128 u128;
+  __shared__ uint32_t s_c[kBuildTile + 1];  // bytes of the tile before each of its keys
+  __shared__ uint32_t s_w[kT / 32];
+  __shared__ uint64_t s_k[2];
+  pdl_wait();
+  pdl_launch();
+  uint64_t t0, t1;
+  build_tiles(a, t0, t1);
+  if (t0 >= t1) return;
+  uint64_t C = a.part[2 * blockIdx.x + 1];
+  // leaves with floor(w S / L) <= c
+  auto leaves_to = [&](uint64_t c) -> uint64_t {
+    const u128 y = (u128)(c + 1) * a.L - 1;
+    const uint64_t w = (y >> 64) ? (uint64_t)(y / a.S) : (uint64_t)y / a.S;
+    return min(a.L, w + 1);
+  };
+  if (threadIdx.x == 0) s_k[1] = C ? leaves_to(C) : 0;
+  const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
+  for (uint64_t t = t0; t < t1; t++) {
+    const uint64_t base = t * kBuildTile;
+    uint64_t x[kBuildItems], prev;
+    uint32_t c[kBuildItems], sum = 0;
+    build_load(a, base, x, prev);
+    build_costs(a, base + (uint64_t)threadIdx.x * kBuildItems, x, prev, c);
+#pragma unroll
+    for (int q = 0; q < kBuildItems; q++) sum += c[q];
+    const uint32_t inc = warp_incl_scan(sum);
+    if (lane == 31) s_w[warp] = inc;
+    __syncthreads();
+    uint32_t run = inc - sum, all = 0;
+#pragma unroll
+    for (unsigned w = 0; w < kT / 32; w++) {
+      if (w < warp) run += s_w[w];
+      all += s_w[w];
+    }
+#pragma unroll
+    for (int q = 0; q < kBuildItems; q++) {
+      s_c[threadIdx.x * kBuildItems + q] = run;
+      run += c[q];
+    }
+    if (threadIdx.x == 0) {
+      s_c[kBuildTile] = all;
+      const uint64_t k0 = s_k[1];
+      s_k[0] = k0;
+      s_k[1] = leaves_to(C + all);
+    }
+    __syncthreads();
+    const uint32_t nk = (uint32_t)min((uint64_t)kBuildTile, a.n - base);
+    for (uint64_t w = s_k[0] + threadIdx.x; w < s_k[1]; w += kT) {
+      const u128 y = (u128)w * a.S;
+      const uint64_t theta = (y >> 64) ? (uint64_t)(y / a.L) : (uint64_t)y / a.L;
+      const uint32_t need = theta > C ? (uint32_t)(theta - C) : 0u;
+      uint32_t lo = 0, m = nk;  // the first of the nk + 1 entries >= need (the last is `all`)
+      while (m > 0) {
+        const uint32_t half = m >> 1;
+        if (s_c[lo + half] < need) { lo += half + 1; m -= half + 1; }
+        else m = half;
+      }
+      a.dstart[w] = base + lo;
+    }
+    C += all;
+    __syncthreads();  // s_c, s_w and s_k are reused
+  }
+}
+
+struct BuildOut {
+  uint8_t* data;
+  uint32_t* used;
+  uint32_t* cnt;
+  uint64_t* heads;
+  uint32_t LB;
+  Status* st;
+};
+
+// A warp per leaf, two keys per lane and step: byte costs, their warp prefix,
+// the codes stored byte by byte into the leaf's image in shared memory, the
+// image to memory whole.  heads[L] is set for a set without empty leaves (the
+// head fix-up runs when there are some).
+__global__ void __launch_bounds__(kT) k_build_encode(BuildArgs a, BuildOut o) {
+  extern __shared__ __align__(16) uint8_t smem[];
+  pdl_wait();
+  pdl_launch();
+  const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
+  uint8_t* buf = smem + (size_t)warp * o.LB;
+  const uint64_t gw = gtid() >> 5, nw = gstride() >> 5;
+  ull added = 0;
+  for (uint64_t w = gw; w < a.L; w += nw) {
+    const uint64_t b = a.dstart[w], e = w + 1 < a.L ? a.dstart[w + 1] : a.n;
+    for (uint32_t p = lane * 16; p < o.LB; p += 512)
+      *reinterpret_cast<uint4*>(buf + p) = make_uint4(0u, 0u, 0u, 0u);
+    __syncwarp();
+    uint32_t pos = 0, cnt = 0;
+    uint64_t last = b ? a.x[b - 1] : 0, head = KEY_MAX;  // the key before this step's
+    bool fits = true;
+    for (uint64_t i0 = b; i0 < e && fits; i0 += 64) {
+      const uint64_t i = i0 + 2 * lane;
+      const uint64_t x0 = i < e ? a.x[i] : 0, x1 = i + 1 < e ? a.x[i + 1] : 0;
+      uint64_t before = __shfl_up_sync(FULL, x1, 1);
+      if (lane == 0) before = last;
+      const bool k0 = i < e && (i == 0 || x0 != before), k1 = i + 1 < e && x1 != x0;
+      const unsigned m0 = __ballot_sync(FULL, k0), m1 = __ballot_sync(FULL, k1);
+      // the leaf's first key is its head, 8 bytes uncoded
+      bool h0 = false, h1 = false;
+      if (cnt == 0 && (m0 | m1)) {
+        const int f0 = m0 ? __ffs(m0) - 1 : 32, f1 = m1 ? __ffs(m1) - 1 : 32;
+        h0 = f0 <= f1 && (int)lane == f0;
+        h1 = f1 < f0 && (int)lane == f1;
+        head = f0 <= f1 ? __shfl_sync(FULL, x0, f0 & 31) : __shfl_sync(FULL, x1, f1 & 31);
+      }
+      const uint64_t d0 = h0 || a.raw ? x0 : x0 - before, d1 = h1 || a.raw ? x1 : x1 - x0;
+      const bool c0 = h0 || a.raw, c1 = h1 || a.raw;  // cells: 8 bytes as they are
+      const uint32_t l0 = !k0 ? 0u : c0 ? 8u : leb_len(d0), l1 = !k1 ? 0u : c1 ? 8u : leb_len(d1);
+      const uint32_t inc = warp_incl_scan(l0 + l1);
+      const uint32_t tot = __shfl_sync(FULL, inc, 31);
+      fits = pos + tot <= o.LB;
+      if (fits) {
+        uint8_t* p = buf + pos + inc - l0 - l1;
+        auto put = [&](uint64_t d, uint32_t l, bool cell) {
+          if (cell) {
+            for (uint32_t q = 0; q < l; q++) p[q] = (uint8_t)(d >> (8 * q));
+          } else {
+#pragma unroll
+            for (uint32_t q = 0; q < 4; q++)
+              if (q < l) p[q] = (uint8_t)(((uint32_t)(d >> (7 * q)) & 0x7Fu) | (q + 1 < l ? 0x80u : 0u));
+            for (uint32_t q = 4; q < l; q++)
+              p[q] = (uint8_t)(((uint32_t)(d >> (7 * q)) & 0x7Fu) | (q + 1 < l ? 0x80u : 0u));
+          }
+          p += l;
+        };
+        put(d0, l0, c0);
+        put(d1, l1, c1);
+      }
+      pos += tot;
+      cnt += __popc(m0) + __popc(m1);
+      last = __shfl_sync(FULL, x1, 31);  // read only when the step was full
+    }
+    if (!fits && lane == 0) atomicOr(&o.st->err, kErrFit);
+    __syncwarp();
+    uint8_t* leafp = o.data + w * o.LB;
+    for (uint32_t p = lane * 16; p < o.LB; p += 512)
+      *reinterpret_cast<uint4*>(leafp + p) = *reinterpret_cast<const uint4*>(buf + p);
+    if (lane == 0) {
+      o.used[w] = pos;
+      o.cnt[w] = cnt;
+      o.heads[w] = head;
+      if (w + 1 == a.L) o.heads[a.L] = w;
+      added += pos;
+      if (cnt == 0) atomicAdd(&o.st->nempty, 1ull);
+    }
+    __syncwarp();
+  }
+  if (lane == 0 && added) atomicAdd(&o.st->bytes_total, added);
+}
+
 // Host-side values the front segment of an update leaves for the rest of it.
 struct Front {
   MergeArgs ma;
@@ -3040,7 +3321,7 @@ int run_front(cpma* h, const uint64_t* d_keys, uint64_t k, int sorted, int is_de
 
 constexpr int kGraphSlots = 8;
 
-constexpr int kSigPtrs = 34;
+constexpr int kSigPtrs = 33;
 
 struct FrontSig {
   const void* p[kSigPtrs];
@@ -3058,7 +3339,7 @@ struct FrontSig {
 FrontSig front_sig(const cpma* h) {
   const Scratch& s = h->s;
   return FrontSig{{s.stage.p,     s.keysA.p,      s.keysB.p,         s.hist.p,      s.partials.p,
-                   s.leaf_of.p,   s.flags.p,      s.flags_scan.p,    s.chunk_begin.p,
+                   s.flags.p,      s.flags_scan.p,    s.chunk_begin.p,
                    s.chunk_leaf.p, s.chunk_tid.p, s.chunk_cnt.p,     s.chunk_off.p, s.T_leaf.p,
                    s.T_begin.p,   s.T_first_chunk.p, s.T_oldcnt.p,   s.T_oldused.p, s.T_newcnt.p,
                    s.T_newbytes.p, s.T_state.p,   s.viol.p,          s.list_lane.p, s.list_v1.p,
@@ -3364,10 +3645,10 @@ int run_rebuild(cpma* h, const uint64_t* d_keys, uint64_t k, int sorted, int is_
   if (hs.err & kErrRoute) return CPMA_ETIMEOUT;
   if (hs.err & kErrUnsorted) return CPMA_EINVAL;
   if (hs.err) return CPMA_EINTERNAL;
-  CPMA_TRY(build_from_sorted_unique(h, P<uint64_t>(s.E), hs.nelem, st));
+  CPMA_TRY(build_measure(h, P<uint64_t>(s.E), hs.nelem, nullptr, st));
+  CPMA_TRY(build_from_sorted(h, P<uint64_t>(s.E), hs.nelem, st));
   prof_end(h, st);
   if (d_delta) {
-    // build_from_sorted_unique reset the status block; the count is on the host
     const uint64_t delta = is_delete ? n - hs.nelem : hs.nelem - n;
     k_put_u64<<<1, 1, 0, st>>>(d_delta, delta);
     h->launches++;
@@ -3479,7 +3760,7 @@ void trim_update_scratch(cpma* h) {
   graph_cache_free(h);
   Scratch& s = h->s;
   for (Buf* b : {&s.keysA, &s.keysB, &s.valsA, &s.valsB, &s.hist, &s.flags, &s.flags_scan,
-                 &s.leaf_of, &s.chunk_begin, &s.chunk_leaf, &s.chunk_tid, &s.chunk_cnt,
+                 &s.chunk_begin, &s.chunk_leaf, &s.chunk_tid, &s.chunk_cnt,
                  &s.chunk_off, &s.T_leaf, &s.T_begin, &s.T_first_chunk, &s.T_oldcnt, &s.T_oldused,
                  &s.T_newcnt, &s.T_newbytes, &s.T_state, &s.viol, &s.list_lane, &s.list_v1,
                  &s.list_gen, &s.list_pend, &s.point_stage, &s.point_rec, &s.cand, &s.wins,
@@ -3660,70 +3941,57 @@ int run_update(cpma* h, const uint64_t* d_keys, uint64_t k, int sorted, int is_d
   return CPMA_OK;
 }
 
-// App. A constructor over sorted distinct keys E[0..n) (already in the E
-// scratch buffer): L = max(1, ceil(1000 S / (build_pm LB - 8000))) leaves for
-// a stream of S bytes, then one byte-balanced spread.
-int build_from_sorted_unique(cpma* h, const uint64_t* E, uint64_t n, cudaStream_t st) {
+// Distinct keys and stream bytes of the sorted keys x[0..n), in the status
+// block once the stream is idle; over: a word to bring along (nullable).
+// Leaves the blocks' prefixes in the scan partials for build_from_sorted.
+static uint32_t build_grid(const cpma* h, uint64_t n) {
+  return (uint32_t)std::max<uint64_t>(
+      1, std::min<uint64_t>((n + kBuildTile - 1) / kBuildTile, (uint64_t)h->num_sms * 8));
+}
+
+int build_measure(cpma* h, const uint64_t* x, uint64_t n, const uint32_t* over, cudaStream_t st) {
+  const uint32_t G = build_grid(h, n);
+  CPMA_TRY(ensure(h, h->s.partials, (size_t)(G + 1) * 16));
+  const BuildArgs a{x, n, P<uint64_t>(h->s.partials), 0, 0, nullptr, (int)h->cfg.codec};
+  CPMA_CUDA(launch_pdl(k_build_sum, G, kT, 0, st, a));
+  CPMA_CUDA(launch_pdl(k_build_totals, 1, 32, 0, st, a, G, over, h->d_status));
+  h->launches += 2;
+  return sync_status(h, st);
+}
+
+// App. A constructor over the sorted keys x[0..n) (repeats allowed), measured
+// by build_measure: L = max(1, ceil(1000 S / (build_pm LB - 8000))) leaves for
+// a stream of S bytes, cut byte-balanced (R10, R8).
+int build_from_sorted(cpma* h, const uint64_t* x, uint64_t n, cudaStream_t st) {
   typedef unsigned __int128 u128;
-  const uint32_t LB = leaf_size_for(h, n);
   Scratch& s = h->s;
-  CPMA_TRY(ensure_win(h, 1));
-  CPMA_TRY(ensure(h, s.cost, n + 1));
-  CPMA_TRY(ensure(h, s.C, (n + 2) * 8));
-  if (E != P<uint64_t>(s.E)) return CPMA_EINTERNAL;
-  // costs and stream bytes (one window, no source leaves)
-  CPMA_CUDA(launch_pdl(k_set_window, (unsigned)(1), 1, 0, st, P<uint64_t>(s.win_src),
-                       P<uint64_t>(s.win_dst), P<uint64_t>(s.win_leaf_off),
-                       P<uint64_t>(s.win_dst_off), 0, 0, 0, 1));
-  h->launches++;
-  uint64_t eo[2] = {0, n};
-  CPMA_CUDA(cudaMemcpyAsync(s.win_elem_off.p, eo, 16, cudaMemcpyHostToDevice, st));
-  CPMA_CUDA(cudaMemcpyAsync(&h->d_status->nelem, &n, 8, cudaMemcpyHostToDevice, st));
-  WinArgs w = win_args(h, 1);
-  CPMA_CUDA(launch_pdl(k_costs, (unsigned)(grid_for(h, n)), kT, 0, st, w, E, &h->d_status->nelem,
-                       P<uint8_t>(s.cost), (int)h->cfg.codec));
-  h->launches++;
-  CPMA_TRY(scan_u8_to_u64(h, P<uint8_t>(s.cost), P<uint64_t>(s.C), n, nullptr, st));
-  CPMA_CUDA(cudaMemcpyAsync(&h->d_status->stream_bytes, P<uint64_t>(s.C) + n, 8,
-                            cudaMemcpyDeviceToDevice, st));
-  CPMA_TRY(sync_status(h, st));
-  const uint64_t S = h->h_status->stream_bytes;
+  const uint64_t nu = h->h_status->nunique, S = h->h_status->stream_bytes;
+  const uint32_t LB = leaf_size_for(h, nu);
   const u128 num = (u128)S * 1000, den = (u128)h->cfg.build_pm * LB - 8000;
   uint64_t L = (uint64_t)((num + den - 1) / den);
   if (L < 1) L = 1;
   Arrays na;
   CPMA_TRY(alloc_arrays(h, L, L * LB, &na, st));
-  CPMA_CUDA(launch_pdl(k_set_window, (unsigned)(1), 1, 0, st, P<uint64_t>(s.win_src),
-                       P<uint64_t>(s.win_dst), P<uint64_t>(s.win_leaf_off),
-                       P<uint64_t>(s.win_dst_off), 0, 0, 0, L));
-  h->launches++;
-  CPMA_TRY(ensure(h, s.dstart, (L + 1) * 8));
-  CPMA_CUDA(launch_pdl(k_starts, (unsigned)(grid_for(h, L)), kT, 0, st, w, P<uint64_t>(s.C), L,
-                       P<uint64_t>(s.dstart)));
-  h->launches++;
-  EncodeArgs ea;
-  ea.w = w;
-  ea.ndst = L;
-  ea.dstart = P<uint64_t>(s.dstart);
-  ea.E = E;
-  ea.C = P<uint64_t>(s.C);
-  ea.data = na.data;
-  ea.used = na.used;
-  ea.cnt = na.cnt;
-  ea.heads = na.heads;
-  ea.LB = LB;
-  ea.st = h->d_status;
-  ea.raw = (int)h->cfg.codec;
-  // the byte total restarts with the new leaves (the encode adds them)
-  int rc = check_cuda(cudaMemsetAsync(&h->d_status->bytes_total, 0, 8, st));
+  int rc = ensure(h, s.dstart, (L + 1) * 8);
+  // the byte total and the count of empty leaves restart with the new leaves
+  if (rc == CPMA_OK) rc = check_cuda(cudaMemsetAsync(&h->d_status->bytes_total, 0, 8, st));
+  if (rc == CPMA_OK) rc = check_cuda(cudaMemsetAsync(&h->d_status->empties, 0, 8, st));
+  if (rc == CPMA_OK) rc = check_cuda(cudaMemsetAsync(&h->d_status->nempty, 0, 8, st));
   if (rc == CPMA_OK) {
-    CPMA_CUDA(launch_pdl(k_encode, (unsigned)(grid_for(h, L * 32)), kT, (size_t)(kT / 32) * LB, st,
-                         ea));
-    h->launches++;
-    rc = check_cuda(cudaGetLastError());
+    const BuildArgs a{x, n, P<uint64_t>(s.partials), L, S, P<uint64_t>(s.dstart),
+                      (int)h->cfg.codec};
+    const BuildOut o{na.data, na.used, na.cnt, na.heads, LB, h->d_status};
+    if (n) rc = check_cuda(launch_pdl(k_build_cuts, build_grid(h, n), kT, 0, st, a));
+    else rc = check_cuda(cudaMemsetAsync(s.dstart.p, 0, 8, st));
+    if (rc == CPMA_OK)
+      rc = check_cuda(launch_pdl(k_build_encode, (unsigned)grid_for(h, L * 32), kT,
+                                 (size_t)(kT / 32) * LB, st, a, o));
+    h->launches += 2;
   }
-  if (rc == CPMA_OK) rc = check_cuda(cudaStreamSynchronize(st));
+  if (rc == CPMA_OK) rc = sync_status(h, st);
+  if (rc == CPMA_OK && h->h_status->err) rc = CPMA_EINTERNAL;
   if (rc != CPMA_OK) {
+    cudaStreamSynchronize(st);
     free_arrays(h, &na);
     return rc;
   }
@@ -3733,13 +4001,13 @@ int build_from_sorted_unique(cpma* h, const uint64_t* E, uint64_t n, cudaStream_
   set_live(h, na);
   h->cfg.leaf_bytes = LB;
   h->L = L;
-  h->n = n;
+  h->n = nu;
   Levels lv;
   CPMA_TRY(ensure_bits(h, st, &lv));
-  h->may_have_empty = true;
-  CPMA_TRY(fix_heads(h, st));
-  CPMA_TRY(sync_status(h, st));
-  if (h->h_status->err) return CPMA_EINTERNAL;
+  if (h->h_status->nempty) {
+    CPMA_TRY(fix_heads(h, st));
+    CPMA_TRY(sync_status(h, st));
+  }
   h->may_have_empty = h->h_status->empties > 0;
   h->t_known = h->h_status->bytes_total;
   h->t_slack = 0;
