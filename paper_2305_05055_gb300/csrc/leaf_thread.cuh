@@ -97,6 +97,14 @@ LT_HD uint32_t clz32(uint32_t x) {  // leading zeros, 32 for x == 0
 #endif
 }
 
+LT_HD uint32_t ctz32(uint32_t x) {  // trailing zeros, x != 0
+#if defined(__CUDA_ARCH__)
+  return (uint32_t)__ffs((int)x) - 1u;
+#else
+  return (uint32_t)__builtin_ctz(x);
+#endif
+}
+
 LT_HD void ld16(const uint8_t* p, uint32_t (&w)[4]) {
 #if defined(__CUDA_ARCH__)
   const uint4 v = *reinterpret_cast<const uint4*>(p);

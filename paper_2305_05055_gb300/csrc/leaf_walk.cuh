@@ -11,12 +11,12 @@
 // the open code's bits.  While no code has more than 4 bytes everything in a
 // group fits 32 bits (at most 11 payload bytes feed it and sum_k acc_k <
 // 9 * 2^28); a group that a longer code touches -- four continuation bytes in
-// a row end in it, or the code carried in has four already -- takes the same
-// steps with 64-bit arithmetic.  The lanes of a warp agree on the form (one
-// vote per group): a set whose codes are all short never pays for the long
-// form, and one with long codes everywhere (edges u << 32 | v, 64-bit hashes)
-// pays 13 instead of 9 integer operations per byte instead of decoding every
-// such leaf twice.
+// a row end in it, or the code carried in has four already -- takes 64 bits,
+// byte by byte for codes of 5 bytes (edges u << 32 | v), code by code for
+// longer ones (64-bit hashes).  The lanes of a warp agree on the form (a vote
+// per group): a set whose codes are all short never pays for the others.
+// 1e5 scans of 64-bit keys: 172 us byte by byte, 137 us code by code; degrees
+// of 2^20 vertices: 484 and 536 us, so codes of 5 bytes stay byte by byte.
 //
 // Which bytes end a code is passed in (term flags, bit 7 of each byte), so
 // bytes past the leaf's used ones are neither codes nor terminators.
@@ -52,15 +52,81 @@ LT_HD bool any_lane(bool p) {
 #endif
 }
 
-// Does a code of more than 4 bytes touch the group (wa, wb)?  Moves the flags
-// carried in k on.
-LT_HD bool long_group(uint32_t wa, uint32_t wb, Walk& k) {
+// The longest codes that touch the group (wa, wb), over the lanes: 0 = at most
+// 4 bytes, 1 = 5, 2 = more.  Moves the flags carried in k on.
+LT_HD int group_form(uint32_t wa, uint32_t wb, Walk& k) {
   const uint32_t ca = wa & kFlags, cb = wb & kFlags;
   const uint32_t ya = ca & fshl(k.c, ca, 8), yb = cb & fshl(ca, cb, 8);
-  const uint32_t z = (ya & fshl(k.y, ya, 16)) | (yb & fshl(ya, yb, 16));
+  const uint32_t za = ya & fshl(k.y, ya, 16), zb = yb & fshl(ya, yb, 16);  // 4 in a row
+  const uint32_t z5 = (za & k.c) | (zb & ca);
   k.c = cb;
   k.y = yb;
-  return z != 0u || k.sh >= 28u;
+  if (!any_lane((za | zb) != 0u || k.sh >= 28u)) return 0;
+  return any_lane(z5 != 0u || k.sh > 28u) ? 2 : 1;
+}
+
+// The group in 32 bits, byte by byte (form 0): step(acc) after each code closed.
+template <class D>
+LT_HD void short_codes(uint32_t pa, uint32_t pb, uint32_t ta, uint32_t tb, Walk& k, D&& done) {
+  uint32_t acc = (uint32_t)k.acc, pw = 1u << k.sh, r = 0;
+#pragma unroll
+  for (int b = 0; b < 8; b++) {
+    acc += byte_of(b < 4 ? pa : pb, b & 3) * pw;
+    const bool term = ((b < 4 ? ta : tb) & (0x80u << (8 * (b & 3)))) != 0u;
+    if (term) done(acc);
+    r = term ? acc : r;
+    pw = term ? 1u : pw << 7;
+  }
+  k.val += r;
+  k.acc = acc - r;
+  k.sh = 31u - leafthr::clz32(pw);
+}
+
+// The same with a 64-bit sum of 32-bit products, for codes of up to 5 bytes
+// (form 1).
+template <class D>
+LT_HD void medium_codes(uint32_t pa, uint32_t pb, uint32_t ta, uint32_t tb, Walk& k, D&& done) {
+  uint64_t acc = k.acc, r = 0;
+  uint32_t pw = 1u << k.sh;
+#pragma unroll
+  for (int b = 0; b < 8; b++) {
+    acc += (uint64_t)byte_of(b < 4 ? pa : pb, b & 3) * pw;
+    const bool term = ((b < 4 ? ta : tb) & (0x80u << (8 * (b & 3)))) != 0u;
+    if (term) done(acc);
+    r = term ? acc : r;
+    pw = term ? 1u : pw << 7;
+  }
+  k.val += r;
+  k.acc = acc - r;
+  k.sh = 31u - leafthr::clz32(pw);
+}
+
+// Codes of any length (form 2): the payloads packed to 56 bits once, then one
+// step per code closed -- codes this long leave few in a group.  done(acc)
+// after each, acc its element less the val the group was entered with.
+template <class D>
+LT_HD void long_codes(uint32_t pa, uint32_t pb, uint32_t ta, uint32_t tb, Walk& k, D&& done) {
+  using leafthr::dp4a;
+  const uint32_t lo = dp4a(pa, 0x00008001u, 0u) + (dp4a(pa, 0x80010000u, 0u) << 14);
+  const uint32_t hi = dp4a(pb, 0x00008001u, 0u) + (dp4a(pb, 0x80010000u, 0u) << 14);
+  const uint64_t v = (uint64_t)lo | ((uint64_t)hi << 28);
+  // terminators as bits 0..7
+  uint32_t t = ((((ta >> 7) * 0x01020408u) >> 24) & 0xFu) |
+               (((((tb >> 7) * 0x01020408u) >> 24) & 0xFu) << 4);
+  uint64_t acc = k.acc, cum = 0;
+  uint32_t sh = k.sh & 63u, pos = 0;
+  while (t) {
+    const uint32_t e = 7u * leafthr::ctz32(t) + 7u;
+    cum += acc | (((v >> pos) & ((1ull << (e - pos)) - 1ull)) << sh);
+    done(cum);
+    acc = 0;
+    sh = 0;
+    pos = e;
+    t &= t - 1u;
+  }
+  k.val += cum;
+  k.acc = acc | ((v >> pos) << sh);
+  k.sh = sh + 56u - pos;
 }
 
 // The group (wa, wb) with terminators ta, tb: T = elements closed, ss = the
@@ -70,35 +136,16 @@ LT_HD void group_sum(uint32_t wa, uint32_t wb, uint32_t ta, uint32_t tb, Walk& k
                      uint64_t& ss) {
   const uint32_t pa = wa & 0x7F7F7F7Fu, pb = wb & 0x7F7F7F7Fu;
   T = popc(ta) + popc(tb);
-  if (!any_lane(long_group(wa, wb, k))) {
-    uint32_t acc = (uint32_t)k.acc, pw = 1u << k.sh, s32 = 0, r = 0;
-#pragma unroll
-    for (int b = 0; b < 8; b++) {
-      acc += byte_of(b < 4 ? pa : pb, b & 3) * pw;
-      const bool term = ((b < 4 ? ta : tb) & (0x80u << (8 * (b & 3)))) != 0u;
-      s32 += term ? acc : 0u;
-      r = term ? acc : r;
-      pw = term ? 1u : pw << 7;
-    }
+  const int form = group_form(wa, wb, k);
+  if (form == 0) {
+    uint32_t s32 = 0;
+    short_codes(pa, pb, ta, tb, k, [&](uint32_t acc) { s32 += acc; });
     ss = s32;
-    k.val += r;
-    k.acc = acc - r;
-    k.sh = 31u - leafthr::clz32(pw);
   } else {
-    uint64_t acc = k.acc, s64 = 0, r = 0;
-    uint32_t sh = k.sh;
-#pragma unroll
-    for (int b = 0; b < 8; b++) {
-      acc += (uint64_t)byte_of(b < 4 ? pa : pb, b & 3) << (sh & 63u);
-      const bool term = ((b < 4 ? ta : tb) & (0x80u << (8 * (b & 3)))) != 0u;
-      s64 += term ? acc : 0ull;
-      r = term ? acc : r;
-      sh = term ? 0u : sh + 7u;
-    }
+    uint64_t s64 = 0;
+    if (form == 1) medium_codes(pa, pb, ta, tb, k, [&](uint64_t acc) { s64 += acc; });
+    else long_codes(pa, pb, ta, tb, k, [&](uint64_t acc) { s64 += acc; });
     ss = s64;
-    k.val += r;
-    k.acc = acc - r;
-    k.sh = sh;
   }
 }
 
@@ -106,34 +153,11 @@ LT_HD void group_sum(uint32_t wa, uint32_t wb, uint32_t ta, uint32_t tb, Walk& k
 template <class F>
 LT_HD void group_visit(uint32_t wa, uint32_t wb, uint32_t ta, uint32_t tb, Walk& k, F&& f) {
   const uint32_t pa = wa & 0x7F7F7F7Fu, pb = wb & 0x7F7F7F7Fu;
-  if (!any_lane(long_group(wa, wb, k))) {
-    uint32_t acc = (uint32_t)k.acc, pw = 1u << k.sh, r = 0;
-#pragma unroll
-    for (int b = 0; b < 8; b++) {
-      acc += byte_of(b < 4 ? pa : pb, b & 3) * pw;
-      const bool term = ((b < 4 ? ta : tb) & (0x80u << (8 * (b & 3)))) != 0u;
-      if (term) f(k.val + acc);
-      r = term ? acc : r;
-      pw = term ? 1u : pw << 7;
-    }
-    k.val += r;
-    k.acc = acc - r;
-    k.sh = 31u - leafthr::clz32(pw);
-  } else {
-    uint64_t acc = k.acc, r = 0;
-    uint32_t sh = k.sh;
-#pragma unroll
-    for (int b = 0; b < 8; b++) {
-      acc += (uint64_t)byte_of(b < 4 ? pa : pb, b & 3) << (sh & 63u);
-      const bool term = ((b < 4 ? ta : tb) & (0x80u << (8 * (b & 3)))) != 0u;
-      if (term) f(k.val + acc);
-      r = term ? acc : r;
-      sh = term ? 0u : sh + 7u;
-    }
-    k.val += r;
-    k.acc = acc - r;
-    k.sh = sh;
-  }
+  const uint64_t v = k.val;
+  const int form = group_form(wa, wb, k);
+  if (form == 0) short_codes(pa, pb, ta, tb, k, [&](uint32_t acc) { f(v + acc); });
+  else if (form == 1) medium_codes(pa, pb, ta, tb, k, [&](uint64_t acc) { f(v + acc); });
+  else long_codes(pa, pb, ta, tb, k, [&](uint64_t acc) { f(v + acc); });
 }
 
 // The 16 bytes of the leaf at p0 (zero past the u used ones) and which of
@@ -141,6 +165,27 @@ LT_HD void group_visit(uint32_t wa, uint32_t wb, uint32_t ta, uint32_t tb, Walk&
 LT_HD void load_chunk(const uint8_t* leafp, uint32_t p0, uint32_t u, uint32_t (&w)[4],
                       uint32_t (&t)[4]) {
   ld16(leafp + p0, w);
+  if (p0 + 16u > u) {
+    const uint32_t keep = u > p0 ? (1u << (u - p0)) - 1u : 0u;
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+      const uint32_t m = bmask4((keep >> (4 * i)) & 0xFu);
+      w[i] &= m;
+      t[i] = ~w[i] & kFlags & m;
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; i++) t[i] = ~w[i] & kFlags;
+  }
+}
+
+// load_chunk for a loop over the leaf: w holds the raw chunk at p0, and the
+// next one is loaded before this one is decoded.
+LT_HD void next_chunk(const uint8_t* leafp, uint32_t p0, uint32_t u, uint32_t (&raw)[4],
+                      uint32_t (&w)[4], uint32_t (&t)[4]) {
+#pragma unroll
+  for (int i = 0; i < 4; i++) w[i] = raw[i];
+  if (p0 + 16u < u) ld16(leafp + p0 + 16u, raw);
   if (p0 + 16u > u) {
     const uint32_t keep = u > p0 ? (1u << (u - p0)) - 1u : 0u;
 #pragma unroll
@@ -315,10 +360,12 @@ LT_HD uint64_t sum_walked(const uint8_t* leafp, uint32_t u) {
   Walk k;
   k.val = leaf_head(leafp);
   uint64_t s = k.val;
+  uint32_t raw[4];
+  ld16(leafp, raw);
   for (uint32_t p0 = 0; p0 < u; p0 += 16) {
     uint32_t w[4], t[4], T;
     uint64_t ss, v;
-    load_chunk(leafp, p0, u, w, t);
+    next_chunk(leafp, p0, u, raw, w, t);
     if (p0) {  // bytes 0-7 are the head
       v = k.val;
       group_sum(w[0], w[1], t[0], t[1], k, T, ss);
@@ -360,9 +407,11 @@ LT_HD void leaf_visit(const uint8_t* leafp, uint32_t u, F&& f) {
   Walk k;
   k.val = leaf_head(leafp);
   f(k.val);
+  uint32_t raw[4];
+  ld16(leafp, raw);
   for (uint32_t p0 = 0; p0 < u; p0 += 16) {
     uint32_t w[4], t[4];
-    load_chunk(leafp, p0, u, w, t);
+    next_chunk(leafp, p0, u, raw, w, t);
     if (p0) group_visit(w[0], w[1], t[0], t[1], k, f);
     group_visit(w[2], w[3], t[2], t[3], k, f);
   }
@@ -406,9 +455,11 @@ LT_HD void leaf_range_sum(const uint8_t* leafp, uint32_t u, uint64_t lo, uint64_
       c += T;
     }
   };
+  uint32_t raw[4];
+  ld16(leafp, raw);
   for (uint32_t p0 = 0; p0 < u && !done; p0 += 16) {
     uint32_t w[4], t[4];
-    load_chunk(leafp, p0, u, w, t);
+    next_chunk(leafp, p0, u, raw, w, t);
     if (p0) step(w[0], w[1], t[0], t[1]);
     if (!done) step(w[2], w[3], t[2], t[3]);
   }
@@ -483,9 +534,11 @@ LT_HD uint32_t leaf_below(const uint8_t* leafp, uint32_t u, uint64_t x) {
     have = k.val >= x;
     if (!have) n += T;
   };
+  uint32_t raw[4];
+  ld16(leafp, raw);
   for (uint32_t p0 = 0; p0 < u && !have; p0 += 16) {
     uint32_t w[4], t[4];
-    load_chunk(leafp, p0, u, w, t);
+    next_chunk(leafp, p0, u, raw, w, t);
     if (p0) step(w[0], w[1], t[0], t[1]);
     if (!have) step(w[2], w[3], t[2], t[3]);
   }
