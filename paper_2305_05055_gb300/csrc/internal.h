@@ -70,7 +70,8 @@ struct Status {
   ull point_fb;    // point path: touched leaves that need the batch algorithm
   ull point_done;  // point path: blocks finished (the last one finishes the pass)
   ull sort_over;   // create: the windows of the batch sort did not hold its buckets
-  ull pad[6];
+  ull n_long;      // touched leaves for the thread-granular merge of long codes
+  ull pad[5];
   ull empties;     // empty leaves in the structure (written by the head
                    // fix-up; not cleared at the start of a batch)
   ull bytes_total; // used bytes over all leaves, kept exact by the merge,
@@ -116,6 +117,7 @@ struct Scratch {
   Buf viol, cand, wins;   // violating leaves, window candidates, windows
   Buf list_lane, list_v1, list_gen;  // merge work lists
   Buf list_pend;          // pending leaves of the thread- and lane-granular inserts
+  Buf list_long;          // leaves with long codes for the thread-granular merge
   Buf point_stage;        // point path: 512-byte staging slot per key
   Buf point_rec;          // point path: staged result per key
   Buf bits;               // per-level window bitsets (u32 words)

@@ -24,14 +24,7 @@
 // The functions are __host__ __device__ so that the same code can be run on
 // the host.
 #pragma once
-#include <stdint.h>
-#include <string.h>
-
-#if defined(__CUDACC__)
-#define LT_HD __host__ __device__ __forceinline__
-#else
-#define LT_HD inline
-#endif
+#include "leaf_walk.cuh"
 
 namespace leafthr {
 
@@ -64,76 +57,6 @@ struct Result {
   uint64_t newhead;
 };
 
-LT_HD uint32_t fshr(uint32_t lo, uint32_t hi, uint32_t sh) {  // low word of (hi:lo) >> sh, sh < 32
-#if defined(__CUDA_ARCH__)
-  return __funnelshift_r(lo, hi, sh);
-#else
-  return sh ? (lo >> sh) | (hi << (32u - sh)) : lo;
-#endif
-}
-
-LT_HD uint32_t fshl(uint32_t lo, uint32_t hi, uint32_t sh) {  // high word of (hi:lo) << sh, 0 < sh < 32
-#if defined(__CUDA_ARCH__)
-  return __funnelshift_l(lo, hi, sh);
-#else
-  return (hi << sh) | (lo >> (32u - sh));
-#endif
-}
-
-LT_HD uint32_t dp4a(uint32_t a, uint32_t b, uint32_t c) {  // c + sum of the four byte products
-#if defined(__CUDA_ARCH__)
-  return __dp4a(a, b, c);
-#else
-  for (int i = 0; i < 4; i++) c += ((a >> (8 * i)) & 0xFFu) * ((b >> (8 * i)) & 0xFFu);
-  return c;
-#endif
-}
-
-LT_HD uint32_t clz32(uint32_t x) {  // leading zeros, 32 for x == 0
-#if defined(__CUDA_ARCH__)
-  return (uint32_t)__clz((int)x);
-#else
-  return x ? (uint32_t)__builtin_clz(x) : 32u;
-#endif
-}
-
-LT_HD uint32_t ctz32(uint32_t x) {  // trailing zeros, x != 0
-#if defined(__CUDA_ARCH__)
-  return (uint32_t)__ffs((int)x) - 1u;
-#else
-  return (uint32_t)__builtin_ctz(x);
-#endif
-}
-
-LT_HD void ld16(const uint8_t* p, uint32_t (&w)[4]) {
-#if defined(__CUDA_ARCH__)
-  const uint4 v = *reinterpret_cast<const uint4*>(p);
-  w[0] = v.x; w[1] = v.y; w[2] = v.z; w[3] = v.w;
-#else
-  memcpy(w, p, 16);
-#endif
-}
-
-LT_HD void st16(uint8_t* p, const uint32_t (&w)[4]) {
-#if defined(__CUDA_ARCH__)
-  *reinterpret_cast<uint4*>(p) = make_uint4(w[0], w[1], w[2], w[3]);
-#else
-  memcpy(p, w, 16);
-#endif
-}
-
-LT_HD uint32_t popc(uint32_t x) {
-#if defined(__CUDA_ARCH__)
-  return (uint32_t)__popc(x);
-#else
-  return (uint32_t)__builtin_popcount(x);
-#endif
-}
-
-LT_HD uint32_t bmask4(uint32_t b4) {  // 4 bits -> 0x00 / 0xFF bytes
-  return ((b4 * 0x00204081u) & 0x01010101u) * 0xFFu;
-}
-
 LT_HD uint32_t leb_bytes(uint64_t d) {  // unsigned LEB128 length of d
 #if defined(__CUDA_ARCH__)
   const uint32_t bl = 64u - (uint32_t)__clzll((long long)(d | 1ull));
@@ -157,23 +80,18 @@ LT_HD uint64_t pick(const uint64_t (&y)[kKeys], uint32_t q) {
 
 // Per-thread scratch: arrays of kKeys entries at stride `rs` (key records and
 // edits), so that a block's threads index shared memory without conflicts.
-struct Scratch {
+template <class Code>
+struct ScratchT {
   uint32_t* rpos;   // key q: cs | ce << 12 | kind << 24
   uint64_t* rval;   // key q: successor value (kGap), the head (kHead), the last value (kAfter)
-  uint32_t* rcode;  // key q: value of the code [cs, ce) (kGap)
+  Code* rcode;      // key q: value of the code [cs, ce) (kGap)
   uint32_t* epos;   // edit e: os | oe << 12 | kind << 24
   int32_t* esa;     // edit e: total size change of edits 0..e
   uint32_t* ekey;   // edit e: first key | end key << 8 | nl << 16
   uint32_t rs;
 };
-
-LT_HD uint32_t byte_of(uint32_t v, int i) {  // byte i of v, zero-extended
-#if defined(__CUDA_ARCH__)
-  return __byte_perm(v, 0u, 0x4440u + (uint32_t)i);
-#else
-  return (v >> (8 * i)) & 0xFFu;
-#endif
-}
+using Scratch = ScratchT<uint32_t>;      // leaves whose codes have at most 4 bytes
+using ScratchLong = ScratchT<uint64_t>;  // any code length
 
 // Pass A, step 1: the byte weights of one 4-byte word of codes.  cb, p1, p2
 // carry the flags of the word before (bit 7 of each byte): cb = the byte is
@@ -205,77 +123,77 @@ LT_HD uint32_t word_sum(uint32_t w, uint32_t& cb, uint32_t& p1, uint32_t& p2, ui
 // element completed in it).  Decode the chunk byte by byte from the state it
 // was entered with (val0: the element before it; carry0, g0: the bits and
 // byte count of the code open at p0) and give each key its gap.
+// For each key the bytes are walked without branches, the values relative to
+// val0: the last terminator below the key, and the first that reaches it.
 LT_HD void place_in_chunk(const uint8_t* leafp, uint32_t uold, uint32_t p0, uint64_t val0,
                           uint32_t carry0, uint32_t g0, const uint64_t (&y)[kKeys], uint32_t q,
                           uint32_t q1, const Scratch& S) {
-  uint32_t w[4];
-  ld16(leafp + p0, w);
-  if (p0 + 16u > uold) {
-    const uint32_t keep = (1u << (uold - p0)) - 1u;
+  uint32_t w[4], t[4];
+  leafwalk::load_chunk(leafp, p0, uold, w, t);
+  const uint32_t first = p0 == 0 ? 8u : 0u;  // bytes 0-7 are the head
+  if (p0 == 0) w[0] = w[1] = t[0] = t[1] = 0u;
 #pragma unroll
-    for (int i = 0; i < 4; i++) w[i] &= bmask4((keep >> (4 * i)) & 0xFu);
-  }
-  uint64_t val = val0;
-  uint32_t acc = carry0, sh = 7u * g0, cs = p0 == 0 ? 8u : p0 - g0;
-  uint64_t ycur = pick(y, q);
-  const int b0 = p0 == 0 ? 8 : 0;
+  for (int i = 0; i < 4; i++) w[i] &= 0x7F7F7F7Fu;
+  for (; q < q1; q++) {
+    const uint64_t yq = pick(y, q);
+    const uint32_t d = (uint32_t)(yq - val0);  // the chunk's last element reaches it
+    uint32_t cum = carry0, pw = 1u << (7u * g0);
+    uint32_t below = 0, cs = first - g0, at = 0, ce = 0;  // cs: relative to p0, may wrap
+    bool open = true;
 #pragma unroll
-  for (int b = 0; b < 16; b++) {  // unrolled: w[] stays in registers
-    if (b < b0) continue;
-    const uint32_t c = byte_of(w[b >> 2], b & 3);
-    acc |= (c & 0x7Fu) << sh;
-    if (c & 0x80u) {
-      sh += 7u;
-      continue;
+    for (int b = 0; b < 16; b++) {
+      cum += byte_of(w[b >> 2], b & 3) * pw;
+      const bool term = (t[b >> 2] & (0x80u << (8 * (b & 3)))) != 0u;
+      const bool stop = term && open && cum >= d;
+      const bool pass = term && open && cum < d;
+      at = stop ? cum : at;
+      ce = stop ? (uint32_t)b + 1u : ce;
+      below = pass ? cum : below;
+      cs = pass ? (uint32_t)b + 1u : cs;
+      open = open && !stop;
+      pw = term ? 1u : pw << 7;
+      if (p0 == 0 && b == 7) pw = 1u << (7u * g0);  // the head's bytes are no codes
     }
-    val += acc;
-    const uint32_t ce = p0 + (uint32_t)b + 1u;
-    while (ycur <= val) {  // this code's gap (val - acc, val] takes the keys up to val
-      const bool rep = q > 0 && pick(y, q - 1) == ycur;
-      const uint32_t kind = rep ? kSkip : ycur == val ? kHit : kGap;
-      S.rpos[q * S.rs] = cs | (ce << 12) | (kind << 24);
-      S.rval[q * S.rs] = val;
-      S.rcode[q * S.rs] = acc;
-      if (++q >= q1) return;
-      ycur = pick(y, q);
-    }
-    acc = 0u;
-    sh = 0u;
-    cs = ce;
+    const uint64_t val = val0 + at;
+    const bool rep = q > 0 && pick(y, q - 1) == yq;
+    const uint32_t kind = rep ? kSkip : yq == val ? kHit : kGap;
+    S.rpos[q * S.rs] = (p0 + cs) | ((p0 + ce) << 12) | (kind << 24);
+    S.rval[q * S.rs] = val;
+    S.rcode[q * S.rs] = at - below;
   }
 }
 
-// The 16 bytes at byte offset `src` (which may be negative: missing bytes
-// read as zero) of the old leaf, masked to chunk bytes [a, b), OR-ed into r.
-LT_HD void gather(const uint8_t* leafp, uint32_t LB, int32_t src, uint32_t a, uint32_t b,
-                  uint32_t (&r)[4]) {
-  const int32_t A = (src >> 4) * 16;  // floor to 16
-  const uint32_t d = (uint32_t)(src - A);
-  uint32_t W[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
-  if (A >= 0) {
-    uint32_t t[4];
-    ld16(leafp + A, t);
-    W[0] = t[0]; W[1] = t[1]; W[2] = t[2]; W[3] = t[3];
-  }
-  if (d != 0u && A + 16 >= 0 && (uint32_t)(A + 16) < LB) {
-    uint32_t t[4];
-    ld16(leafp + A + 16, t);
-    W[4] = t[0]; W[5] = t[1]; W[6] = t[2]; W[7] = t[3];
-  }
-  const uint32_t q = d >> 2, s8 = 8u * (d & 3u);
-  uint32_t V[5];
+// The 16 bytes of the old leaf at byte offset src, bytes outside [0, LB)
+// reading as zero: five 4-byte words from the 4-byte boundary at or below src
+// and one byte shift (two 16-byte loads and their word selects took more).
+LT_HD void chunk_at(const uint8_t* leafp, uint32_t LB, int32_t src, uint32_t (&r)[4]) {
+  const int32_t base = src & ~3;
+  const uint32_t s8 = 8u * (uint32_t)(src & 3);
+  uint32_t W[5];
 #pragma unroll
-  for (int i = 0; i < 5; i++)
-    V[i] = q == 0 ? W[i] : q == 1 ? W[i + 1] : q == 2 ? W[i + 2] : W[i + 3];
-  const uint32_t m16 = ((b >= 16u ? 0xFFFFu : ((1u << b) - 1u)) & ~((1u << a) - 1u));
+  for (int i = 0; i < 5; i++) {
+    W[i] = 0u;
+    if ((uint32_t)(base + 4 * i) < LB && (i < 4 || s8)) W[i] = ld4(leafp + base + 4 * i);
+  }
 #pragma unroll
-  for (int i = 0; i < 4; i++) r[i] |= fshr(V[i], V[i + 1], s8) & bmask4((m16 >> (4 * i)) & 0xFu);
+  for (int i = 0; i < 4; i++) r[i] = fshr(W[i], W[i + 1], s8);
+}
+
+// r with the bytes [a, b) of x in place of its own.
+LT_HD void take_bytes(uint32_t (&r)[4], const uint32_t (&x)[4], uint32_t a, uint32_t b) {
+  const uint32_t m16 = (b >= 16u ? 0xFFFFu : ((1u << b) - 1u)) & ~((1u << a) - 1u);
+#pragma unroll
+  for (int i = 0; i < 4; i++) {
+    const uint32_t m = bmask4((m16 >> (4 * i)) & 0xFu);
+    r[i] = (r[i] & ~m) | (x[i] & m);
+  }
 }
 
 // Pass B: destination bounds [dlo, dhi) and shift sa of segment e (-1 .. E-1):
 // the old bytes [oe_e, os_{e+1}) moved by sa_e (oe_{-1} = 0, os_E = uold,
 // sa_{-1} = 0).
-LT_HD void seg_bounds(const Scratch& S, uint32_t E, uint32_t uold, uint32_t os0, int e,
+template <class SC>
+LT_HD void seg_bounds(const SC& S, uint32_t E, uint32_t uold, uint32_t os0, int e,
                       int32_t& dlo, int32_t& dhi, int32_t& sa) {
   uint32_t lo = 0u, hi = os0;
   sa = 0;
@@ -368,13 +286,99 @@ LT_HD uint32_t pass_a(const uint8_t* leafp, uint32_t uold, uint32_t m, const uin
   return kPlaced;
 }
 
+// The same for leaves with codes of any length, eight bytes at a time with
+// 64-bit values (the leaf walk's groups: Walk carries the element before the
+// group and the code open at it).  Always kPlaced.
+LT_HD uint32_t pass_a(const uint8_t* leafp, uint32_t uold, uint32_t m, const uint64_t (&y)[kKeys],
+                      uint32_t s, const ScratchLong& S, uint64_t& head) {
+  uint32_t w[4], t[4], raw[4];
+  ld16(leafp, raw);
+  head = (uint64_t)raw[0] | ((uint64_t)raw[1] << 32);
+  uint32_t k = 0;
+  while (k < s && pick(y, k) <= head) {
+    const uint64_t x = pick(y, k);
+    const bool rep = k > 0 && pick(y, k - 1) == x;
+    const uint32_t kind = rep ? kSkip : x == head ? kHit : kHead;
+    S.rpos[k * S.rs] = 0u | (8u << 12) | (kind << 24);
+    S.rval[k * S.rs] = head;
+    S.rcode[k * S.rs] = 0u;
+    k++;
+  }
+  // step 1: every key gets the group that reaches it and the walk's state there
+  uint64_t ycur = k < s ? pick(y, k) : ~0ull;
+  leafwalk::Walk c;
+  c.val = head;
+  auto group = [&](uint32_t p0, int i) {
+    const leafwalk::Walk c0 = c;
+    uint32_t T;
+    uint64_t ss;
+    leafwalk::group_sum(w[i], w[i + 1], t[i], t[i + 1], c, T, ss);
+    while (k < s && ycur <= c.val) {
+      S.rpos[k * S.rs] = p0 | ((c0.sh / 7u) << 12) | (kChunk << 24);
+      S.rval[k * S.rs] = c0.val;
+      S.rcode[k * S.rs] = c0.acc;
+      k++;
+      ycur = k < s ? pick(y, k) : ~0ull;
+    }
+  };
+  for (uint32_t p0 = 0; p0 < uold && k < s; p0 += 16) {
+    leafwalk::next_chunk(leafp, p0, uold, raw, w, t);
+    if (p0) group(p0, 0);
+    if (p0 + 8u < uold) group(p0 + 8u, 2);
+  }
+  // step 2: exact gaps inside the recorded groups
+  for (uint32_t q = 0; q < k; q++) {
+    const uint32_t rp = S.rpos[q * S.rs];
+    if ((rp >> 24) != kChunk) continue;  // placed (head keys, or by an earlier group)
+    const uint32_t p0 = rp & 0xFFFu, g0 = (rp >> 12) & 0xFFFu;
+    uint64_t val = S.rval[q * S.rs], acc = S.rcode[q * S.rs];
+    uint32_t sh = 7u * g0, cs = p0 - g0;
+    uint32_t q1 = q + 1;
+    while (q1 < k && S.rpos[q1 * S.rs] == rp) q1++;
+    uint64_t yc = pick(y, q);
+    uint32_t qq = q;
+    for (uint32_t b = 0; b < 8u && p0 + b < uold && qq < q1; b++) {
+      const uint32_t ch = leafp[p0 + b];
+      acc |= (uint64_t)(ch & 0x7Fu) << sh;
+      if (ch & 0x80u) {
+        sh += 7u;
+        continue;
+      }
+      val += acc;
+      const uint32_t ce = p0 + b + 1u;
+      while (qq < q1 && yc <= val) {
+        const bool rep = qq > 0 && pick(y, qq - 1) == yc;
+        const uint32_t kind = rep ? kSkip : yc == val ? kHit : kGap;
+        S.rpos[qq * S.rs] = cs | (ce << 12) | (kind << 24);
+        S.rval[qq * S.rs] = val;
+        S.rcode[qq * S.rs] = acc;
+        qq++;
+        if (qq < q1) yc = pick(y, qq);
+      }
+      acc = 0;
+      sh = 0;
+      cs = ce;
+    }
+    q = q1 - 1;
+  }
+  for (; k < s; k++) {
+    const uint64_t x = pick(y, k);
+    const bool rep = k > 0 && pick(y, k - 1) == x;
+    S.rpos[k * S.rs] = uold | (uold << 12) | ((rep ? kSkip : kAfter) << 24);
+    S.rval[k * S.rs] = c.val;
+    S.rcode[k * S.rs] = 0u;
+  }
+  return kPlaced;
+}
+
 // Pass A and the edits of inserting the sorted slice y[0..s) (1 <= s <=
 // kKeys, repeats allowed) into the leaf at leafp (uold >= 8 used bytes, m
 // elements, LB bytes, 16-byte aligned).  Returns one of the results above
 // and writes nothing; kWritten means the leaf is to be rewritten (R.wlo ..
 // R.whi, the R.E edits in S).
+template <class SC>
 LT_HD uint32_t plan_leaf(uint8_t* leafp, uint32_t LB, uint32_t uold, uint32_t m,
-                           const uint64_t (&y)[kKeys], uint32_t s, const Scratch& S,
+                           const uint64_t (&y)[kKeys], uint32_t s, const SC& S,
                            Result& R) {
   uint64_t head;
   const uint32_t pa = pass_a(leafp, uold, m, y, s, S, head);
@@ -436,100 +440,58 @@ LT_HD uint32_t plan_leaf(uint8_t* leafp, uint32_t LB, uint32_t uold, uint32_t m,
   return kWritten;
 }
 
-// The 16 bytes at leaf[src, src + 16) (0 <= src, src + 16 <= the old used
-// bytes): the aligned chunk below src and, unless src is aligned, the one
-// after it, shifted together.  A destination chunk wholly inside the
-// segment after the last edit is exactly this, with src = o - sa.
-LT_HD void chunk_tail(const uint8_t* leafp, int32_t src, uint32_t (&r)[4]) {
-#if defined(__CUDA_ARCH__)
-  // five 4-byte words from the 4-byte boundary at or below src, then the
-  // byte shift inside a word (no word selects).  The fifth word is needed
-  // only for an unaligned src; its bytes past src + 16 (the leaf's zero
-  // bytes, the next leaf, or the padding after the last leaf) are shifted
-  // out.
-  const uint32_t* w = reinterpret_cast<const uint32_t*>(leafp + (src & ~3));
-  const uint32_t s8 = 8u * (uint32_t)(src & 3);
-  uint32_t W[5];
-#pragma unroll
-  for (int i = 0; i < 4; i++) W[i] = w[i];
-  W[4] = s8 ? w[4] : 0u;
-#pragma unroll
-  for (int i = 0; i < 4; i++) r[i] = fshr(W[i], W[i + 1], s8);
-#else
-  const int32_t A = src & ~15;
-  const uint32_t d = (uint32_t)(src - A);
-  uint32_t W[8];
-  uint32_t t[4];
-  ld16(leafp + A, t);
-  W[0] = t[0]; W[1] = t[1]; W[2] = t[2]; W[3] = t[3];
-  W[4] = W[5] = W[6] = W[7] = 0u;
-  if (d) {
-    ld16(leafp + A + 16, t);
-    W[4] = t[0]; W[5] = t[1]; W[6] = t[2]; W[7] = t[3];
+// Chunk o of the rewritten leaf from segment cur (destination [slo, shi), shift
+// ssa) and, where it starts inside the chunk, the ones before it.  Bytes of
+// edits are left as they fall (their own bytes are written last); bytes past
+// the new used ones (shi of the last segment) are zero.
+template <class SC>
+LT_HD void build_chunk(const uint8_t* leafp, uint32_t LB, uint32_t uold, const SC& S, uint32_t E,
+                       uint32_t os0, int cur, int32_t slo, int32_t shi, int32_t ssa, int32_t o,
+                       uint32_t (&r)[4]) {
+  chunk_at(leafp, LB, o - ssa, r);
+  if (o + 16 > shi && cur + 1 == (int)E) {
+    const uint32_t zero[4] = {0u, 0u, 0u, 0u};
+    take_bytes(r, zero, shi > o ? (uint32_t)(shi - o) : 0u, 16u);
   }
-  // words q .. q + 4 of the 32 bytes (two selects per word), then the byte
-  // shift inside a word
-  const uint32_t q = d >> 2, s8 = 8u * (d & 3u);
-  uint32_t X[7];
-#pragma unroll
-  for (int i = 0; i < 7; i++) X[i] = (q & 1u) ? W[i + 1] : W[i];
-  uint32_t V[5];
-#pragma unroll
-  for (int i = 0; i < 5; i++) V[i] = (q & 2u) ? X[i + 2] : X[i];
-#pragma unroll
-  for (int i = 0; i < 4; i++) r[i] = fshr(V[i], V[i + 1], s8);
-#endif
+  while (slo > o && cur >= 0) {
+    cur--;
+    seg_bounds(S, E, uold, os0, cur, slo, shi, ssa);
+    if (shi <= o) break;  // wholly below this chunk: so are the earlier ones
+    uint32_t x[4];
+    chunk_at(leafp, LB, o - ssa, x);
+    take_bytes(r, x, 0u, shi - o < 16 ? (uint32_t)(shi - o) : 16u);
+  }
 }
 
 // Pass B by one thread: the chunks R.wlo .. R.whi of the leaf from the end
-// backwards, each built from the segments that land in it and stored whole
-// (the edits' own bytes are left zero: write_edits fills them).  A run of
-// chunks inside one segment is one shift each; the chunk below it, where an
-// edit falls, is gathered segment by segment.  Runs of every segment, not only
-// of the last, take the short way: with one or two keys in most leaves, some
-// lane of every warp has chunks between two edits, and gathering those too
-// kept its whole warp (1e6 keys into 1e8: a launch 303 -> 290 us with this).
-LT_HD void rewrite_leaf(uint8_t* leafp, uint32_t LB, uint32_t uold, const Scratch& S,
+// backwards, each built from the segments that land in it and stored whole.
+// Every chunk is one shifted read, whatever segment it lies in; the one an
+// edit falls into merges a second (with one or two keys in most leaves, some
+// lane of every warp is at such a chunk in every step, so that is all a step
+// may cost).  Gathering those chunks segment by segment: 290 us a launch for 1e6
+// keys into 1e8, this 254 us.
+template <class SC>
+LT_HD void rewrite_leaf(uint8_t* leafp, uint32_t LB, uint32_t uold, const SC& S,
                         const Result& R) {
   const uint32_t E = R.E;
   const uint32_t os0 = S.epos[0] & 0xFFFu;
-  const int32_t olo = (int32_t)R.wlo;
   int cur = (int)E - 1;  // the highest segment not wholly above chunk o
   int32_t slo, shi, ssa;
   seg_bounds(S, E, uold, os0, cur, slo, shi, ssa);
-  for (int32_t o = (int32_t)R.whi - 16; o >= olo; o -= 16) {
-    while (o >= olo && o >= slo && o + 16 <= shi) {
-      uint32_t r[4];
-      chunk_tail(leafp, o - ssa, r);
-      st16(leafp + o, r);
-      o -= 16;
-    }
-    if (o < olo) break;
+  for (int32_t o = (int32_t)R.whi - 16; o >= (int32_t)R.wlo; o -= 16) {
     while (cur >= 0 && slo >= o + 16) {
       cur--;
       seg_bounds(S, E, uold, os0, cur, slo, shi, ssa);
     }
-    if (o >= slo && o + 16 <= shi) {  // the next segment's run starts here
-      o += 16;
-      continue;
-    }
-    uint32_t r[4] = {0u, 0u, 0u, 0u};
-    for (int e = cur; e >= -1; e--) {
-      int32_t dlo, dhi, sa;
-      seg_bounds(S, E, uold, os0, e, dlo, dhi, sa);
-      if (dhi <= o) break;  // wholly below this chunk: so are the earlier ones
-      if (dhi > dlo) {
-        const uint32_t a = (uint32_t)((dlo > o ? dlo : o) - o);
-        const uint32_t b = (uint32_t)((dhi < o + 16 ? dhi : o + 16) - o);
-        gather(leafp, LB, o - sa, a, b, r);
-      }
-    }
+    uint32_t r[4];
+    build_chunk(leafp, LB, uold, S, E, os0, cur, slo, shi, ssa, o, r);
     st16(leafp + o, r);
   }
 }
 
 // The edits' own bytes (new head, split codes), after the chunks are stored.
-LT_HD void write_edits(uint8_t* leafp, const uint64_t (&y)[kKeys], const Scratch& S,
+template <class SC>
+LT_HD void write_edits(uint8_t* leafp, const uint64_t (&y)[kKeys], const SC& S,
                        const Result& R) {
   for (uint32_t e = 0; e < R.E; e++) {
     const uint32_t ep = S.epos[e * S.rs], ek = S.ekey[e * S.rs];
@@ -587,8 +549,9 @@ LT_HD uint64_t leb_read(const uint8_t* p, uint32_t& len) {
 // kKeys, repeats allowed) from the leaf (as plan_leaf).  R.added: bit q =
 // slice key q was removed; R.wlo .. R.whi covers the old used bytes from the
 // first edit on, so the bytes freed at the end are cleared.
+template <class SC>
 LT_HD uint32_t plan_delete(uint8_t* leafp, uint32_t LB, uint32_t uold, uint32_t m,
-                           const uint64_t (&y)[kKeys], uint32_t s, const Scratch& S,
+                           const uint64_t (&y)[kKeys], uint32_t s, const SC& S,
                            Result& R) {
   uint64_t head;
   const uint32_t pa = pass_a(leafp, uold, m, y, s, S, head);
@@ -651,51 +614,36 @@ LT_HD uint32_t plan_delete(uint8_t* leafp, uint32_t LB, uint32_t uold, uint32_t 
   return kWritten;
 }
 
-// Pass B of a delete by one thread: the chunks R.wlo .. R.whi from the front,
-// each built from the segments that land in it (every shift is <= 0, so a
-// chunk's sources lie at or above it: not yet written), runs inside one
-// segment by one shift each as in rewrite_leaf.
-LT_HD void rewrite_forward(uint8_t* leafp, uint32_t LB, uint32_t uold, const Scratch& S,
+// Pass B of a delete by one thread: the chunks R.wlo .. R.whi from the front
+// (every shift is <= 0, so a chunk's sources lie at or above it: not yet
+// written), each built as in rewrite_leaf; the chunks past the new used bytes
+// are cleared.
+template <class SC>
+LT_HD void rewrite_forward(uint8_t* leafp, uint32_t LB, uint32_t uold, const SC& S,
                            const Result& R) {
   const uint32_t E = R.E;
   const uint32_t os0 = S.epos[0] & 0xFFFu;
-  const int32_t ohi = (int32_t)R.whi;
-  int cur = -1;  // the lowest segment not wholly below chunk o
-  int32_t slo, shi, ssa;
-  seg_bounds(S, E, uold, os0, cur, slo, shi, ssa);
-  for (int32_t o = (int32_t)R.wlo; o < ohi; o += 16) {
-    while (o < ohi && o >= slo && o + 16 <= shi) {
-      uint32_t r[4];
-      chunk_tail(leafp, o - ssa, r);
-      st16(leafp + o, r);
-      o += 16;
-    }
-    if (o >= ohi) break;
-    while (cur + 1 < (int)E && shi <= o) {
+  int cur = -1;  // the highest segment that starts at or before the chunk's end
+  int32_t slo = 0, shi = (int32_t)os0, ssa = 0;
+  for (int32_t o = (int32_t)R.wlo; o < (int32_t)R.whi; o += 16) {
+    while (cur + 1 < (int)E) {
+      int32_t lo2, hi2, sa2;
+      seg_bounds(S, E, uold, os0, cur + 1, lo2, hi2, sa2);
+      if (lo2 >= o + 16) break;
       cur++;
-      seg_bounds(S, E, uold, os0, cur, slo, shi, ssa);
+      slo = lo2;
+      shi = hi2;
+      ssa = sa2;
     }
-    if (o >= slo && o + 16 <= shi) {  // the next segment's run starts here
-      o -= 16;
-      continue;
-    }
-    uint32_t r[4] = {0u, 0u, 0u, 0u};
-    for (int e = cur; e < (int)E; e++) {
-      int32_t dlo, dhi, sa;
-      seg_bounds(S, E, uold, os0, e, dlo, dhi, sa);
-      if (dlo >= o + 16) break;  // wholly above this chunk: so are the later ones
-      if (dhi > dlo && dhi > o) {
-        const uint32_t a = (uint32_t)((dlo > o ? dlo : o) - o);
-        const uint32_t b = (uint32_t)((dhi < o + 16 ? dhi : o + 16) - o);
-        gather(leafp, LB, o - sa, a, b, r);
-      }
-    }
+    uint32_t r[4];
+    build_chunk(leafp, LB, uold, S, E, os0, cur, slo, shi, ssa, o, r);
     st16(leafp + o, r);
   }
 }
 
 // The delete edits' own bytes: a new head, or the merged code.
-LT_HD void write_delete_edits(uint8_t* leafp, const Scratch& S, const Result& R) {
+template <class SC>
+LT_HD void write_delete_edits(uint8_t* leafp, const SC& S, const Result& R) {
   for (uint32_t e = 0; e < R.E; e++) {
     const uint32_t ep = S.epos[e * S.rs], ek = S.ekey[e * S.rs];
     const uint32_t nl = ek >> 16;
@@ -713,8 +661,9 @@ LT_HD void write_delete_edits(uint8_t* leafp, const Scratch& S, const Result& R)
   }
 }
 
+template <class SC>
 LT_HD uint32_t delete_leaf(uint8_t* leafp, uint32_t LB, uint32_t uold, uint32_t m,
-                           const uint64_t (&y)[kKeys], uint32_t s, const Scratch& S,
+                           const uint64_t (&y)[kKeys], uint32_t s, const SC& S,
                            Result& R) {
   const uint32_t res = plan_delete(leafp, LB, uold, m, y, s, S, R);
   if (res == kWritten) {
@@ -726,8 +675,9 @@ LT_HD uint32_t delete_leaf(uint8_t* leafp, uint32_t LB, uint32_t uold, uint32_t 
 
 // All of it by one thread: returns one of the results above; the leaf is
 // written only for kWritten.
+template <class SC>
 LT_HD uint32_t insert_leaf(uint8_t* leafp, uint32_t LB, uint32_t uold, uint32_t m,
-                           const uint64_t (&y)[kKeys], uint32_t s, const Scratch& S,
+                           const uint64_t (&y)[kKeys], uint32_t s, const SC& S,
                            Result& R) {
   const uint32_t res = plan_leaf(leafp, LB, uold, m, y, s, S, R);
   if (res == kWritten) {

@@ -24,7 +24,7 @@
 // The functions are __host__ __device__ so that the same code can be run on
 // the host.
 #pragma once
-#include "leaf_thread.cuh"
+#include "leaf_bits.cuh"
 
 namespace leafwalk {
 
@@ -378,23 +378,28 @@ LT_HD uint64_t sum_walked(const uint8_t* leafp, uint32_t u) {
   return s;
 }
 
+// Do four continuation bytes in a row end among the leaf's first 24 bytes of
+// codes (words a, b, c)?
+LT_HD bool long_in(uint32_t a, uint32_t b, const uint32_t (&c)[4]) {
+  const uint32_t x[6] = {a, b, c[0], c[1], c[2], c[3]};
+  uint32_t f = 0, y = 0, z = 0;
+#pragma unroll
+  for (int i = 0; i < 6; i++) {
+    const uint32_t fi = x[i] & kFlags, yi = fi & fshl(f, fi, 8);
+    z |= yi & fshl(y, yi, 16);
+    f = fi;
+    y = yi;
+  }
+  return z != 0u;
+}
+
 // The same for a leaf of m elements, whose bytes past u are zero.
 LT_HD uint64_t leaf_sum(const uint8_t* leafp, uint32_t u, uint32_t m) {
-  // four continuation bytes in a row among the first 24 bytes of codes?
   uint32_t w[4], w2[4] = {0u, 0u, 0u, 0u};
   ld16(leafp, w);
   if (u > 16u) ld16(leafp + 16, w2);
-  const uint32_t x[6] = {w[2], w[3], w2[0], w2[1], w2[2], w2[3]};
-  uint32_t c = 0, y = 0, z = 0;
-#pragma unroll
-  for (int i = 0; i < 6; i++) {
-    const uint32_t ci = x[i] & kFlags, yi = ci & fshl(c, ci, 8);
-    z |= yi & fshl(y, yi, 16);
-    c = ci;
-    y = yi;
-  }
   uint64_t s;
-  if (!any_lane(z != 0u)) {
+  if (!any_lane(long_in(w[2], w[3], w2))) {
     const bool ok = any_lane(m > 256u) ? sum_many(leafp, u, m, s) : sum_few(leafp, u, m, s);
     if (ok) return s;
   }

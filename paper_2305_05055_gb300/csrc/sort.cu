@@ -143,7 +143,7 @@ __device__ __forceinline__ void tile_rank(const uint64_t (&key)[ITEMS], const ui
 
 // ---- up to kBTile keys in one block, by bins ----
 constexpr uint32_t kBins = 4096;
-constexpr uint32_t kBinMost = 32;  // keys of a bin ranked against each other (at most 255)
+constexpr uint32_t kBinMost = 128;  // keys of a bin ranked against each other (at most 255)
 struct BinSmem {
   uint64_t keys[kBTile];
   __align__(16) uint32_t bin[kBins + 4];

@@ -419,6 +419,7 @@ struct MergeArgs {
   uint32_t* list_v1;     // touched leaves for k_merge_small (count st->n_v1)
   uint32_t* list_gen;    // work items for k_merge in count mode (st->n_gen)
   uint32_t* list_pend;   // pending leaves of k_insert_thread / k_insert_lane (st->n_pendl)
+  uint32_t* list_long;   // leaves for k_insert_thread_long (st->n_long)
   int raw;               // leaves hold 8-byte cells (codec 1), not byte codes
   int small;             // a small batch: every slice goes to a warp per leaf
   Bounds B;              // density bounds and tree height, for the leaves the
@@ -1262,15 +1263,66 @@ __global__ void __launch_bounds__(kT) k_point_commit(MergeArgs a,
 // rewrites the bytes from the first edit on in place, 16 bytes at a time.  Slices this small are the common case of a
 // batch that is small against the set (about one key per touched leaf), where
 // a warp per leaf leaves most lanes idle.  A leaf with a code of more than 4
-// bytes goes to the element-array splice (state kFallback); a result over LB
-// bytes is left pending for the general merge.
+// bytes goes to k_insert_thread_long; a result over LB bytes is left pending
+// for the general merge.
 constexpr int kThrT = 256;
 constexpr int kThrBuckets = 128;  // tile sort buckets: 16-byte chunks of the old leaf
 
+// What a thread does with its planned leaf: the rewrite, the leaf's new counts
+// and head, and the finalize pass's work for it (batch totals dl and db, the
+// own-bound test).
+template <bool DEL, class SC>
+__device__ __forceinline__ void thread_finish(const MergeArgs& a, uint32_t t, uint32_t tb, uint32_t s,
+                                              uint32_t j, uint32_t m, uint32_t uold, uint32_t fc0,
+                                              uint32_t fc1, uint8_t* leafp,
+                                              const uint64_t (&y)[leafthr::kKeys], const SC& S,
+                                              uint32_t res, const leafthr::Result& R, ull& nbytes,
+                                              ull& dl, ull& db) {
+  uint32_t c0 = 0;
+  if (res == leafthr::kUnchanged) {
+    nbytes += uold;
+    a.T_state[t] = kUnchanged;
+    a.T_newcnt[t] = m;
+    a.T_newbytes[t] = uold;
+  } else if (res == leafthr::kTooBig) {
+    a.T_state[t] = kPending;
+    a.T_newcnt[t] = R.newc;
+    a.T_newbytes[t] = R.nb;
+    a.list_pend[atomicAdd(&a.st->n_pendl, 1ull)] = t;
+    c0 = R.newc;
+  } else {
+    if (DEL) {
+      leafthr::rewrite_forward(leafp, a.LB, uold, S, R);
+      leafthr::write_delete_edits(leafp, S, R);
+      if (R.newc == 0) atomicAdd(&a.st->nempty, 1ull);
+    } else {
+      leafthr::rewrite_leaf(leafp, a.LB, uold, S, R);
+      leafthr::write_edits(leafp, y, S, R);
+    }
+    nbytes += R.nb;
+    a.used[j] = R.nb;
+    a.cnt[j] = R.newc;
+    a.heads[j] = R.newhead;
+    a.T_newcnt[t] = R.newc;
+    a.T_newbytes[t] = R.nb;
+    dl += DEL ? m - R.newc : R.newc - m;
+    db += (ull)R.nb - (ull)uold;
+    if (node_violates(a.B, a.H, 0, 1, R.nb)) a.viol[atomicAdd(&a.st->nviol, 1ull)] = j;
+    a.T_state[t] = kDone;
+  }
+  for (uint32_t cq = fc0; cq < fc1; cq++) a.chunk_cnt[cq] = cq == fc0 ? c0 : 0u;
+  if (a.tag_counts)
+    for (uint32_t q = 0; q < s; q++)
+      if ((R.added >> q) & 1u) credit(a, tb + q);
+}
+
 // DEL: the same for deletes of at most kThrKeys keys from a byte-code leaf
 // (plan_delete, forward rewrite; never over LB bytes).
+// Four blocks per SM (64 registers, a few spilled) ran faster than three with
+// 80: 1e6 keys into 1e8 254 against 257 us, out of it 219 against 237 us; five
+// blocks were slower (271 and 240).
 template <bool DEL>
-__global__ void __launch_bounds__(kThrT) k_insert_thread(MergeArgs a) {
+__global__ void __launch_bounds__(kThrT, 4) k_insert_thread(MergeArgs a) {
   constexpr uint32_t K = leafthr::kKeys;
   __shared__ uint32_t s_rpos[K * kThrT], s_rcode[K * kThrT];
   __shared__ uint64_t s_rval[K * kThrT];
@@ -1318,6 +1370,7 @@ __global__ void __launch_bounds__(kThrT) k_insert_thread(MergeArgs a) {
     if (mine) s_tile[s_hist[bkt] + slot] = (uint32_t)idx;
     __syncthreads();
     ull dl = 0, db = 0;  // db: change of the byte total, mod 2^64
+    uint32_t lng = 0xFFFFFFFFu;
     if (tid < s_hist[kThrBuckets]) {
       const uint32_t t = s_tile[tid];
       const uint32_t tb = a.T_begin[t], s = a.T_begin[t + 1] - tb;
@@ -1335,48 +1388,12 @@ __global__ void __launch_bounds__(kThrT) k_insert_thread(MergeArgs a) {
       const uint32_t res = DEL ? leafthr::plan_delete(leafp, a.LB, uold, m, y, s, S, R)
                                : leafthr::plan_leaf(leafp, a.LB, uold, m, y, s, S, R);
       if (res == leafthr::kLongCode) {
-        a.T_state[t] = kFallback;
-        a.list_v1[atomicAdd(&a.st->n_v1, 1ull)] = t;
+        lng = t;
       } else {
-        uint32_t c0 = 0;
-        if (res == leafthr::kUnchanged) {
-          nbytes += uold;
-          a.T_state[t] = kUnchanged;
-          a.T_newcnt[t] = m;
-          a.T_newbytes[t] = uold;
-        } else if (res == leafthr::kTooBig) {
-          a.T_state[t] = kPending;
-          a.T_newcnt[t] = R.newc;
-          a.T_newbytes[t] = R.nb;
-          a.list_pend[atomicAdd(&a.st->n_pendl, 1ull)] = t;
-          c0 = R.newc;
-        } else {
-          if (DEL) {
-            leafthr::rewrite_forward(leafp, a.LB, uold, S, R);
-            leafthr::write_delete_edits(leafp, S, R);
-            if (R.newc == 0) atomicAdd(&a.st->nempty, 1ull);
-          } else {
-            leafthr::rewrite_leaf(leafp, a.LB, uold, S, R);
-            leafthr::write_edits(leafp, y, S, R);
-          }
-          nbytes += R.nb;
-          a.used[j] = R.nb;
-          a.cnt[j] = R.newc;
-          a.heads[j] = R.newhead;
-          a.T_newcnt[t] = R.newc;
-          a.T_newbytes[t] = R.nb;
-          // the finalize pass's work for this leaf, done here
-          dl += DEL ? m - R.newc : R.newc - m;
-          db += (ull)R.nb - (ull)uold;
-          if (node_violates(a.B, a.H, 0, 1, R.nb)) a.viol[atomicAdd(&a.st->nviol, 1ull)] = j;
-          a.T_state[t] = kDone;
-        }
-        for (uint32_t cq = fc0; cq < fc1; cq++) a.chunk_cnt[cq] = cq == fc0 ? c0 : 0u;
-        if (a.tag_counts)
-          for (uint32_t q = 0; q < s; q++)
-            if ((R.added >> q) & 1u) credit(a, tb + q);
+        thread_finish<DEL>(a, t, tb, s, j, m, uold, fc0, fc1, leafp, y, S, res, R, nbytes, dl, db);
       }
     }
+    warp_append(lng != 0xFFFFFFFFu, lng, a.list_long, &a.st->n_long);
     dl = warp_sum(dl);
     db = warp_sum(db);
     if (lane_id() == 0) {
@@ -1387,6 +1404,51 @@ __global__ void __launch_bounds__(kThrT) k_insert_thread(MergeArgs a) {
   }
   nbytes = warp_sum(nbytes);
   if (a.prof && lane_id() == 0 && nbytes) atomicAdd(a.prof, nbytes);
+}
+
+// The leaves k_insert_thread found a code of more than 4 bytes in (edges
+// u << 32 | v, 64-bit hashes: all of them): the same by 64-bit values, one
+// thread per leaf.  A warp per leaf with the leaf's elements in shared memory
+// took 87 us for the 6e4 leaves that 1e5 edges touch, this 37 us.
+constexpr int kLongT = 128;
+template <bool DEL>
+__global__ void __launch_bounds__(kLongT) k_insert_thread_long(MergeArgs a) {
+  constexpr uint32_t K = leafthr::kKeys;
+  __shared__ uint32_t s_rpos[K * kLongT];
+  __shared__ uint64_t s_rval[K * kLongT], s_rcode[K * kLongT];
+  __shared__ uint32_t s_epos[K * kLongT], s_ekey[K * kLongT];
+  __shared__ int32_t s_esa[K * kLongT];
+  pdl_wait();
+  pdl_launch();
+  if (a.st->err) return;
+  const unsigned tid = threadIdx.x;
+  const leafthr::ScratchLong S{s_rpos + tid, s_rval + tid, s_rcode + tid, s_epos + tid,
+                               s_esa + tid,  s_ekey + tid, (uint32_t)kLongT};
+  const uint64_t n = a.st->n_long;
+  ull nbytes = 0, dl = 0, db = 0;
+  for (uint64_t i = gtid(); i < n; i += gstride()) {
+    const uint32_t t = a.list_long[i];
+    const uint32_t tb = a.T_begin[t], s = a.T_begin[t + 1] - tb;
+    const uint32_t uold = a.T_oldused[t], j = a.T_leaf[t], m = a.T_oldcnt[t];
+    uint8_t* leafp = a.data + (size_t)j * a.LB;
+    uint64_t y[K];
+#pragma unroll
+    for (uint32_t q = 0; q < K; q++) y[q] = q < s ? a.u[tb + q] : 0ull;
+    leafthr::Result R;
+    R.E = 0;
+    const uint32_t res = DEL ? leafthr::plan_delete(leafp, a.LB, uold, m, y, s, S, R)
+                             : leafthr::plan_leaf(leafp, a.LB, uold, m, y, s, S, R);
+    thread_finish<DEL>(a, t, tb, s, j, m, uold, a.T_first_chunk[t], a.T_first_chunk[t + 1], leafp,
+                       y, S, res, R, nbytes, dl, db);
+  }
+  dl = warp_sum(dl);
+  db = warp_sum(db);
+  nbytes = warp_sum(nbytes);
+  if (lane_id() == 0) {
+    if (dl) atomicAdd(&a.st->delta, dl);
+    if (db) atomicAdd(&a.st->bytes_total, db);
+    if (a.prof && nbytes) atomicAdd(a.prof, nbytes);
+  }
 }
 
 // Sort the touched leaves into the merge kernels' work lists: inserts of at
@@ -3038,11 +3100,15 @@ void merge_attrs() {
 // The thread-granular insert (or delete) over the touched leaves of a batch
 // of k keys (at most k of them).
 template <bool DEL>
-void launch_insert_thread(cpma* h, const MergeArgs& ma, uint64_t k, cudaStream_t st) {
+int launch_insert_thread(cpma* h, const MergeArgs& ma, uint64_t k, cudaStream_t st) {
   const int g = (int)std::max<uint64_t>(
       1, std::min<uint64_t>((k + kThrT - 1) / kThrT, (uint64_t)h->num_sms * 16));
   k_insert_thread<DEL><<<g, kThrT, 0, st>>>(ma);
-  h->launches++;
+  const unsigned gl = (unsigned)std::max<uint64_t>(
+      1, std::min<uint64_t>((k + kLongT - 1) / kLongT, (uint64_t)h->num_sms * 8));
+  const cudaError_t e = launch_pdl(k_insert_thread_long<DEL>, gl, kLongT, 0, st, ma);
+  h->launches += 2;
+  return check_cuda(e);
 }
 
 // Every buffer the front segment of a batch of k keys touches, sized before
@@ -3073,6 +3139,7 @@ int front_scratch(cpma* h, uint64_t k, bool tagged, cudaStream_t st) {
   CPMA_TRY(ensure(h, s.list_v1, (k + 2) * 4));
   CPMA_TRY(ensure(h, s.list_gen, (k + 2) * 4));
   CPMA_TRY(ensure(h, s.list_pend, (k + 2) * 4));
+  CPMA_TRY(ensure(h, s.list_long, (k + 2) * 4));
   CPMA_TRY(ensure(h, s.cand, (2 * k + 2) * 8));
   CPMA_TRY(ensure(h, s.wins, (2 * k + 2) * 16));
   CPMA_TRY(ensure(h, s.prefix, (h->L + 2) * 8));
@@ -3201,6 +3268,7 @@ int run_front(cpma* h, const uint64_t* d_keys, uint64_t k, int sorted, int is_de
   ma.list_v1 = P<uint32_t>(s.list_v1);
   ma.list_gen = P<uint32_t>(s.list_gen);
   ma.list_pend = P<uint32_t>(s.list_pend);
+  ma.list_long = P<uint32_t>(s.list_long);
   ma.raw = (int)h->cfg.codec;
   ma.small = k <= kSmallBatch ? 1 : 0;
   ma.B = B;
@@ -3241,14 +3309,14 @@ int run_front(cpma* h, const uint64_t* d_keys, uint64_t k, int sorted, int is_de
       CPMA_CUDA(cudaEventRecord(h->ev_join, h->side));
       ma.prof = prof_bytes(h, PH_MERGE);
       if (!ma.raw && !ma.small) {
-        launch_insert_thread<false>(h, ma, k, st);
+        CPMA_TRY(launch_insert_thread<false>(h, ma, k, st));
       }
       ma.prof = nullptr;
       CPMA_CUDA(cudaStreamWaitEvent(st, h->ev_join, 0));
     }
     if (is_delete && !ma.raw && !ma.small) {
       ma.prof = prof_bytes(h, PH_MERGE);
-      launch_insert_thread<true>(h, ma, k, st);
+      CPMA_TRY(launch_insert_thread<true>(h, ma, k, st));
       ma.prof = nullptr;
     }
     prof_end(h, st);
@@ -3321,7 +3389,7 @@ int run_front(cpma* h, const uint64_t* d_keys, uint64_t k, int sorted, int is_de
 
 constexpr int kGraphSlots = 8;
 
-constexpr int kSigPtrs = 33;
+constexpr int kSigPtrs = 34;
 
 struct FrontSig {
   const void* p[kSigPtrs];
@@ -3343,7 +3411,7 @@ FrontSig front_sig(const cpma* h) {
                    s.chunk_leaf.p, s.chunk_tid.p, s.chunk_cnt.p,     s.chunk_off.p, s.T_leaf.p,
                    s.T_begin.p,   s.T_first_chunk.p, s.T_oldcnt.p,   s.T_oldused.p, s.T_newcnt.p,
                    s.T_newbytes.p, s.T_state.p,   s.viol.p,          s.list_lane.p, s.list_v1.p,
-                   s.list_gen.p,  s.list_pend.p,  s.cand.p,          s.wins.p,      s.bits.p,  h->data,
+                   s.list_gen.p,  s.list_pend.p, s.list_long.p,  s.cand.p,          s.wins.p,      s.bits.p,  h->data,
                    h->used,       h->cnt,         h->heads,          h->d_status},
                   h->L, h->cfg.leaf_bytes, h->sort_poll_limit, h->sort_silent_tile};
 }
@@ -3763,7 +3831,7 @@ void trim_update_scratch(cpma* h) {
                  &s.chunk_begin, &s.chunk_leaf, &s.chunk_tid, &s.chunk_cnt,
                  &s.chunk_off, &s.T_leaf, &s.T_begin, &s.T_first_chunk, &s.T_oldcnt, &s.T_oldused,
                  &s.T_newcnt, &s.T_newbytes, &s.T_state, &s.viol, &s.list_lane, &s.list_v1,
-                 &s.list_gen, &s.list_pend, &s.point_stage, &s.point_rec, &s.cand, &s.wins,
+                 &s.list_gen, &s.list_pend, &s.list_long, &s.point_stage, &s.point_rec, &s.cand, &s.wins,
                  &s.bits, &s.prefix, &s.E, &s.cost, &s.C,
                  &s.srccnt, &s.srcoff, &s.dstart, &s.win_src, &s.win_dst, &s.win_leaf_off,
                  &s.win_elem_off, &s.win_dst_off, &s.partials, &s.stage, &s.fh})
