@@ -56,11 +56,11 @@ void dev_free(cpma* h, void* p, size_t bytes, cudaStream_t st) {
   h->mem_held -= bytes;
 }
 
-int ensure(cpma* h, Buf& b, size_t bytes, cudaStream_t st) {
+int ensure(cpma* h, Buf& b, size_t bytes, cudaStream_t st, int grow) {
   if (bytes == 0) bytes = 16;
   if (b.cap >= bytes) return CPMA_OK;
   if (h->no_alloc || g_capturing) return CPMA_EINTERNAL;
-  size_t want = std::max(bytes, b.cap + b.cap / 2);
+  size_t want = std::max(bytes, b.cap + b.cap / grow);
   want = (want + 255) & ~(size_t)255;
   if (b.p) {
     // growth only: the old contents are dead, but queued kernels may still
@@ -118,8 +118,23 @@ void free_arrays(cpma* h, Arrays* a) {
   *a = Arrays{};
 }
 
-int sync_status(cpma* h, cudaStream_t st) {
-  CPMA_CUDA(cudaMemcpyAsync(h->h_status, h->d_status, sizeof(Status), cudaMemcpyDeviceToHost, st));
+// The status block to the host's pinned copy and, unless the batch was
+// rejected, the number of keys it changed to the caller.  A kernel chained to
+// the one before it instead of two copies, one of them issued only after the
+// host had woken up: 6 us less between an update's last kernel and the next
+// call's first.
+__global__ void k_report(const Status* st, Status* host, uint64_t* d_delta) {
+  pdl_wait();
+  static_assert(sizeof(Status) % 8 == 0 && sizeof(Status) / 8 <= 64, "a word per thread");
+  if (threadIdx.x < sizeof(Status) / 8)
+    reinterpret_cast<volatile ull*>(host)[threadIdx.x] =
+        reinterpret_cast<const ull*>(st)[threadIdx.x];
+  if (d_delta && threadIdx.x == 0 && !st->err) *d_delta = st->delta;
+}
+
+int sync_status(cpma* h, cudaStream_t st, uint64_t* d_delta) {
+  CPMA_CUDA(launch_pdl(k_report, 1, 64, 0, st, h->d_status, h->h_status, d_delta));
+  h->launches++;
   CPMA_CUDA(cudaStreamSynchronize(st));
   prof_resolve(h);
   return CPMA_OK;
@@ -325,7 +340,7 @@ void release_all(cpma* h) {
                  &s.wins, &s.bits, &s.prefix, &s.E, &s.cost, &s.C, &s.srccnt, &s.srcoff, &s.dstart,
                  &s.win_src, &s.win_dst, &s.win_leaf_off, &s.win_elem_off, &s.win_dst_off,
                  &s.partials, &s.partials_q, &s.q_first, &s.q_items, &s.q_off, &s.stage, &s.q_lo,
-                 &s.q_hi, &s.q_rank, &s.q_pre, &s.q_tiles, &s.fh})
+                 &s.q_hi, &s.q_rank, &s.q_pre, &s.fh})
     release(h, *b);
   prof_resolve(h);  // before the graphs (and their events) go
   graph_cache_free(h);
@@ -671,7 +686,7 @@ int cpma_reserve(cpma_t* h, uint64_t max_batch, uint64_t max_queries, int tagged
     CPMA_TRY(ensure(h, s.partials_q, (size_t)(2 * h->num_sms + 2) * 8));
     // range_map runs without its leaf prefix when there is no room for it
     if (max_queries > 1 && !h->cfg.codec) {
-      const int rc = reserve_leaf_prefix(h, std::max(h->L, h->spare.cap_leaves));
+      const int rc = reserve_leaf_prefix(h);
       if (rc != CPMA_OK && rc != CPMA_ENOMEM) return rc;
     }
   }

@@ -131,7 +131,7 @@ struct Scratch {
                           // on another stream while an update sorts
   Buf q_first, q_items, q_off; // range queries
   Buf q_lo, q_hi, q_rank;       // rank-space queries: rank bounds, leaf-count prefix
-  Buf q_pre, q_tiles;           // range queries: reductions before each leaf, and each tile
+  Buf q_pre;                    // range queries: the prefix over the leaves, when E is too small
   Buf stage;              // padded batch of a graph-launched update
   Buf fh;                 // head fix-up: per-tile summaries
 };
@@ -228,7 +228,7 @@ namespace cpmaimpl {
 // set, it refuses to allocate (CPMA_EINTERNAL) instead.
 int dev_alloc(cpma* h, void** p, size_t bytes, cudaStream_t st);
 void dev_free(cpma* h, void* p, size_t bytes, cudaStream_t st);
-int ensure(cpma* h, Buf& b, size_t bytes, cudaStream_t st = nullptr);
+int ensure(cpma* h, Buf& b, size_t bytes, cudaStream_t st = nullptr, int grow = 2);
 void release(cpma* h, Buf& b);
 int alloc_arrays(cpma* h, uint64_t leaves, uint64_t data_bytes, Arrays* a, cudaStream_t st);
 void free_arrays(cpma* h, Arrays* a);
@@ -259,11 +259,15 @@ int scan_u64_given_partials(cpma* h, const uint64_t* in, uint64_t* out, uint64_t
 // and set the kernels' shared-memory attributes.
 int sort_scratch(cpma* h, uint64_t k, bool vals);
 // sort.cu: sort k keys ascending into *out (one of the scratch buffers).
+// cleared: the words sort_control names are zero already.
 int sort_keys(cpma* h, const uint64_t* d_in, uint64_t k, const uint64_t** out,
-              cudaStream_t st);
+              cudaStream_t st, bool cleared = false);
 // the same, moving a 32-bit payload with every key (stable)
 int sort_pairs(cpma* h, const uint64_t* d_in, const uint32_t* v_in, uint64_t k,
-               const uint64_t** out, const uint32_t** vout, cudaStream_t st);
+               const uint64_t** out, const uint32_t** vout, cudaStream_t st,
+               bool cleared = false);
+// The control words a sort of k keys starts from zero (null: none).
+uint32_t* sort_control(cpma* h, uint64_t k, uint32_t* nwords);
 // sort.cu: sort_keys without the passes that a large batch needs only when a
 // window did not hold its buckets: *over (device; null when there is nothing
 // to decide) is then not zero once the work queued here is done, and
@@ -297,14 +301,16 @@ int run_range_reduce(const cpma* h, const uint64_t* lo, const uint64_t* hi, uint
 int run_range_noalloc(const cpma* h, const uint64_t* lo, const uint64_t* hi, uint64_t q,
                       uint64_t* sum, uint64_t* count, cudaStream_t st);
 
-// The buffers of the range queries' prefix over the leaves, for L leaves (the
-// queries run without them when they cannot be had), and giving them back:
-// true when there was something to give (the device is then idle).
-int reserve_leaf_prefix(cpma* h, uint64_t L);
+// The memory of the range queries' prefix over the leaves (the queries run
+// without it when it cannot be had), and giving it back: true when there was
+// something to give (the device is then idle).
+int reserve_leaf_prefix(cpma* h);
 bool release_leaf_prefix(cpma* h);
 
 int check_cuda(cudaError_t e);
-int sync_status(cpma* h, cudaStream_t st);
+// Waits for the stream with the status block brought to h->h_status; d_delta
+// (nullable, device) receives the number of keys changed unless there is an error.
+int sync_status(cpma* h, cudaStream_t st, uint64_t* d_delta = nullptr);
 
 // profiling (no-ops unless enabled)
 void prof_begin(const cpma* h, int phase, cudaStream_t st);

@@ -1035,6 +1035,9 @@ int query_grid(const cpma* h, uint64_t q, int block, uint64_t per_sm) {
       1, std::min<uint64_t>((q + block - 1) / block, (uint64_t)h->num_sms * per_sm));
 }
 
+// Per leaf a reduction and a count, per tile both again.
+size_t leaf_prefix_bytes(uint64_t L) { return L * 12 + (L + kT - 1) / kT * 16; }
+
 // Grows a query buffer; the leaf prefix, which the queries can do without, is
 // given back when there is no room for it.
 int ensure_query(cpma* h, Buf& b, size_t bytes) {
@@ -1043,10 +1046,12 @@ int ensure_query(cpma* h, Buf& b, size_t bytes) {
   return rc;
 }
 
-// The leaf prefix's buffers for this call, or none (the inner leaves are then
-// walked): one query covers no leaf twice, a set without room for them under
-// its memory budget does without, and so does a stream that is being captured
-// while they would have to grow.
+// The leaf prefix's memory for this call, or none (the inner leaves are then
+// walked): one query covers no leaf twice, a set without room for it under its
+// memory budget does without, and so does a stream that is being captured (a
+// graph would keep the address, and the memory may move with the set's size).
+// A set that has been updated holds it already: the redistribution's element
+// buffer, which only an update uses, and none may overlap a query.
 //
 // The rule of the kernels: the prefix is taken when the inner leaves of all
 // queries number more than the set's leaves.  Both forms decode a leaf in the
@@ -1056,20 +1061,19 @@ int ensure_query(cpma* h, Buf& b, size_t bytes) {
 LeafPrefix leaf_prefix(cpma* h, uint64_t q, cudaStream_t st) {
   LeafPrefix p;
   if (q < 2) return p;
-  Scratch& s = h->s;
-  const uint64_t nt = (h->L + kT - 1) / kT;
-  if (s.q_pre.cap < h->L * 12 + 16 || s.q_tiles.cap < nt * 16) {
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
-      cudaGetLastError();
-      return p;
-    }
-    if (reserve_leaf_prefix(h, h->L) != CPMA_OK) return p;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return p;
   }
-  p.val = (uint64_t*)s.q_pre.p;
-  p.cnt = (uint32_t*)(p.val + h->L);
-  p.tval = (uint64_t*)s.q_tiles.p;
+  Scratch& s = h->s;
+  const size_t need = leaf_prefix_bytes(h->L);
+  if (s.E.cap < need && ensure(h, s.q_pre, need) != CPMA_OK) return p;
+  const uint64_t nt = (h->L + kT - 1) / kT;
+  p.val = (uint64_t*)(s.E.cap < need ? s.q_pre.p : s.E.p);
+  p.tval = p.val + h->L;
   p.tcnt = p.tval + nt;
+  p.cnt = (uint32_t*)(p.tcnt + nt);
   p.most = h->L;
   return p;
 }
@@ -1163,19 +1167,18 @@ int raw_prep(cpma* h, const uint64_t* lo, const uint64_t* hi, uint64_t q, uint64
 }  // namespace
 
 bool release_leaf_prefix(cpma* h) {
-  if (!h->s.q_pre.p && !h->s.q_tiles.p) return false;
+  if (!h->s.q_pre.p) return false;
   if (cudaDeviceSynchronize() != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
   release(h, h->s.q_pre);
-  release(h, h->s.q_tiles);
   return true;
 }
 
-int reserve_leaf_prefix(cpma* h, uint64_t L) {
-  CPMA_TRY(ensure(h, h->s.q_pre, L * 12 + 16));
-  return ensure(h, h->s.q_tiles, (L + kT - 1) / kT * 16);
+int reserve_leaf_prefix(cpma* h) {
+  const size_t need = leaf_prefix_bytes(h->L);
+  return h->s.E.cap < need ? ensure(h, h->s.q_pre, need) : CPMA_OK;
 }
 
 int run_range(const cpma* h, const uint64_t* lo, const uint64_t* hi, uint64_t q, uint64_t* sum,

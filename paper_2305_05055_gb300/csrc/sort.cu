@@ -896,7 +896,7 @@ int sort_digits(cpma* h, const uint64_t* d_in, const uint32_t* v_in, uint64_t k,
 // most: a large batch without sort_digits (the caller looks at ctl->rest)
 template <bool VALS>
 int sort_impl(cpma* h, const uint64_t* d_in, const uint32_t* v_in, uint64_t k, const uint64_t** out,
-              const uint32_t** vout, cudaStream_t st, bool most = false) {
+              const uint32_t** vout, cudaStream_t st, bool cleared, bool most = false) {
   *out = d_in;
   if (vout) *vout = v_in;
   if (k <= 1) return CPMA_OK;
@@ -929,11 +929,11 @@ int sort_impl(cpma* h, const uint64_t* d_in, const uint32_t* v_in, uint64_t k, c
   SortCtl* ctl = reinterpret_cast<SortCtl*>(h->s.hist.p);
   const uint32_t G = pass_blocks<VALS>(h, k);
   const Pass a = pass_of<VALS>(h, d_in, v_in, k);
-  CPMA_CUDA(cudaMemsetAsync(ctl, 0, sizeof(SortCtl), st));
+  if (!cleared) CPMA_CUDA(cudaMemsetAsync(ctl, 0, sizeof(SortCtl), st));
   // about eight keys per thread: one step of the unrolled loop
   const int ogrid = (int)std::max<uint64_t>(
       1, std::min<uint64_t>((uint64_t)h->num_sms * 8, (k + 8 * kT - 1) / (8 * kT)));
-  k_orand<<<ogrid, kT, 0, st>>>(d_in, k, ctl, VALS);
+  CPMA_CUDA(launch_pdl(k_orand, ogrid, kT, 0, st, d_in, k, ctl, VALS));
   h->launches++;
   if (k <= kBucketMax) {
     CPMA_TRY(digit_pass<VALS>(h, a, G, kField, VALS, st));
@@ -964,19 +964,24 @@ int sort_impl(cpma* h, const uint64_t* d_in, const uint32_t* v_in, uint64_t k, c
 }
 
 int sort_keys(cpma* h, const uint64_t* d_in, uint64_t k, const uint64_t** out,
-              cudaStream_t st) {
-  return sort_impl<false>(h, d_in, nullptr, k, out, nullptr, st);
+              cudaStream_t st, bool cleared) {
+  return sort_impl<false>(h, d_in, nullptr, k, out, nullptr, st, cleared);
 }
 
 int sort_pairs(cpma* h, const uint64_t* d_in, const uint32_t* v_in, uint64_t k,
-               const uint64_t** out, const uint32_t** vout, cudaStream_t st) {
-  return sort_impl<true>(h, d_in, v_in, k, out, vout, st);
+               const uint64_t** out, const uint32_t** vout, cudaStream_t st, bool cleared) {
+  return sort_impl<true>(h, d_in, v_in, k, out, vout, st, cleared);
+}
+
+uint32_t* sort_control(cpma* h, uint64_t k, uint32_t* nwords) {
+  *nwords = k > (uint64_t)kTile ? (uint32_t)(sizeof(SortCtl) / 4) : 0u;
+  return *nwords ? reinterpret_cast<uint32_t*>(h->s.hist.p) : nullptr;
 }
 
 int sort_keys_most(cpma* h, const uint64_t* d_in, uint64_t k, const uint64_t** out,
                    const uint32_t** over, cudaStream_t st) {
   *over = nullptr;
-  CPMA_TRY(sort_impl<false>(h, d_in, nullptr, k, out, nullptr, st, true));
+  CPMA_TRY(sort_impl<false>(h, d_in, nullptr, k, out, nullptr, st, false, true));
   if (k > kBucketMax) *over = &reinterpret_cast<SortCtl*>(h->s.hist.p)->rest;
   return CPMA_OK;
 }

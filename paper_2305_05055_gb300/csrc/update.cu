@@ -3147,6 +3147,51 @@ int front_scratch(cpma* h, uint64_t k, bool tagged, cudaStream_t st) {
   return ensure_bits(h, st, &lv);
 }
 
+// What the front segment of a batch starts from zero: the status block's
+// batch words, the routing's tile counter and look-back words, the sort's
+// control words.
+struct FrontReset {
+  Status* st;
+  uint64_t* look;
+  uint64_t nlook;
+  uint32_t* ctl;
+  uint32_t nctl;
+};
+
+__device__ __forceinline__ void front_reset(const FrontReset& r) {
+  for (uint64_t i = gtid(); i < offsetof(Status, empties) / 8; i += gstride())
+    reinterpret_cast<uint64_t*>(r.st)[i] = 0;
+  for (uint64_t i = gtid(); i < r.nlook; i += gstride()) r.look[i] = 0;
+  for (uint64_t i = gtid(); i < r.nctl; i += gstride()) r.ctl[i] = 0;
+}
+
+__global__ void __launch_bounds__(kT) k_reset(FrontReset r) { front_reset(r); }
+
+// Routing tiles: keys per thread, the most (8, 4, 2) that still gives two
+// tiles per SM when the batch is dense against the leaves (a tile then
+// reaches about as many heads as it has keys), one otherwise.
+int route_kpt(const cpma* h, uint64_t k) {
+  if (2 * k >= h->L)
+    for (int c = 8; c > 1; c >>= 1)
+      if (k >= (uint64_t)h->num_sms * 2 * kRT * c) return c;
+  return 1;
+}
+
+uint64_t route_tiles(const cpma* h, uint64_t k) {
+  const uint64_t tile_keys = (uint64_t)kRT * route_kpt(h, k);
+  return (k + tile_keys - 1) / tile_keys;
+}
+
+FrontReset reset_of(cpma* h, uint64_t k, int sorted) {
+  FrontReset r;
+  r.st = h->d_status;
+  r.look = P<uint64_t>(h->s.flags);
+  r.nlook = route_tiles(h, k) + 1;
+  r.nctl = 0;
+  r.ctl = sorted ? nullptr : sort_control(h, k, &r.nctl);
+  return r;
+}
+
 // The front segment of an update: status reset, tag check, sort, route,
 // work lists, the in-place merges, finalize and the overflow-offset scan --
 // everything before the first host read of the status block.  It reads the
@@ -3156,22 +3201,18 @@ int front_scratch(cpma* h, uint64_t k, bool tagged, cudaStream_t st) {
 // needs.
 int run_front(cpma* h, const uint64_t* d_keys, uint64_t k, int sorted, int is_delete,
               cudaStream_t st, const uint32_t* tags, uint64_t* tag_counts, uint64_t ntags,
-              Front* f) {
+              Front* f, bool reset_done) {
   Status* ds = h->d_status;
-  CPMA_CUDA(cudaMemsetAsync(ds, 0, offsetof(Status, empties), st));
-  // routing tiles: keys per thread, the most (8, 4, 2) that still gives two
-  // tiles per SM when the batch is dense against the leaves (a tile then
-  // reaches about as many heads as it has keys), one otherwise.  The tile
-  // counter and look-back words are cleared now, so that the routing kernel
-  // directly follows the sort's last kernel.
-  int kpt = 1;
-  if (2 * k >= h->L)
-    for (int c = 8; c > 1 && kpt == 1; c >>= 1)
-      if (k >= (uint64_t)h->num_sms * 2 * kRT * c) kpt = c;
-  const uint64_t tile_keys = (uint64_t)kRT * kpt;
-  const uint64_t ntiles = (k + tile_keys - 1) / tile_keys;
+  // one kernel clears what the segment starts from (the graph's staging kernel
+  // does it there): three memory sets and the gaps between them took 18 us
+  if (!reset_done) {
+    const FrontReset r = reset_of(h, k, sorted);
+    k_reset<<<grid_for(h, r.nlook), kT, 0, st>>>(r);
+    h->launches++;
+  }
+  const int kpt = route_kpt(h, k);
+  const uint64_t ntiles = route_tiles(h, k);
   uint64_t* look = P<uint64_t>(h->s.flags);
-  CPMA_CUDA(cudaMemsetAsync(look, 0, (ntiles + 1) * 8, st));
   const uint64_t* u = d_keys;
   const uint32_t* ut = tags;
   if (tags) {
@@ -3180,8 +3221,8 @@ int run_front(cpma* h, const uint64_t* d_keys, uint64_t k, int sorted, int is_de
   }
   if (!sorted) {
     prof_begin(h, PH_SORT, st);
-    if (tags) CPMA_TRY(sort_pairs(h, d_keys, tags, k, &u, &ut, st));
-    else CPMA_TRY(sort_keys(h, d_keys, k, &u, st));
+    if (tags) CPMA_TRY(sort_pairs(h, d_keys, tags, k, &u, &ut, st, true));
+    else CPMA_TRY(sort_keys(h, d_keys, k, &u, st, true));
     prof_end(h, st);
   }
   Scratch& s = h->s;
@@ -3279,55 +3320,45 @@ int run_front(cpma* h, const uint64_t* d_keys, uint64_t k, int sorted, int is_de
   const size_t msmem = per * mwarps;
   const int mgrid = (int)std::max<uint64_t>(
       1, std::min<uint64_t>((k + kChunk + mwarps - 1) / mwarps, (uint64_t)h->num_sms * 4));
-  // inserts: k_classify runs on the side stream, ahead of the lane kernel
-  // and beside the thread kernel (which walks the touched leaves itself)
-  if (is_delete) {
-    k_classify<<<grid_for(h, k), kT, 0, st>>>(ma);
-    h->launches++;
-  }
   prof_end(h, st);
-  prof_begin(h, PH_MERGE, st);
   {
+    // The thread-granular merge on st; on the side stream meanwhile the work
+    // lists and the merges of the other slices (a warp per leaf or per work
+    // item): disjoint leaves and outputs, shared counters by atomics.  Their
+    // few leaves are latency-bound.
     const size_t sper = small_warp_bytes(LB);
     const int swarps = (int)std::max<size_t>(1, std::min<size_t>(8, (216 * 1024) / (4 * sper)));
     const int sgrid = (int)std::max<uint64_t>(
         1, std::min<uint64_t>((k + swarps - 1) / swarps, (uint64_t)h->num_sms * 8));
-    if (!is_delete) {
-      // the thread-granular insert on st and the work lists plus the
-      // lane-granular insert on the side stream at the same time: disjoint
-      // leaves and outputs (shared counters by atomics); the lane kernel's
-      // few leaves are latency-bound
-      CPMA_CUDA(cudaEventRecord(h->ev_fork, st));
-      CPMA_CUDA(cudaStreamWaitEvent(h->side, h->ev_fork, 0));
-      prof_begin_side(h, PH_MERGE_LANE, h->side);
-      MergeArgs ml = ma;
-      ml.prof = prof_bytes(h, PH_MERGE_LANE);
-      k_classify<<<grid_for(h, k), kT, 0, h->side>>>(ma);
-      k_insert_lane<kLaneSeg><<<sgrid, 256, lane_warp_bytes(kLaneSeg) * 8, h->side>>>(ml);
-      h->launches += 2;
-      prof_end_side(h, h->side);
-      CPMA_CUDA(cudaEventRecord(h->ev_join, h->side));
-      ma.prof = prof_bytes(h, PH_MERGE);
-      if (!ma.raw && !ma.small) {
-        CPMA_TRY(launch_insert_thread<false>(h, ma, k, st));
-      }
-      ma.prof = nullptr;
-      CPMA_CUDA(cudaStreamWaitEvent(st, h->ev_join, 0));
-    }
-    if (is_delete && !ma.raw && !ma.small) {
-      ma.prof = prof_bytes(h, PH_MERGE);
-      CPMA_TRY(launch_insert_thread<true>(h, ma, k, st));
-      ma.prof = nullptr;
-    }
-    prof_end(h, st);
-    prof_begin(h, PH_MERGE2, st);
-    ma.prof = prof_bytes(h, PH_MERGE2);
-    k_merge_small<<<sgrid, swarps * 32, sper * swarps, st>>>(ma);
+    CPMA_CUDA(cudaEventRecord(h->ev_fork, st));
+    CPMA_CUDA(cudaStreamWaitEvent(h->side, h->ev_fork, 0));
+    prof_begin_side(h, PH_MERGE_LANE, h->side);
+    k_classify<<<grid_for(h, k), kT, 0, h->side>>>(ma);
     h->launches++;
+    if (!is_delete) {
+      ma.prof = prof_bytes(h, PH_MERGE_LANE);
+      k_insert_lane<kLaneSeg><<<sgrid, 256, lane_warp_bytes(kLaneSeg) * 8, h->side>>>(ma);
+      h->launches++;
+    }
+    prof_end_side(h, h->side);
+    prof_begin_side(h, PH_MERGE2, h->side);
+    ma.prof = prof_bytes(h, PH_MERGE2);
+    k_merge_small<<<sgrid, swarps * 32, sper * swarps, h->side>>>(ma);
     ma.prof = nullptr;
+    CPMA_CUDA(launch_pdl(k_merge<false>, (unsigned)mgrid, (unsigned)(mwarps * 32), msmem, h->side,
+                         ma));
+    h->launches += 2;
+    prof_end_side(h, h->side);
+    CPMA_CUDA(cudaEventRecord(h->ev_join, h->side));
+    prof_begin(h, PH_MERGE, st);
+    if (!ma.raw && !ma.small) {
+      ma.prof = prof_bytes(h, PH_MERGE);
+      if (is_delete) CPMA_TRY(launch_insert_thread<true>(h, ma, k, st));
+      else CPMA_TRY(launch_insert_thread<false>(h, ma, k, st));
+      ma.prof = nullptr;
+    }
+    CPMA_CUDA(cudaStreamWaitEvent(st, h->ev_join, 0));
   }
-  CPMA_CUDA(launch_pdl(k_merge<false>, (unsigned)mgrid, (unsigned)(mwarps * 32), msmem, st, ma));
-  h->launches++;
   CPMA_CUDA(cudaGetLastError());
   prof_end(h, st);
   prof_begin(h, PH_COUNT, st);
@@ -3454,7 +3485,9 @@ uint64_t graph_bucket(uint64_t k) {  // k rounded up to 5 significant bits
 // floor(j k / K) or one less (j < 2^31, so the error j (2^32 k / K - r) is
 // below 2^32), fixed by one comparison; no division on the device
 __global__ void __launch_bounds__(kT) k_stage(const uint64_t* __restrict__ in, uint64_t k,
-                                              uint64_t* __restrict__ out, uint64_t K, uint64_t r) {
+                                              uint64_t* __restrict__ out, uint64_t K, uint64_t r,
+                                              FrontReset z) {
+  front_reset(z);
   for (uint64_t j = gtid(); j < K; j += gstride()) {
     uint64_t i = (j * r) >> 32;
     if ((i + 1) * K <= j * k) i++;
@@ -3470,7 +3503,7 @@ int run_front_graph(cpma* h, const uint64_t* d_keys, uint64_t k, int sorted, int
   CPMA_TRY(front_scratch(h, K, false, st));
   uint64_t* stage = P<uint64_t>(h->s.stage);
   const uint64_t r = (uint64_t)(((unsigned __int128)k << 32) / K);  // 2^32 when K == k
-  k_stage<<<grid_for(h, K), kT, 0, st>>>(d_keys, k, stage, K, r);
+  k_stage<<<grid_for(h, K), kT, 0, st>>>(d_keys, k, stage, K, r, reset_of(h, K, sorted));
   h->launches++;
   CPMA_CUDA(cudaGetLastError());
   if (!h->graphs) h->graphs = new GraphCache();
@@ -3504,7 +3537,7 @@ int run_front_graph(cpma* h, const uint64_t* d_keys, uint64_t k, int sorted, int
     CPMA_CUDA(cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
     set_capturing(true);
     int rc = run_front(h, stage, K, sorted, is_delete, h->cap_stream, nullptr, nullptr, 0,
-                       &slot->f);
+                       &slot->f, true);
     set_capturing(false);
     if (prof) {
       pr.capturing = false;
@@ -3756,6 +3789,8 @@ int reserve(cpma* h, uint64_t max_batch, int tagged, cudaStream_t st) {
 // fail; the used bytes after the merge lie within t_known -+ t_slack (the
 // redistribution after the last merge) and 10 bytes per key (an inserted
 // key adds at most a 10-byte code, a deleted one removes at most one).
+constexpr int kSetGrow = 4;  // set-sized buffers grow by at least a quarter (a half held
+                             // a third more memory than a set ever used of it)
 int reserve_update(cpma* h, uint64_t k, int is_delete, cudaStream_t st, bool as_if_resizing) {
   Scratch& s = h->s;
   const uint64_t n = h->n, L = h->L;
@@ -3763,9 +3798,9 @@ int reserve_update(cpma* h, uint64_t k, int is_delete, cudaStream_t st, bool as_
   // grown with an eighth to spare, so that a set growing batch by batch
   // does not reallocate them at every step
   const uint64_t n_res = n_hi + n_hi / 8;
-  if (s.E.cap < (n_hi + 1) * 8) CPMA_TRY(ensure(h, s.E, (n_res + 1) * 8, st));
-  if (s.cost.cap < n_hi + 1) CPMA_TRY(ensure(h, s.cost, n_res + 1, st));
-  if (s.C.cap < (n_hi + 2) * 8) CPMA_TRY(ensure(h, s.C, (n_res + 2) * 8, st));
+  if (s.E.cap < (n_hi + 1) * 8) CPMA_TRY(ensure(h, s.E, (n_res + 1) * 8, st, kSetGrow));
+  if (s.cost.cap < n_hi + 1) CPMA_TRY(ensure(h, s.cost, n_res + 1, st, kSetGrow));
+  if (s.C.cap < (n_hi + 2) * 8) CPMA_TRY(ensure(h, s.C, (n_res + 2) * 8, st, kSetGrow));
   const uint64_t dk = 10 * k;
   const uint64_t t_hi = h->t_known + h->t_slack + (is_delete ? 0 : dk);
   const uint64_t sub = h->t_slack + (is_delete ? dk : 0);
@@ -3898,7 +3933,7 @@ int run_update(cpma* h, const uint64_t* d_keys, uint64_t k, int sorted, int is_d
   if (graph) {
     CPMA_TRY(run_front_graph(h, d_keys, k, sorted, is_delete, st, &f));
   } else {
-    CPMA_TRY(run_front(h, d_keys, k, sorted, is_delete, st, tags, tag_counts, ntags, &f));
+    CPMA_TRY(run_front(h, d_keys, k, sorted, is_delete, st, tags, tag_counts, ntags, &f, false));
   }
   const NoAlloc guard(h);  // from here on everything needed is reserved
   MergeArgs& ma = f.ma;
@@ -3908,7 +3943,7 @@ int run_update(cpma* h, const uint64_t* d_keys, uint64_t k, int sorted, int is_d
   const Bounds B = bounds_of(h);
   const int mgrid = f.mgrid, mwarps = f.mwarps;
   const size_t msmem = f.msmem;
-  CPMA_TRY(sync_status(h, st));
+  CPMA_TRY(sync_status(h, st, d_delta));
   prof_begin(h, PH_COUNT, st);
   Status hs = *h->h_status;
   if (hs.err & kErrRoute) return CPMA_ETIMEOUT;
@@ -4002,8 +4037,6 @@ int run_update(cpma* h, const uint64_t* d_keys, uint64_t k, int sorted, int is_d
   // reverse), per leaf of the larger side
   h->t_known = t_merged;
   h->t_slack = t_slack;
-  if (d_delta)
-    CPMA_CUDA(cudaMemcpyAsync(d_delta, &ds->delta, 8, cudaMemcpyDeviceToDevice, st));
   CPMA_CUDA(cudaGetLastError());
   prof_end(h, st);
   return CPMA_OK;
