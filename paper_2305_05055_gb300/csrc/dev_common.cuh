@@ -397,83 +397,6 @@ __device__ __forceinline__ void lane_codes(const uint32_t (&w)[NW], int b_lo, in
   }
 }
 
-// Bytes of w past u - p0 cleared (the leaf's zero padding, read as such).
-__device__ __forceinline__ void mask_past(uint32_t (&w)[4], uint32_t p0, uint32_t u) {
-  if (p0 + 16u > u) {
-    const uint32_t keep = u > p0 ? (1u << (u - p0)) - 1u : 0u;
-#pragma unroll
-    for (int i = 0; i < 4; i++) w[i] &= bytemask4((keep >> (4 * i)) & 0xFu);
-  }
-}
-
-// Is x an element of the byte-code leaf at leafp (u used bytes)?  One
-// thread decodes the leaf from its head, 16 bytes at a time, until the
-// running value passes x.  The bytes are taken eight at a time as in
-// leaf_walk.cuh: the element closed at a terminator is val + acc with a
-// 32-bit acc, so it equals x exactly when acc equals x - val (no element of
-// the group can when x - val >= 2^32, since acc stays below 9 * 2^28).
-// Zero bytes after u repeat the last value, which is an element.  A leaf
-// with a code over 4 bytes is decoded again exactly, byte by byte.
-__device__ __forceinline__ void leaf_has_group(uint32_t wa, uint32_t wb, uint64_t x,
-                                               uint64_t& val, bool& found, uint32_t& acc,
-                                               uint32_t& pw, uint32_t& pwor) {
-  const uint64_t dx = x - val;  // wraps past 2^32 once val > x: no match then
-  const uint32_t d32 = dx > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)dx;
-  const uint32_t pa = wa & 0x7F7F7F7Fu, pb = wb & 0x7F7F7F7Fu;
-  uint32_t r = 0;
-#pragma unroll
-  for (int b = 0; b < 8; b++) {
-    const uint32_t wv = b < 4 ? wa : wb, pv = b < 4 ? pa : pb;
-    acc += __byte_perm(pv, 0u, 0x4440u + (uint32_t)(b & 3)) * pw;
-    const bool term = (wv & (0x80u << (8 * (b & 3)))) == 0u;
-    pwor |= pw;
-    found |= term && acc == d32;
-    r = term ? acc : r;
-    pw = term ? 1u : pw << 7;
-  }
-  val += r;
-  acc -= r;
-}
-
-__device__ __forceinline__ bool thread_leaf_has(const uint8_t* __restrict__ leafp, uint32_t u,
-                                                uint64_t x) {
-  if (u == 0) return false;
-  uint4 v = *reinterpret_cast<const uint4*>(leafp);
-  uint32_t w[4] = {v.x, v.y, v.z, v.w};
-  uint64_t val = (uint64_t)w[0] | ((uint64_t)w[1] << 32);
-  if (x <= val) return x == val;
-  bool found = false;
-  uint32_t acc = 0, pw = 1, pwor = 0;
-  for (uint32_t p0 = 0; p0 < u && val < x; p0 += 16) {
-    if (p0) {
-      v = *reinterpret_cast<const uint4*>(leafp + p0);
-      w[0] = v.x; w[1] = v.y; w[2] = v.z; w[3] = v.w;
-    }
-    mask_past(w, p0, u);
-    if (p0) leaf_has_group(w[0], w[1], x, val, found, acc, pw, pwor);  // bytes 0-7: the head
-    leaf_has_group(w[2], w[3], x, val, found, acc, pw, pwor);
-  }
-  if (pwor >= (1u << 28)) {  // a long code: exact 64-bit decode
-    val = *reinterpret_cast<const uint64_t*>(leafp);
-    found = false;
-    uint64_t a64 = 0;
-    uint32_t sh = 0;
-    for (uint32_t p = 8; p < u && val < x; p++) {
-      const uint32_t c = leafp[p];
-      if (sh < 64) a64 |= (uint64_t)(c & 0x7Fu) << sh;
-      if (c & 0x80u) {
-        sh += 7;
-      } else {
-        val += a64;
-        found |= val == x;
-        a64 = 0;
-        sh = 0;
-      }
-    }
-  }
-  return found;
-}
-
 // ---------------------------------------------------------------------------
 // Sum (mod 2^64) and count of every element of the leaves [j0, j1), added to
 // the calling lane's partials (the caller reduces them over the warp).

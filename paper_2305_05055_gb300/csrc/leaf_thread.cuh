@@ -118,6 +118,62 @@ LT_HD uint32_t word_sum(uint32_t w, uint32_t& cb, uint32_t& p1, uint32_t& p2, ui
   return dp4a(pay, w01, 0u) + (dp4a(pay, w23, 0u) << 14);
 }
 
+// Is x an element of the byte-code leaf of u >= 8 used bytes (bytes past them
+// zero)?  The leaf is summed chunk by chunk as in pass A, to the one whose
+// last element reaches x; that chunk's elements are then compared one by one,
+// by all lanes of a warp together.  A leaf that turns out to hold a code of
+// more than 4 bytes before x is walked instead.
+LT_HD bool leaf_has(const uint8_t* leafp, uint32_t u, uint64_t x) {
+  uint32_t w[4], raw[4];
+  ld16(leafp, raw);
+  uint64_t val = (uint64_t)raw[0] | ((uint64_t)raw[1] << 32);
+  if (x <= val) return x == val;
+  uint32_t carry = 0, lc = 0, cb = 0, p1 = 0, p2 = 0, g0 = 0, p0 = 0;
+  for (;; p0 += 16) {
+#pragma unroll
+    for (int i = 0; i < 4; i++) w[i] = raw[i];
+    if (p0 + 16u < u) ld16(leafp + p0 + 16u, raw);  // on its way while this one is summed
+    const uint32_t cb_in = cb;
+    uint32_t tsum = 0, pay = 0, w01 = 0, w23 = 0;
+    if (p0) {
+      tsum += word_sum(w[0], cb, p1, p2, lc, pay, w01, w23);
+      tsum += word_sum(w[1], cb, p1, p2, lc, pay, w01, w23);
+    }
+    tsum += word_sum(w[2], cb, p1, p2, lc, pay, w01, w23);
+    tsum += word_sum(w[3], cb, p1, p2, lc, pay, w01, w23);
+    const uint32_t tw = ~cb & 0x80808080u;
+    const uint32_t ps = pay & (tw ? ~(0xFFFFFFFFu >> clz32(tw)) : 0xFFFFFFFFu);
+    const uint32_t cnew = dp4a(ps, w01, 0u) + (dp4a(ps, w23, 0u) << 14);
+    lc |= tw ? 0u : 1u;
+    const uint64_t vend = val + (uint32_t)(carry + tsum - cnew);
+    g0 = clz32(~cb_in & 0x80808080u) >> 3;
+    if (vend >= x || lc || p0 + 16u >= u) break;
+    val = vend;
+    carry = cnew;
+  }
+  if (lc) {
+    bool found = false;
+    leafwalk::leaf_visit(leafp, u, [&](uint64_t v) { found |= v == x; });
+    return found;
+  }
+  // the chunk's elements relative to the one before it (zero bytes past the
+  // used ones repeat the last, which is an element)
+  const uint64_t dx = x - val;
+  const uint32_t d = dx > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)dx;
+  uint32_t cum = carry, pw = 1u << (7u * g0);
+  bool found = false;
+#pragma unroll
+  for (int b = 0; b < 16; b++) {
+    const uint32_t c = byte_of(w[b >> 2], b & 3);
+    const bool code = b >= 8 || p0 != 0;  // bytes 0-7 of the leaf are the head
+    cum += code ? (c & 0x7Fu) * pw : 0u;
+    const bool term = code && !(c & 0x80u);
+    found |= term && cum == d;
+    pw = !code ? pw : (c & 0x80u) ? pw << 7 : 1u;
+  }
+  return found;
+}
+
 // Pass A, step 2: the codes of the chunk at p0 take keys q..q1-1 (all of
 // them: their values lie between the element before the chunk and the last
 // element completed in it).  Decode the chunk byte by byte from the state it

@@ -1,6 +1,6 @@
 // Queries over the compressed leaves.
 //  has (Sec. 5 "Point queries"): binary search on the uncompressed heads, then
-//    one warp-cooperative pass over the leaf.
+//    one pass over the leaf.
 //  range_map (Sec. 3: a search for the first element, then a scan to the end
 //    of the range) with f = (sum mod 2^64, count).  A query covers parts of its
 //    first and last leaf and all of the leaves between them.  The parts are
@@ -25,6 +25,7 @@
 
 #include "dev_common.cuh"
 #include "internal.h"
+#include "leaf_thread.cuh"
 #include "leaf_walk.cuh"
 
 using namespace cpmadev;
@@ -39,35 +40,39 @@ __device__ __forceinline__ uint64_t gtid() {
 }
 __device__ __forceinline__ uint64_t gstride() { return (uint64_t)gridDim.x * blockDim.x; }
 
-// Warp per query key, 32 keys routed per step.  A key equal to its leaf's
-// head, below it or above the leaf's last element needs no decode beyond the
-// lane summaries; otherwise only the lane whose value interval holds the key
-// is decoded (one byte position per lane).  Leaves with codes longer than 4
-// bytes or more than 512 used bytes go through the general decoder.
+// Byte codes: a thread per query key routes it and searches its leaf
+// (leafthr::leaf_has) up to the key.  Bound by instruction issue: a warp runs
+// as long as its deepest search.  1e6 keys against 1e8: 156 us, 195 us when the
+// leaf was decoded code by code.  (A block ordering its 256 keys by how deep
+// each is likely to lie: 154 us, and 1.9 us more on 1e3 keys.)
 __global__ void __launch_bounds__(kT) k_has(const uint64_t* __restrict__ keys, uint64_t q,
                                             const uint8_t* __restrict__ data,
                                             const uint32_t* __restrict__ used,
                                             const uint64_t* __restrict__ heads, uint64_t L,
-                                            uint32_t LB, uint8_t* __restrict__ out,
-                                            ull* prof, int raw) {
+                                            uint32_t LB, uint8_t* __restrict__ out, ull* prof) {
+  ull nbytes = 0;
+  for (uint64_t i = (uint64_t)blockIdx.x * kT + threadIdx.x; i < q;
+       i += (uint64_t)gridDim.x * kT) {
+    const uint64_t x = keys[i], j = route_leaf(heads, L, x);
+    const uint32_t u = min(used[j], LB);
+    out[i] = u && leafthr::leaf_has(data + j * LB, u, x) ? 1u : 0u;
+    nbytes += u + 9;
+  }
+  nbytes = warp_sum(nbytes);
+  if (prof && lane_id() == 0 && nbytes) atomicAdd(prof, nbytes);
+}
+
+// Cells (codec 1): a warp per key, 32 routed per step.
+__global__ void __launch_bounds__(kT) k_has_cells(const uint64_t* __restrict__ keys, uint64_t q,
+                                                  const uint8_t* __restrict__ data,
+                                                  const uint32_t* __restrict__ used,
+                                                  const uint64_t* __restrict__ heads, uint64_t L,
+                                                  uint32_t LB, uint8_t* __restrict__ out,
+                                                  ull* prof) {
   const unsigned lane = lane_id();
-  const uint64_t gw = gtid() >> 5, nw = gstride() >> 5;
   ull nbytes = 0;
   uint64_t r0, r1;
-  warp_share(q, gw, nw, r0, r1);
-  if (!raw) {
-    // byte codes: one key per thread, its leaf decoded up to the key
-    for (uint64_t qi = r0 + lane; qi < r1; qi += 32) {
-      const uint64_t x = keys[qi];
-      const uint64_t j = route_leaf(heads, L, x);
-      const uint32_t u = min(used[j], LB);
-      nbytes += u + 9;
-      out[qi] = thread_leaf_has(data + j * LB, u, x) ? 1u : 0u;
-    }
-    nbytes = warp_sum(nbytes);
-    if (prof && lane == 0 && nbytes) atomicAdd(prof, nbytes);
-    return;
-  }
+  warp_share(q, gtid() >> 5, gstride() >> 5, r0, r1);
   for (uint64_t base = r0; base < r1; base += 32) {
     const uint64_t qi = base + lane;
     uint64_t xi = 0, ji = 0;
@@ -83,66 +88,10 @@ __global__ void __launch_bounds__(kT) k_has(const uint64_t* __restrict__ keys, u
       const uint64_t x = __shfl_sync(FULL, xi, k);
       const uint64_t j = __shfl_sync(FULL, ji, k);
       const uint32_t u = __shfl_sync(FULL, ui, k);
-      const uint8_t* leaf = data + j * LB;
       nbytes += u + 9;
-      bool found = false;
-      if (raw) {  // codec 1: compare the cells
-        bool f = false;
-        warp_decode(leaf, u, [&](uint32_t, uint64_t val) { f |= (val == x); }, true);
-        found = __any_sync(FULL, f);
-      } else if (u > 0) {
-        const uint32_t p0 = lane * 16u;
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (p0 < u) v = __ldg(reinterpret_cast<const uint4*>(leaf + p0));
-        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-        const int b_lo = lane == 0 ? 8 : 0;
-        const int b_hi = (u > p0) ? (int)min(16u, u - p0) : 0;
-        LaneCodes lc;
-        lane_codes<false>(w, b_lo, b_hi, lc);
-        bool bad = lc.bad || u > 512;  // one 16-byte chunk per lane covers 512 bytes
-        uint32_t pv = __shfl_up_sync(FULL, lc.tail, 1);
-        uint32_t ps = __shfl_up_sync(FULL, lc.tail_sh, 1);
-        if (lane == 0) { pv = 0; ps = 0; }
-        uint32_t D = 0;
-        if (lc.term) {
-          if (ps / 7u + lc.first_len > 4u) bad = true;
-          D = lc.D - lc.first_own + pv + (lc.first_own << ps);
-        }
-        if (__any_sync(FULL, bad)) {
-          bool f = false;
-          warp_decode(leaf, u, [&](uint32_t, uint64_t val) { f |= (val == x); });
-          found = __any_sync(FULL, f);
-        } else {
-          const uint64_t head = __shfl_sync(FULL, (uint64_t)w[0] | ((uint64_t)w[1] << 32), 0);
-          const uint64_t Dinc = warp_incl_scan((uint64_t)D);
-          const uint64_t V = head + (Dinc - D);
-          const uint64_t lastv = head + __shfl_sync(FULL, Dinc, 31);
-          if (x == head) {
-            found = true;
-          } else if (x > head && x <= lastv) {
-            const unsigned own = __ballot_sync(FULL, lc.term != 0 && V < x && x <= V + D);
-            const unsigned o = __ffs(own) - 1;
-            uint32_t xo[4];
-#pragma unroll
-            for (int t = 0; t < 4; t++) xo[t] = __shfl_sync(FULL, lc.x[t], o);
-            const uint32_t term_o = __shfl_sync(FULL, lc.term, o);
-            const uint32_t pv_o = __shfl_sync(FULL, pv, o), ps_o = __shfl_sync(FULL, ps, o);
-            const uint64_t V_o = __shfl_sync(FULL, V, o);
-            const bool is_t = lane < 16 && ((term_o >> lane) & 1u);
-            const uint32_t before = lane < 16 ? (term_o & ((1u << lane) - 1u)) : 0u;
-            const bool firstc = before == 0;
-            const uint32_t st0 = firstc ? (o == 0 ? 8u : 0u) : (32u - (uint32_t)__clz(before));
-            uint32_t code = 0;
-            if (is_t) {
-              const uint32_t own_bits = compact7(window32(xo, st0)) & mask7(lane + 1u - st0);
-              code = firstc ? pv_o + (own_bits << ps_o) : own_bits;
-            }
-            const uint64_t val = V_o + warp_incl_scan(code);
-            found = __any_sync(FULL, is_t && val == x);
-          }
-        }
-      }
-      if (found) found_bits |= 1u << k;
+      bool f = false;
+      warp_decode(data + j * LB, u, [&](uint32_t, uint64_t val) { f |= (val == x); }, true);
+      if (__any_sync(FULL, f)) found_bits |= 1u << k;
     }
     if (qi < r1) out[qi] = (found_bits >> lane) & 1u;
   }
@@ -644,12 +593,12 @@ __device__ __forceinline__ uint64_t block_scan_op(uint64_t v, uint64_t* ws, uint
   return op_apply<OP>(carry, e);
 }
 
-constexpr uint32_t kSumShift = 4;      // sort key of a leaf: used bytes / 16
+constexpr uint32_t kSumShift = 4;      // sort key of a leaf: bytes to decode / 16
 constexpr uint32_t kSumBuckets = 128;  // enough for 2048-byte leaves (a multiple of 32)
 
-// Order of the nt <= kT leaves of a tile by used bytes (a counting sort in
-// shared memory), so the 32 leaves a warp decodes side by side take about the
-// same number of steps: order[i] = the tile's leaf that thread i takes.
+// Order of the nt <= kT leaves of a tile by the bytes u to decode of each (a
+// counting sort in shared memory), so the 32 leaves a warp decodes side by
+// side take about the same number of steps: order[i] = the one thread i takes.
 __device__ __forceinline__ void order_tile(uint32_t u, uint32_t nt, uint32_t* hist,
                                            uint32_t* order) {
   for (uint32_t i = threadIdx.x; i < kSumBuckets; i += kT) hist[i] = 0;
@@ -1014,8 +963,9 @@ int run_has(const cpma* h, const uint64_t* d_keys, uint64_t q, uint8_t* d_out, c
   const int grid = (int)std::max<uint64_t>(
       1, std::min<uint64_t>((q + kT - 1) / kT, (uint64_t)persistent_grid(h)));
   prof_begin(h, PH_HAS, st);
-  k_has<<<grid, kT, 0, st>>>(d_keys, q, h->data, h->used, h->heads, h->L, h->cfg.leaf_bytes,
-                             d_out, prof_bytes(h, PH_HAS), (int)h->cfg.codec);
+  const auto kern = h->cfg.codec ? k_has_cells : k_has;
+  kern<<<grid, kT, 0, st>>>(d_keys, q, h->data, h->used, h->heads, h->L, h->cfg.leaf_bytes, d_out,
+                            prof_bytes(h, PH_HAS));
   CPMA_LAUNCHED(h);
   prof_end(h, st);
   return check_cuda(cudaGetLastError());

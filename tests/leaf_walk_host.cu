@@ -1,5 +1,6 @@
-// Host build of a thread's walk over a leaf (leaf_walk.cuh) for the CPU tests.
-#include "../paper_2305_05055_gb300/csrc/leaf_walk.cuh"
+// Host build of a thread's walk over a leaf (leaf_walk.cuh) and of its
+// membership test (leaf_thread.cuh) for the CPU tests.
+#include "../paper_2305_05055_gb300/csrc/leaf_thread.cuh"
 
 extern "C" uint64_t lw_sum(const uint8_t* leaf, uint32_t u, uint32_t m, int form) {
   uint64_t s = 0;
@@ -29,4 +30,8 @@ extern "C" void lw_take(const uint8_t* leaf, uint32_t u, uint64_t lo, uint64_t m
 
 extern "C" uint32_t lw_below(const uint8_t* leaf, uint32_t u, uint64_t x) {
   return leafwalk::leaf_below(leaf, u, x);
+}
+
+extern "C" int lw_has(const uint8_t* leaf, uint32_t u, uint64_t x) {
+  return leafthr::leaf_has(leaf, u, x) ? 1 : 0;
 }

@@ -35,6 +35,7 @@ def lw(tmp_path_factory):
     lib.lw_range.argtypes = [u8, u32, u64, u64, p64]
     lib.lw_take.argtypes = [u8, u32, u64, u64, p64]
     lib.lw_below.restype, lib.lw_below.argtypes = u32, [u8, u32, u64]
+    lib.lw_has.argtypes = [u8, u32, u64]
     return lib
 
 
@@ -121,6 +122,7 @@ def test_walk_against_keys(lw, LB):
         res = (C.c_uint64 * 3)()
         for lo in marks:
             assert lw.lw_below(p, u, lo) == bisect.bisect_left(keys, lo)
+            assert lw.lw_has(p, u, lo) == (lo in keys)
             for hi in rng.sample(marks, 6):
                 if lo >= hi:
                     continue
