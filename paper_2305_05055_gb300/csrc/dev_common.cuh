@@ -261,12 +261,6 @@ __device__ __forceinline__ uint32_t warp_encode(const uint64_t* z, uint32_t r, u
   return pos;
 }
 
-// Byte cost of z[i] in a stream: 8 for the first element, else its code
-// (8 for every element of the uncompressed format).
-__device__ __forceinline__ uint32_t elem_cost(const uint64_t* z, uint32_t i, bool raw = false) {
-  return (i == 0 || raw) ? 8u : leb_len(z[i] - z[i - 1]);
-}
-
 // ---------------------------------------------------------------------------
 // Bit-parallel summary of the codes in one lane's 16 bytes of a leaf, for
 // leaves whose codes are at most 4 bytes long (deltas < 2^28).
@@ -317,7 +311,6 @@ struct LaneCodesN {
   uint32_t x[NW];     // the lane's bytes, zero outside [b_lo, b_hi)
   uint32_t term;      // bit b: byte b ends a code
   uint32_t D;         // own bits of the codes ending here (first one without carry)
-  uint32_t W;         // sum over those codes of (index among them) * own bits
   uint32_t first_own; // own bits of the first code ending here
   uint32_t first_len; // its own byte count
   uint32_t tail;      // bits of the partial code after the last terminator
@@ -325,10 +318,8 @@ struct LaneCodesN {
   bool bad;           // a code longer than 4 bytes, or no terminator
 };
 
-using LaneCodes = LaneCodesN<4>;
-
 // NW words (4*NW <= 32 bytes) per lane; b_lo, b_hi in bytes of the lane.
-template <bool WANT_W, int NW = 4>
+template <int NW>
 __device__ __forceinline__ void lane_codes(const uint32_t (&w)[NW], int b_lo, int b_hi,
                                            LaneCodesN<NW>& L) {
   uint32_t range = 0;
@@ -349,8 +340,8 @@ __device__ __forceinline__ void lane_codes(const uint32_t (&w)[NW], int b_lo, in
   // before it, at most 3) of its code.  With 0/1 byte masks m_i of g_b == i,
   // dp4a with multipliers m0 + 128 m1 and m2 + 128 m3 gives S0 + (S1 << 7)
   // and S2 + (S3 << 7) directly, S_i the sum of the group-i payloads.
-  uint32_t S01 = 0, S23 = 0, W0 = 0, W1 = 0, W2 = 0, W3 = 0;
-  uint32_t badm = 0, base = 0;
+  uint32_t S01 = 0, S23 = 0;
+  uint32_t badm = 0;
 #pragma unroll
   for (int q = 0; q < NW; q++) {
     const uint32_t prev = q ? cb[q - 1] : 0u;
@@ -363,15 +354,6 @@ __device__ __forceinline__ void lane_codes(const uint32_t (&w)[NW], int b_lo, in
     const uint32_t m0 = ~p1 & 0x01010101u, m1 = p1 ^ a12, m2 = a12 ^ a123, m3 = a123;
     S01 = __dp4a(v, m0 | (m1 << 7), S01);
     S23 = __dp4a(v, m2 | (m3 << 7), S23);
-    if constexpr (WANT_W) {
-      // terminators before each byte of the word (bytes), plus the earlier words'
-      const uint32_t lidx = tb[q] * 0x01010100u + base * 0x01010101u;
-      W0 = __dp4a(v & (m0 * 0x7Fu), lidx, W0);
-      W1 = __dp4a(v & (m1 * 0x7Fu), lidx, W1);
-      W2 = __dp4a(v & (m2 * 0x7Fu), lidx, W2);
-      W3 = __dp4a(v & (m3 * 0x7Fu), lidx, W3);
-      base += __popc(tb[q]);
-    }
   }
   const uint32_t Dall = S01 + (S23 << 14);
   L.bad = badm != 0 || (range != 0 && L.term == 0);
@@ -380,7 +362,6 @@ __device__ __forceinline__ void lane_codes(const uint32_t (&w)[NW], int b_lo, in
   L.first_own = 0;
   L.first_len = 0;
   L.D = 0;
-  L.W = 0;
   if (L.term) {
     const uint32_t lt = 31u - (uint32_t)__clz(L.term);
     const uint32_t tl = (uint32_t)b_hi - 1u - lt;
@@ -390,10 +371,6 @@ __device__ __forceinline__ void lane_codes(const uint32_t (&w)[NW], int b_lo, in
     L.first_len = ft + 1u - (uint32_t)b_lo;
     L.first_own = compact7(b_lo == 0 ? L.x[0] : L.x[2]) & mask7(L.first_len);
     L.D = Dall - L.tail;
-    if constexpr (WANT_W) {
-      const uint32_t c = __popc(L.term);
-      L.W = (W0 + (W1 << 7) + (W2 << 14) + (W3 << 21)) - c * L.tail;
-    }
   }
 }
 

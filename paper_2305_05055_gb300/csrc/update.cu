@@ -686,7 +686,7 @@ __device__ __forceinline__ uint32_t lane_leaf(const MergeArgs& a, uint8_t* wbase
   const int b_lo = sl == 0 ? 8 : 0;
   const int b_hi = (uold > p0) ? (int)min(kLB, uold - p0) : 0;
   LaneCodesN<NW> lc;
-  lane_codes<false, NW>(w, b_lo, b_hi, lc);
+  lane_codes<NW>(w, b_lo, b_hi, lc);
   bool bad = lc.bad;
   uint32_t pv = __shfl_up_sync(seg, lc.tail, 1, SEG);
   uint32_t ps = __shfl_up_sync(seg, lc.tail_sh, 1, SEG);
