@@ -340,7 +340,7 @@ void release_all(cpma* h) {
                  &s.wins, &s.bits, &s.prefix, &s.E, &s.cost, &s.C, &s.srccnt, &s.srcoff, &s.dstart,
                  &s.win_src, &s.win_dst, &s.win_leaf_off, &s.win_elem_off, &s.win_dst_off,
                  &s.partials, &s.partials_q, &s.q_first, &s.q_items, &s.q_off, &s.stage, &s.q_lo,
-                 &s.q_hi, &s.q_rank, &s.q_pre, &s.fh})
+                 &s.q_hi, &s.q_rank, &s.q_pre, &s.q_marks, &s.fh})
     release(h, *b);
   prof_resolve(h);  // before the graphs (and their events) go
   graph_cache_free(h);
@@ -686,7 +686,7 @@ int cpma_reserve(cpma_t* h, uint64_t max_batch, uint64_t max_queries, int tagged
     CPMA_TRY(ensure(h, s.partials_q, (size_t)(2 * h->num_sms + 2) * 8));
     // range_map runs without its leaf prefix when there is no room for it
     if (max_queries > 1 && !h->cfg.codec) {
-      const int rc = reserve_leaf_prefix(h);
+      const int rc = reserve_leaf_prefix(h, max_queries);
       if (rc != CPMA_OK && rc != CPMA_ENOMEM) return rc;
     }
   }

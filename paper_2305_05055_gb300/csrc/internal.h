@@ -131,6 +131,7 @@ struct Scratch {
                           // on another stream while an update sorts
   Buf q_first, q_items, q_off; // range queries
   Buf q_lo, q_hi, q_rank;       // rank-space queries: rank bounds, leaf-count prefix
+  Buf q_marks;                  // the same queries: marks inside the leaves, when E is too small
   Buf q_pre;                    // range queries: the prefix over the leaves, when E is too small
   Buf stage;              // padded batch of a graph-launched update
   Buf fh;                 // head fix-up: per-tile summaries
@@ -301,10 +302,11 @@ int run_range_reduce(const cpma* h, const uint64_t* lo, const uint64_t* hi, uint
 int run_range_noalloc(const cpma* h, const uint64_t* lo, const uint64_t* hi, uint64_t q,
                       uint64_t* sum, uint64_t* count, cudaStream_t st);
 
-// The memory of the range queries' prefix over the leaves (the queries run
-// without it when it cannot be had), and giving it back: true when there was
-// something to give (the device is then idle).
-int reserve_leaf_prefix(cpma* h);
+// The memory of the range queries' prefix over the leaves, and of the marks
+// inside them for q or more queries (the queries run without them when it
+// cannot be had), and giving it back: true when there was something to give
+// (the device is then idle).
+int reserve_leaf_prefix(cpma* h, uint64_t q);
 bool release_leaf_prefix(cpma* h);
 
 int check_cuda(cudaError_t e);

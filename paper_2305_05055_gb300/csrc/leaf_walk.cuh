@@ -552,4 +552,99 @@ LT_HD uint32_t leaf_below(const uint8_t* leafp, uint32_t u, uint64_t x) {
   return n;
 }
 
+// ---- marks: the walk's state at every kMark-th byte of a leaf ----
+//
+// For many queries on one leaf the walk is done once and kept at every 32nd
+// byte: a query then starts at the last mark whose element is below its bound
+// and walks at most 32 bytes instead of half the leaf.  (Every 64th byte:
+// degrees of 2^20 vertices 192 us instead of 150.)
+constexpr uint32_t kMark = 32;
+
+struct alignas(16) Mark {
+  uint64_t val;  // the last element closed before the mark
+  uint64_t sum;  // the sum of those elements, the head included
+  uint64_t acc;  // the open code, as in Walk
+  uint32_t cnt;
+  uint32_t sh;
+};
+
+// Walks a leaf of u >= 8 used bytes: put(i, its state at byte kMark * i) for
+// 0 < kMark * i < u; s and c = the sum and the number of its elements.
+template <class F>
+LT_HD void leaf_marks(const uint8_t* leafp, uint32_t u, uint64_t& s, uint32_t& c, F&& put) {
+  Walk k;
+  k.val = leaf_head(leafp);
+  s = k.val;
+  c = 1;
+  uint32_t raw[4];
+  ld16(leafp, raw);
+  for (uint32_t p0 = 0; p0 < u; p0 += 16) {
+    uint32_t w[4], t[4], T;
+    uint64_t ss, v;
+    next_chunk(leafp, p0, u, raw, w, t);
+    if (p0) {  // bytes 0-7 are the head
+      if (p0 % kMark == 0) put(p0 / kMark, Mark{k.val, s, k.acc, c, k.sh});
+      v = k.val;
+      group_sum(w[0], w[1], t[0], t[1], k, T, ss);
+      s += T * v + ss;
+      c += T;
+    }
+    v = k.val;
+    group_sum(w[2], w[3], t[2], t[3], k, T, ss);
+    s += T * v + ss;
+    c += T;
+  }
+}
+
+// The walk at a mark: the flags carried in follow from the open code's bytes.
+LT_HD Walk walk_at(const Mark& m) {
+  Walk k;
+  k.val = m.val;
+  k.acc = m.acc;
+  k.sh = m.sh;
+  const uint32_t n = m.sh / 7u;  // continuation bytes right before the mark
+  k.c = n >= 4u ? kFlags : n ? kFlags << (8u * (4u - n)) : 0u;
+  k.y = n >= 5u ? kFlags : n > 1u ? kFlags << (8u * (5u - n)) : 0u;
+  return k;
+}
+
+// Adds the sum and the number of the elements < x that the walk k closes from
+// byte p (a multiple of 16) on to s and c.  k.val < x.  With this few groups
+// to go each is compared element by element, instead of being summed whole and
+// the last one decoded again.
+LT_HD void below_sum(const uint8_t* leafp, uint32_t u, uint32_t p, Walk k, uint64_t x, uint64_t& s,
+                     uint64_t& c) {
+  auto step = [&](uint32_t wa, uint32_t wb, uint32_t ta, uint32_t tb) {
+    const uint32_t pa = wa & 0x7F7F7F7Fu, pb = wb & 0x7F7F7F7Fu;
+    const uint64_t v = k.val, d = x - v;  // elements val + acc with acc < d
+    uint32_t n = 0;
+    uint64_t ss = 0;
+    const int form = group_form(wa, wb, k);
+    if (form == 0) {
+      const uint32_t d32 = d >> 32 ? 0xFFFFFFFFu : (uint32_t)d;
+      uint32_t s32 = 0;
+      short_codes(pa, pb, ta, tb, k, [&](uint32_t acc) {
+        if (acc < d32) { n++; s32 += acc; }
+      });
+      ss = s32;
+    } else {
+      auto take = [&](uint64_t acc) {
+        if (acc < d) { n++; ss += acc; }
+      };
+      if (form == 1) medium_codes(pa, pb, ta, tb, k, take);
+      else long_codes(pa, pb, ta, tb, k, take);
+    }
+    s += n * v + ss;
+    c += n;
+  };
+  uint32_t raw[4];
+  if (p < u) ld16(leafp + p, raw);
+  for (uint32_t p0 = p; p0 < u && k.val < x; p0 += 16) {
+    uint32_t w[4], t[4];
+    next_chunk(leafp, p0, u, raw, w, t);
+    if (p0) step(w[0], w[1], t[0], t[1]);
+    if (k.val < x) step(w[2], w[3], t[2], t[3]);
+  }
+}
+
 }  // namespace leafwalk

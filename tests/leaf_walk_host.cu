@@ -35,3 +35,21 @@ extern "C" uint32_t lw_below(const uint8_t* leaf, uint32_t u, uint64_t x) {
 extern "C" int lw_has(const uint8_t* leaf, uint32_t u, uint64_t x) {
   return leafthr::leaf_has(leaf, u, x) ? 1 : 0;
 }
+
+// Elements < x and their sum, from the last mark below x.
+extern "C" void lw_marked(const uint8_t* leaf, uint32_t u, uint64_t x, uint64_t* out) {
+  leafwalk::Mark m[2048 / leafwalk::kMark];
+  uint32_t n = 0, at = 0;
+  leafwalk::leaf_marks(leaf, u, out[2], n, [&](uint32_t i, const leafwalk::Mark& v) { m[i] = v; });
+  out[0] = out[1] = 0;
+  out[3] = n;
+  leafwalk::Walk k;
+  k.val = leafwalk::leaf_head(leaf);
+  if (k.val >= x) return;
+  for (uint32_t i = 1; i * leafwalk::kMark < u; i++)
+    if (m[i].val < x) at = i;
+  out[0] = at ? m[at].sum : k.val;
+  out[1] = at ? m[at].cnt : 1;
+  if (at) k = leafwalk::walk_at(m[at]);
+  leafwalk::below_sum(leaf, u, at * leafwalk::kMark, k, x, out[0], out[1]);
+}

@@ -84,6 +84,38 @@ def test_total_at_the_line():
             check(g, p, np.full(q, lo, U), np.full(q, hi, U), q)
 
 
+@pytest.mark.parametrize("LB", [256, 272, 2048])
+@pytest.mark.parametrize("kind", [40, 64, "edges", "mixed"])
+def test_a_query_per_leaf_and_more(kind, LB):
+    # the leaves are marked from L queries on; some leaves hold nothing
+    base = keys_of(kind, 30_000, 8)
+    p, g = oracle.PlainSet(base), cp.CPMA(T(base), leaf_bytes=LB, rho_leaf=0, rho_root=1)
+    gone = p.S[p.S.size // 4:p.S.size // 2].copy()
+    assert int(g.delete_batch(T(gone)).item()) == p.delete_batch(gone)
+    L, S = g.leaves(), p.S
+    for q in (L - 1, L, 3 * L + 1):
+        lo, hi, _ = W.range_queries_by_rank(S, 5 + q, q, 1, 60)
+        lo[::5] += U(1)
+        hi[::7] -= U(1)
+        lo[0], hi[0] = 0, 0xFFFFFFFFFFFFFFFF
+        lo[-1], hi[-1] = gone[0], gone[-1]
+        tl, th = T(lo), T(hi)
+        want = p.range_map(lo, hi)
+        same(g.range_map(tl, th), want, (L, q))
+        g.set_mem_budget(g.mem_held())               # the memory it holds is enough
+        same(g.range_map(tl, th), want, (L, q, "again"))
+        g.set_mem_budget(0)
+    h = cp.CPMA(T(S), leaf_bytes=LB)
+    h.set_mem_budget(h.mem_held() + 64 * q)          # room for the queries, not for the marks
+    lo, hi, _ = W.range_queries_by_rank(S, 4, 4 * q, 1, 60)
+    same(h.range_map(T(lo[:q]), T(hi[:q])), p.range_map(lo[:q], hi[:q]), "within the budget")
+    h.set_mem_budget(0)
+    h.reserve(1, 4 * q)
+    held = h.mem_held()
+    same(h.range_map(T(lo), T(hi)), p.range_map(lo, hi), "reserved")
+    assert h.mem_held() == held
+
+
 def test_empty_leaves_inside():
     base = np.arange(40_000, dtype=U) * U(1000)
     p, g = oracle.PlainSet(base), cp.CPMA(T(base), leaf_bytes=256, rho_leaf=0, rho_root=1)

@@ -36,6 +36,7 @@ def lw(tmp_path_factory):
     lib.lw_take.argtypes = [u8, u32, u64, u64, p64]
     lib.lw_below.restype, lib.lw_below.argtypes = u32, [u8, u32, u64]
     lib.lw_has.argtypes = [u8, u32, u64]
+    lib.lw_marked.argtypes = [u8, u32, u64, p64]
     return lib
 
 
@@ -119,8 +120,11 @@ def test_walk_against_keys(lw, LB):
         for _ in range(6):
             x = rng.choice(keys)
             marks += [x, (x + 1) & M64, max(x - 1, 0), rng.randrange(keys[0], keys[-1] + 1)]
-        res = (C.c_uint64 * 3)()
+        res = (C.c_uint64 * 4)()
         for lo in marks:
+            a = bisect.bisect_left(keys, lo)
+            lw.lw_marked(p, u, lo, res)
+            assert list(res) == [sum(keys[:a]) & M64, a, sum(keys) & M64, len(keys)]
             assert lw.lw_below(p, u, lo) == bisect.bisect_left(keys, lo)
             assert lw.lw_has(p, u, lo) == (lo in keys)
             for hi in rng.sample(marks, 6):
