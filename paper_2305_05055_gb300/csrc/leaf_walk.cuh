@@ -406,6 +406,85 @@ LT_HD uint64_t leaf_sum(const uint8_t* leafp, uint32_t u, uint32_t m) {
   return sum_walked(leafp, u);
 }
 
+// The walk's state at a byte of the leaf.
+struct alignas(16) Mark {
+  uint64_t val;  // the last element closed before it
+  uint64_t sum;  // the sum of those elements, the head included (or as said)
+  uint64_t acc;  // the open code, as in Walk
+  uint32_t cnt;
+  uint32_t sh;
+};
+
+// The flags carried in follow from the open code's bytes.
+LT_HD Walk walk_at(const Mark& m) {
+  Walk k;
+  k.val = m.val;
+  k.acc = m.acc;
+  k.sh = m.sh;
+  const uint32_t n = m.sh / 7u;  // continuation bytes right before it
+  k.c = n >= 4u ? kFlags : n ? kFlags << (8u * (4u - n)) : 0u;
+  k.y = n >= 5u ? kFlags : n > 1u ? kFlags << (8u * (5u - n)) : 0u;
+  return k;
+}
+
+// Chunks of 16 bytes whose elements are all below x, passed over whole: k and
+// n (the elements closed) move past them, raw holds the chunk at the byte
+// returned, where the walk goes on.  From the leaf's start, raw its first
+// chunk.  With codes of up to 5 bytes a chunk is five sums of byte products
+// (payloads at position 0 to 4 of their code), no step per byte: about 110
+// operations, 150 by groups of 8 while codes are short and 220 when a lane has
+// a longer one.  (Not before a loop over the range itself, as in
+// leaf_range_sum: a warp then takes its longest skip and its longest range one
+// after the other; 1e5 ranges 189 -> 200 us.)  It stops before a chunk with a code of more than 5 bytes, and
+// before the last, partial one.
+LT_HD uint32_t skip_below(const uint8_t* leafp, uint32_t u, uint64_t x, Walk& k, uint32_t& n,
+                          uint32_t (&raw)[4]) {
+  using leafthr::dp4a;
+  uint32_t c = 0, q1 = 0, q2 = 0, q3 = 0, lng = 0, p0 = 0;
+  for (; p0 + 16u <= u; p0 += 16u) {
+    uint32_t next[4] = {0u, 0u, 0u, 0u};
+    if (p0 + 16u < u) ld16(leafp + p0 + 16u, next);  // on its way while this one is summed
+    uint32_t s01 = 0, s23 = 0, s4 = 0, conts = 0, pay = 0, w01 = 0, w23 = 0;
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+      if (i < 2 && p0 == 0) continue;  // the head
+      const uint32_t cw = raw[i] & kFlags;
+      const uint32_t b1 = fshl(c, cw, 8);  // position in its code >= 1, .. >= 4
+      const uint32_t b2 = b1 & fshl(q1, b1, 8);
+      const uint32_t b3 = b2 & fshl(q2, b2, 8);
+      const uint32_t b4 = b3 & fshl(q3, b3, 8);
+      lng |= b4 & cw;
+      pay = raw[i] & 0x7F7F7F7Fu;
+      w01 = ((~b1 & kFlags) >> 7) | (b1 ^ b2);
+      w23 = ((b2 ^ b3) >> 7) | (b3 ^ b4);
+      s01 = dp4a(pay, w01, s01);
+      s23 = dp4a(pay, w23, s23);
+      s4 = dp4a(pay, b4 >> 7, s4);
+      conts += popc(cw);
+      c = cw;
+      q1 = b1;
+      q2 = b2;
+      q3 = b3;
+    }
+    // the open code: it starts in the last word, or lng is set
+    const uint32_t tw = ~c & kFlags;
+    const uint32_t ps = pay & (tw ? ~(0xFFFFFFFFu >> leafthr::clz32(tw)) : 0xFFFFFFFFu);
+    const uint32_t open = dp4a(ps, w01, 0u) + (dp4a(ps, w23, 0u) << 14);
+    const uint64_t end =
+        k.val + (k.acc + s01 + ((uint64_t)s23 << 14) + ((uint64_t)s4 << 28) - open);
+    if (lng || end >= x) break;
+    n += (p0 ? 16u : 8u) - conts;
+    k.val = end;
+    k.acc = open;
+    k.sh = tw ? 7u * (leafthr::clz32(tw) >> 3) : 28u;
+    k.c = c;
+    k.y = c & q1;
+#pragma unroll
+    for (int i = 0; i < 4; i++) raw[i] = next[i];
+  }
+  return p0;
+}
+
 // f(element) for every element of a leaf of u >= 8 used bytes, in order.
 template <class F>
 LT_HD void leaf_visit(const uint8_t* leafp, uint32_t u, F&& f) {
@@ -419,6 +498,21 @@ LT_HD void leaf_visit(const uint8_t* leafp, uint32_t u, F&& f) {
     next_chunk(leafp, p0, u, raw, w, t);
     if (p0) group_visit(w[0], w[1], t[0], t[1], k, f);
     group_visit(w[2], w[3], t[2], t[3], k, f);
+  }
+}
+
+// f(element) for the elements that the walk k closes from byte p (a multiple
+// of 8, past the head) on, until done() holds after a group.
+template <class F, class D>
+LT_HD void visit_from(const uint8_t* leafp, uint32_t u, uint32_t p, Walk k, F&& f, D&& done) {
+  uint32_t p0 = p & ~15u;
+  uint32_t raw[4];
+  if (p0 < u) ld16(leafp + p0, raw);
+  for (; p0 < u && !done(); p0 += 16) {
+    uint32_t w[4], t[4];
+    next_chunk(leafp, p0, u, raw, w, t);
+    if (p0 >= p) group_visit(w[0], w[1], t[0], t[1], k, f);
+    if (!done()) group_visit(w[2], w[3], t[2], t[3], k, f);
   }
 }
 
@@ -489,6 +583,12 @@ LT_HD void leaf_take_sum(const uint8_t* leafp, uint32_t u, uint64_t lo, uint64_t
   };
   take(k.val);
   uint32_t p = 8;
+  if (k.val < lo) {
+    uint32_t raw[4];
+    ld16(leafp, raw);
+    const uint32_t p0 = skip_below(leafp, u, lo, k, below, raw);
+    if (p0) p = p0;
+  }
   // up to the group that reaches lo, counted; that group; then whole groups
   // while they fit; then the group that does not
   Held g;
@@ -523,14 +623,18 @@ LT_HD void leaf_take_sum(const uint8_t* leafp, uint32_t u, uint64_t lo, uint64_t
   if (have) group_visit(g.wa, g.wb, g.ta, g.tb, g.k, take);
 }
 
-// Elements < x of a leaf of u >= 8 used bytes.
-LT_HD uint32_t leaf_below(const uint8_t* leafp, uint32_t u, uint64_t x) {
+// Elements < x of a leaf of u >= 8 used bytes.  at = where the first element
+// >= x is closed, if the leaf has one past its head: the state before its
+// group of 8 bytes, `sum` the group's byte and `cnt` the elements before it;
+// else the byte is 0.
+LT_HD uint32_t leaf_below(const uint8_t* leafp, uint32_t u, uint64_t x, Mark& at) {
   Walk k;
   k.val = leaf_head(leafp);
-  uint32_t n = k.val < x ? 1u : 0u;
+  at = Mark{0, 0, 0, 0, 0};
+  if (k.val >= x) return 0;
+  uint32_t n = 1, p = 0;
   Held g;
-  bool have = k.val >= x;
-  const bool none = have;
+  bool have = false;
   auto step = [&](uint32_t wa, uint32_t wb, uint32_t ta, uint32_t tb) {
     g = Held{k, wa, wb, ta, tb};
     uint32_t T;
@@ -541,14 +645,21 @@ LT_HD uint32_t leaf_below(const uint8_t* leafp, uint32_t u, uint64_t x) {
   };
   uint32_t raw[4];
   ld16(leafp, raw);
-  for (uint32_t p0 = 0; p0 < u && !have; p0 += 16) {
+  uint32_t p0 = skip_below(leafp, u, x, k, n, raw);
+  for (; p0 < u && !have; p0 += 16) {
     uint32_t w[4], t[4];
     next_chunk(leafp, p0, u, raw, w, t);
+    p = p0;
     if (p0) step(w[0], w[1], t[0], t[1]);
-    if (!have) step(w[2], w[3], t[2], t[3]);
+    if (!have) {
+      p = p0 + 8u;
+      step(w[2], w[3], t[2], t[3]);
+    }
   }
-  if (have && !none)
+  if (have) {
+    at = Mark{g.k.val, p, g.k.acc, n, g.k.sh};
     group_visit(g.wa, g.wb, g.ta, g.tb, g.k, [&](uint64_t v) { n += v < x ? 1u : 0u; });
+  }
   return n;
 }
 
@@ -559,14 +670,6 @@ LT_HD uint32_t leaf_below(const uint8_t* leafp, uint32_t u, uint64_t x) {
 // and walks at most 32 bytes instead of half the leaf.  (Every 64th byte:
 // degrees of 2^20 vertices 192 us instead of 150.)
 constexpr uint32_t kMark = 32;
-
-struct alignas(16) Mark {
-  uint64_t val;  // the last element closed before the mark
-  uint64_t sum;  // the sum of those elements, the head included
-  uint64_t acc;  // the open code, as in Walk
-  uint32_t cnt;
-  uint32_t sh;
-};
 
 // Walks a leaf of u >= 8 used bytes: put(i, its state at byte kMark * i) for
 // 0 < kMark * i < u; s and c = the sum and the number of its elements.
@@ -594,18 +697,6 @@ LT_HD void leaf_marks(const uint8_t* leafp, uint32_t u, uint64_t& s, uint32_t& c
     s += T * v + ss;
     c += T;
   }
-}
-
-// The walk at a mark: the flags carried in follow from the open code's bytes.
-LT_HD Walk walk_at(const Mark& m) {
-  Walk k;
-  k.val = m.val;
-  k.acc = m.acc;
-  k.sh = m.sh;
-  const uint32_t n = m.sh / 7u;  // continuation bytes right before the mark
-  k.c = n >= 4u ? kFlags : n ? kFlags << (8u * (4u - n)) : 0u;
-  k.y = n >= 5u ? kFlags : n > 1u ? kFlags << (8u * (5u - n)) : 0u;
-  return k;
 }
 
 // Adds the sum and the number of the elements < x that the walk k closes from

@@ -208,6 +208,7 @@ struct ExtractArgs {
   uint32_t LB;
   uint64_t* out;
   uint64_t cap;
+  const leafwalk::Mark* start = nullptr;  // where each query's first key lies (leaf_below)
 };
 
 __global__ void __launch_bounds__(kT) k_extract(ExtractArgs a) {
@@ -721,6 +722,21 @@ __global__ void __launch_bounds__(kT) k_tile_scan(const uint64_t* __restrict__ t
   }
 }
 
+// The warp's equal contiguous share of N items that its lanes take one each:
+// as many warps as have 32 of them, spread over the blocks, so that few items
+// do not leave most lanes of every warp idle (with shares over all 9728 warps
+// of the grid, the 2.4e4 inner leaves of 1e5 short scans ran 2.3 lanes a warp:
+// 54 us, now 16; the 1e5 leaves that a packed neighbour query extracts 5.4
+// lanes: 73 us, now 41, the start of each first leaf's walk included).
+__device__ __forceinline__ void lane_share(uint64_t N, uint64_t& g0, uint64_t& g1) {
+  const uint64_t w = (uint64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+  const uint64_t nw = max((uint64_t)1, min(gstride() >> 5, (N + 31) >> 5));
+  g0 = g1 = 0;
+  if (w >= nw) return;
+  g0 = N * w / nw;
+  g1 = N * (w + 1) / nw;
+}
+
 // The leaves strictly inside the ranges.  From the prefix: a thread per
 // query.  Otherwise the (query, leaf) items in equal contiguous shares per
 // warp, one leaf per lane: a lane keeps its partial while it stays on one
@@ -753,8 +769,8 @@ __global__ void __launch_bounds__(kT) k_range_inner(Leaves t, Reduce<OP, PLAIN> 
     return;
   }
   const unsigned lane = lane_id();
-  const uint64_t gw = gtid() >> 5, nw = gstride() >> 5;
-  const uint64_t g0 = N * gw / nw, g1 = N * (gw + 1) / nw;
+  uint64_t g0, g1;
+  lane_share(N, g0, g1);
   if (g0 >= g1) return;
   uint64_t qi = 0, qend = 0, qoff = 0, fl = 0;
   uint64_t r = op_identity<OP>(), c = 0;
@@ -926,18 +942,20 @@ __global__ void __launch_bounds__(kT) k_rank_ends(const uint64_t* __restrict__ A
                                                   uint64_t* __restrict__ r1o,
                                                   uint64_t* __restrict__ first,
                                                   uint64_t* __restrict__ items,
-                                                  uint64_t* __restrict__ count) {
+                                                  uint64_t* __restrict__ count,
+                                                  leafwalk::Mark* __restrict__ start) {
   pdl_wait();
   pdl_launch();
   // whole warps stay in the loop: both lanes of a query take part in it
   for (uint64_t g = gtid() & ~31ull; g < 2 * q; g += gstride()) {
     const uint64_t e = g + lane_id(), i = e >> 1;
     uint64_t r = 0, j = 0;
+    leafwalk::Mark at{0, 0, 0, 0, 0};
     if (i < q) {
       const uint64_t x = (e & 1) ? B[i] : A[i];
       j = route_leaf(t.heads, t.L, x);
       const uint32_t u = min(t.used[j], t.LB);
-      r = P[j] + (u ? leafwalk::leaf_below(t.data + j * t.LB, u, x) : 0u);
+      r = P[j] + (u ? leafwalk::leaf_below(t.data + j * t.LB, u, x, at) : 0u);
     }
     const uint64_t r1 = __shfl_down_sync(FULL, r, 1);
     if (i < q && !(e & 1)) {
@@ -953,19 +971,21 @@ __global__ void __launch_bounds__(kT) k_rank_ends(const uint64_t* __restrict__ A
       first[i] = fl;
       items[i] = it;
       count[i] = hi - r;
+      if (start) start[i] = at;  // its byte is 0 unless fl == j
     }
   }
 }
 
 // The keys of ranks [r0, r1) of every query, one (query, leaf) item per lane:
 // out[off + r - r0] = key of rank r (entries at or past cap are dropped).  A
+// query's first leaf is walked from where the search for its first key ended
+// (a.start, null without room for it), the others from their heads.  A
 // lane stores its leaf's keys one after another; the eight bytes of
 // neighbouring keys meet in the L2's lines.
 __global__ void __launch_bounds__(kT) k_extract_leaf(ExtractArgs a) {
   pdl_wait();
-  const uint64_t gw = gtid() >> 5, nw = gstride() >> 5;
-  const uint64_t N = a.item_off[a.q];
-  const uint64_t g0 = N * gw / nw, g1 = N * (gw + 1) / nw;
+  uint64_t g0, g1;
+  lane_share(a.item_off[a.q], g0, g1);
   uint64_t qi = 0, qend = 0;
   for (uint64_t g = g0 + lane_id(); g < g1; g += 32) {
     if (g >= qend) {
@@ -990,12 +1010,25 @@ __global__ void __launch_bounds__(kT) k_extract_leaf(ExtractArgs a) {
       stop = min(stop, room - before);
     }
     uint64_t* dst = a.out + (int64_t)(o + base - r0);
-    uint32_t idx = 0;
+    uint32_t idx = 0, p = 8;
     const uint32_t st = (uint32_t)min(stop, (uint64_t)0xFFFFFFFFu);
-    leafwalk::leaf_visit(a.data + j * a.LB, u, [&](uint64_t v) {
+    const uint8_t* leafp = a.data + j * a.LB;
+    auto put = [&](uint64_t v) {
       if (idx >= skip && idx < st) dst[idx] = v;
       idx++;
-    });
+    };
+    leafwalk::Walk k;
+    leafwalk::Mark m{0, 0, 0, 0, 0};
+    if (a.start && r0 >= base) m = a.start[qi];
+    if (m.sum) {  // from where the first key's search ended
+      k = leafwalk::walk_at(m);
+      p = (uint32_t)m.sum;
+      idx = m.cnt;
+    } else {
+      k.val = leafwalk::leaf_head(leafp);
+      put(k.val);
+    }
+    leafwalk::visit_from(leafp, u, p, k, put, [&] { return idx >= st; });
   }
 }
 
@@ -1399,6 +1432,10 @@ int run_range_extract(const cpma* h, const uint64_t* lo, const uint64_t* hi, uin
   uint64_t* P = (uint64_t*)s.q_rank.p;
   uint64_t* r0 = (uint64_t*)s.q_lo.p;
   uint64_t* r1 = (uint64_t*)s.q_hi.p;
+  // where each query's first key lies in its leaf, when there is room
+  leafwalk::Mark* start = nullptr;
+  if (!h->cfg.codec && out && cap)
+    start = (leafwalk::Mark*)prefix_memory(hm, s.q_marks, q * sizeof(leafwalk::Mark), st);
   prof_begin(h, PH_RANGE_PREP, st);
   CPMA_TRY(scan_u32_query(hm, h->cnt, P, h->L, st));
   // the counts (r1 - r0) go to `offsets` first
@@ -1408,7 +1445,7 @@ int run_range_extract(const cpma* h, const uint64_t* lo, const uint64_t* hi, uin
         nullptr, offsets);
   } else {
     CPMA_CUDA(launch_pdl(k_rank_ends, (unsigned)query_grid(h, 2 * q, kT, 8), kT, 0, st, lo, hi, q,
-                         leaves_of(h), P, r0, r1, r.first, r.items, offsets));
+                         leaves_of(h), P, r0, r1, r.first, r.items, offsets, start));
   }
   CPMA_LAUNCHED(h);
   CPMA_TRY(scan_u64_query(hm, offsets, offsets, q, st));
@@ -1417,6 +1454,7 @@ int run_range_extract(const cpma* h, const uint64_t* lo, const uint64_t* hi, uin
   prof_end(h, st);
   if (!emit) return check_cuda(cudaGetLastError());
   ExtractArgs a;
+  a.start = start;
   a.r0 = r0;
   a.r1 = r1;
   a.q = q;

@@ -29,7 +29,8 @@ extern "C" void lw_take(const uint8_t* leaf, uint32_t u, uint64_t lo, uint64_t m
 }
 
 extern "C" uint32_t lw_below(const uint8_t* leaf, uint32_t u, uint64_t x) {
-  return leafwalk::leaf_below(leaf, u, x);
+  leafwalk::Mark at;
+  return leafwalk::leaf_below(leaf, u, x, at);
 }
 
 extern "C" int lw_has(const uint8_t* leaf, uint32_t u, uint64_t x) {
@@ -52,4 +53,16 @@ extern "C" void lw_marked(const uint8_t* leaf, uint32_t u, uint64_t x, uint64_t*
   out[1] = at ? m[at].cnt : 1;
   if (at) k = leafwalk::walk_at(m[at]);
   leafwalk::below_sum(leaf, u, at * leafwalk::kMark, k, x, out[0], out[1]);
+}
+
+// The elements from lo on, starting where the search for it ended; returns
+// how many (0 when it did not end at a code).
+extern "C" uint32_t lw_from(const uint8_t* leaf, uint32_t u, uint64_t lo, uint64_t* out) {
+  leafwalk::Mark at;
+  const uint32_t r = leafwalk::leaf_below(leaf, u, lo, at);
+  uint32_t n = 0, idx = at.cnt;
+  if (at.sum)
+    leafwalk::visit_from(leaf, u, (uint32_t)at.sum, leafwalk::walk_at(at),
+                         [&](uint64_t v) { if (idx++ >= r) out[n++] = v; }, [] { return false; });
+  return n;
 }

@@ -36,6 +36,7 @@ def lw(tmp_path_factory):
     lib.lw_take.argtypes = [u8, u32, u64, u64, p64]
     lib.lw_below.restype, lib.lw_below.argtypes = u32, [u8, u32, u64]
     lib.lw_has.argtypes = [u8, u32, u64]
+    lib.lw_from.restype, lib.lw_from.argtypes = u32, [u8, u32, u64, p64]
     lib.lw_marked.argtypes = [u8, u32, u64, p64]
     return lib
 
@@ -134,6 +135,8 @@ def test_walk_against_keys(lw, LB):
                 lw.lw_range(p, u, lo, hi, res)
                 assert (res[0], res[1]) == (sum(keys[a:b]) & M64, b - a)
             a = bisect.bisect_left(keys, lo)
+            n = lw.lw_from(p, u, lo, out)
+            assert list(out[:n]) == (keys[a:] if 0 < a else [])
             for most in (0, 1, 2, rng.randint(0, len(keys)), len(keys) - a, 1 << 40, M64):
                 got = keys[a:a + most]
                 lw.lw_take(p, u, lo, most, res)
