@@ -3954,9 +3954,12 @@ int run_update(cpma* h, const uint64_t* d_keys, uint64_t k, int sorted, int is_d
   const uint64_t delta = hs.delta;
   const uint64_t n_after = is_delete ? h->n - delta : h->n + delta;
   // empty leaves: made by this batch's merges, or left when the last head
-  // fix-up ran (a window redistribution never empties a leaf: each gets
-  // about S/W >= rho_leaf LB > 10 bytes, more than one code)
-  h->may_have_empty = hs.nempty || hs.empties;
+  // fix-up ran.  A window redistribution empties none while each leaf gets
+  // about S/W >= rho_leaf LB > 10 bytes, more than one code; with a lower
+  // bound below that, a leaf left pending by a delete may be rewritten empty.
+  h->may_have_empty = hs.nempty || hs.empties ||
+                      (is_delete && hs.npend &&
+                       (uint64_t)h->cfg.rho_leaf * h->cfg.leaf_bytes <= 20000);
 
   // ---- pending leaves: materialise their merged elements ----
   if (hs.npend) {

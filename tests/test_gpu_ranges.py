@@ -127,6 +127,26 @@ def test_empty_leaves_inside():
     check(g, p, lo, hi, 2)
 
 
+@pytest.mark.parametrize("LB,a,b", [(2048, 2, 3), (2048, 1, 7), (256, 1, 7)])
+def test_leaves_emptied_by_slices_of_many_keys(LB, a, b):
+    # (slices of more keys than one work item holds: the leaf is left pending
+    # and rewritten, empty, by the redistribution; no lower density bound)
+    base = keys_of("edges", 30_000, 8)
+    p, g = oracle.PlainSet(base), cp.CPMA(T(base), leaf_bytes=LB, rho_leaf=0, rho_root=1)
+    gone = p.S[p.S.size * a // 8:p.S.size * b // 8].copy()
+    assert int(g.delete_batch(T(gone)).item()) == p.delete_batch(gone)
+    _, used, heads = g.layout()
+    heads, used = cp.to_u64(heads)[:used.numel()], used.cpu().numpy()
+    assert (used == 0).sum() > 1
+    want = [U(0xFFFFFFFFFFFFFFFF)]           # an empty leaf's head: the next one's
+    for h, u in zip(heads[::-1], used[::-1]):
+        want.append(h if u else want[-1])
+    assert np.array_equal(heads, np.array(want[:0:-1], U))
+    assert bool(g.has_batch(T(p.S)).all()) and not bool(g.has_batch(T(gone)).any())
+    lo, hi, _ = W.range_queries_by_rank(p.S, 9, 500, 1, 60)
+    check(g, p, lo, hi, 2)
+
+
 def test_without_room_for_the_prefix_and_in_a_capture():
     base = W.uniform_keys(13, 200_000, bits=40)
     p, g = oracle.PlainSet(base), cp.CPMA(T(base))
