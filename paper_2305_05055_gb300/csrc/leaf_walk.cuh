@@ -516,6 +516,29 @@ LT_HD void visit_from(const uint8_t* leafp, uint32_t u, uint32_t p, Walk k, F&& 
   }
 }
 
+// f(element) for the elements v with lo <= v < hi of a leaf of u >= 8 used
+// bytes, in order.
+template <class F>
+LT_HD void leaf_range_visit(const uint8_t* leafp, uint32_t u, uint64_t lo, uint64_t hi, F&& f) {
+  Walk k;
+  k.val = leaf_head(leafp);
+  if (k.val >= hi) return;
+  uint32_t p = 8;
+  if (k.val >= lo) {
+    f(k.val);
+  } else {
+    uint32_t raw[4], n = 0;
+    ld16(leafp, raw);
+    p = skip_below(leafp, u, lo, k, n, raw);
+    if (!p) p = 8;
+  }
+  uint64_t last = k.val;
+  visit_from(leafp, u, p, k, [&](uint64_t v) {
+    if (v >= lo && v < hi) f(v);
+    last = v;
+  }, [&] { return last >= hi; });
+}
+
 // A group set aside: the walk as it was before it, and its words.  The few
 // groups that a bound falls into are decoded after the loop over the leaf, by
 // all lanes of a warp together, instead of inside it, where each lane would
@@ -661,6 +684,64 @@ LT_HD uint32_t leaf_below(const uint8_t* leafp, uint32_t u, uint64_t x, Mark& at
     group_visit(g.wa, g.wb, g.ta, g.tb, g.k, [&](uint64_t v) { n += v < x ? 1u : 0u; });
   }
   return n;
+}
+
+// ---- a leaf walked by a team of lanes ----
+//
+// One lane walks a leaf in some 30 steps that wait for one another; with few
+// queries on the GPU that chain is what a call waits for.  Here each of kTeam
+// lanes takes an equal run of 16-byte chunks: it enters with the code open at
+// its first byte (found by walking the chunk before from any state: every code
+// has at most 10 bytes, so one ends in it), sums its deltas, learns from a scan
+// over the team the element before its run, and then visits its elements.
+constexpr uint32_t kTeam = 8;
+
+struct Run {
+  Walk k;               // at byte b0; val 0 until the scan over the team
+  uint32_t b0, b1;      // the lane's bytes
+  uint64_t delta = 0;   // what its codes add up to
+  uint32_t codes = 0;
+};
+
+// Lane tl's run of a leaf of u used bytes (0: no leaf).
+LT_HD Run team_run(const uint8_t* leafp, uint32_t u, uint32_t tl) {
+  const uint32_t per = 16u * (((u + 15u) / 16u + kTeam - 1u) / kTeam);
+  Run r;
+  r.b0 = per * tl;
+  r.b1 = r.b0 + per < u ? r.b0 + per : u;
+  uint32_t w[4], t[4], T;
+  uint64_t ss;
+  Walk k;
+  if (tl && r.b0 < u) {
+    load_chunk(leafp, r.b0 - 16u, u, w, t);
+    if (r.b0 > 16u) group_sum(w[0], w[1], t[0], t[1], k, T, ss);  // else the head
+    group_sum(w[2], w[3], t[2], t[3], k, T, ss);
+    k.val = 0;
+  }
+  r.k = k;
+  for (uint32_t p0 = r.b0; p0 < r.b1; p0 += 16) {
+    load_chunk(leafp, p0, u, w, t);
+    if (p0) {
+      group_sum(w[0], w[1], t[0], t[1], k, T, ss);
+      r.codes += T;
+    }
+    group_sum(w[2], w[3], t[2], t[3], k, T, ss);
+    r.codes += T;
+  }
+  r.delta = k.val;
+  return r;
+}
+
+// f(element) for the run's elements (its k.val set), the head not among them.
+template <class F>
+LT_HD void run_visit(const uint8_t* leafp, uint32_t u, const Run& r, F&& f) {
+  Walk k = r.k;
+  for (uint32_t p0 = r.b0; p0 < r.b1; p0 += 16) {
+    uint32_t w[4], t[4];
+    load_chunk(leafp, p0, u, w, t);
+    if (p0) group_visit(w[0], w[1], t[0], t[1], k, f);
+    group_visit(w[2], w[3], t[2], t[3], k, f);
+  }
 }
 
 // ---- marks: the walk's state at every kMark-th byte of a leaf ----

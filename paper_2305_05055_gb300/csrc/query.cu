@@ -62,6 +62,91 @@ __global__ void __launch_bounds__(kT) k_has(const uint64_t* __restrict__ keys, u
   if (prof && lane_id() == 0 && nbytes) atomicAdd(prof, nbytes);
 }
 
+// ---- few queries: a team of lanes per leaf (leafwalk::team_run) ----
+
+constexpr unsigned kTeam = leafwalk::kTeam;
+static_assert(kTeam == 8, "four teams to a warp");
+
+__device__ __forceinline__ unsigned team_lane() { return lane_id() & (kTeam - 1); }
+__device__ __forceinline__ unsigned team_mask() { return 0xFFu << (lane_id() & ~(kTeam - 1)); }
+
+// upper_count by a team: each step its lanes probe eight entries, so the
+// search waits for 6 loads where one lane would for 18 (2e5 entries).
+__device__ __forceinline__ uint64_t team_upper_count(const uint64_t* __restrict__ a, uint64_t n,
+                                                     uint64_t x) {
+  const unsigned tl = team_lane(), m = team_mask();
+  uint64_t base = 0, len = n;
+  while (len) {
+    const uint64_t step = len / (kTeam + 1) + 1, at = (tl + 1) * step - 1;
+    const uint64_t c = __popc(__ballot_sync(m, at < len && __ldg(a + base + at) <= x));
+    base += c * step;
+    len = min(step - 1, len - c * step);
+  }
+  return base;
+}
+
+__device__ __forceinline__ uint64_t team_route(const uint64_t* __restrict__ heads, uint64_t L,
+                                               uint64_t x) {
+  if (x == KEY_MAX) return heads[L];
+  const uint64_t c = team_upper_count(heads, L, x);
+  return c ? c - 1 : 0;
+}
+
+// The lane's run with the element before it (in k.val) and the number of
+// elements before it (the head included); a whole warp calls.
+__device__ __forceinline__ leafwalk::Run team_leaf(const uint8_t* leafp, uint32_t u,
+                                                   uint32_t& idx) {
+  const unsigned tl = team_lane();
+  leafwalk::Run r = leafwalk::team_run(leafp, u, tl);
+  __syncwarp();
+  uint64_t d = r.delta;
+  uint32_t n = r.codes;
+#pragma unroll
+  for (unsigned o = 1; o < kTeam; o <<= 1) {
+    const uint64_t y = __shfl_up_sync(FULL, d, o, kTeam);
+    const uint32_t z = __shfl_up_sync(FULL, n, o, kTeam);
+    if (tl >= o) { d += y; n += z; }
+  }
+  r.k.val = (u ? leafwalk::leaf_head(leafp) : 0) + (d - r.delta);
+  idx = 1 + n - r.codes;
+  return r;
+}
+
+// The thread-per-key kernel's work by a team per key.
+__global__ void __launch_bounds__(kT) k_has_team(const uint64_t* __restrict__ keys, uint64_t q,
+                                                 const uint8_t* __restrict__ data,
+                                                 const uint32_t* __restrict__ used,
+                                                 const uint64_t* __restrict__ heads, uint64_t L,
+                                                 uint32_t LB, uint8_t* __restrict__ out,
+                                                 ull* prof) {
+  ull nbytes = 0;
+  const unsigned tl = team_lane(), team = lane_id() / kTeam;
+  for (uint64_t i0 = (gtid() >> 5) * (32 / kTeam); i0 < q; i0 += (gstride() >> 5) * (32 / kTeam)) {
+    const uint64_t i = i0 + team;
+    uint64_t x = 0, j = 0;
+    uint32_t u = 0, idx;
+    if (i < q) {
+      x = keys[i];
+      j = team_route(heads, L, x);
+      u = min(used[j], LB);
+    }
+    __syncwarp();
+    const uint8_t* leafp = data + j * LB;
+    const leafwalk::Run r = team_leaf(leafp, u, idx);
+    bool found = u && tl == 0 && r.k.val == x;  // the head
+    if (r.k.val < x && x - r.k.val <= r.delta)
+      leafwalk::run_visit(leafp, u, r, [&](uint64_t v) { found |= v == x; });
+    __syncwarp();
+    const unsigned hit = __ballot_sync(FULL, found) & team_mask();
+    if (i < q && tl == 0) {
+      out[i] = hit ? 1u : 0u;
+      nbytes += u + 9;
+    }
+  }
+  nbytes = warp_sum(nbytes);
+  if (prof && lane_id() == 0 && nbytes) atomicAdd(prof, nbytes);
+}
+
 // Cells (codec 1): a warp per key, 32 routed per step.
 __global__ void __launch_bounds__(kT) k_has_cells(const uint64_t* __restrict__ keys, uint64_t q,
                                                   const uint8_t* __restrict__ data,
@@ -412,8 +497,8 @@ struct Reduce {
     if constexpr (PLAIN) {
       leafwalk::leaf_range_sum(leafp, u, lo, hi, r, c);
     } else {
-      leafwalk::leaf_visit(leafp, u, [&](uint64_t v) {
-        if (v >= lo && v < hi && (v & mask) == value) { r = op_apply<OP>(r, v); c++; }
+      leafwalk::leaf_range_visit(leafp, u, lo, hi, [&](uint64_t v) {
+        if ((v & mask) == value) { r = op_apply<OP>(r, v); c++; }
       });
     }
   }
@@ -431,7 +516,8 @@ __global__ void __launch_bounds__(kT) k_range_ends(const uint64_t* __restrict__ 
                                                    uint64_t* __restrict__ first,
                                                    uint64_t* __restrict__ items,
                                                    uint64_t* __restrict__ out,
-                                                   uint64_t* __restrict__ count, ull* prof) {
+                                                   uint64_t* __restrict__ count, uint32_t* ticket, ull* prof) {
+  if (ticket && gtid() == 0) *ticket = 0;
   __shared__ uint64_t s_hi[kT], s_r[kT], s_c[kT];
   __shared__ uint32_t s_leaf[kT], s_q[kT];
   __shared__ uint32_t s_n;
@@ -486,6 +572,65 @@ __global__ void __launch_bounds__(kT) k_range_ends(const uint64_t* __restrict__ 
   if (prof && lane_id() == 0 && nbytes) atomicAdd(prof, nbytes);
 }
 
+template <int OP>
+__device__ __forceinline__ void team_reduce(uint64_t& r, uint64_t& c) {
+#pragma unroll
+  for (unsigned o = kTeam / 2; o; o >>= 1) {
+    r = op_apply<OP>(r, __shfl_xor_sync(FULL, r, o));
+    c += __shfl_xor_sync(FULL, c, o);
+  }
+}
+
+// k_range_ends by a team per end: the two teams of a query sit side by side.
+template <int OP, bool PLAIN>
+__global__ void __launch_bounds__(kT) k_range_ends_team(const uint64_t* __restrict__ lo,
+                                                        const uint64_t* __restrict__ hi, uint64_t q,
+                                                        Leaves t, Reduce<OP, PLAIN> f,
+                                                        uint64_t* __restrict__ first,
+                                                        uint64_t* __restrict__ items,
+                                                        uint64_t* __restrict__ out,
+                                                        uint64_t* __restrict__ count, uint32_t* ticket, ull* prof) {
+  if (ticket && gtid() == 0) *ticket = 0;
+  ull nbytes = 0;
+  const unsigned tl = team_lane(), team = lane_id() / kTeam;
+  for (uint64_t e0 = (gtid() >> 5) * (32 / kTeam); e0 < 2 * q;
+       e0 += (gstride() >> 5) * (32 / kTeam)) {
+    const uint64_t i = (e0 + team) >> 1;
+    const bool side = (team & 1u) != 0u;
+    uint64_t a = 0, b = 0, j = 0;
+    if (i < q) { a = lo[i]; b = hi[i]; }
+    if (a < b) j = team_route(t.heads, t.L, side ? b - 1 : a);
+    __syncwarp();
+    const uint64_t other = __shfl_xor_sync(FULL, j, kTeam);
+    const uint64_t fl = side ? other : j, ll = side ? j : other;
+    const uint32_t u = a < b && (!side || ll > fl) ? min(t.used[j], t.LB) : 0u;
+    const uint8_t* leafp = t.data + j * t.LB;
+    uint32_t idx;
+    const leafwalk::Run run = team_leaf(leafp, u, idx);
+    uint64_t r = op_identity<OP>(), c = 0;
+    auto take = [&](uint64_t v) {
+      if (v >= a && v < b && (PLAIN || (v & f.mask) == f.value)) { r = op_apply<OP>(r, v); c++; }
+    };
+    if (u && tl == 0) take(run.k.val);
+    if (u && run.k.val < b && run.k.val + run.delta >= a) leafwalk::run_visit(leafp, u, run, take);
+    __syncwarp();
+    team_reduce<OP>(r, c);
+    r = op_apply<OP>(r, __shfl_down_sync(FULL, r, kTeam));
+    c += __shfl_down_sync(FULL, c, kTeam);
+    if (tl == 0) {
+      nbytes += u;
+      if (!side && i < q) {
+        first[i] = fl + 1;
+        items[i] = ll > fl ? ll - fl - 1 : 0;
+        out[i] = r;
+        count[i] = c;
+      }
+    }
+  }
+  nbytes = warp_sum(nbytes);
+  if (prof && lane_id() == 0 && nbytes) atomicAdd(prof, nbytes);
+}
+
 // The same for map_range_length: thread i takes the first length[i] elements
 // from start[i] on as far as its first leaf holds them; P (elements before
 // each leaf) then names the leaf of the last one and how many it gives.
@@ -495,7 +640,8 @@ __global__ void __launch_bounds__(kT) k_length_ends(const uint64_t* __restrict__
                                                     uint64_t* __restrict__ first,
                                                     uint64_t* __restrict__ items,
                                                     uint64_t* __restrict__ sum,
-                                                    uint64_t* __restrict__ count, ull* prof) {
+                                                    uint64_t* __restrict__ count, uint32_t* ticket, ull* prof) {
+  if (ticket && gtid() == 0) *ticket = 0;
   pdl_wait();
   pdl_launch();
   __shared__ uint64_t s_s[kT];
@@ -554,6 +700,80 @@ __global__ void __launch_bounds__(kT) k_length_ends(const uint64_t* __restrict__
   if (prof && lane_id() == 0 && nbytes) atomicAdd(prof, nbytes);
 }
 
+// k_length_ends by a team per query.
+__global__ void __launch_bounds__(kT) k_length_ends_team(
+    const uint64_t* __restrict__ start, const uint64_t* __restrict__ length, uint64_t q, Leaves t,
+    const uint64_t* __restrict__ P, uint64_t* __restrict__ first, uint64_t* __restrict__ items,
+    uint64_t* __restrict__ sum, uint64_t* __restrict__ count, uint32_t* ticket, ull* prof) {
+  if (ticket && gtid() == 0) *ticket = 0;
+  pdl_wait();
+  pdl_launch();
+  ull nbytes = 0;
+  const uint64_t n = P[t.L];
+  const unsigned tl = team_lane(), team = lane_id() / kTeam;
+  for (uint64_t i0 = (gtid() >> 5) * (32 / kTeam); i0 < q; i0 += (gstride() >> 5) * (32 / kTeam)) {
+    const uint64_t i = i0 + team;
+    uint64_t x = 0, len = 0, fl = 0, s = 0, c = 0;
+    uint32_t u = 0, idx;
+    if (i < q) len = length[i];
+    if (len) {
+      x = start[i];
+      fl = team_route(t.heads, t.L, x);
+      u = min(t.used[fl], t.LB);
+    }
+    __syncwarp();
+    const uint8_t* leafp = t.data + fl * t.LB;
+    leafwalk::Run run = team_leaf(leafp, u, idx);
+    const uint64_t head = __shfl_sync(FULL, run.k.val, 0, kTeam);
+    uint64_t below = u && tl == 0 && head < x ? 1u : 0u;
+    // the run's elements below x: none, all or, for one lane, some
+    if (u && run.k.val < x) {
+      if (run.k.val + run.delta < x) below += run.codes;
+      else leafwalk::run_visit(leafp, u, run, [&](uint64_t v) { below += v < x ? 1u : 0u; });
+    }
+    __syncwarp();
+    team_reduce<CPMA_OP_SUM>(s, below);
+    const uint64_t r0 = P[fl] + below;  // rank of the first key >= x
+    const uint64_t r1 = len >= n - r0 ? n : r0 + len;
+    // the elements of ranks [r0, r1) in two leaves: its first, and its last one
+    uint64_t j = fl, ll = fl;
+    for (int end = 0; end < 2; end++) {
+      const uint64_t p = P[j];
+      const uint64_t from = r0 > p ? r0 - p : 0, to = u ? r1 - p : 0;  // of the leaf's elements
+      uint32_t at = idx;
+      auto take = [&](uint64_t v) {
+        if (at >= from && at < to) { s += v; c++; }
+        at++;
+      };
+      if (u && tl == 0) {
+        at = 0;
+        take(run.k.val);
+      }
+      if (u && idx < to && idx + run.codes > from) leafwalk::run_visit(leafp, u, run, take);
+      __syncwarp();
+      if (tl == 0) nbytes += u;
+      if (end) break;
+      u = 0;
+      if (len && r1 > r0 && r1 > P[fl + 1]) {  // more in later leaves
+        ll = j = last_from(P, fl, t.L + 1, r1 - 1);
+        u = min(t.used[j], t.LB);
+      }
+      __syncwarp();
+      leafp = t.data + j * t.LB;
+      run = team_leaf(leafp, u, idx);
+    }
+    team_reduce<CPMA_OP_SUM>(s, c);
+    if (tl == 0 && i < q) {
+      first[i] = fl + 1;
+      items[i] = ll > fl ? ll - fl - 1 : 0;
+      sum[i] = s;
+      count[i] = c;
+    }
+  }
+  nbytes = warp_sum(nbytes);
+  if (prof && lane_id() == 0 && nbytes) atomicAdd(prof, nbytes);
+}
+
 // Reductions before (min: from) each leaf, in two levels: val / cnt inside
 // the tile of kT leaves, tval / tcnt over the tiles.  Unused (null) when its
 // memory cannot be had; taken when the queries' inner leaves number more than
@@ -563,6 +783,7 @@ struct LeafPrefix {
   uint32_t* cnt = nullptr;   // per leaf: matches before it in its tile
   uint64_t* tval = nullptr;  // per tile
   uint64_t* tcnt = nullptr;
+  uint32_t* ticket = nullptr;  // blocks done, cleared by the kernel before
   uint64_t most = ~0ull;
 };
 
@@ -621,8 +842,76 @@ __device__ __forceinline__ void order_tile(uint32_t u, uint32_t nt, uint32_t* hi
   __syncthreads();
 }
 
-// Every leaf reduced once, scanned inside tiles of kT leaves (when the
-// queries cover more than p.most leaves; otherwise nothing).
+// The tiles' reductions scanned in place by one block: exclusive from the
+// front (min: from the back).
+template <int OP>
+__device__ void tile_scan(const LeafPrefix& p, uint64_t nt, uint64_t* s_ws) {
+  constexpr bool REV = OP == CPMA_OP_MIN;
+  // a contiguous run of tiles per thread: reduced, scanned over the block,
+  // rescanned
+  const uint64_t per = (nt + kT - 1) / kT;
+  const uint64_t b0 = min(nt, threadIdx.x * per), b1 = min(nt, b0 + per);
+  uint64_t r = op_identity<OP>(), c = 0;
+  for (uint64_t b = b0; b < b1; b++) {
+    r = op_apply<OP>(r, p.tval[b]);
+    c += p.tcnt[b];
+  }
+  uint64_t all;
+  uint64_t x;
+  if (REV) {  // exclusive from the back: the inclusive one of the next thread
+    const uint64_t inc = block_scan_op<OP, true>(r, s_ws, &all);
+    __shared__ uint64_t s_inc[kT + 1];
+    s_inc[threadIdx.x] = inc;
+    if (threadIdx.x == 0) s_inc[kT] = op_identity<OP>();
+    __syncthreads();
+    x = s_inc[threadIdx.x + 1];
+  } else {
+    x = block_scan_op<OP, false>(r, s_ws, &all);
+  }
+  uint64_t y = block_scan_op<CPMA_OP_SUM, false>(c, s_ws, &all);
+  for (uint64_t b = b0; b < b1; b++) {
+    const uint64_t v = p.tcnt[b];
+    p.tcnt[b] = y;
+    y += v;
+  }
+  if (REV) {
+    for (uint64_t b = b1; b-- > b0;) {
+      const uint64_t v = p.tval[b];
+      p.tval[b] = x;
+      x = op_apply<OP>(x, v);
+    }
+  } else {
+    for (uint64_t b = b0; b < b1; b++) {
+      const uint64_t v = p.tval[b];
+      p.tval[b] = x;
+      x = op_apply<OP>(x, v);
+    }
+  }
+}
+
+// Is this block the last of the grid to come here?  Then it sees what the
+// others wrote before.
+__device__ __forceinline__ bool last_block(uint32_t* ticket) {
+  __shared__ uint32_t s_last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+  __syncthreads();
+  const bool last = s_last != 0;
+  if (last) __threadfence();
+  return last;
+}
+
+__global__ void __launch_bounds__(kT) k_tile_scan(LeafPrefix p, uint64_t nt) {
+  __shared__ uint64_t s_ws[kT / 32];
+  pdl_wait();
+  pdl_launch();
+  tile_scan<CPMA_OP_SUM>(p, nt, s_ws);
+}
+
+// Every leaf reduced once, scanned inside tiles of kT leaves, and the tiles by
+// the last block to finish (when the queries cover more than p.most leaves;
+// otherwise nothing).
 template <int OP, bool PLAIN>
 __global__ void __launch_bounds__(kT) k_leaf_prefix(Leaves t, Reduce<OP, PLAIN> f,
                                                     const uint64_t* __restrict__ total,
@@ -668,58 +957,7 @@ __global__ void __launch_bounds__(kT) k_leaf_prefix(Leaves t, Reduce<OP, PLAIN> 
   }
   nbytes = warp_sum(nbytes);
   if (prof && lane_id() == 0 && nbytes) atomicAdd(prof, nbytes);
-}
-
-// The tiles' reductions scanned in place by one block: exclusive from the
-// front (min: from the back).
-template <int OP>
-__global__ void __launch_bounds__(kT) k_tile_scan(const uint64_t* __restrict__ total, LeafPrefix p,
-                                                  uint64_t nt) {
-  __shared__ uint64_t s_ws[kT / 32];
-  pdl_wait();
-  pdl_launch();
-  if (total && *total <= p.most) return;
-  constexpr bool REV = OP == CPMA_OP_MIN;
-  // a contiguous run of tiles per thread: reduced, scanned over the block,
-  // rescanned
-  const uint64_t per = (nt + kT - 1) / kT;
-  const uint64_t b0 = min(nt, threadIdx.x * per), b1 = min(nt, b0 + per);
-  uint64_t r = op_identity<OP>(), c = 0;
-  for (uint64_t b = b0; b < b1; b++) {
-    r = op_apply<OP>(r, p.tval[b]);
-    c += p.tcnt[b];
-  }
-  uint64_t all;
-  uint64_t x;
-  if (REV) {  // exclusive from the back: the inclusive one of the next thread
-    const uint64_t inc = block_scan_op<OP, true>(r, s_ws, &all);
-    __shared__ uint64_t s_inc[kT + 1];
-    s_inc[threadIdx.x] = inc;
-    if (threadIdx.x == 0) s_inc[kT] = op_identity<OP>();
-    __syncthreads();
-    x = s_inc[threadIdx.x + 1];
-  } else {
-    x = block_scan_op<OP, false>(r, s_ws, &all);
-  }
-  uint64_t y = block_scan_op<CPMA_OP_SUM, false>(c, s_ws, &all);
-  for (uint64_t b = b0; b < b1; b++) {
-    const uint64_t v = p.tcnt[b];
-    p.tcnt[b] = y;
-    y += v;
-  }
-  if (REV) {
-    for (uint64_t b = b1; b-- > b0;) {
-      const uint64_t v = p.tval[b];
-      p.tval[b] = x;
-      x = op_apply<OP>(x, v);
-    }
-  } else {
-    for (uint64_t b = b0; b < b1; b++) {
-      const uint64_t v = p.tval[b];
-      p.tval[b] = x;
-      x = op_apply<OP>(x, v);
-    }
-  }
+  if (last_block(p.ticket)) tile_scan<OP>(p, nt, s_ws);
 }
 
 // The warp's equal contiguous share of N items that its lanes take one each:
@@ -769,6 +1007,35 @@ __global__ void __launch_bounds__(kT) k_range_inner(Leaves t, Reduce<OP, PLAIN> 
     return;
   }
   const unsigned lane = lane_id();
+  if (N * kTeam * 4 <= gstride()) {  // few: a team per item
+    const uint64_t e0 = ((uint64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * (32 / kTeam);
+    if (e0 >= N) return;
+    const uint64_t e = e0 + lane / kTeam;
+    uint64_t qi = 0, j = 0;
+    uint32_t u = 0, idx;
+    if (e < N) {
+      qi = team_upper_count(off, q + 1, e) - 1;
+      j = first[qi] + (e - off[qi]);
+      u = min(t.used[j], t.LB);
+    }
+    __syncwarp();
+    const uint8_t* leafp = t.data + j * t.LB;
+    const leafwalk::Run run = team_leaf(leafp, u, idx);
+    uint64_t r = op_identity<OP>(), c = 0;
+    auto take = [&](uint64_t v) {
+      if (PLAIN || (v & f.mask) == f.value) { r = op_apply<OP>(r, v); c++; }
+    };
+    if (u && team_lane() == 0) take(run.k.val);
+    leafwalk::run_visit(leafp, u, run, take);
+    __syncwarp();
+    team_reduce<OP>(r, c);
+    if (team_lane() == 0 && c) {
+      op_atomic<OP>(&out[qi], r);
+      atomicAdd((ull*)&count[qi], (ull)c);
+    }
+    if (prof && team_lane() == 0 && u) atomicAdd(prof, (ull)u);
+    return;
+  }
   uint64_t g0, g1;
   lane_share(N, g0, g1);
   if (g0 >= g1) return;
@@ -1078,6 +1345,14 @@ __global__ void __launch_bounds__(kT) k_sum(const uint8_t* __restrict__ data,
 
 int persistent_grid(const cpma* h) { return h->num_sms * 8; }
 
+// Few enough queries for a team of lanes per leaf.  A team spends about twice
+// a thread's instructions on a leaf in a third of its time.  Team / thread per
+// leaf, us (about 35 of them the call's own), 1e7 keys: masked ranges of 50
+// elements, 1e3 queries 36 / 52, 1e4 47 / 57, 4e4 74 / 70; plain ones 38 / 42,
+// 45 / 44, 72 / 53; scans by length 33 / 43, 42 / 49, 84 / 66.  With leaves of
+// 2048 bytes masked ones, 1e4 queries, 60 / 63 and 2e4 93 / 69.
+bool few_queries(const cpma* h, uint64_t q) { return q <= (uint64_t)h->num_sms * 64; }
+
 // Scratch of the allocation-free range_map: per-query first leaf, item count
 // and item offsets, plus the partial sums of the offset scan.  It lives in the
 // library's own device image, so every GPU that loads the library holds these
@@ -1116,10 +1391,14 @@ int scratch_address(int dev, uint8_t** out) {
 
 int run_has(const cpma* h, const uint64_t* d_keys, uint64_t q, uint8_t* d_out, cudaStream_t st) {
   if (q == 0) return CPMA_OK;
+  // (a lookup is half a range: 2048-byte leaves, 4e3 keys 15 us by teams and
+  // 19 by threads, 9e3 21 and 19)
+  const bool few = !h->cfg.codec && few_queries(h, 2 * q);
+  const uint64_t per = few ? kT / kTeam : kT;  // keys a block
   const int grid = (int)std::max<uint64_t>(
-      1, std::min<uint64_t>((q + kT - 1) / kT, (uint64_t)persistent_grid(h)));
+      1, std::min<uint64_t>((q + per - 1) / per, (uint64_t)persistent_grid(h)));
   prof_begin(h, PH_HAS, st);
-  const auto kern = h->cfg.codec ? k_has_cells : k_has;
+  const auto kern = h->cfg.codec ? k_has_cells : few ? k_has_team : k_has;
   kern<<<grid, kT, 0, st>>>(d_keys, q, h->data, h->used, h->heads, h->L, h->cfg.leaf_bytes, d_out,
                             prof_bytes(h, PH_HAS));
   CPMA_LAUNCHED(h);
@@ -1142,7 +1421,7 @@ int query_grid(const cpma* h, uint64_t q, int block, uint64_t per_sm) {
 }
 
 // Per leaf a reduction and a count, per tile both again.
-size_t leaf_prefix_bytes(uint64_t L) { return L * 12 + (L + kT - 1) / kT * 16; }
+size_t leaf_prefix_bytes(uint64_t L) { return L * 12 + (L + kT - 1) / kT * 16 + 4; }
 
 // Grows a query buffer; the leaf prefix, which the queries can do without, is
 // given back when there is no room for it.
@@ -1183,6 +1462,7 @@ LeafPrefix leaf_prefix(cpma* h, uint64_t q, cudaStream_t st) {
   p.tval = p.val + h->L;
   p.tcnt = p.tval + nt;
   p.cnt = (uint32_t*)(p.tcnt + nt);
+  p.ticket = p.cnt + h->L;
   p.most = h->L;
   return p;
 }
@@ -1219,7 +1499,7 @@ int range_marked(cpma* h, const uint64_t* lo, const uint64_t* hi, uint64_t q, co
   const unsigned g = (unsigned)std::min<uint64_t>(nt, (uint64_t)persistent_grid(h));
   k_marks<<<g, kT, 0, st>>>(t, m, prof);
   CPMA_CUDA(cudaGetLastError());
-  CPMA_CUDA(launch_pdl(k_tile_scan<CPMA_OP_SUM>, 1, kT, 0, st, nullptr, m.tiles, nt));
+  CPMA_CUDA(launch_pdl(k_tile_scan, 1, kT, 0, st, m.tiles, nt));
   const int b = query_block(h, q);
   CPMA_CUDA(launch_pdl(k_range_marked, (unsigned)query_grid(h, q, b, 8), (unsigned)b, 0, st, lo, hi,
                        q, t, m, sum, count, prof));
@@ -1264,8 +1544,7 @@ int range_inner(cpma* h, Reduce<OP, PLAIN> f, uint64_t q, uint64_t* out, uint64_
     const unsigned g = (unsigned)std::min<uint64_t>(nt, (uint64_t)persistent_grid(h));
     const uint64_t* total = r.off + q;
     CPMA_CUDA(launch_pdl(k_leaf_prefix<OP, PLAIN>, g, kT, 0, st, t, f, total, p, prof));
-    CPMA_CUDA(launch_pdl(k_tile_scan<OP>, 1, kT, 0, st, total, p, nt));
-    h->launches += 2;
+    h->launches++;
   }
   CPMA_CUDA(launch_pdl(k_range_inner<OP, PLAIN>, (unsigned)persistent_grid(h), kT, 0, st, t, f, q,
                        r.first, r.off, p, out, count, prof));
@@ -1278,9 +1557,15 @@ int range_leaves(cpma* h, const uint64_t* lo, const uint64_t* hi, uint64_t q, ui
                  uint64_t value, uint64_t* out, uint64_t* count, const RangeScratch& r,
                  const LeafPrefix& p, cudaStream_t st, ull* prof) {
   const Reduce<OP, PLAIN> f{mask, value};
-  const int b = query_block(h, q);
-  k_range_ends<OP, PLAIN><<<query_grid(h, q, b, 8), b, 0, st>>>(lo, hi, q, leaves_of(h), f, r.first,
-                                                                r.items, out, count, prof);
+  if (few_queries(h, q)) {
+    k_range_ends_team<OP, PLAIN><<<query_grid(h, 2 * q * kTeam, 64, 32), 64, 0, st>>>(
+        lo, hi, q, leaves_of(h), f, r.first, r.items, out, count, p.ticket, prof);
+  } else {
+    const int b = query_block(h, q);
+    k_range_ends<OP, PLAIN><<<query_grid(h, q, b, 8), b, 0, st>>>(lo, hi, q, leaves_of(h), f,
+                                                                  r.first, r.items, out, count,
+                                                                  p.ticket, prof);
+  }
   CPMA_LAUNCHED(h);
   CPMA_CUDA(cudaGetLastError());
   return range_inner<OP, PLAIN>(h, f, q, out, count, r, p, st, prof);
@@ -1392,9 +1677,12 @@ int run_range_length(const cpma* h, const uint64_t* start, const uint64_t* lengt
     const LeafPrefix p = leaf_prefix(hm, q, st);
     ull* prof = prof_bytes(h, PH_RANGE);
     prof_begin(h, PH_RANGE, st);
-    const int b = query_block(h, q);
-    CPMA_CUDA(launch_pdl(k_length_ends, (unsigned)query_grid(h, q, b, 8), (unsigned)b, 0, st, start,
-                         length, q, leaves_of(h), P, r.first, r.items, sum, count, prof));
+    const bool few = few_queries(h, q);
+    const int b = few ? 64 : query_block(h, q);
+    const int g = few ? query_grid(h, q * kTeam, b, 32) : query_grid(h, q, b, 8);
+    CPMA_CUDA(launch_pdl(few ? k_length_ends_team : k_length_ends, (unsigned)g, (unsigned)b, 0, st,
+                         start, length, q, leaves_of(h), P, r.first, r.items, sum, count, p.ticket,
+                         prof));
     CPMA_LAUNCHED(h);
     const int rc = range_inner<CPMA_OP_SUM, true>(hm, Reduce<CPMA_OP_SUM, true>{0, 0}, q, sum,
                                                   count, r, p, st, prof);

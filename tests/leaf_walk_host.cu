@@ -55,6 +55,13 @@ extern "C" void lw_marked(const uint8_t* leaf, uint32_t u, uint64_t x, uint64_t*
   leafwalk::below_sum(leaf, u, at * leafwalk::kMark, k, x, out[0], out[1]);
 }
 
+extern "C" uint32_t lw_between(const uint8_t* leaf, uint32_t u, uint64_t lo, uint64_t hi,
+                               uint64_t* out) {
+  uint32_t n = 0;
+  leafwalk::leaf_range_visit(leaf, u, lo, hi, [&](uint64_t v) { out[n++] = v; });
+  return n;
+}
+
 // The elements from lo on, starting where the search for it ended; returns
 // how many (0 when it did not end at a code).
 extern "C" uint32_t lw_from(const uint8_t* leaf, uint32_t u, uint64_t lo, uint64_t* out) {
@@ -64,5 +71,21 @@ extern "C" uint32_t lw_from(const uint8_t* leaf, uint32_t u, uint64_t lo, uint64
   if (at.sum)
     leafwalk::visit_from(leaf, u, (uint32_t)at.sum, leafwalk::walk_at(at),
                          [&](uint64_t v) { if (idx++ >= r) out[n++] = v; }, [] { return false; });
+  return n;
+}
+
+// A team's runs one after another: the elements in order, and whether each
+// run's own count and sum of deltas say the same.
+extern "C" uint32_t lw_team(const uint8_t* leaf, uint32_t u, uint64_t* out) {
+  uint32_t n = 0;
+  uint64_t v = out[n++] = leafwalk::leaf_head(leaf);
+  for (uint32_t tl = 0; tl < leafwalk::kTeam; tl++) {
+    leafwalk::Run r = leafwalk::team_run(leaf, u, tl);
+    const uint32_t n0 = n;
+    r.k.val = v;
+    leafwalk::run_visit(leaf, u, r, [&](uint64_t x) { out[n++] = x; });
+    v += r.delta;
+    if (n - n0 != r.codes || out[n - 1] != v) return 0;
+  }
   return n;
 }

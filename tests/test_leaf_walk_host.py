@@ -36,6 +36,8 @@ def lw(tmp_path_factory):
     lib.lw_take.argtypes = [u8, u32, u64, u64, p64]
     lib.lw_below.restype, lib.lw_below.argtypes = u32, [u8, u32, u64]
     lib.lw_has.argtypes = [u8, u32, u64]
+    lib.lw_team.restype, lib.lw_team.argtypes = u32, [u8, u32, p64]
+    lib.lw_between.restype, lib.lw_between.argtypes = u32, [u8, u32, u64, u64, p64]
     lib.lw_from.restype, lib.lw_from.argtypes = u32, [u8, u32, u64, p64]
     lib.lw_marked.argtypes = [u8, u32, u64, p64]
     return lib
@@ -117,6 +119,7 @@ def test_walk_against_keys(lw, LB):
         assert sums(lw, p, u, keys)
         out = (C.c_uint64 * (len(keys) + 8))()
         assert lw.lw_visit(p, u, out) == len(keys) and list(out[:len(keys)]) == keys
+        assert lw.lw_team(p, u, out) == len(keys) and list(out[:len(keys)]) == keys
         marks = [0, M64, keys[0], keys[-1], (keys[-1] + 1) & M64]
         for _ in range(6):
             x = rng.choice(keys)
@@ -134,6 +137,8 @@ def test_walk_against_keys(lw, LB):
                 a, b = bisect.bisect_left(keys, lo), bisect.bisect_left(keys, hi)
                 lw.lw_range(p, u, lo, hi, res)
                 assert (res[0], res[1]) == (sum(keys[a:b]) & M64, b - a)
+                n = lw.lw_between(p, u, lo, hi, out)
+                assert list(out[:n]) == keys[a:b]
             a = bisect.bisect_left(keys, lo)
             n = lw.lw_from(p, u, lo, out)
             assert list(out[:n]) == (keys[a:] if 0 < a else [])
