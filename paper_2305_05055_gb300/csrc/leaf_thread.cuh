@@ -7,10 +7,11 @@
 // word-parallel arithmetic (each byte's position inside its code from the
 // continuation flags of the bytes before it, then two dot products per word
 // with byte weights 1 / 128 and 2^14 / 2^21), recording for every key of
-// the slice the chunk it lands in; those chunks are then decoded byte by
-// byte to place each key: before the head (a new head), inside the gap that one code spans
-// (the code is split), or after the last element (appended); a key equal to
-// an element or to the slice key before it is skipped.  Keys sharing a gap
+// the slice the chunk it lands in; each key's chunk is then decoded byte by
+// byte (by any thread: the record holds the state) to find its place: before
+// the head (a new head), inside the gap that one code spans (the code is
+// split), or after the last element (appended); a key equal to an element or
+// to the slice key before it is skipped.  Keys sharing a gap
 // form one edit: old bytes [os, oe) replaced by nl new bytes.  Every edit of
 // an insert grows or keeps the size (a split code never needs more bytes
 // than its two parts), so pass B rewrites the leaf in place from the end
@@ -174,49 +175,45 @@ LT_HD bool leaf_has(const uint8_t* leafp, uint32_t u, uint64_t x) {
   return found;
 }
 
-// Pass A, step 2: the codes of the chunk at p0 take keys q..q1-1 (all of
-// them: their values lie between the element before the chunk and the last
-// element completed in it).  Decode the chunk byte by byte from the state it
-// was entered with (val0: the element before it; carry0, g0: the bits and
-// byte count of the code open at p0) and give each key its gap.
-// For each key the bytes are walked without branches, the values relative to
-// val0: the last terminator below the key, and the first that reaches it.
-LT_HD void place_in_chunk(const uint8_t* leafp, uint32_t uold, uint32_t p0, uint64_t val0,
-                          uint32_t carry0, uint32_t g0, const uint64_t (&y)[kKeys], uint32_t q,
-                          uint32_t q1, const Scratch& S) {
+// Pass A, step 2, for key yq of the slice (rep: a repeat of the one before it),
+// whose record (rpos, rval, rcode) names the chunk it lands in and the state
+// that was entered with: val0 the element before it, carry0 and g0 the bits and
+// byte count of the code open at its start.  The chunk is walked byte by byte
+// without branches, the values relative to val0: the last terminator below the
+// key, and the first that reaches it.  The record becomes the key's gap.
+LT_HD void place_key(const uint8_t* leafp, uint32_t uold, uint64_t yq, bool rep, uint32_t& rpos,
+                     uint64_t& rval, uint32_t& rcode) {
+  const uint32_t p0 = rpos & 0xFFFu, g0 = (rpos >> 12) & 0xFFFu;
+  const uint64_t val0 = rval;
   uint32_t w[4], t[4];
   leafwalk::load_chunk(leafp, p0, uold, w, t);
   const uint32_t first = p0 == 0 ? 8u : 0u;  // bytes 0-7 are the head
   if (p0 == 0) w[0] = w[1] = t[0] = t[1] = 0u;
 #pragma unroll
   for (int i = 0; i < 4; i++) w[i] &= 0x7F7F7F7Fu;
-  for (; q < q1; q++) {
-    const uint64_t yq = pick(y, q);
-    const uint32_t d = (uint32_t)(yq - val0);  // the chunk's last element reaches it
-    uint32_t cum = carry0, pw = 1u << (7u * g0);
-    uint32_t below = 0, cs = first - g0, at = 0, ce = 0;  // cs: relative to p0, may wrap
-    bool open = true;
+  const uint32_t d = (uint32_t)(yq - val0);  // the chunk's last element reaches it
+  uint32_t cum = rcode, pw = 1u << (7u * g0);
+  uint32_t below = 0, cs = first - g0, at = 0, ce = 0;  // cs: relative to p0, may wrap
+  bool open = true;
 #pragma unroll
-    for (int b = 0; b < 16; b++) {
-      cum += byte_of(w[b >> 2], b & 3) * pw;
-      const bool term = (t[b >> 2] & (0x80u << (8 * (b & 3)))) != 0u;
-      const bool stop = term && open && cum >= d;
-      const bool pass = term && open && cum < d;
-      at = stop ? cum : at;
-      ce = stop ? (uint32_t)b + 1u : ce;
-      below = pass ? cum : below;
-      cs = pass ? (uint32_t)b + 1u : cs;
-      open = open && !stop;
-      pw = term ? 1u : pw << 7;
-      if (p0 == 0 && b == 7) pw = 1u << (7u * g0);  // the head's bytes are no codes
-    }
-    const uint64_t val = val0 + at;
-    const bool rep = q > 0 && pick(y, q - 1) == yq;
-    const uint32_t kind = rep ? kSkip : yq == val ? kHit : kGap;
-    S.rpos[q * S.rs] = (p0 + cs) | ((p0 + ce) << 12) | (kind << 24);
-    S.rval[q * S.rs] = val;
-    S.rcode[q * S.rs] = at - below;
+  for (int b = 0; b < 16; b++) {
+    cum += byte_of(w[b >> 2], b & 3) * pw;
+    const bool term = (t[b >> 2] & (0x80u << (8 * (b & 3)))) != 0u;
+    const bool stop = term && open && cum >= d;
+    const bool pass = term && open && cum < d;
+    at = stop ? cum : at;
+    ce = stop ? (uint32_t)b + 1u : ce;
+    below = pass ? cum : below;
+    cs = pass ? (uint32_t)b + 1u : cs;
+    open = open && !stop;
+    pw = term ? 1u : pw << 7;
+    if (p0 == 0 && b == 7) pw = 1u << (7u * g0);  // the head's bytes are no codes
   }
+  const uint64_t val = val0 + at;
+  const uint32_t kind = rep ? kSkip : yq == val ? kHit : kGap;
+  rpos = (p0 + cs) | ((p0 + ce) << 12) | (kind << 24);
+  rval = val;
+  rcode = at - below;
 }
 
 // The 16 bytes of the old leaf at byte offset src, bytes outside [0, LB)
@@ -267,8 +264,11 @@ LT_HD void seg_bounds(const SC& S, uint32_t E, uint32_t uold, uint32_t os0, int 
 // else kLongCode (the leaf holds a code of more than 4 bytes).  head
 // receives the leaf's first element.
 constexpr uint32_t kPlaced = kWritten;
-LT_HD uint32_t pass_a(const uint8_t* leafp, uint32_t uold, uint32_t m, const uint64_t (&y)[kKeys],
-                      uint32_t s, const Scratch& S, uint64_t& head) {
+
+// Step 1: keys before, at and after the leaf's elements get their records, the
+// others (kChunk) the chunk that takes them.
+LT_HD uint32_t pass_a_sum(const uint8_t* leafp, uint32_t uold, const uint64_t (&y)[kKeys],
+                          uint32_t s, const Scratch& S, uint64_t& head) {
   uint32_t w[4];
   ld16(leafp, w);
   head = (uint64_t)w[0] | ((uint64_t)w[1] << 32);
@@ -282,7 +282,7 @@ LT_HD uint32_t pass_a(const uint8_t* leafp, uint32_t uold, uint32_t m, const uin
     S.rcode[k * S.rs] = 0u;
     k++;
   }
-  // step 1: chunk sums over the whole leaf (a warp's threads then take the
+  // chunk sums over the whole leaf (a warp's threads then take the
   // same number of steps); every key gets the chunk (p0, entry state) of
   // the code it falls in, or stays for the end
   uint64_t ycur = k < s ? pick(y, k) : ~0ull;
@@ -320,17 +320,6 @@ LT_HD uint32_t pass_a(const uint8_t* leafp, uint32_t uold, uint32_t m, const uin
     carry = cnew;
   }
   if (lc) return kLongCode;
-  // step 2: exact gaps inside the recorded chunks
-  for (uint32_t q = 0; q < k; q++) {
-    const uint32_t rp = S.rpos[q * S.rs];
-    if ((rp >> 24) != kChunk) continue;  // placed (head keys, or by an earlier chunk)
-    const uint32_t p0 = rp & 0xFFFu;
-    uint32_t q1 = q + 1;
-    while (q1 < k && S.rpos[q1 * S.rs] == rp) q1++;
-    place_in_chunk(leafp, uold, p0, S.rval[q * S.rs], S.rcode[q * S.rs], (rp >> 12) & 0xFFFu, y,
-                   q, q1, S);
-    q = q1 - 1;
-  }
   const uint64_t lastv = val;
   for (; k < s; k++) {
     const uint64_t x = pick(y, k);
@@ -342,11 +331,24 @@ LT_HD uint32_t pass_a(const uint8_t* leafp, uint32_t uold, uint32_t m, const uin
   return kPlaced;
 }
 
+LT_HD uint32_t pass_a(const uint8_t* leafp, uint32_t uold, const uint64_t (&y)[kKeys], uint32_t s,
+                      const Scratch& S, uint64_t& head) {
+  const uint32_t res = pass_a_sum(leafp, uold, y, s, S, head);
+  if (res != kPlaced) return res;
+  // step 2: exact gaps inside the recorded chunks
+  for (uint32_t q = 0; q < s; q++) {
+    if ((S.rpos[q * S.rs] >> 24) != kChunk) continue;
+    place_key(leafp, uold, pick(y, q), q > 0 && pick(y, q - 1) == pick(y, q), S.rpos[q * S.rs],
+              S.rval[q * S.rs], S.rcode[q * S.rs]);
+  }
+  return kPlaced;
+}
+
 // The same for leaves with codes of any length, eight bytes at a time with
 // 64-bit values (the leaf walk's groups: Walk carries the element before the
 // group and the code open at it).  Always kPlaced.
-LT_HD uint32_t pass_a(const uint8_t* leafp, uint32_t uold, uint32_t m, const uint64_t (&y)[kKeys],
-                      uint32_t s, const ScratchLong& S, uint64_t& head) {
+LT_HD uint32_t pass_a(const uint8_t* leafp, uint32_t uold, const uint64_t (&y)[kKeys], uint32_t s,
+                      const ScratchLong& S, uint64_t& head) {
   uint32_t w[4], t[4], raw[4];
   ld16(leafp, raw);
   head = (uint64_t)raw[0] | ((uint64_t)raw[1] << 32);
@@ -427,18 +429,14 @@ LT_HD uint32_t pass_a(const uint8_t* leafp, uint32_t uold, uint32_t m, const uin
   return kPlaced;
 }
 
-// Pass A and the edits of inserting the sorted slice y[0..s) (1 <= s <=
-// kKeys, repeats allowed) into the leaf at leafp (uold >= 8 used bytes, m
+// The edits of inserting the sorted slice y[0..s) (1 <= s <= kKeys, repeats
+// allowed), placed by pass A, into the leaf at leafp (uold >= 8 used bytes, m
 // elements, LB bytes, 16-byte aligned).  Returns one of the results above
 // and writes nothing; kWritten means the leaf is to be rewritten (R.wlo ..
 // R.whi, the R.E edits in S).
 template <class SC>
-LT_HD uint32_t plan_leaf(uint8_t* leafp, uint32_t LB, uint32_t uold, uint32_t m,
-                           const uint64_t (&y)[kKeys], uint32_t s, const SC& S,
-                           Result& R) {
-  uint64_t head;
-  const uint32_t pa = pass_a(leafp, uold, m, y, s, S, head);
-  if (pa != kPlaced) return pa;
+LT_HD uint32_t plan_insert(uint32_t LB, uint32_t uold, uint32_t m, const uint64_t (&y)[kKeys],
+                           uint32_t s, uint64_t head, const SC& S, Result& R) {
   // ---- edits: new keys grouped by the gap they fall in ----
   uint32_t E = 0, nn = 0, added = 0, mc = 0;
   int32_t tot = 0;
@@ -525,7 +523,7 @@ LT_HD void build_chunk(const uint8_t* leafp, uint32_t LB, uint32_t uold, const S
 // edit falls into merges a second (with one or two keys in most leaves, some
 // lane of every warp is at such a chunk in every step, so that is all a step
 // may cost).  Gathering those chunks segment by segment: 290 us a launch for 1e6
-// keys into 1e8, this 254 us.
+// keys into 1e8, this 254 us (then; 238 us by now).
 template <class SC>
 LT_HD void rewrite_leaf(uint8_t* leafp, uint32_t LB, uint32_t uold, const SC& S,
                         const Result& R) {
@@ -601,17 +599,14 @@ LT_HD uint64_t leb_read(const uint8_t* p, uint32_t& len) {
   return v;
 }
 
-// Pass A and the edits of deleting the sorted slice y[0..s) (1 <= s <=
-// kKeys, repeats allowed) from the leaf (as plan_leaf).  R.added: bit q =
+// The edits of deleting the sorted slice y[0..s) (1 <= s <= kKeys, repeats
+// allowed), placed by pass A, from the leaf (as plan_insert).  R.added: bit q =
 // slice key q was removed; R.wlo .. R.whi covers the old used bytes from the
 // first edit on, so the bytes freed at the end are cleared.
 template <class SC>
-LT_HD uint32_t plan_delete(uint8_t* leafp, uint32_t LB, uint32_t uold, uint32_t m,
-                           const uint64_t (&y)[kKeys], uint32_t s, const SC& S,
+LT_HD uint32_t plan_delete(const uint8_t* leafp, uint32_t uold, uint32_t m,
+                           const uint64_t (&y)[kKeys], uint32_t s, uint64_t head, const SC& S,
                            Result& R) {
-  uint64_t head;
-  const uint32_t pa = pass_a(leafp, uold, m, y, s, S, head);
-  if (pa != kPlaced) return pa;
   uint32_t E = 0, nn = 0, removed = 0;
   int32_t tot = 0;
   uint64_t newhead = head;
@@ -717,11 +712,22 @@ LT_HD void write_delete_edits(uint8_t* leafp, const SC& S, const Result& R) {
   }
 }
 
+// Pass A and the edits (DEL: of the delete) by one thread.
+template <bool DEL, class SC>
+LT_HD uint32_t plan(const uint8_t* leafp, uint32_t LB, uint32_t uold, uint32_t m,
+                    const uint64_t (&y)[kKeys], uint32_t s, const SC& S, Result& R) {
+  uint64_t head;
+  const uint32_t res = pass_a(leafp, uold, y, s, S, head);
+  if (res != kPlaced) return res;
+  return DEL ? plan_delete(leafp, uold, m, y, s, head, S, R)
+             : plan_insert(LB, uold, m, y, s, head, S, R);
+}
+
 template <class SC>
 LT_HD uint32_t delete_leaf(uint8_t* leafp, uint32_t LB, uint32_t uold, uint32_t m,
                            const uint64_t (&y)[kKeys], uint32_t s, const SC& S,
                            Result& R) {
-  const uint32_t res = plan_delete(leafp, LB, uold, m, y, s, S, R);
+  const uint32_t res = plan<true>(leafp, LB, uold, m, y, s, S, R);
   if (res == kWritten) {
     rewrite_forward(leafp, LB, uold, S, R);
     write_delete_edits(leafp, S, R);
@@ -735,7 +741,7 @@ template <class SC>
 LT_HD uint32_t insert_leaf(uint8_t* leafp, uint32_t LB, uint32_t uold, uint32_t m,
                            const uint64_t (&y)[kKeys], uint32_t s, const SC& S,
                            Result& R) {
-  const uint32_t res = plan_leaf(leafp, LB, uold, m, y, s, S, R);
+  const uint32_t res = plan<false>(leafp, LB, uold, m, y, s, S, R);
   if (res == kWritten) {
     rewrite_leaf(leafp, LB, uold, S, R);
     write_edits(leafp, y, S, R);

@@ -1133,7 +1133,7 @@ __device__ __forceinline__ uint32_t point_stage_delete(const MergeArgs& a, uint8
     for (uint32_t q = 0; q < K; q++) y[q] = q < s ? a.u[i + q] : 0ull;
     leafthr::Result R;
     R.E = 0;
-    const uint32_t res = leafthr::plan_delete(slot, a.LB, uold, m, y, s, S, R);
+    const uint32_t res = leafthr::plan<true>(slot, a.LB, uold, m, y, s, S, R);
     if (res == leafthr::kUnchanged) {
       verdict = kLeafSame;
     } else if (res == leafthr::kWritten && R.newc > 0 &&
@@ -1318,9 +1318,12 @@ __device__ __forceinline__ void thread_finish(const MergeArgs& a, uint32_t t, ui
 
 // DEL: the same for deletes of at most kThrKeys keys from a byte-code leaf
 // (plan_delete, forward rewrite; never over LB bytes).
+// Bound by instruction issue at half the lanes (ncu: 0.63 issued per cycle and
+// scheduler, 14.6 threads each).  1e6 keys into 1e8: 238 us, out of it 191 us;
+// with each thread placing its own leaf's keys 254 and 224 us.  (Sorting the
+// block's leaves once more, by chunks to rewrite: 245 and 225 us.)
 // Four blocks per SM (64 registers, a few spilled) ran faster than three with
-// 80: 1e6 keys into 1e8 254 against 257 us, out of it 219 against 237 us; five
-// blocks were slower (271 and 240).
+// 80 (254 against 257 and 219 against 237 us before) and than five (271, 240).
 template <bool DEL>
 __global__ void __launch_bounds__(kThrT, 4) k_insert_thread(MergeArgs a) {
   constexpr uint32_t K = leafthr::kKeys;
@@ -1330,8 +1333,10 @@ __global__ void __launch_bounds__(kThrT, 4) k_insert_thread(MergeArgs a) {
   __shared__ int32_t s_esa[K * kThrT];
   __shared__ uint32_t s_tile[kThrT];
   __shared__ uint32_t s_hist[kThrBuckets + 1];
+  __shared__ uint16_t s_task[K * kThrT];
   if (a.st->err) return;
   const unsigned tid = threadIdx.x;
+  uint16_t* task = s_task + (tid & ~31u) * K;  // the warp's
   const leafthr::Scratch S{s_rpos + tid, s_rval + tid, s_rcode + tid, s_epos + tid,
                            s_esa + tid,  s_ekey + tid, (uint32_t)kThrT};
   const uint64_t n = a.st->nT;
@@ -1371,26 +1376,59 @@ __global__ void __launch_bounds__(kThrT, 4) k_insert_thread(MergeArgs a) {
     __syncthreads();
     ull dl = 0, db = 0;  // db: change of the byte total, mod 2^64
     uint32_t lng = 0xFFFFFFFFu;
-    if (tid < s_hist[kThrBuckets]) {
-      const uint32_t t = s_tile[tid];
-      const uint32_t tb = a.T_begin[t], s = a.T_begin[t + 1] - tb;
-      const uint32_t uold = a.T_oldused[t], j = a.T_leaf[t], m = a.T_oldcnt[t];
-      const uint32_t fc0 = a.T_first_chunk[t], fc1 = a.T_first_chunk[t + 1];
-      uint8_t* leafp = a.data + (size_t)j * a.LB;
+    const bool act = tid < s_hist[kThrBuckets];
+    uint32_t t = 0, tb = 0, s = 0, uold = 0, j = 0, res = leafthr::kLongCode;
+    uint64_t y[K], head = 0;
+    if (act) {
+      t = s_tile[tid];
+      tb = a.T_begin[t];
+      s = a.T_begin[t + 1] - tb;
+      uold = a.T_oldused[t];
+      j = a.T_leaf[t];
       // algorithmic bytes of a touched leaf: the old leaf, the new one and
       // 24 bytes of metadata (the new leaf added below once it is known)
       nbytes += uold + 24u;
-      uint64_t y[K];
 #pragma unroll
       for (uint32_t q = 0; q < K; q++) y[q] = q < s ? a.u[tb + q] : 0ull;
-      leafthr::Result R;
-      R.E = 0;
-      const uint32_t res = DEL ? leafthr::plan_delete(leafp, a.LB, uold, m, y, s, S, R)
-                               : leafthr::plan_leaf(leafp, a.LB, uold, m, y, s, S, R);
+      res = leafthr::pass_a_sum(a.data + (size_t)j * a.LB, uold, y, s, S, head);
+    }
+    __syncwarp();
+    // the warp's keys that lie inside a chunk, one per lane: most leaves have
+    // one or two, but some lane of nearly every warp has four
+    uint32_t nk = 0;
+#pragma unroll
+    for (uint32_t q = 0; q < K; q++) {
+      const bool mid = res == leafthr::kPlaced && q < s &&
+                       (s_rpos[q * kThrT + tid] >> 24) == leafthr::kChunk;
+      const unsigned mk = __ballot_sync(FULL, mid);
+      if (mid) task[nk + __popc(mk & lanemask_lt())] = (uint16_t)(q * kThrT + tid);
+      nk += __popc(mk);
+    }
+    __syncwarp();
+    for (uint32_t i0 = 0; i0 < nk; i0 += 32) {
+      const bool on = i0 + lane_id() < nk;
+      const uint32_t r = on ? task[i0 + lane_id()] : 0u, q = r / kThrT, own = r & 31u;
+      const uint32_t jo = __shfl_sync(FULL, j, own), uo = __shfl_sync(FULL, uold, own);
+      const uint32_t at = __shfl_sync(FULL, tb, own) + q;
+      if (on) {
+        const uint64_t yq = a.u[at];
+        leafthr::place_key(a.data + (size_t)jo * a.LB, uo, yq, q > 0 && a.u[at - 1] == yq,
+                           s_rpos[r], s_rval[r], s_rcode[r]);
+      }
+    }
+    __syncwarp();
+    if (act) {
       if (res == leafthr::kLongCode) {
         lng = t;
       } else {
-        thread_finish<DEL>(a, t, tb, s, j, m, uold, fc0, fc1, leafp, y, S, res, R, nbytes, dl, db);
+        const uint32_t m = a.T_oldcnt[t];
+        uint8_t* leafp = a.data + (size_t)j * a.LB;
+        leafthr::Result R;
+        R.E = 0;
+        res = DEL ? leafthr::plan_delete(leafp, uold, m, y, s, head, S, R)
+                  : leafthr::plan_insert(a.LB, uold, m, y, s, head, S, R);
+        thread_finish<DEL>(a, t, tb, s, j, m, uold, a.T_first_chunk[t], a.T_first_chunk[t + 1],
+                           leafp, y, S, res, R, nbytes, dl, db);
       }
     }
     warp_append(lng != 0xFFFFFFFFu, lng, a.list_long, &a.st->n_long);
@@ -1436,8 +1474,7 @@ __global__ void __launch_bounds__(kLongT) k_insert_thread_long(MergeArgs a) {
     for (uint32_t q = 0; q < K; q++) y[q] = q < s ? a.u[tb + q] : 0ull;
     leafthr::Result R;
     R.E = 0;
-    const uint32_t res = DEL ? leafthr::plan_delete(leafp, a.LB, uold, m, y, s, S, R)
-                             : leafthr::plan_leaf(leafp, a.LB, uold, m, y, s, S, R);
+    const uint32_t res = leafthr::plan<DEL>(leafp, a.LB, uold, m, y, s, S, R);
     thread_finish<DEL>(a, t, tb, s, j, m, uold, a.T_first_chunk[t], a.T_first_chunk[t + 1], leafp,
                        y, S, res, R, nbytes, dl, db);
   }
