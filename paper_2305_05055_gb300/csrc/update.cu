@@ -2842,7 +2842,7 @@ __global__ void __launch_bounds__(kT) k_rebuild_scatter(const uint64_t* __restri
 // (k_build_encode).  A repeat costs no bytes and is skipped wherever it falls.
 // Two reads of the keys and one of them with the leaves' bytes out; flags,
 // their scan, a compaction, costs, their scan and a search per leaf took 820
-// us of 3e7 keys, these three 320 us.
+// us of 3e7 keys, these three 335 us.
 constexpr int kBuildItems = 8;
 constexpr uint32_t kBuildTile = kT * kBuildItems;  // keys per block step
 
@@ -3030,86 +3030,207 @@ struct BuildOut {
   uint32_t* cnt;
   uint64_t* heads;
   uint32_t LB;
+  uint32_t per;  // leaves a warp takes at a time
   Status* st;
 };
 
-// A warp per leaf, two keys per lane and step: byte costs, their warp prefix,
-// the codes stored byte by byte into the leaf's image in shared memory, the
-// image to memory whole.  heads[L] is set for a set without empty leaves (the
-// head fix-up runs when there are some).
+// A warp writes leaf w, two keys per lane and step: byte costs, their warp
+// prefix, the codes stored byte by byte into the leaf's image in shared memory,
+// the image to memory whole.
+__device__ __forceinline__ void build_leaf_warp(const BuildArgs& a, const BuildOut& o, uint64_t w,
+                                                uint64_t b, uint64_t e, uint8_t* buf, ull& added) {
+  const unsigned lane = lane_id();
+  for (uint32_t p = lane * 16; p < o.LB; p += 512)
+    *reinterpret_cast<uint4*>(buf + p) = make_uint4(0u, 0u, 0u, 0u);
+  __syncwarp();
+  uint32_t pos = 0, cnt = 0;
+  uint64_t last = b ? a.x[b - 1] : 0, head = KEY_MAX;  // the key before this step's
+  bool fits = true;
+  for (uint64_t i0 = b; i0 < e && fits; i0 += 64) {
+    const uint64_t i = i0 + 2 * lane;
+    const uint64_t x0 = i < e ? a.x[i] : 0, x1 = i + 1 < e ? a.x[i + 1] : 0;
+    uint64_t before = __shfl_up_sync(FULL, x1, 1);
+    if (lane == 0) before = last;
+    const bool k0 = i < e && (i == 0 || x0 != before), k1 = i + 1 < e && x1 != x0;
+    const unsigned m0 = __ballot_sync(FULL, k0), m1 = __ballot_sync(FULL, k1);
+    // the leaf's first key is its head, 8 bytes uncoded
+    bool h0 = false, h1 = false;
+    if (cnt == 0 && (m0 | m1)) {
+      const int f0 = m0 ? __ffs(m0) - 1 : 32, f1 = m1 ? __ffs(m1) - 1 : 32;
+      h0 = f0 <= f1 && (int)lane == f0;
+      h1 = f1 < f0 && (int)lane == f1;
+      head = f0 <= f1 ? __shfl_sync(FULL, x0, f0 & 31) : __shfl_sync(FULL, x1, f1 & 31);
+    }
+    const uint64_t d0 = h0 || a.raw ? x0 : x0 - before, d1 = h1 || a.raw ? x1 : x1 - x0;
+    const bool c0 = h0 || a.raw, c1 = h1 || a.raw;  // cells: 8 bytes as they are
+    const uint32_t l0 = !k0 ? 0u : c0 ? 8u : leb_len(d0), l1 = !k1 ? 0u : c1 ? 8u : leb_len(d1);
+    const uint32_t inc = warp_incl_scan(l0 + l1);
+    const uint32_t tot = __shfl_sync(FULL, inc, 31);
+    fits = pos + tot <= o.LB;
+    if (fits) {
+      uint8_t* p = buf + pos + inc - l0 - l1;
+      auto put = [&](uint64_t d, uint32_t l, bool cell) {
+        for (uint32_t q = 0; q < l; q++)
+          p[q] = cell ? (uint8_t)(d >> (8 * q))
+                      : (uint8_t)(((uint32_t)(d >> (7 * q)) & 0x7Fu) | (q + 1 < l ? 0x80u : 0u));
+        p += l;
+      };
+      put(d0, l0, c0);
+      put(d1, l1, c1);
+    }
+    pos += tot;
+    cnt += __popc(m0) + __popc(m1);
+    last = __shfl_sync(FULL, x1, 31);  // read only when the step was full
+  }
+  if (!fits && lane == 0) atomicOr(&o.st->err, kErrFit);
+  __syncwarp();
+  uint8_t* leafp = o.data + w * o.LB;
+  for (uint32_t p = lane * 16; p < o.LB; p += 512)
+    *reinterpret_cast<uint4*>(leafp + p) = *reinterpret_cast<const uint4*>(buf + p);
+  if (lane == 0) {
+    o.used[w] = pos;
+    o.cnt[w] = cnt;
+    o.heads[w] = head;
+    if (w + 1 == a.L) o.heads[a.L] = w;
+    added += pos;
+    if (cnt == 0) atomicAdd(&o.st->nempty, 1ull);
+  }
+  __syncwarp();
+}
+
+// One thread's bytes of a leaf on their way out: eight gathered in acc, two of
+// those to a 16-byte store.  Stores past the leaf are left out (the byte count
+// then says that it does not fit).
+struct ByteOut {
+  uint8_t* p;
+  uint32_t LB, n = 0;       // bytes so far
+  uint64_t acc = 0, w0 = 0;
+  __device__ __forceinline__ void word() {  // acc is full; n counts its bytes
+    const uint32_t at = n & ~7u;            // the byte after it
+    if (at & 8u) w0 = acc;
+    else if (at <= LB) *reinterpret_cast<ulonglong2*>(p + at - 16u) = make_ulonglong2(w0, acc);
+  }
+  __device__ __forceinline__ void put(uint64_t c, uint32_t l) {  // 1 <= l <= 8 bytes of c
+    const uint32_t f = n & 7u;
+    acc |= c << (8u * f);
+    n += l;
+    if (f + l >= 8u) {
+      word();
+      acc = f ? c >> (8u * (8u - f)) : 0ull;
+    }
+  }
+};
+
+// Writes leaf w from its keys [b, e): at most LB of them, byte codes.
+__device__ __forceinline__ void build_leaf_thread(const BuildArgs& a, const BuildOut& o, uint64_t w,
+                                                  uint64_t b, uint64_t e, ull& added) {
+  ByteOut out;
+  out.p = o.data + w * o.LB;
+  out.LB = o.LB;
+  uint32_t cnt = 0;
+  uint64_t prev = b ? a.x[b - 1] : 0, head = KEY_MAX;
+  // four keys at a time in two 16-byte loads (a lane's loads hit lines of their
+  // own, so their number is what counts), the next four on their way meanwhile;
+  // the first four may start before b
+  const uint64_t i0 = b & ~1ull;
+  const bool vec = (reinterpret_cast<uintptr_t>(a.x) & 15u) == 0;
+  uint64_t nx[4];
+  auto load = [&](uint64_t i) {
+#pragma unroll
+    for (int q = 0; q < 4; q += 2) {
+      if (vec && i + q + 1 < a.n && i + q < e) {
+        const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(a.x + i + q);
+        nx[q] = v.x;
+        nx[q + 1] = v.y;
+      } else {
+        nx[q] = i + q < e ? a.x[i + q] : 0;
+        nx[q + 1] = i + q + 1 < e ? a.x[i + q + 1] : 0;
+      }
+    }
+  };
+  load(i0);
+  for (uint64_t i = i0; i < e; i += 4) {
+    uint64_t x[4];
+#pragma unroll
+    for (int q = 0; q < 4; q++) x[q] = nx[q];
+    load(i + 4);
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+      if (i + q < b || i + q >= e || (x[q] == prev && i + q)) continue;  // (a repeat)
+      uint64_t d = x[q] - prev;
+      prev = x[q];
+      if (!cnt++) {  // the head: 8 bytes as they are
+        head = x[q];
+        out.put(head, 8);
+        continue;
+      }
+      while (d >> 28) {  // four bytes, all continued
+        const uint32_t v = (uint32_t)d;
+        out.put((v & 0x7Fu) | ((v << 1) & 0x7F00u) | ((v << 2) & 0x7F0000u) |
+                    ((v << 3) & 0x7F000000u) | 0x80808080u, 4);
+        d >>= 28;
+      }
+      const uint32_t v = (uint32_t)d;
+      const uint32_t l = 1u + (v >= 1u << 7) + (v >= 1u << 14) + (v >= 1u << 21);
+      out.put(((v & 0x7Fu) | ((v << 1) & 0x7F00u) | ((v << 2) & 0x7F0000u) | ((v << 3) & 0x7F000000u)) +
+                  (0x00808080u & ((1u << (8u * (l - 1u))) - 1u)), l);
+    }
+  }
+  const uint32_t used = out.n;
+  // the rest of the leaf
+  if (used & 15u) {
+    if (used & 8u) {
+      if ((used & ~15u) + 16u <= o.LB)
+        *reinterpret_cast<ulonglong2*>(out.p + (used & ~15u)) = make_ulonglong2(out.w0, out.acc);
+    } else if ((used & ~15u) + 16u <= o.LB) {
+      *reinterpret_cast<ulonglong2*>(out.p + (used & ~15u)) = make_ulonglong2(out.acc, 0ull);
+    }
+  }
+  for (uint32_t p = (used + 15u) & ~15u; p < o.LB; p += 16)
+    *reinterpret_cast<uint4*>(out.p + p) = make_uint4(0u, 0u, 0u, 0u);
+  if (used > o.LB) atomicOr(&o.st->err, kErrFit);
+  o.used[w] = used;
+  o.cnt[w] = cnt;
+  o.heads[w] = head;
+  if (w + 1 == a.L) o.heads[a.L] = w;
+  added += used;
+  if (cnt == 0) atomicAdd(&o.st->nempty, 1ull);
+}
+
+// A thread per leaf (o.per = 32 to a warp).  A leaf of more keys than bytes is
+// full of repeats, which one thread would take a long time to pass over: the
+// warp then writes it together, as it does cells, and all leaves of a set with
+// few of them (o.per = 1), where a thread's chain of keys is what it waits for
+// (4.3e3 leaves 8 us by warps and 20 by threads, 1.3e4 17 and 23, 3.6e4 41 and
+// 46, 3.2e5 239 and 181).  heads[L] is set for a set without empty leaves (the
+// head fix-up runs when there are some).  By warps it takes 650 instructions
+// for a leaf's 107 keys, by threads 105e6 in all for 3e7 keys; then the lanes'
+// scattered 16-byte loads and stores bound it (L2 at 67 % of its rate).
 __global__ void __launch_bounds__(kT) k_build_encode(BuildArgs a, BuildOut o) {
   extern __shared__ __align__(16) uint8_t smem[];
   pdl_wait();
   pdl_launch();
-  const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
-  uint8_t* buf = smem + (size_t)warp * o.LB;
-  const uint64_t gw = gtid() >> 5, nw = gstride() >> 5;
+  const unsigned lane = lane_id();
+  uint8_t* buf = smem + (size_t)(threadIdx.x >> 5) * o.LB;
   ull added = 0;
-  for (uint64_t w = gw; w < a.L; w += nw) {
-    const uint64_t b = a.dstart[w], e = w + 1 < a.L ? a.dstart[w + 1] : a.n;
-    for (uint32_t p = lane * 16; p < o.LB; p += 512)
-      *reinterpret_cast<uint4*>(buf + p) = make_uint4(0u, 0u, 0u, 0u);
-    __syncwarp();
-    uint32_t pos = 0, cnt = 0;
-    uint64_t last = b ? a.x[b - 1] : 0, head = KEY_MAX;  // the key before this step's
-    bool fits = true;
-    for (uint64_t i0 = b; i0 < e && fits; i0 += 64) {
-      const uint64_t i = i0 + 2 * lane;
-      const uint64_t x0 = i < e ? a.x[i] : 0, x1 = i + 1 < e ? a.x[i + 1] : 0;
-      uint64_t before = __shfl_up_sync(FULL, x1, 1);
-      if (lane == 0) before = last;
-      const bool k0 = i < e && (i == 0 || x0 != before), k1 = i + 1 < e && x1 != x0;
-      const unsigned m0 = __ballot_sync(FULL, k0), m1 = __ballot_sync(FULL, k1);
-      // the leaf's first key is its head, 8 bytes uncoded
-      bool h0 = false, h1 = false;
-      if (cnt == 0 && (m0 | m1)) {
-        const int f0 = m0 ? __ffs(m0) - 1 : 32, f1 = m1 ? __ffs(m1) - 1 : 32;
-        h0 = f0 <= f1 && (int)lane == f0;
-        h1 = f1 < f0 && (int)lane == f1;
-        head = f0 <= f1 ? __shfl_sync(FULL, x0, f0 & 31) : __shfl_sync(FULL, x1, f1 & 31);
-      }
-      const uint64_t d0 = h0 || a.raw ? x0 : x0 - before, d1 = h1 || a.raw ? x1 : x1 - x0;
-      const bool c0 = h0 || a.raw, c1 = h1 || a.raw;  // cells: 8 bytes as they are
-      const uint32_t l0 = !k0 ? 0u : c0 ? 8u : leb_len(d0), l1 = !k1 ? 0u : c1 ? 8u : leb_len(d1);
-      const uint32_t inc = warp_incl_scan(l0 + l1);
-      const uint32_t tot = __shfl_sync(FULL, inc, 31);
-      fits = pos + tot <= o.LB;
-      if (fits) {
-        uint8_t* p = buf + pos + inc - l0 - l1;
-        auto put = [&](uint64_t d, uint32_t l, bool cell) {
-          if (cell) {
-            for (uint32_t q = 0; q < l; q++) p[q] = (uint8_t)(d >> (8 * q));
-          } else {
-#pragma unroll
-            for (uint32_t q = 0; q < 4; q++)
-              if (q < l) p[q] = (uint8_t)(((uint32_t)(d >> (7 * q)) & 0x7Fu) | (q + 1 < l ? 0x80u : 0u));
-            for (uint32_t q = 4; q < l; q++)
-              p[q] = (uint8_t)(((uint32_t)(d >> (7 * q)) & 0x7Fu) | (q + 1 < l ? 0x80u : 0u));
-          }
-          p += l;
-        };
-        put(d0, l0, c0);
-        put(d1, l1, c1);
-      }
-      pos += tot;
-      cnt += __popc(m0) + __popc(m1);
-      last = __shfl_sync(FULL, x1, 31);  // read only when the step was full
+  for (uint64_t w0 = (gtid() >> 5) * o.per; w0 < a.L; w0 += (gstride() >> 5) * o.per) {
+    const uint64_t w = w0 + lane;
+    const bool mine = lane < o.per && w < a.L;
+    uint64_t b = 0, e = 0;
+    if (mine) {
+      b = a.dstart[w];
+      e = w + 1 < a.L ? a.dstart[w + 1] : a.n;
     }
-    if (!fits && lane == 0) atomicOr(&o.st->err, kErrFit);
+    const bool together = mine && (o.per == 1 || a.raw || e - b > o.LB);
+    if (mine && !together) build_leaf_thread(a, o, w, b, e, added);
     __syncwarp();
-    uint8_t* leafp = o.data + w * o.LB;
-    for (uint32_t p = lane * 16; p < o.LB; p += 512)
-      *reinterpret_cast<uint4*>(leafp + p) = *reinterpret_cast<const uint4*>(buf + p);
-    if (lane == 0) {
-      o.used[w] = pos;
-      o.cnt[w] = cnt;
-      o.heads[w] = head;
-      if (w + 1 == a.L) o.heads[a.L] = w;
-      added += pos;
-      if (cnt == 0) atomicAdd(&o.st->nempty, 1ull);
+    for (unsigned m = __ballot_sync(FULL, together); m; m &= m - 1u) {
+      const int src = __ffs(m) - 1;
+      build_leaf_warp(a, o, w0 + src, __shfl_sync(FULL, b, src), __shfl_sync(FULL, e, src), buf,
+                      added);
     }
-    __syncwarp();
   }
+  added = warp_sum(added);
   if (lane == 0 && added) atomicAdd(&o.st->bytes_total, added);
 }
 
@@ -4121,11 +4242,12 @@ int build_from_sorted(cpma* h, const uint64_t* x, uint64_t n, cudaStream_t st) {
   if (rc == CPMA_OK) {
     const BuildArgs a{x, n, P<uint64_t>(s.partials), L, S, P<uint64_t>(s.dstart),
                       (int)h->cfg.codec};
-    const BuildOut o{na.data, na.used, na.cnt, na.heads, LB, h->d_status};
+    const uint32_t per = L <= (uint64_t)h->num_sms * 256 ? 1u : 32u;
+    const BuildOut o{na.data, na.used, na.cnt, na.heads, LB, per, h->d_status};
     if (n) rc = check_cuda(launch_pdl(k_build_cuts, build_grid(h, n), kT, 0, st, a));
     else rc = check_cuda(cudaMemsetAsync(s.dstart.p, 0, 8, st));
     if (rc == CPMA_OK)
-      rc = check_cuda(launch_pdl(k_build_encode, (unsigned)grid_for(h, L * 32), kT,
+      rc = check_cuda(launch_pdl(k_build_encode, (unsigned)grid_for(h, L * 32 / per), kT,
                                  (size_t)(kT / 32) * LB, st, a, o));
     h->launches += 2;
   }

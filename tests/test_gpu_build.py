@@ -54,3 +54,24 @@ def test_build_shapes(kind, LB):
         keys = np.concatenate([W.full_range_keys(5, 5_000), np.arange(60_000, dtype=U),
                                np.array([0, 2**64 - 1, 2**63, 2**64 - 1], U)])
     same(keys, leaf_bytes=LB)
+
+
+@pytest.mark.parametrize("kind", ["uniform", "mixed", "long", "runs"])
+def test_build_of_many_leaves(kind):
+    # a thread writes each leaf from 256 leaves per SM on; one of more keys
+    # than bytes (a run of repeats) is written by a warp
+    if kind == "uniform":
+        keys = W.uniform_keys(11, 2_600_001, bits=40)
+    elif kind == "mixed":   # codes of 1 to 10 bytes, every shift of the 8-byte words
+        keys = np.concatenate([W.uniform_keys(12, 1_500_000, bits=24), W.full_range_keys(13, 700_001),
+                               W.uniform_keys(14, 600_000, bits=46)])
+    elif kind == "long":
+        keys = W.full_range_keys(15, 1_000_003)
+    else:
+        keys = W.uniform_keys(16, 2_700_000, bits=40)
+        keys[100_000:103_000] = keys[5]
+        keys[200_000:200_200] = keys[6]
+    g = cp.CPMA(torch.from_numpy(np.ascontiguousarray(keys).view(np.int64)).cuda(), leaf_bytes=256)
+    assert g.leaves() > 256 * torch.cuda.get_device_properties(0).multi_processor_count
+    del g
+    same(keys, leaf_bytes=256)
