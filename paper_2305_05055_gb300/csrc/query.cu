@@ -454,6 +454,13 @@ struct Leaves {
   uint32_t LB;
 };
 
+// No two elements of leaf j lie this far apart: the next leaf's head (an empty
+// one's is that of the next with elements, or 2^64 - 1) is above them all.
+__device__ __forceinline__ uint64_t leaf_span(const uint64_t* __restrict__ heads, uint64_t L,
+                                              uint64_t j) {
+  return j + 1 < L ? __ldg(heads + j + 1) - __ldg(heads + j) : ~0ull;
+}
+
 // Last index i in [a, n) with p[i] <= x, p sorted; a when p[a] > x too.  The
 // next few entries are tried first: most ranges end in their first leaf or
 // the one after it.
@@ -480,14 +487,19 @@ __device__ __forceinline__ uint64_t last_from(const uint64_t* __restrict__ p, ui
 template <int OP, bool PLAIN>
 struct Reduce {
   uint64_t mask, value;
-  __device__ __forceinline__ void leaf(const uint8_t* leafp, uint32_t u, const uint32_t* cnt,
-                                       uint64_t& r, uint64_t& c) const {
+  __device__ __forceinline__ void leaf(const Leaves& t, uint64_t j, uint32_t u, uint64_t& r,
+                                       uint64_t& c) const {
     if constexpr (PLAIN) {
-      const uint32_t m = *cnt;
-      r += leafwalk::leaf_sum(leafp, u, m);
+      const uint32_t m = t.cnt[j];
+      r += leafwalk::leaf_sum(t.data + j * t.LB, u, m, leaf_span(t.heads, t.L, j));
       c += m;
     } else {
-      leafwalk::leaf_visit(leafp, u, [&](uint64_t v) {
+      if (OP == CPMA_OP_SUM && !((mask | value) >> 32) &&
+          !leafwalk::any_lane(leaf_span(t.heads, t.L, j) > 1ull << 28)) {
+        leafwalk::leaf_masked_sum(t.data + j * t.LB, u, (uint32_t)mask, (uint32_t)value, r, c);
+        return;
+      }
+      leafwalk::leaf_visit(t.data + j * t.LB, u, [&](uint64_t v) {
         if ((v & mask) == value) { r = op_apply<OP>(r, v); c++; }
       });
     }
@@ -508,9 +520,10 @@ struct Reduce {
 // its part of the first leaf; the queries that reach another leaf put their
 // last one on the block's list, which the first threads then take, so a warp
 // runs the second decode only when 32 of them have one.  Writes the ends'
-// reduction and count and the leaves strictly between (first, items).
+// reduction and count and the leaves strictly between (first, items).  Three
+// blocks per SM for plain sums (1e5 ranges 73 us; 84 with two, 77 with four).
 template <int OP, bool PLAIN>
-__global__ void __launch_bounds__(kT) k_range_ends(const uint64_t* __restrict__ lo,
+__global__ void __launch_bounds__(kT, PLAIN ? 3 : 1) k_range_ends(const uint64_t* __restrict__ lo,
                                                    const uint64_t* __restrict__ hi, uint64_t q,
                                                    Leaves t, Reduce<OP, PLAIN> f,
                                                    uint64_t* __restrict__ first,
@@ -912,8 +925,11 @@ __global__ void __launch_bounds__(kT) k_tile_scan(LeafPrefix p, uint64_t nt) {
 // Every leaf reduced once, scanned inside tiles of kT leaves, and the tiles by
 // the last block to finish (when the queries cover more than p.most leaves;
 // otherwise nothing).
+// Four blocks per SM: the lanes' scattered loads are what it waits for (plain,
+// 1e8 keys: 106 us with the registers it would take, 76 us; masked sums, 5e7
+// keys: 157 and 109 us).
 template <int OP, bool PLAIN>
-__global__ void __launch_bounds__(kT) k_leaf_prefix(Leaves t, Reduce<OP, PLAIN> f,
+__global__ void __launch_bounds__(kT, 4) k_leaf_prefix(Leaves t, Reduce<OP, PLAIN> f,
                                                     const uint64_t* __restrict__ total,
                                                     LeafPrefix p, ull* prof) {
   __shared__ uint32_t s_hist[kSumBuckets], s_order[kT];
@@ -936,7 +952,7 @@ __global__ void __launch_bounds__(kT) k_leaf_prefix(Leaves t, Reduce<OP, PLAIN> 
       const uint32_t u = min(t.used[j0 + o], t.LB);
       uint64_t r = op_identity<OP>(), c = 0;
       if (u) {
-        f.leaf(t.data + (j0 + o) * t.LB, u, t.cnt + j0 + o, r, c);
+        f.leaf(t, j0 + o, u, r, c);
         nbytes += u;
       }
       s_r[o] = r;
@@ -1061,7 +1077,7 @@ __global__ void __launch_bounds__(kT) k_range_inner(Leaves t, Reduce<OP, PLAIN> 
     const uint64_t j = fl + (g - qoff);
     const uint32_t u = min(t.used[j], t.LB);
     nbytes += u;
-    if (u) f.leaf(t.data + j * t.LB, u, t.cnt + j, r, c);
+    if (u) f.leaf(t, j, u, r, c);
   }
   const uint64_t q0 = __shfl_sync(FULL, qi, 0);
   if (__all_sync(FULL, qi == q0 || c == 0)) {
@@ -1299,9 +1315,10 @@ __global__ void __launch_bounds__(kT) k_extract_leaf(ExtractArgs a) {
   }
 }
 
-__global__ void __launch_bounds__(kT) k_sum(const uint8_t* __restrict__ data,
+__global__ void __launch_bounds__(kT, 4) k_sum(const uint8_t* __restrict__ data,
                                             const uint32_t* __restrict__ used,
-                                            const uint32_t* __restrict__ cnt, uint64_t L,
+                                            const uint32_t* __restrict__ cnt,
+                                            const uint64_t* __restrict__ heads, uint64_t L,
                                             uint32_t LB, uint64_t* sum, uint64_t* count,
                                             ull* prof, int raw) {
   const unsigned lane = lane_id();
@@ -1325,7 +1342,7 @@ __global__ void __launch_bounds__(kT) k_sum(const uint8_t* __restrict__ data,
         nbytes += 8;  // its used and element counts
         if (uu) {
           const uint32_t m = cnt[jj];
-          s += leafwalk::leaf_sum(data + jj * LB, uu, m);
+          s += leafwalk::leaf_sum(data + jj * LB, uu, m, leaf_span(heads, L, jj));
           c += m;
           nbytes += uu;
         }
@@ -1857,8 +1874,8 @@ int run_sum(const cpma* h, uint64_t* sum, uint64_t* count, cudaStream_t st) {
   CPMA_CUDA(cudaMemsetAsync(sum, 0, 8, st));
   if (count) CPMA_CUDA(cudaMemsetAsync(count, 0, 8, st));
   prof_begin(h, PH_SUM, st);
-  k_sum<<<persistent_grid(h), kT, 0, st>>>(h->data, h->used, h->cnt, h->L, h->cfg.leaf_bytes, sum,
-                                           count, prof_bytes(h, PH_SUM), (int)h->cfg.codec);
+  k_sum<<<persistent_grid(h), kT, 0, st>>>(h->data, h->used, h->cnt, h->heads, h->L,
+                                           h->cfg.leaf_bytes, sum, count, prof_bytes(h, PH_SUM), (int)h->cfg.codec);
   CPMA_LAUNCHED(h);
   prof_end(h, st);
   return check_cuda(cudaGetLastError());

@@ -2,11 +2,12 @@
 // membership test (leaf_thread.cuh) for the CPU tests.
 #include "../paper_2305_05055_gb300/csrc/leaf_thread.cuh"
 
-extern "C" uint64_t lw_sum(const uint8_t* leaf, uint32_t u, uint32_t m, int form) {
+extern "C" uint64_t lw_sum(const uint8_t* leaf, uint32_t u, uint32_t m, int form,
+                           uint64_t span) {
   uint64_t s = 0;
-  if (form == 0) return leafwalk::leaf_sum(leaf, u, m);
+  if (form == 0) return leafwalk::leaf_sum(leaf, u, m, span);
   if (form == 1) return leafwalk::sum_walked(leaf, u);
-  return (form == 2 ? leafwalk::sum_few(leaf, u, m, s) : leafwalk::sum_many(leaf, u, m, s)) ? s : ~0ull;
+  return (form == 2 ? leafwalk::sum_few<4>(leaf, u, m, s) : leafwalk::sum_many(leaf, u, m, s)) ? s : ~0ull;
 }
 
 extern "C" uint32_t lw_visit(const uint8_t* leaf, uint32_t u, uint64_t* out) {
@@ -60,6 +61,12 @@ extern "C" uint32_t lw_between(const uint8_t* leaf, uint32_t u, uint64_t lo, uin
   uint32_t n = 0;
   leafwalk::leaf_range_visit(leaf, u, lo, hi, [&](uint64_t v) { out[n++] = v; });
   return n;
+}
+
+extern "C" void lw_masked(const uint8_t* leaf, uint32_t u, uint32_t mask, uint32_t value,
+                          uint64_t* out) {
+  out[0] = out[1] = 0;
+  leafwalk::leaf_masked_sum(leaf, u, mask, value, out[0], out[1]);
 }
 
 // The elements from lo on, starting where the search for it ended; returns

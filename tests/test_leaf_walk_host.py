@@ -30,12 +30,13 @@ def lw(tmp_path_factory):
                     os.path.join(HERE, "leaf_walk_host.cu")], check=True)
     lib = C.CDLL(out)
     u8, u32, u64, p64 = C.c_void_p, C.c_uint32, C.c_uint64, C.POINTER(C.c_uint64)
-    lib.lw_sum.restype, lib.lw_sum.argtypes = u64, [u8, u32, u32, C.c_int]
+    lib.lw_sum.restype, lib.lw_sum.argtypes = u64, [u8, u32, u32, C.c_int, u64]
     lib.lw_visit.restype, lib.lw_visit.argtypes = u32, [u8, u32, p64]
     lib.lw_range.argtypes = [u8, u32, u64, u64, p64]
     lib.lw_take.argtypes = [u8, u32, u64, u64, p64]
     lib.lw_below.restype, lib.lw_below.argtypes = u32, [u8, u32, u64]
     lib.lw_has.argtypes = [u8, u32, u64]
+    lib.lw_masked.argtypes = [u8, u32, u32, u32, p64]
     lib.lw_team.restype, lib.lw_team.argtypes = u32, [u8, u32, p64]
     lib.lw_between.restype, lib.lw_between.argtypes = u32, [u8, u32, u64, u64, p64]
     lib.lw_from.restype, lib.lw_from.argtypes = u32, [u8, u32, u64, p64]
@@ -86,18 +87,24 @@ def sums(lw, p, u, keys):
     two in 32 bits say so when a code is too long for them."""
     want, m = sum(keys) & M64, len(keys)
     short = all(b - a < 1 << 28 for a, b in zip(keys, keys[1:]))
-    few = lw.lw_sum(p, u, m, 2) if m <= 256 else want
-    return (lw.lw_sum(p, u, m, 0) == lw.lw_sum(p, u, m, 1) == want and
+    few = lw.lw_sum(p, u, m, 2, M64) if m <= 256 else want
+    span = keys[-1] - keys[0] + 1   # the least the next leaf's head can leave
+    return (lw.lw_sum(p, u, m, 0, M64) == lw.lw_sum(p, u, m, 0, span) == want and
+            lw.lw_sum(p, u, m, 1, 0) == want and
             (few if short else want) == want and
-            lw.lw_sum(p, u, m, 3) == (want if short else M64))
+            lw.lw_sum(p, u, m, 3, 0) == (want if short else M64))
 
 
 @pytest.mark.parametrize("m", [1, 2, 3, 60, 127, 128, 129, 130, 254, 255, 256, 257, 258, 400, 2040])
 def test_leaf_sum_by_number_of_codes(lw, m):
     rng = random.Random(m)
-    for ln in (1, 2, 3, 4, 0):
+    for ln in (1, 2, 3, 4, 0, -1, -2):
         keys = [rng.randrange(1 << 40)]
-        while len(keys) < m:
+        top = {-1: 1 << 14, -2: 1 << 21}.get(ln)   # spans at the edge of two and three planes
+        if top and m > 1:
+            keys += sorted(keys[0] + d for d in rng.sample(range(1, top - 1), min(m - 2, 250)))
+            keys.append(keys[0] + top - 1)
+        while len(keys) < m and not top:
             n = ln or rng.choice([1, 1, 1, 2, 3, 4])
             keys.append(keys[-1] + rng.choice([(1 << (7 * n)) - 1, max(1, 1 << (7 * (n - 1)))]))
         while oracle.leaf_bytes(np.array(keys, dtype=np.uint64)) > 2048:
@@ -120,6 +127,12 @@ def test_walk_against_keys(lw, LB):
         out = (C.c_uint64 * (len(keys) + 8))()
         assert lw.lw_visit(p, u, out) == len(keys) and list(out[:len(keys)]) == keys
         assert lw.lw_team(p, u, out) == len(keys) and list(out[:len(keys)]) == keys
+        if all(b - a < 1 << 28 for a, b in zip(keys, keys[1:])):
+            for mask in (0, 1, 255, 0xFFFFFFFF):
+                value = rng.choice(keys) & mask
+                got = [x for x in keys if x & mask == value]
+                lw.lw_masked(p, u, mask, value, out)
+                assert list(out[:2]) == [sum(got) & M64, len(got)]
         marks = [0, M64, keys[0], keys[-1], (keys[-1] + 1) & M64]
         for _ in range(6):
             x = rng.choice(keys)
