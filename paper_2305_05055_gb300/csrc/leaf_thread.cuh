@@ -232,6 +232,46 @@ LT_HD void chunk_at(const uint8_t* leafp, uint32_t LB, int32_t src, uint32_t (&r
   for (int i = 0; i < 4; i++) r[i] = fshr(W[i], W[i + 1], s8);
 }
 
+// The same for a run of chunks 16 bytes apart, downwards: of the two aligned
+// blocks it spans the upper one was read for the chunk before, and is kept.
+struct Block {
+  uint32_t w[4] = {0u, 0u, 0u, 0u};
+  int32_t at = -64;
+};
+
+LT_HD void block_at(const uint8_t* leafp, uint32_t LB, int32_t at, const Block& kept,
+                    uint32_t (&r)[4]) {
+  if (at == kept.at) {
+#pragma unroll
+    for (int i = 0; i < 4; i++) r[i] = kept.w[i];
+  } else if ((uint32_t)at < LB) {
+    ld16(leafp + at, r);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; i++) r[i] = 0u;
+  }
+}
+
+LT_HD void next_chunk_at(const uint8_t* leafp, uint32_t LB, int32_t src, Block& kept,
+                         uint32_t (&r)[4]) {
+  const int32_t base = src & ~15;
+  const uint32_t s = (uint32_t)src & 15u;
+  uint32_t lo[4], hi[4] = {0u, 0u, 0u, 0u};
+  block_at(leafp, LB, base, kept, lo);
+  if (s) block_at(leafp, LB, base + 16, kept, hi);
+  const bool two = (s & 8u) != 0u, one = (s & 4u) != 0u;
+  const uint32_t y[6] = {two ? lo[2] : lo[0], two ? lo[3] : lo[1], two ? hi[0] : lo[2],
+                         two ? hi[1] : lo[3], two ? hi[2] : hi[0], two ? hi[3] : hi[1]};
+  uint32_t z[5];
+#pragma unroll
+  for (int i = 0; i < 5; i++) z[i] = one ? y[i + 1] : y[i];
+#pragma unroll
+  for (int i = 0; i < 4; i++) r[i] = fshr(z[i], z[i + 1], 8u * (s & 3u));
+  kept.at = base;
+#pragma unroll
+  for (int i = 0; i < 4; i++) kept.w[i] = lo[i];
+}
+
 // r with the bytes [a, b) of x in place of its own.
 LT_HD void take_bytes(uint32_t (&r)[4], const uint32_t (&x)[4], uint32_t a, uint32_t b) {
   const uint32_t m16 = (b >= 16u ? 0xFFFFu : ((1u << b) - 1u)) & ~((1u << a) - 1u);
@@ -288,8 +328,8 @@ LT_HD uint32_t pass_a_sum(const uint8_t* leafp, uint32_t uold, const uint64_t (&
   uint64_t ycur = k < s ? pick(y, k) : ~0ull;
   uint64_t val = head;
   uint32_t carry = 0, lc = 0, cb = 0, p1 = 0, p2 = 0;
-  for (uint32_t p0 = 0; p0 < uold; p0 += 16) {
-    if (p0) ld16(leafp + p0, w);  // bytes past the used ones are zero (packed left)
+  // (bytes past the used ones are zero: packed left)
+  auto chunk = [&](uint32_t p0, const uint32_t (&w)[4]) {
     const uint32_t cb_in = cb;    // flags of the last word before p0
     uint32_t tsum = 0, pay = 0, w01 = 0, w23 = 0;
     if (p0) {
@@ -318,6 +358,21 @@ LT_HD uint32_t pass_a_sum(const uint8_t* leafp, uint32_t uold, const uint64_t (&
     }
     val = vend;
     carry = cnew;
+  };
+  // 32 bytes at a time: a lane's loads hit lines of their own, so their number
+  // counts
+  const bool wide = (reinterpret_cast<uintptr_t>(leafp) & 31u) == 0;
+  uint32_t w2[4];
+  for (uint32_t p0 = 0; p0 < uold; p0 += 32) {
+    const bool two = p0 + 16u < uold;
+    if (wide && two) {
+      leafwalk::ld32(leafp + p0, w, w2);
+    } else {
+      if (p0) ld16(leafp + p0, w);
+      if (two) ld16(leafp + p0 + 16u, w2);
+    }
+    chunk(p0, w);
+    if (two) chunk(p0 + 16u, w2);
   }
   if (lc) return kLongCode;
   const uint64_t lastv = val;
@@ -498,11 +553,13 @@ LT_HD uint32_t plan_insert(uint32_t LB, uint32_t uold, uint32_t m, const uint64_
 // ssa) and, where it starts inside the chunk, the ones before it.  Bytes of
 // edits are left as they fall (their own bytes are written last); bytes past
 // the new used ones (shi of the last segment) are zero.
+// kept: null, or the block read for the chunk after this one (next_chunk_at).
 template <class SC>
 LT_HD void build_chunk(const uint8_t* leafp, uint32_t LB, uint32_t uold, const SC& S, uint32_t E,
                        uint32_t os0, int cur, int32_t slo, int32_t shi, int32_t ssa, int32_t o,
-                       uint32_t (&r)[4]) {
-  chunk_at(leafp, LB, o - ssa, r);
+                       Block* kept, uint32_t (&r)[4]) {
+  if (kept) next_chunk_at(leafp, LB, o - ssa, *kept, r);
+  else chunk_at(leafp, LB, o - ssa, r);
   if (o + 16 > shi && cur + 1 == (int)E) {
     const uint32_t zero[4] = {0u, 0u, 0u, 0u};
     take_bytes(r, zero, shi > o ? (uint32_t)(shi - o) : 0u, 16u);
@@ -522,8 +579,10 @@ LT_HD void build_chunk(const uint8_t* leafp, uint32_t LB, uint32_t uold, const S
 // Every chunk is one shifted read, whatever segment it lies in; the one an
 // edit falls into merges a second (with one or two keys in most leaves, some
 // lane of every warp is at such a chunk in every step, so that is all a step
-// may cost).  Gathering those chunks segment by segment: 290 us a launch for 1e6
-// keys into 1e8, this 254 us (then; 238 us by now).
+// may cost).  1e6 keys into 1e8, the kernel: 290 us gathering those chunks
+// segment by segment, 254 so; 230 then became 197 with one 16-byte load per
+// chunk instead of five words (32 lanes' loads hit 32 lines; the deletes' way,
+// forwards, gained nothing: 189 and 193).
 template <class SC>
 LT_HD void rewrite_leaf(uint8_t* leafp, uint32_t LB, uint32_t uold, const SC& S,
                         const Result& R) {
@@ -532,13 +591,14 @@ LT_HD void rewrite_leaf(uint8_t* leafp, uint32_t LB, uint32_t uold, const SC& S,
   int cur = (int)E - 1;  // the highest segment not wholly above chunk o
   int32_t slo, shi, ssa;
   seg_bounds(S, E, uold, os0, cur, slo, shi, ssa);
+  Block kept;
   for (int32_t o = (int32_t)R.whi - 16; o >= (int32_t)R.wlo; o -= 16) {
     while (cur >= 0 && slo >= o + 16) {
       cur--;
       seg_bounds(S, E, uold, os0, cur, slo, shi, ssa);
     }
     uint32_t r[4];
-    build_chunk(leafp, LB, uold, S, E, os0, cur, slo, shi, ssa, o, r);
+    build_chunk(leafp, LB, uold, S, E, os0, cur, slo, shi, ssa, o, &kept, r);
     st16(leafp + o, r);
   }
 }
@@ -687,7 +747,7 @@ LT_HD void rewrite_forward(uint8_t* leafp, uint32_t LB, uint32_t uold, const SC&
       ssa = sa2;
     }
     uint32_t r[4];
-    build_chunk(leafp, LB, uold, S, E, os0, cur, slo, shi, ssa, o, r);
+    build_chunk(leafp, LB, uold, S, E, os0, cur, slo, shi, ssa, o, nullptr, r);
     st16(leafp + o, r);
   }
 }
