@@ -585,6 +585,53 @@ __global__ void __launch_bounds__(kT, PLAIN ? 3 : 1) k_range_ends(const uint64_t
   if (prof && lane_id() == 0 && nbytes) atomicAdd(prof, nbytes);
 }
 
+// Is this block the last of the grid to come here?  Then it sees what the
+// others wrote before.
+__device__ __forceinline__ bool last_block(uint32_t* ticket) {
+  __shared__ uint32_t s_last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+  __syncthreads();
+  const bool last = s_last != 0;
+  if (last) __threadfence();
+  return last;
+}
+
+// The items' offsets by the last block of the ends' kernel (64 threads) instead
+// of a scan of its own: a call with few queries waits for its launches.
+constexpr uint64_t kEndsScan = 1024;  // queries at most: 16 items per thread
+struct EndsScan {
+  uint64_t* off = nullptr;       // q + 1 entries; null: not here
+  ull* done = nullptr;           // Status::query_done
+};
+
+__device__ __forceinline__ void scan_ends(const EndsScan& z, const uint64_t* items, uint64_t q) {
+  __shared__ uint64_t s_w[2];
+  __shared__ uint32_t s_last;
+  if (!z.off) return;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(z.done, 1ull) == gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  const uint32_t per = (uint32_t)((q + 63) / 64);
+  const uint64_t i0 = min(q, (uint64_t)threadIdx.x * per), i1 = min(q, i0 + per);
+  uint64_t v = 0;
+  for (uint64_t i = i0; i < i1; i++) v += items[i];
+  const uint64_t inc = warp_incl_scan(v);
+  if (lane_id() == 31) s_w[threadIdx.x >> 5] = inc;
+  __syncthreads();
+  uint64_t run = inc - v + (threadIdx.x >= 32 ? s_w[0] : 0ull);
+  for (uint64_t i = i0; i < i1; i++) {
+    z.off[i] = run;
+    run += items[i];
+  }
+  if (threadIdx.x == 63) z.off[q] = run;
+  if (threadIdx.x == 0) *z.done = 0;
+}
+
 template <int OP>
 __device__ __forceinline__ void team_reduce(uint64_t& r, uint64_t& c) {
 #pragma unroll
@@ -602,7 +649,7 @@ __global__ void __launch_bounds__(kT) k_range_ends_team(const uint64_t* __restri
                                                         uint64_t* __restrict__ first,
                                                         uint64_t* __restrict__ items,
                                                         uint64_t* __restrict__ out,
-                                                        uint64_t* __restrict__ count, uint32_t* ticket, ull* prof) {
+                                                        uint64_t* __restrict__ count, uint32_t* ticket, EndsScan z, ull* prof) {
   if (ticket && gtid() == 0) *ticket = 0;
   ull nbytes = 0;
   const unsigned tl = team_lane(), team = lane_id() / kTeam;
@@ -642,6 +689,7 @@ __global__ void __launch_bounds__(kT) k_range_ends_team(const uint64_t* __restri
   }
   nbytes = warp_sum(nbytes);
   if (prof && lane_id() == 0 && nbytes) atomicAdd(prof, nbytes);
+  scan_ends(z, items, q);
 }
 
 // The same for map_range_length: thread i takes the first length[i] elements
@@ -717,7 +765,7 @@ __global__ void __launch_bounds__(kT) k_length_ends(const uint64_t* __restrict__
 __global__ void __launch_bounds__(kT) k_length_ends_team(
     const uint64_t* __restrict__ start, const uint64_t* __restrict__ length, uint64_t q, Leaves t,
     const uint64_t* __restrict__ P, uint64_t* __restrict__ first, uint64_t* __restrict__ items,
-    uint64_t* __restrict__ sum, uint64_t* __restrict__ count, uint32_t* ticket, ull* prof) {
+    uint64_t* __restrict__ sum, uint64_t* __restrict__ count, uint32_t* ticket, EndsScan z, ull* prof) {
   if (ticket && gtid() == 0) *ticket = 0;
   pdl_wait();
   pdl_launch();
@@ -785,6 +833,7 @@ __global__ void __launch_bounds__(kT) k_length_ends_team(
   }
   nbytes = warp_sum(nbytes);
   if (prof && lane_id() == 0 && nbytes) atomicAdd(prof, nbytes);
+  scan_ends(z, items, q);
 }
 
 // Reductions before (min: from) each leaf, in two levels: val / cnt inside
@@ -900,19 +949,6 @@ __device__ void tile_scan(const LeafPrefix& p, uint64_t nt, uint64_t* s_ws) {
       x = op_apply<OP>(x, v);
     }
   }
-}
-
-// Is this block the last of the grid to come here?  Then it sees what the
-// others wrote before.
-__device__ __forceinline__ bool last_block(uint32_t* ticket) {
-  __shared__ uint32_t s_last;
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
-  __syncthreads();
-  const bool last = s_last != 0;
-  if (last) __threadfence();
-  return last;
 }
 
 __global__ void __launch_bounds__(kT) k_tile_scan(LeafPrefix p, uint64_t nt) {
@@ -1544,6 +1580,16 @@ int range_scratch(cpma* h, uint64_t q, RangeScratch* r) {
   return CPMA_OK;
 }
 
+// Whether the ends' kernel leaves the offsets (scan_ends), and with what.
+EndsScan ends_scan(const cpma* h, const RangeScratch& r, uint64_t q) {
+  EndsScan z;
+  if (few_queries(h, q) && q <= kEndsScan) {
+    z.off = r.off;
+    z.done = &h->d_status->query_done;
+  }
+  return z;
+}
+
 int scan_items(cpma* h, const RangeScratch& r, uint64_t q, cudaStream_t st) {
   if (r.partials)
     return scan_u64_given_partials(h, r.items, r.off, q, r.partials, r.partials_cap, st);
@@ -1555,7 +1601,7 @@ template <int OP, bool PLAIN>
 int range_inner(cpma* h, Reduce<OP, PLAIN> f, uint64_t q, uint64_t* out, uint64_t* count,
                 const RangeScratch& r, const LeafPrefix& p, cudaStream_t st, ull* prof) {
   const Leaves t = leaves_of(h);
-  CPMA_TRY(scan_items(h, r, q, st));
+  if (!ends_scan(h, r, q).off) CPMA_TRY(scan_items(h, r, q, st));
   const uint64_t nt = (t.L + kT - 1) / kT;
   if (p.val) {
     const unsigned g = (unsigned)std::min<uint64_t>(nt, (uint64_t)persistent_grid(h));
@@ -1576,7 +1622,8 @@ int range_leaves(cpma* h, const uint64_t* lo, const uint64_t* hi, uint64_t q, ui
   const Reduce<OP, PLAIN> f{mask, value};
   if (few_queries(h, q)) {
     k_range_ends_team<OP, PLAIN><<<query_grid(h, 2 * q * kTeam, 64, 32), 64, 0, st>>>(
-        lo, hi, q, leaves_of(h), f, r.first, r.items, out, count, p.ticket, prof);
+        lo, hi, q, leaves_of(h), f, r.first, r.items, out, count, p.ticket, ends_scan(h, r, q),
+        prof);
   } else {
     const int b = query_block(h, q);
     k_range_ends<OP, PLAIN><<<query_grid(h, q, b, 8), b, 0, st>>>(lo, hi, q, leaves_of(h), f,
@@ -1697,9 +1744,13 @@ int run_range_length(const cpma* h, const uint64_t* start, const uint64_t* lengt
     const bool few = few_queries(h, q);
     const int b = few ? 64 : query_block(h, q);
     const int g = few ? query_grid(h, q * kTeam, b, 32) : query_grid(h, q, b, 8);
-    CPMA_CUDA(launch_pdl(few ? k_length_ends_team : k_length_ends, (unsigned)g, (unsigned)b, 0, st,
-                         start, length, q, leaves_of(h), P, r.first, r.items, sum, count, p.ticket,
-                         prof));
+    if (few)
+      CPMA_CUDA(launch_pdl(k_length_ends_team, (unsigned)g, (unsigned)b, 0, st, start, length, q,
+                           leaves_of(h), P, r.first, r.items, sum, count, p.ticket,
+                           ends_scan(h, r, q), prof));
+    else
+      CPMA_CUDA(launch_pdl(k_length_ends, (unsigned)g, (unsigned)b, 0, st, start, length, q,
+                           leaves_of(h), P, r.first, r.items, sum, count, p.ticket, prof));
     CPMA_LAUNCHED(h);
     const int rc = range_inner<CPMA_OP_SUM, true>(hm, Reduce<CPMA_OP_SUM, true>{0, 0}, q, sum,
                                                   count, r, p, st, prof);
