@@ -209,9 +209,11 @@ LT_HD uint64_t leaf_head(const uint8_t* leafp) {
 // 32 bytes at p (32-byte aligned) in one load.
 LT_HD void ld32(const uint8_t* p, uint32_t (&a)[4], uint32_t (&b)[4]) {
 #if defined(__CUDA_ARCH__)
-  asm("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-      : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]), "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3])
-      : "l"(p));
+  const ulonglong4_32a v = *reinterpret_cast<const ulonglong4_32a*>(p);
+  a[0] = (uint32_t)v.x; a[1] = (uint32_t)(v.x >> 32);
+  a[2] = (uint32_t)v.y; a[3] = (uint32_t)(v.y >> 32);
+  b[0] = (uint32_t)v.z; b[1] = (uint32_t)(v.z >> 32);
+  b[2] = (uint32_t)v.w; b[3] = (uint32_t)(v.w >> 32);
 #else
   ld16(p, a);
   ld16(p + 16, b);
