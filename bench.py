@@ -485,7 +485,7 @@ def measure_extra(a, g, ins_batches, dev, st, hbm_peak, peak_kind, T):
         torch.cuda.synchronize()
         return e0.elapsed_time(e1) / reps, r
 
-    kname = {"range": "k_range", "sum": "k_sum", "has": "k_has", "merge": "k_insert_thread",
+    kname = {"range": "k_range_ends+k_leaf_prefix+k_range_inner", "sum": "k_sum", "has": "k_has", "merge": "k_insert_thread",
              "merge_lane": "k_insert_lane",
              "merge_other": "k_merge_small+k_merge"}
     def roof(prof, p):

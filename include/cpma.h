@@ -205,8 +205,14 @@ int cpma_has_batch(const cpma_t* h, const uint64_t* d_keys, uint64_t q,
 /* Sec. 3 range_map(start, end, f) with f = (sum, count), batched: for every
  * i < q, d_sum[i] = sum of the keys x with d_lo[i] <= x < d_hi[i], modulo
  * 2^64, and d_count[i] = how many there are (both device uint64 arrays of q
- * entries).  lo >= hi gives 0 and 0.  All q queries run in one load-balanced
- * launch over (query, leaf) work items. */
+ * entries).  lo >= hi gives 0 and 0.  The queries' end leaves are
+ * decoded, the leaves between them walked in equal shares; when two or more
+ * queries together cover more leaves than the set has, every leaf is reduced
+ * once instead (12 bytes of scratch per leaf), and from a query per leaf on the
+ * walk of every leaf is kept at each 32nd byte (as much scratch as leaves) and
+ * a query looks up its two ends.  Without memory for either (budget, a stream
+ * being captured) the queries walk: same results.  The scratch is held by the
+ * handle and given back when an update or a query needs the memory. */
 int cpma_range_map(const cpma_t* h, const uint64_t* d_lo, const uint64_t* d_hi,
                    uint64_t q, uint64_t* d_sum, uint64_t* d_count,
                    cpma_stream_t stream);
@@ -217,8 +223,7 @@ int cpma_range_map(const cpma_t* h, const uint64_t* d_lo, const uint64_t* d_hi,
  * (all device uint64 arrays of q entries).  Length 1 gives the successor of
  * start (Sec. 3 search); start 0 and length 1 the minimum.  One prefix sum of
  * the leaves' element counts per call turns every query into a range of
- * global ranks; the ranks then run through the same load-balanced leaf walk
- * as cpma_range_map.  Errors: CPMA_EINVAL (null handle or array with q > 0),
+ * global ranks; the rest is as for cpma_range_map.  Errors: CPMA_EINVAL (null handle or array with q > 0),
  * CPMA_ENOMEM (scratch). */
 int cpma_range_map_length(const cpma_t* h, const uint64_t* d_start,
                           const uint64_t* d_length, uint64_t q, uint64_t* d_sum,
@@ -232,8 +237,8 @@ int cpma_range_map_length(const cpma_t* h, const uint64_t* d_start,
  * out_cap are not written; with d_out NULL or out_cap 0 only d_offsets is
  * computed, so a caller sizes d_out from d_offsets[q] and calls again.  Both
  * range ends are turned into global ranks (a prefix sum of the leaves'
- * element counts, then one leaf decode per end), and the leaves between them
- * are decoded by the load-balanced walk of cpma_range_map.  Errors:
+ * element counts, then one leaf search per end), and the leaves from the first
+ * to the last are decoded, shared evenly over the GPU.  Errors:
  * CPMA_EINVAL (null handle, d_offsets NULL, or d_lo / d_hi NULL with q > 0),
  * CPMA_ENOMEM. */
 int cpma_range_extract(const cpma_t* h, const uint64_t* d_lo, const uint64_t* d_hi,
@@ -249,9 +254,8 @@ int cpma_range_extract(const cpma_t* h, const uint64_t* d_lo, const uint64_t* d_
 /* Sec. 3 range_map(start, end, f) with f one of the CPMA_OP_* reductions over
  * a filter, batched: for every i < q, over the keys x with d_lo[i] <= x <
  * d_hi[i] and (x & mask) == value, d_out[i] = the reduction and d_count[i] =
- * how many keys passed (so mask/value filters give filter-counts).  Every
- * covered leaf is decoded; with CPMA_OP_SUM and mask = value = 0 this is
- * cpma_range_map.  Errors: CPMA_EINVAL (null handle or array with q > 0, op
+ * how many keys passed (so mask/value filters give filter-counts).  Runs as
+ * cpma_range_map, which it is with CPMA_OP_SUM and mask = value = 0.  Errors: CPMA_EINVAL (null handle or array with q > 0, op
  * not a CPMA_OP_*), CPMA_ENOMEM. */
 int cpma_range_reduce(const cpma_t* h, const uint64_t* d_lo, const uint64_t* d_hi,
                       uint64_t q, int op, uint64_t mask, uint64_t value,
@@ -334,9 +338,11 @@ int cpma_export_layout(const cpma_t* h, uint8_t* d_data, uint32_t* d_used,
 /* Pre-size the scratch that an update of up to max_batch keys (tagged != 0:
  * with request tags) and a range_map of up to max_queries queries use, so
  * that those calls do not allocate: the batch's sort, routing and merge
- * buffers, the redistribution buffers for the whole set plus the batch, and
- * spare leaf arrays for the resize the batch could cause (held until a
- * resize uses them, or until 64 updates in a row could not have resized).
+ * buffers, the redistribution buffers for the whole set plus the batch, the
+ * queries' prefix over the leaves (and marks inside them, when max_queries
+ * reaches the leaf count; both only if there is memory), and spare leaf arrays
+ * for the resize the batch could cause (held until a resize uses them, or until
+ * 64 updates in a row could not have resized).
  * Later updates that grow the set past these sizes reserve more before they
  * change anything.  With graphs on (cpma_use_graphs) it also sizes the
  * staging buffer of the padded batch.  Errors: CPMA_EINVAL (null handle,
