@@ -677,10 +677,10 @@ LT_HD void leaf_take_sum(const uint8_t* leafp, uint32_t u, uint64_t lo, uint64_t
     else if (taken < most) { s += v; taken++; }
   };
   take(k.val);
-  uint32_t p = 8;
+  uint32_t p = 8;  // the next group's byte
+  uint32_t raw[4];
+  ld16(leafp, raw);
   if (k.val < lo) {
-    uint32_t raw[4];
-    ld16(leafp, raw);
     const uint32_t p0 = skip_below(leafp, u, lo, k, below, raw);
     if (p0) p = p0;
   }
@@ -688,32 +688,41 @@ LT_HD void leaf_take_sum(const uint8_t* leafp, uint32_t u, uint64_t lo, uint64_t
   // while they fit; then the group that does not
   Held g;
   bool have = false;
-  for (; p < u && k.val < lo; p += 8) {
-    uint32_t w[4], t[4];
-    load_chunk(leafp, p & ~15u, u, w, t);
-    const bool hi8 = (p & 8u) != 0u;
-    g = Held{k, hi8 ? w[2] : w[0], hi8 ? w[3] : w[1], hi8 ? t[2] : t[0], hi8 ? t[3] : t[1]};
+  auto before = [&](uint32_t wa, uint32_t wb, uint32_t ta, uint32_t tb) {
+    g = Held{k, wa, wb, ta, tb};
     uint32_t T;
     uint64_t ss;
-    group_sum(g.wa, g.wb, g.ta, g.tb, k, T, ss);
+    group_sum(wa, wb, ta, tb, k, T, ss);
     have = k.val >= lo;
     if (!have) below += T;
+    p += 8;
+  };
+  for (uint32_t p0 = p & ~15u; p < u && k.val < lo; p0 += 16) {
+    uint32_t w[4], t[4];
+    next_chunk(leafp, p0, u, raw, w, t);
+    if (p0 == p) before(w[0], w[1], t[0], t[1]);
+    if (p < u && k.val < lo) before(w[2], w[3], t[2], t[3]);
   }
   if (have) group_visit(g.wa, g.wb, g.ta, g.tb, g.k, take);
   have = false;
-  for (; p < u && !have && taken < most; p += 8) {
-    uint32_t w[4], t[4];
-    load_chunk(leafp, p & ~15u, u, w, t);
-    const bool hi8 = (p & 8u) != 0u;
-    g = Held{k, hi8 ? w[2] : w[0], hi8 ? w[3] : w[1], hi8 ? t[2] : t[0], hi8 ? t[3] : t[1]};
+  auto within = [&](uint32_t wa, uint32_t wb, uint32_t ta, uint32_t tb) {
+    g = Held{k, wa, wb, ta, tb};
     uint32_t T;
     uint64_t ss;
-    group_sum(g.wa, g.wb, g.ta, g.tb, k, T, ss);
+    group_sum(wa, wb, ta, tb, k, T, ss);
     have = taken + T > most;
     if (!have) {
       s += T * g.k.val + ss;
       taken += T;
     }
+    p += 8;
+  };
+  if (p < u) ld16(leafp + (p & ~15u), raw);
+  for (uint32_t p0 = p & ~15u; p < u && !have && taken < most; p0 += 16) {
+    uint32_t w[4], t[4];
+    next_chunk(leafp, p0, u, raw, w, t);
+    if (p0 == p) within(w[0], w[1], t[0], t[1]);
+    if (p < u && !have && taken < most) within(w[2], w[3], t[2], t[3]);
   }
   if (have) group_visit(g.wa, g.wb, g.ta, g.tb, g.k, take);
 }
