@@ -76,7 +76,8 @@ struct Status {
                    // fix-up; not cleared at the start of a batch)
   ull bytes_total; // used bytes over all leaves, kept exact by the merge,
                    // redistribution and build kernels (not cleared either)
-  ull query_done;  // range queries: blocks done (the last one puts it back to 0)
+  ull query_done;  // range queries with the handle's scratch: blocks done (the
+                   // last one puts it back to 0)
 };
 
 constexpr ull kErrUnsorted = 1;   // a batch promised sorted was not

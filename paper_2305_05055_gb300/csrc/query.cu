@@ -603,7 +603,7 @@ __device__ __forceinline__ bool last_block(uint32_t* ticket) {
 constexpr uint64_t kEndsScan = 1024;  // queries at most: 16 items per thread
 struct EndsScan {
   uint64_t* off = nullptr;       // q + 1 entries; null: not here
-  ull* done = nullptr;           // Status::query_done
+  ull* done = nullptr;           // blocks done: 0 between calls
 };
 
 __device__ __forceinline__ void scan_ends(const EndsScan& z, const uint64_t* items, uint64_t q) {
@@ -1566,6 +1566,7 @@ struct RangeScratch {
   uint64_t *first, *items, *off;   // q, q, q + 1 entries
   uint64_t* partials = nullptr;    // given partials of the offset scan (else the handle's)
   uint64_t partials_cap = 0;
+  ull* done = nullptr;             // EndsScan::done (none with given scratch: it outlives a call)
 };
 
 int range_scratch(cpma* h, uint64_t q, RangeScratch* r) {
@@ -1577,15 +1578,18 @@ int range_scratch(cpma* h, uint64_t q, RangeScratch* r) {
   r->first = (uint64_t*)s.q_first.p;
   r->items = (uint64_t*)s.q_items.p;
   r->off = (uint64_t*)s.q_off.p;
+  r->done = &h->d_status->query_done;
   return CPMA_OK;
 }
 
-// Whether the ends' kernel leaves the offsets (scan_ends), and with what.
+// Whether the ends' kernel leaves the offsets (scan_ends), and with what.  Not
+// in the allocation-free call: it may overlap the handle's range calls, and
+// carries nothing over from one call to the next.
 EndsScan ends_scan(const cpma* h, const RangeScratch& r, uint64_t q) {
   EndsScan z;
-  if (few_queries(h, q) && q <= kEndsScan) {
+  if (r.done && few_queries(h, q) && q <= kEndsScan) {
     z.off = r.off;
-    z.done = &h->d_status->query_done;
+    z.done = r.done;
   }
   return z;
 }
