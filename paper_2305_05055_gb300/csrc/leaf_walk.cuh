@@ -429,13 +429,13 @@ LT_HD bool long_in(uint32_t a, uint32_t b, const uint32_t (&c)[4]) {
 }
 
 // The same for a leaf of m elements, whose bytes past u are zero; span: no two
-// of its elements lie this far apart (the next leaf's head less its own), which
+// of its elements lie further apart (the next leaf's head less its own), which
 // bounds its codes: below 2^21 they have at most 3 bytes, below 2^14 two, and
 // the planes of the others are left out for a warp of such leaves.
 LT_HD uint64_t leaf_sum(const uint8_t* leafp, uint32_t u, uint32_t m, uint64_t span) {
-  if (!any_lane(m > 256u || span > 1ull << 21)) {
+  if (!any_lane(m > 256u || span >= 1ull << 21)) {
     uint64_t s = 0;
-    if (any_lane(span > 1ull << 14)) sum_few<3>(leafp, u, m, s);
+    if (any_lane(span >= 1ull << 14)) sum_few<3>(leafp, u, m, s);
     else sum_few<2>(leafp, u, m, s);
     return s;
   }

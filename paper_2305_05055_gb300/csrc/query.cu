@@ -454,8 +454,9 @@ struct Leaves {
   uint32_t LB;
 };
 
-// No two elements of leaf j lie this far apart: the next leaf's head (an empty
-// one's is that of the next with elements, or 2^64 - 1) is above them all.
+// No two elements of leaf j lie further apart: the next leaf's head (an empty
+// one's is that of the next with elements, or 2^64 - 1, which may itself be the
+// last element of j) is not below any of them.
 __device__ __forceinline__ uint64_t leaf_span(const uint64_t* __restrict__ heads, uint64_t L,
                                               uint64_t j) {
   return j + 1 < L ? __ldg(heads + j + 1) - __ldg(heads + j) : ~0ull;
@@ -495,7 +496,7 @@ struct Reduce {
       c += m;
     } else {
       if (OP == CPMA_OP_SUM && !((mask | value) >> 32) &&
-          !leafwalk::any_lane(leaf_span(t.heads, t.L, j) > 1ull << 28)) {
+          !leafwalk::any_lane(leaf_span(t.heads, t.L, j) >= 1ull << 28)) {
         leafwalk::leaf_masked_sum(t.data + j * t.LB, u, (uint32_t)mask, (uint32_t)value, r, c);
         return;
       }

@@ -88,8 +88,9 @@ def sums(lw, p, u, keys):
     want, m = sum(keys) & M64, len(keys)
     short = all(b - a < 1 << 28 for a, b in zip(keys, keys[1:]))
     few = lw.lw_sum(p, u, m, 2, M64) if m <= 256 else want
-    span = keys[-1] - keys[0] + 1   # the least the next leaf's head can leave
-    return (lw.lw_sum(p, u, m, 0, M64) == lw.lw_sum(p, u, m, 0, span) == want and
+    span = keys[-1] - keys[0]   # the least: 2^64 - 1 in this leaf, the next one empty
+    return (lw.lw_sum(p, u, m, 0, M64) == lw.lw_sum(p, u, m, 0, span) ==
+            lw.lw_sum(p, u, m, 0, span + 1) == want and
             lw.lw_sum(p, u, m, 1, 0) == want and
             (few if short else want) == want and
             lw.lw_sum(p, u, m, 3, 0) == (want if short else M64))
@@ -114,6 +115,18 @@ def test_leaf_sum_by_number_of_codes(lw, m):
         at = -leaf.ctypes.data % 16
         leaf[at:at + 2048] = buf[:2048]
         assert sums(lw, leaf[at:].ctypes.data, u, keys)
+
+
+@pytest.mark.parametrize("d", [1 << 7, 1 << 14, 1 << 21, 1 << 28])
+def test_leaf_sum_of_two_elements_a_span_apart(lw, d):
+    # the second is 2^64 - 1 and the next leaf empty: its head says d as well
+    for gap in (d - 1, d):
+        keys = [M64 - gap, M64]
+        buf, u = oracle.leaf_encode(np.array(keys, dtype=np.uint64), 256)
+        leaf = np.zeros(256 + 64, dtype=np.uint8)
+        at = -leaf.ctypes.data % 16
+        leaf[at:at + 256] = buf[:256]
+        assert lw.lw_sum(leaf[at:].ctypes.data, u, 2, 0, gap) == sum(keys) & M64
 
 
 @pytest.mark.parametrize("LB", [256, 512, 2048])
