@@ -11,6 +11,10 @@
 //    prefix over the leaves, and a query takes the difference at its two ends
 //    (k_leaf_prefix, k_tile_scan, k_range_inner): each leaf is then decoded
 //    once however often the queries overlap.
+//    From one query per leaf on, every leaf is walked once with its state kept
+//    at every 32nd byte, and a query looks up its two ends (k_marks,
+//    k_range_marked).  A few thousand queries and fewer take eight lanes per
+//    leaf instead of one.
 //  sum (App. A sum()): every leaf once.
 //  map_range_length (App. A: f on at most `length` elements from the first
 //    key >= start): a prefix sum of the leaves' element counts gives the leaf

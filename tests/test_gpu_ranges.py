@@ -1,7 +1,8 @@
 """Range queries over byte-code leaves, bit for bit against the plain sorted
 set: queries that together cover more leaves than the set has (the leaves are
 then reduced once and differenced) and fewer (walked), around that line, over
-codes of one to ten bytes, and with leaves that deletions left empty."""
+codes of one to ten bytes, and with leaves that deletions left empty; few
+queries (eight lanes per leaf), at least one per leaf (marks inside the leaves)."""
 import ctypes as C
 
 import numpy as np
