@@ -9,7 +9,7 @@
 //    lane of equal shares -- or, when the queries together cover more leaves
 //    than the set has, every leaf is reduced once, those reductions become a
 //    prefix over the leaves, and a query takes the difference at its two ends
-//    (k_leaf_prefix, k_tile_scan, k_range_inner): each leaf is then decoded
+//    (k_leaf_prefix, k_range_inner): each leaf is then decoded
 //    once however often the queries overlap.
 //    From one query per leaf on, every leaf is walked once with its state kept
 //    at every 32nd byte, and a query looks up its two ends (k_marks,
