@@ -4112,13 +4112,14 @@ int run_update(cpma* h, const uint64_t* d_keys, uint64_t k, int sorted, int is_d
   uint64_t t_slack = 0;
   const uint64_t delta = hs.delta;
   const uint64_t n_after = is_delete ? h->n - delta : h->n + delta;
-  // empty leaves: made by this batch's merges, or left when the last head
-  // fix-up ran.  A window redistribution empties none while each leaf gets
-  // about S/W >= rho_leaf LB > 10 bytes, more than one code; with a lower
-  // bound below that, a leaf left pending by a delete may be rewritten empty.
-  h->may_have_empty = hs.nempty || hs.empties ||
-                      (is_delete && hs.npend &&
-                       (uint64_t)h->cfg.rho_leaf * h->cfg.leaf_bytes <= 20000);
+  // empty leaves: made by this batch's merges, left when the last head fix-up
+  // ran, or made by the redistribution below.  That encodes every source leaf's
+  // head but the window's first as a code, so a window of W leaves and B used
+  // bytes is a stream of S > B - 7 W, cut every S / W bytes: a leaf is sure of an
+  // element while S / W is at least a code's 10 bytes: from a lower bound of 17
+  // bytes a leaf on (20 here).
+  const bool sparse = (uint64_t)h->cfg.rho_leaf * h->cfg.leaf_bytes <= 20000;
+  h->may_have_empty = hs.nempty || hs.empties || (sparse && (hs.nviol || hs.npend));
 
   // ---- pending leaves: materialise their merged elements ----
   if (hs.npend) {
