@@ -486,6 +486,8 @@ int cpma_clone(const cpma_t* src, cpma_t** out, cpma_stream_t stream) {
   const uint64_t L = src->L, LB = src->cfg.leaf_bytes;
   Arrays a;
   int rc = alloc_arrays(h, L, L * LB, &a, st);
+  if (rc == CPMA_ENOMEM && release_leaf_prefix(const_cast<cpma*>(src)))
+    rc = alloc_arrays(h, L, L * LB, &a, st);
   if (rc != CPMA_OK) {
     release_all(h);
     delete h;
@@ -555,6 +557,7 @@ int cpma_sort_batch(cpma_t* h, const uint64_t* d_keys, const uint32_t* d_tags, u
   cudaStream_t st = (cudaStream_t)stream;
   const uint64_t* u = nullptr;
   const uint32_t* ut = nullptr;
+  CPMA_TRY(with_query_room(h, [&] { return sort_scratch(h, k, d_tags != nullptr); }));
   if (d_tags) CPMA_TRY(sort_pairs(h, d_keys, d_tags, k, &u, &ut, st));
   else CPMA_TRY(sort_keys(h, d_keys, k, &u, st));
   CPMA_CUDA(cudaMemcpyAsync(d_keys_out, u, k * 8, cudaMemcpyDeviceToDevice, st));
@@ -677,13 +680,16 @@ int cpma_stats(const cpma_t* h, uint64_t* launches) {
 int cpma_reserve(cpma_t* h, uint64_t max_batch, uint64_t max_queries, int tagged,
                  cpma_stream_t stream) {
   if (!h) return CPMA_EINVAL;
-  CPMA_TRY(reserve(h, max_batch, tagged, (cudaStream_t)stream));
-  if (max_queries) {
+  CPMA_TRY(with_query_room(h, [&] {
+    CPMA_TRY(reserve(h, max_batch, tagged, (cudaStream_t)stream));
+    if (!max_queries) return (int)CPMA_OK;
     Scratch& s = h->s;
     CPMA_TRY(ensure(h, s.q_first, max_queries * 8));
     CPMA_TRY(ensure(h, s.q_items, (max_queries + 1) * 8));
     CPMA_TRY(ensure(h, s.q_off, (max_queries + 1) * 8));
-    CPMA_TRY(ensure(h, s.partials_q, (size_t)(2 * h->num_sms + 2) * 8));
+    return ensure(h, s.partials_q, (size_t)(2 * h->num_sms + 2) * 8);
+  }));
+  if (max_queries) {
     // range_map runs without its leaf prefix when there is no room for it
     if (max_queries > 1 && !h->cfg.codec) {
       const int rc = reserve_leaf_prefix(h, max_queries);
@@ -730,7 +736,10 @@ int cpma_profile(cpma_t* h, int enable) {
   if (cudaDeviceSynchronize() != cudaSuccess) return CPMA_ECUDA;
   prof_resolve(h);
   Prof& p = h->prof;
-  if (!p.d_bytes) CPMA_TRY(dev_alloc(h, (void**)&p.d_bytes, sizeof(unsigned long long) * PH_N, nullptr));
+  if (!p.d_bytes)
+    CPMA_TRY(with_query_room(h, [&] {
+      return dev_alloc(h, (void**)&p.d_bytes, sizeof(unsigned long long) * PH_N, nullptr);
+    }));
   CPMA_CUDA(cudaMemset(p.d_bytes, 0, sizeof(unsigned long long) * PH_N));
   for (int i = 0; i < PH_N; i++) { p.ms[i] = 0; p.calls[i] = 0; p.host_bytes[i] = 0; }
   p.on = enable != 0;

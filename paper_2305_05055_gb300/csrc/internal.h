@@ -311,6 +311,15 @@ int run_range_noalloc(const cpma* h, const uint64_t* lo, const uint64_t* hi, uin
 int reserve_leaf_prefix(cpma* h, uint64_t q);
 bool release_leaf_prefix(cpma* h);
 
+// take() (which changes nothing when it runs out of memory), once more without
+// the range queries' prefix and marks if it does: whatever else a handle needs
+// memory for goes before them.
+template <class F>
+int with_query_room(cpma* h, F&& take) {
+  const int rc = take();
+  return rc == CPMA_ENOMEM && release_leaf_prefix(h) ? take() : rc;
+}
+
 int check_cuda(cudaError_t e);
 // Waits for the stream with the status block brought to h->h_status; d_delta
 // (nullable, device) receives the number of keys changed unless there is an error.

@@ -1481,12 +1481,9 @@ int query_grid(const cpma* h, uint64_t q, int block, uint64_t per_sm) {
 // Per leaf a reduction and a count, per tile both again.
 size_t leaf_prefix_bytes(uint64_t L) { return L * 12 + (L + kT - 1) / kT * 16 + 4; }
 
-// Grows a query buffer; the leaf prefix, which the queries can do without, is
-// given back when there is no room for it.
+// Grows a query buffer.
 int ensure_query(cpma* h, Buf& b, size_t bytes) {
-  int rc = ensure(h, b, bytes);
-  if (rc == CPMA_ENOMEM && release_leaf_prefix(h)) rc = ensure(h, b, bytes);
-  return rc;
+  return with_query_room(h, [&] { return ensure(h, b, bytes); });
 }
 
 // The leaf prefix's memory for this call, or none (the inner leaves are then

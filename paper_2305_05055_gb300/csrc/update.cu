@@ -2503,6 +2503,7 @@ int ensure_bits(cpma* h, cudaStream_t st, Levels* lv) {
   uint64_t words = 0;
   *lv = levels_of(h->L, H, &words);
   if (words != h->bits_words) {
+    h->bits_words = 0;
     CPMA_TRY(ensure(h, h->s.bits, words * 4));
     CPMA_CUDA(cudaMemsetAsync(h->s.bits.p, 0, words * 4, st));
     h->bits_words = words;
@@ -3852,7 +3853,8 @@ void graph_cache_free(cpma* h) {
 
 // R14: apply the batch by merging it with every element and building the
 // result like the constructor.  Nothing is replaced before the new arrays
-// are complete, so a rejected batch leaves the set unchanged.
+// are complete, so a rejected batch leaves the set unchanged (and one refused
+// for want of memory can be run again).
 int run_rebuild(cpma* h, const uint64_t* d_keys, uint64_t k, int sorted, int is_delete,
                 uint64_t* d_delta, cudaStream_t st) {
   Status* ds = h->d_status;
@@ -3922,9 +3924,7 @@ int reserve(cpma* h, uint64_t max_batch, int tagged, cudaStream_t st) {
   if (max_batch >= (1ull << 31)) return CPMA_EINVAL;
   if (max_batch == 0) return CPMA_OK;
   // everything an insert of max_batch keys reserves, a growing resize included
-  int rc = reserve_update(h, max_batch, 0, st, true);
-  if (rc == CPMA_ENOMEM && release_leaf_prefix(h)) rc = reserve_update(h, max_batch, 0, st, true);
-  CPMA_TRY(rc);
+  CPMA_TRY(reserve_update(h, max_batch, 0, st, true));
   CPMA_TRY(front_scratch(h, max_batch, tagged != 0, st));
   if (!tagged && h->point_max) CPMA_TRY(point_scratch(h, std::min(max_batch, h->point_max), st));
   if (h->graph_max_batch && !tagged) {
@@ -4053,10 +4053,11 @@ int run_update(cpma* h, const uint64_t* d_keys, uint64_t k, int sorted, int is_d
   if (k >= (1ull << 31)) return CPMA_EINVAL;
   if (h->cfg.rebuild_pm && !tags &&
       (unsigned __int128)1000 * k >= (unsigned __int128)h->cfg.rebuild_pm * h->n)
-    return run_rebuild(h, d_keys, k, sorted, is_delete, d_delta, st);
+    return with_query_room(
+        h, [&] { return run_rebuild(h, d_keys, k, sorted, is_delete, d_delta, st); });
   Scratch& s = h->s;
   const bool graph = k <= h->graph_max_batch && !tags && graph_bucket(k) < (1ull << 31);
-  auto take = [&] {
+  int rc = with_query_room(h, [&] {
     int e = reserve_update(h, k, is_delete, st, false);
     if (e == CPMA_OK && graph) {
       e = ensure(h, s.stage, graph_bucket(k) * 8, st);
@@ -4065,10 +4066,7 @@ int run_update(cpma* h, const uint64_t* d_keys, uint64_t k, int sorted, int is_d
       e = front_scratch(h, k, tags != nullptr, st);
     }
     return e;
-  };
-  int rc = take();
-  // the range queries' prefix makes room first: they run without it
-  if (rc == CPMA_ENOMEM && release_leaf_prefix(h)) rc = take();
+  });
   if (rc == CPMA_ENOMEM) {
     // refused before any change; give back the scratch grown so far, so
     // that a smaller batch after this one starts from the structure alone
@@ -4079,7 +4077,9 @@ int run_update(cpma* h, const uint64_t* d_keys, uint64_t k, int sorted, int is_d
   // the point path; the batch algorithm below when its scratch cannot be
   // had within the memory budget, or when some touched leaf cannot change
   // in place (nothing has been written then)
-  const int prc = point_ok(h, k, is_delete, tags) ? point_scratch(h, k, st) : CPMA_ENOMEM;
+  const int prc = point_ok(h, k, is_delete, tags)
+                      ? with_query_room(h, [&] { return point_scratch(h, k, st); })
+                      : CPMA_ENOMEM;
   if (prc != CPMA_OK && prc != CPMA_ENOMEM) return prc;
   if (prc == CPMA_OK) {
     bool fb = false;
@@ -4237,6 +4237,13 @@ int build_from_sorted(cpma* h, const uint64_t* x, uint64_t n, cudaStream_t st) {
   Arrays na;
   CPMA_TRY(alloc_arrays(h, L, L * LB, &na, st));
   int rc = ensure(h, s.dstart, (L + 1) * 8);
+  // (what the update path needs for these leaves, while a refusal changes nothing)
+  uint64_t words = 0;
+  levels_of(L, ceil_log2(L), &words);
+  if (rc == CPMA_OK && s.bits.cap < words * 4) {
+    h->bits_words = 0;
+    rc = ensure(h, s.bits, words * 4);
+  }
   // the byte total and the count of empty leaves restart with the new leaves
   if (rc == CPMA_OK) rc = check_cuda(cudaMemsetAsync(&h->d_status->bytes_total, 0, 8, st));
   if (rc == CPMA_OK) rc = check_cuda(cudaMemsetAsync(&h->d_status->empties, 0, 8, st));
@@ -4255,6 +4262,8 @@ int build_from_sorted(cpma* h, const uint64_t* x, uint64_t n, cudaStream_t st) {
   }
   if (rc == CPMA_OK) rc = sync_status(h, st);
   if (rc == CPMA_OK && h->h_status->err) rc = CPMA_EINTERNAL;
+  if (rc == CPMA_OK && h->h_status->nempty)
+    rc = ensure(h, s.fh, (L + kFHTile - 1) / kFHTile * sizeof(FHTile));
   if (rc != CPMA_OK) {
     cudaStreamSynchronize(st);
     free_arrays(h, &na);
