@@ -210,9 +210,10 @@ int cpma_has_batch(const cpma_t* h, const uint64_t* d_keys, uint64_t q,
  * queries together cover more leaves than the set has, every leaf is reduced
  * once instead (12 bytes of scratch per leaf), and from a query per leaf on the
  * walk of every leaf is kept at each 32nd byte (as much scratch as leaves) and
- * a query looks up its two ends.  Without memory for either (budget, a stream
- * being captured) the queries walk: same results.  The scratch is held by the
- * handle and given back when an update or a query needs the memory. */
+ * a query looks up its two ends.  Without memory for either (budget, less than
+ * twice as much free on the device, a stream being captured) the queries walk:
+ * same results.  The scratch is held by the handle and given back when another
+ * call on it needs the memory, or by cpma_set_mem_budget. */
 int cpma_range_map(const cpma_t* h, const uint64_t* d_lo, const uint64_t* d_hi,
                    uint64_t q, uint64_t* d_sum, uint64_t* d_count,
                    cpma_stream_t stream);
@@ -316,8 +317,11 @@ int cpma_mem_held(const cpma_t* h, uint64_t* out);
  * arrays). */
 int cpma_mem_peak(const cpma_t* h, uint64_t* out);
 
-/* Change the memory budget of a live handle (0 = no cap).  Memory already
- * held is kept; the cap applies to the next allocations. */
+/* Change the memory budget of a live handle (0 = no cap).  The cap applies to
+ * the next allocations; memory already held is kept, except that a budget below
+ * it gives back the range queries' prefix and marks (cpma_range_map), which
+ * synchronises the device.  So a budget of 1 byte followed by the old one frees
+ * what queries took for their speed. */
 int cpma_set_mem_budget(cpma_t* h, uint64_t bytes);
 
 /* For tests of the bounded wait (no counterpart in the paper): poll_limit

@@ -649,6 +649,8 @@ int cpma_mem_peak(const cpma_t* h, uint64_t* out) {
 int cpma_set_mem_budget(cpma_t* h, uint64_t bytes) {
   if (!h) return CPMA_EINVAL;
   h->cfg.mem_budget_bytes = bytes;
+  // what the range queries can do without goes first
+  if (bytes && h->mem_held > bytes) release_leaf_prefix(h);
   return CPMA_OK;
 }
 

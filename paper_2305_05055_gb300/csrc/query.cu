@@ -1491,7 +1491,8 @@ int ensure_query(cpma* h, Buf& b, size_t bytes) {
 // memory budget does without, and so does a stream that is being captured (a
 // graph would keep the address, and the memory may move with the set's size).
 // A set that has been updated holds it already: the redistribution's element
-// buffer, which only an update uses, and none may overlap a query.
+// buffer, which only an update uses, and none may overlap a query.  A budget
+// below what the handle holds (cpma_set_mem_budget) gives it back.
 //
 // The rule of the kernels: the prefix is taken when the inner leaves of all
 // queries number more than the set's leaves.  Both forms decode a leaf in the
@@ -1505,6 +1506,16 @@ void* prefix_memory(cpma* h, Buf& b, size_t need, cudaStream_t st) {
     return nullptr;
   }
   if (h->s.E.cap >= need) return h->s.E.p;
+  // Memory that a query takes of its own accord is no other handle's or
+  // allocator's to get back: at most half of what the device has free.
+  if (b.cap < need && !h->cfg.alloc) {
+    size_t free_bytes = 0, all = 0;
+    if (cudaMemGetInfo(&free_bytes, &all) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    if (need > (free_bytes + b.cap) / 2) return nullptr;
+  }
   return ensure(h, b, need) == CPMA_OK ? b.p : nullptr;
 }
 

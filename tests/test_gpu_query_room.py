@@ -119,3 +119,45 @@ def test_clone_of_a_set_that_holds_marks():
         assert torch.equal(x, y)
     del c, g
     assert not held
+
+
+def test_a_lower_budget_gives_the_queries_memory_back():
+    base = W.uniform_keys(46, N, bits=40)
+    p, g = oracle.PlainSet(base), cp.CPMA(T(base), leaf_bytes=512)
+    q = 2 * g.leaves()
+    lo, hi, _ = W.range_queries_by_rank(p.S, 47, q, 1, 50)
+    alone = g.mem_held()
+    want = p.range_map(lo, hi)
+    for rnd in range(2):
+        for got, w in zip(g.range_map(T(lo), T(hi)), want):
+            assert np.array_equal(cp.to_u64(got), w)
+        held = g.mem_held()
+        assert held - alone > query_scratch(q) + 4096
+        g.set_mem_budget(held)                   # not below: kept
+        assert g.mem_held() == held
+        g.set_mem_budget(1)
+        assert g.mem_held() - alone <= query_scratch(q)
+        g.set_mem_budget(0)
+
+
+def test_a_query_leaves_half_of_the_free_memory():
+    # all but a few MB of the device taken: the marks (some 300 MB) are not
+    base = W.uniform_keys(48, 40_000_000, bits=40)
+    g = cp.CPMA(T(base), leaf_bytes=512)
+    L = g.leaves()
+    lo = torch.arange(L + 1, dtype=torch.int64, device="cuda") << 18
+    hi = lo + (1 << 20)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    marks = L * 512
+    free = torch.cuda.mem_get_info()[0]
+    taken = torch.empty(free - marks - marks // 2, dtype=torch.uint8, device="cuda")
+    before = g.mem_held()
+    want = g.range_map(lo, hi)
+    assert g.mem_held() - before < marks // 2
+    del taken
+    torch.cuda.empty_cache()
+    got = g.range_map(lo, hi)
+    assert g.mem_held() - before > marks
+    for a, b in zip(got, want):
+        assert torch.equal(a, b)
