@@ -852,8 +852,11 @@ int sort_scratch(cpma* h, uint64_t k, bool vals) {
   if (k <= (uint64_t)kTile) return CPMA_OK;
   CPMA_TRY(ensure(h, h->s.keysB, k * 8));
   if (vals) CPMA_TRY(ensure(h, h->s.valsB, k * 4));
-  const uint32_t G = vals ? pass_blocks<true>(h, k) : pass_blocks<false>(h, k);
-  return ensure(h, h->s.hist, ctl_bytes() + (size_t)G * 256 * 4);
+  // (fewer keys may take more blocks, and keys alone more than keys with tags:
+  // room for all that a reservation for k covers)
+  const uint64_t most = std::min<uint64_t>(
+      (k + kTile - 1) / kTile, (uint64_t)h->num_sms * (uint64_t)scatter_blocks_per_sm<false>());
+  return ensure(h, h->s.hist, ctl_bytes() + (size_t)most * 256 * 4);
 }
 
 template <bool VALS>
