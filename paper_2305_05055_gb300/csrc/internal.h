@@ -15,8 +15,9 @@ typedef unsigned long long ull;
 // serialisation (launch_pdl) may be scheduled while the kernel before it in
 // the stream still runs.  pdl_wait() returns once that kernel has completed
 // and its memory operations are visible (at once when the launch carried no
-// such dependency), so a kernel calls it before reading anything its
-// predecessor wrote -- and every kernel so launched calls it, so that its
+// such dependency), so a kernel calls it before it reads anything its
+// predecessor wrote or writes anything a predecessor may still use (scratch
+// buffers are shared) -- and every kernel so launched calls it, so that its
 // own completion implies its predecessors'.  pdl_launch() lets the next
 // kernel be scheduled.
 #if defined(__CUDACC__)

@@ -707,9 +707,9 @@ __global__ void __launch_bounds__(kT) k_length_ends(const uint64_t* __restrict__
                                                     uint64_t* __restrict__ items,
                                                     uint64_t* __restrict__ sum,
                                                     uint64_t* __restrict__ count, uint32_t* ticket, ull* prof) {
-  if (ticket && gtid() == 0) *ticket = 0;
   pdl_wait();
   pdl_launch();
+  if (ticket && gtid() == 0) *ticket = 0;
   __shared__ uint64_t s_s[kT];
   __shared__ uint32_t s_leaf[kT], s_q[kT], s_k[kT];
   __shared__ uint32_t s_n;
@@ -771,9 +771,9 @@ __global__ void __launch_bounds__(kT) k_length_ends_team(
     const uint64_t* __restrict__ start, const uint64_t* __restrict__ length, uint64_t q, Leaves t,
     const uint64_t* __restrict__ P, uint64_t* __restrict__ first, uint64_t* __restrict__ items,
     uint64_t* __restrict__ sum, uint64_t* __restrict__ count, uint32_t* ticket, EndsScan z, ull* prof) {
-  if (ticket && gtid() == 0) *ticket = 0;
   pdl_wait();
   pdl_launch();
+  if (ticket && gtid() == 0) *ticket = 0;
   ull nbytes = 0;
   const uint64_t n = P[t.L];
   const unsigned tl = team_lane(), team = lane_id() / kTeam;
