@@ -402,11 +402,10 @@ __global__ void __launch_bounds__(kT) k_digit_scan(Pass a, uint32_t G) {
   if (threadIdx.x == 0) a.ctl->tot[blockIdx.x] = carry;
 }
 
-// Partition of the tile by digit with no order among equal digits: one
-// atomic per key.
-template <bool VALS>
+// Partition of the tile by digit with no order among equal digits (keys
+// alone): one atomic per key.
 __device__ __forceinline__ void tile_rank_any(const uint64_t (&key)[kItems], uint32_t nvalid,
-                                              int shift, TileSmemT<VALS>& sm) {
+                                              int shift, TileSmemT<false>& sm) {
   const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
   uint32_t* cnt = sm.wcnt[0];
   cnt[threadIdx.x] = 0;
@@ -435,6 +434,7 @@ __device__ __forceinline__ void tile_rank_any(const uint64_t (&key)[kItems], uin
 // the block's earlier keys of every digit.
 template <bool VALS, bool STABLE>
 __global__ void __launch_bounds__(kT, 3) k_digit_scatter(Pass a) {
+  static_assert(STABLE || !VALS, "tags move stably");
   extern __shared__ __align__(16) uint8_t smem_raw[];
   TileSmemT<VALS>& sm = *reinterpret_cast<TileSmemT<VALS>*>(smem_raw);
   __shared__ uint32_t s_off[256];  // where the tile's keys of a digit go, less their tile index
@@ -467,7 +467,7 @@ __global__ void __launch_bounds__(kT, 3) k_digit_scatter(Pass a) {
       else val[j] = 0u;
     }
     if constexpr (STABLE) tile_rank<VALS>(key, val, nvalid, io.shift, sm);
-    else tile_rank_any<VALS>(key, nvalid, io.shift, sm);
+    else tile_rank_any(key, nvalid, io.shift, sm);
     s_off[d] = run - sm.dstart[d];
     run += (d < 255 ? sm.dstart[d + 1] : nvalid) - sm.dstart[d];
     __syncthreads();
@@ -770,7 +770,6 @@ __global__ void __launch_bounds__(kBitT) k_sort_bitonic(const uint64_t* __restri
 // below it and the equal keys before it, and the sum of their counts (a
 // shuffle reduction) is where the key (and its tag) goes.
 constexpr int kRankT = 256;
-template <bool VALS>
 __global__ void __launch_bounds__(kRankT) k_sort_rank(const uint64_t* __restrict__ in,
                                                       uint64_t* __restrict__ out,
                                                       const uint32_t* __restrict__ vin,
@@ -797,7 +796,7 @@ __global__ void __launch_bounds__(kRankT) k_sort_rank(const uint64_t* __restrict
   for (uint32_t o = 1; o < P; o <<= 1) r += __shfl_xor_sync(FULL, r, o);
   if (valid && part == 0) {
     out[r] = x;
-    if constexpr (VALS) vout[r] = vin[i];
+    vout[r] = vin[i];
   }
 }
 
@@ -817,8 +816,9 @@ void sort_attrs() {
   const int smem = (int)sizeof(TileSmemT<VALS>);
   cudaFuncSetAttribute(k_digit_scatter<VALS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        smem);
-  cudaFuncSetAttribute(k_digit_scatter<VALS, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       smem);
+  if constexpr (!VALS)
+    cudaFuncSetAttribute(k_digit_scatter<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         smem);
   cudaFuncSetAttribute(k_bucket_sort<VALS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        (int)sizeof(FinishSmem<VALS>));
   cudaFuncSetAttribute(k_window_sort, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -876,8 +876,9 @@ int digit_pass(cpma* h, Pass a, uint32_t G, int p, bool stable, cudaStream_t st)
   a.p = p;
   CPMA_CUDA(launch_pdl(k_digit_count, G, kT, 0, st, a));
   CPMA_CUDA(launch_pdl(k_digit_scan, 256, kT, 0, st, a, G));
-  CPMA_CUDA(stable ? launch_pdl(k_digit_scatter<VALS, true>, G, kT, smem, st, a)
-                   : launch_pdl(k_digit_scatter<VALS, false>, G, kT, smem, st, a));
+  if constexpr (VALS) stable = true;
+  CPMA_CUDA(launch_pdl(stable ? k_digit_scatter<VALS, true> : k_digit_scatter<false, false>, G, kT,
+                       smem, st, a));
   h->launches += 3;
   return CPMA_OK;
 }
@@ -916,12 +917,12 @@ int sort_impl(cpma* h, const uint64_t* d_in, const uint32_t* v_in, uint64_t k, c
     return check_cuda(cudaGetLastError());
   }
   if (k <= (uint64_t)kTile) {
-    prof_add_bytes(h, PH_SORT, (VALS ? 24ull : 16ull) * k);
+    prof_add_bytes(h, PH_SORT, 24ull * k);
     // threads per key: a power of two keeping each thread's share at 256 keys
     uint32_t P = 1;
     while (P < 32 && k > 256ull * P) P <<= 1;
     const uint32_t nb = (uint32_t)((k * P + kRankT - 1) / kRankT);
-    k_sort_rank<VALS><<<nb, kRankT, k * 8, st>>>(d_in, A, v_in, VA, (uint32_t)k, P);
+    k_sort_rank<<<nb, kRankT, k * 8, st>>>(d_in, A, v_in, VA, (uint32_t)k, P);
     h->launches++;
     *out = A;
     if (vout) *vout = VA;

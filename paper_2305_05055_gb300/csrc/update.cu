@@ -2840,8 +2840,8 @@ __global__ void __launch_bounds__(kT) k_rebuild_scatter(const uint64_t* __restri
 // copy, element costs or their prefix in memory: one pass adds up the distinct
 // keys and the bytes of their stream per block (k_build_sum), which give the
 // leaf count; a second one prefixes the bytes again tile by tile and finds the
-// key each leaf starts at (k_build_cuts); a warp per leaf then writes it
-// (k_build_encode).  A repeat costs no bytes and is skipped wherever it falls.
+// key each leaf starts at (k_build_cuts); a thread per leaf (a warp when they
+// are few) then writes it (k_build_encode).  A repeat costs no bytes and is skipped wherever it falls.
 // Two reads of the keys and one of them with the leaves' bytes out; flags,
 // their scan, a compaction, costs, their scan and a search per leaf took 820
 // us of 3e7 keys, these three 335 us.
@@ -3739,8 +3739,7 @@ int run_front_graph(cpma* h, const uint64_t* d_keys, uint64_t k, int sorted, int
 // May an update take the point path?  Untagged updates of 1 .. point_max
 // keys on a non-empty set of byte-code leaves of at most 512 bytes (the
 // lane-granular insert's buffer, the staging slot), unless a test of the
-// bounded waits is set up (those waits are in the batch algorithm's sort and
-// routing).
+// bounded waits is set up (they are in the batch algorithm's routing).
 bool point_ok(const cpma* h, uint64_t k, int is_delete, const uint32_t* tags) {
   return !tags && k >= 1 &&
          k <= std::min<uint64_t>(h->point_max, is_delete ? kPointDelMax : kPointMax) &&
