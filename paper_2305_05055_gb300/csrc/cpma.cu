@@ -5,6 +5,9 @@
 #include <cstring>
 #include <mutex>
 #include <new>
+#include <utility>
+
+#include <cuda.h>
 
 #include "internal.h"
 
@@ -283,19 +286,57 @@ void prof_push(const cpma* hc, const Prof::Rec* recs, int n, const unsigned long
 
 namespace {
 
-// Pinned status blocks of destroyed handles, kept for the next ones (pinning
-// and unpinning one took 250 us of a build of 3e7 keys): at most kPinned of
-// them, 256 bytes each; more go back at once.  A block belongs to no device,
-// stream or handle while it is here.
+// The current context's id, never used twice in a process (a reset device's next
+// context has another one); 0 when the driver does not say.
+uint64_t context_id() {
+  typedef CUresult (*Current)(CUcontext*);
+  typedef CUresult (*Id)(CUcontext, unsigned long long*);
+  static const Current current = (Current)[] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult r;
+    if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &f, 12000, cudaEnableDefault, &r) !=
+        cudaSuccess)
+      cudaGetLastError();
+    return f;
+  }();
+  static const Id id = (Id)[] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult r;
+    if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &f, 12000, cudaEnableDefault, &r) !=
+        cudaSuccess)
+      cudaGetLastError();
+    return f;
+  }();
+  CUcontext c = nullptr;
+  unsigned long long v = 0;
+  if (!current || !id || current(&c) != CUDA_SUCCESS || !c || id(c, &v) != CUDA_SUCCESS) return 0;
+  return v;
+}
+
+// Pinned status blocks of destroyed handles, kept for the next ones of the same
+// context (pinning and unpinning one took 250 us of a build of 3e7 keys): at most
+// kPinned of them, 256 bytes each; more go back at once.  cudaDeviceReset ends
+// the context and its pinned memory with it, so a block is taken again only in
+// the context it was pinned in; one of another context makes way when the pool is
+// full.
 constexpr int kPinned = 64;
+struct PinnedStatus {
+  Status* p;
+  uint64_t ctx;
+};
 std::mutex g_pinned_mu;
-Status* g_pinned[kPinned];
+PinnedStatus g_pinned[kPinned];
 int g_npinned = 0;
 
-Status* take_pinned() {
-  {
+Status* take_pinned(uint64_t ctx) {
+  if (ctx) {
     std::lock_guard<std::mutex> lock(g_pinned_mu);
-    if (g_npinned) return g_pinned[--g_npinned];
+    for (int i = g_npinned; i-- > 0;)
+      if (g_pinned[i].ctx == ctx) {
+        Status* p = g_pinned[i].p;
+        g_pinned[i] = g_pinned[--g_npinned];
+        return p;
+      }
   }
   void* p = nullptr;
   if (cudaHostAlloc(&p, sizeof(Status), cudaHostAllocPortable) != cudaSuccess) {
@@ -305,16 +346,22 @@ Status* take_pinned() {
   return static_cast<Status*>(p);
 }
 
-void give_pinned(Status* p) {
+void give_pinned(Status* p, uint64_t ctx) {
   if (!p) return;
-  {
+  if (ctx) {
     std::lock_guard<std::mutex> lock(g_pinned_mu);
     if (g_npinned < kPinned) {
-      g_pinned[g_npinned++] = p;
+      g_pinned[g_npinned++] = PinnedStatus{p, ctx};
       return;
     }
+    for (int i = 0; i < kPinned; i++)
+      if (g_pinned[i].ctx != ctx) {
+        std::swap(g_pinned[i].p, p);
+        g_pinned[i].ctx = ctx;
+        break;
+      }
   }
-  cudaFreeHost(p);
+  if (cudaFreeHost(p) != cudaSuccess) cudaGetLastError();  // (its context may be gone)
 }
 
 int validate(const cpma_config& c) {
@@ -354,7 +401,7 @@ void release_all(cpma* h) {
   free_arrays(h, &cur);
   free_arrays(h, &h->spare);
   dev_free(h, h->d_status, sizeof(Status), nullptr);
-  give_pinned(h->h_status);
+  give_pinned(h->h_status, h->status_ctx);
   prof_resolve(h);
   for (int i = 0; i < h->prof.npool; i++) cudaEventDestroy(h->prof.pool[i]);
   delete[] h->prof.pool;
@@ -397,7 +444,8 @@ int new_handle(const cpma_config* cfg, cpma** out) {
     delete h;
     return rc;
   }
-  h->h_status = take_pinned();
+  h->status_ctx = context_id();
+  h->h_status = take_pinned(h->status_ctx);
   if (!h->h_status) {
     release_all(h);
     delete h;

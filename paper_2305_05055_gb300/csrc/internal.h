@@ -203,6 +203,7 @@ struct cpma {
   bool may_have_empty = false;      // some leaf may be empty (head fix-up)
   cpmaimpl::Status* d_status = nullptr;
   cpmaimpl::Status* h_status = nullptr;  // pinned
+  uint64_t status_ctx = 0;               // the context it was pinned in
   cpmaimpl::Scratch s;
   // kernels launched; atomic because const queries on one handle may be
   // issued from several host threads
