@@ -1,17 +1,17 @@
 // Batch sort (Sec. 4: "an unsorted batch can be converted into a sorted batch
 // in O(k log k) work") as a radix sort over 8-bit digits.
 //
-// One digit pass is three kernels.  Every block owns a contiguous run of
-// 4096-key tiles.  It counts its keys per digit (k_digit_count); a block per
-// digit turns the blocks' counts into offsets (k_digit_scan); every block then
-// takes its tiles in order, ranks each in shared memory and writes every
-// digit's run of the tile contiguously behind the ones before it
-// (k_digit_scatter).  No block waits for another.  (Reading the keys once and
-// joining the tiles by decoupled look-back instead was slower: several hundred
-// tiles start together, so each had to add up most of its predecessors'
-// counts, 8 per round trip to the L2: 343 us a pass over 3e7 keys, against
-// 63 + 3 + 180 us for the three kernels.)  A stable rank takes eight ballots
-// per key and warp (115 instructions per 32 keys bound the scatter); where
+// One digit pass is two kernels.  Every block owns an equal contiguous run of the
+// keys, in tiles of at most 4096.  It counts its keys per digit (k_digit_count),
+// for itself and, by atomics, for its group of 32 blocks; every block then adds up
+// the groups and the blocks of its group before it, takes its tiles in order,
+// ranks each in shared memory and writes every digit's run of the tile
+// contiguously behind the ones before it (k_digit_scatter).  No block waits for
+// another.  (Reading the keys once and joining the tiles by decoupled look-back
+// instead was slower on large batches: several hundred tiles start together, so
+// each had to add up most of its predecessors' counts, 8 per round trip to the L2:
+// 343 us a pass over 3e7 keys, against 42 + 182 us.)  A stable rank takes eight
+// ballots per key and warp (115 instructions per 32 keys bound the scatter); where
 // order among equal digits does not matter it is one atomic.
 //
 // Keys alone go most significant bits first, so that few passes cross memory:
@@ -21,10 +21,12 @@
 //   (k_bucket_sort);
 // - above, when more than 24 bits vary: two passes by the 16 highest of them,
 //   then each block finishes the buckets that start in its 4096 keys
-//   (k_window_sort), at most 6144 keys.  A bucket of more than 2048 keys
-//   (heavy repeats or skew) does not fit that: it raises a flag, and the
-//   passes over all varying digits, lowest first, run after all.  3e7 40-bit
-//   keys: 735 us, 1650 us for the five look-back passes.
+//   (k_window_sort), at most 6144 keys.  A bucket of more than 2048 keys (heavy
+//   repeats or skew) does not fit that.  One key in 128 is counted by its bucket
+//   first (k_sample): when that shows such a bucket, the passes over all varying
+//   digits, lowest first, run instead, and otherwise after all if a window meets
+//   one.  3e7 40-bit keys: 710 us, 1650 us for the five look-back passes; 4e6
+//   R-MAT edges (six varying digits): 285, 320 and, by windows first, 540 us.
 // A block finishes up to 6144 keys in shared memory in one counting pass: bins
 // by the highest bits in which the keys differ, about as many as keys, one
 // atomic per key, then every key's rank among the few keys of its bin.  Bins
@@ -35,6 +37,7 @@
 // Keys with tags (which must move stably) take the digit passes: buckets up
 // to 1.25M, all varying digits from the lowest up above.
 #include <algorithm>
+#include <cmath>
 
 #include "dev_common.cuh"
 #include "internal.h"
@@ -56,6 +59,10 @@ constexpr int kBTile = kBT * kBItems;  // 6144 keys
 // Batches of more than one tile and at most this many keys take the
 // top-digit buckets (k / 256 keys per bucket on average, far below kBTile).
 constexpr uint64_t kBucketMax = 1280ull * 1024;
+// Larger batches of keys alone, and at most this many (1700 per bucket of the 16
+// highest bits on average, eight standard deviations below the 2048 that fit),
+// go by those bits and in windows.
+constexpr uint64_t kMsdMax = 1700ull << 16;
 
 template <bool VALS, int KT = kT, int ITEMS = kItems>
 struct TileSmemT {
@@ -225,7 +232,7 @@ struct SortCtl {
   uint32_t done;           // OR/AND blocks finished
   uint32_t msd;            // large batch: top 16 varying bits, then windows
   uint32_t rest;           // the passes over all digits are needed: few bits vary, or a
-                           // window did not hold its buckets
+                           // bucket is too large for a window
   uint32_t pad;
   ull or_all, nand_all;    // OR of the keys and of their complements
 };
@@ -270,11 +277,13 @@ __device__ __forceinline__ void vary_of(ull o, ull na, SortCtl* ctl, bool digits
   }
 }
 
-// Bucket path, first kernel: the bits that vary.
+// First kernel: the bits that vary; nz words at z to zero (the passes' group
+// counts, the sample's buckets).
 __global__ void __launch_bounds__(kT) k_orand(const uint64_t* __restrict__ in, uint64_t k,
-                                              SortCtl* ctl, bool digits) {
+                                              SortCtl* ctl, bool digits, uint32_t* z, uint32_t nz) {
   pdl_wait();
   pdl_launch();
+  for (uint32_t i = blockIdx.x * kT + threadIdx.x; i < nz; i += gridDim.x * kT) z[i] = 0;
   ull o = 0, na = 0;
   // eight keys per thread and step, loaded together
   const uint64_t stride = (uint64_t)gridDim.x * kT;
@@ -294,6 +303,34 @@ __global__ void __launch_bounds__(kT) k_orand(const uint64_t* __restrict__ in, u
   vary_of(o, na, ctl, digits);
 }
 
+// Large batches: one key in kSampleEvery, at a scattered place of each run of as
+// many, counted by the 16 highest bits that vary.  `most` keys in one bucket: the
+// batch takes the digit passes.
+constexpr uint32_t kSampleEvery = 128, kSampleBins = 1u << 16;
+__global__ void __launch_bounds__(kT) k_sample(const uint64_t* __restrict__ in, uint64_t k,
+                                               SortCtl* ctl, uint32_t* bins, uint32_t most) {
+  pdl_wait();
+  pdl_launch();
+  if (!ctl->msd) return;
+  const int sh = (int)ctl->fshift - 8;
+  const uint64_t n = k / kSampleEvery;
+  const unsigned lane = lane_id();
+  // whole warps stay in the loop
+  for (uint64_t j0 = ((uint64_t)blockIdx.x * kT + threadIdx.x) & ~31ull; j0 < n;
+       j0 += (uint64_t)gridDim.x * kT) {
+    if (__any_sync(FULL, *((volatile uint32_t*)&ctl->rest) != 0)) return;  // decided
+    const uint64_t j = j0 + lane;
+    const uint32_t at = ((uint32_t)j * 0x9E3779B1u) >> 25;  // in [0, kSampleEvery)
+    const bool ok = j < n;
+    const uint32_t b = ok ? (uint32_t)(in[j * kSampleEvery + at] >> sh) & (kSampleBins - 1) : ~0u;
+    const unsigned same = __match_any_sync(FULL, b);
+    if (ok && lane == (unsigned)__ffs(same) - 1u) {
+      const uint32_t c = __popc(same);
+      if (atomicAdd(&bins[b], c) + c >= most) ctl->rest = 1;
+    }
+  }
+}
+
 // What a digit pass reads and writes.  p >= 0: digit p of the passes from the
 // lowest up, which take the input, then A and B alternately, arranged so that
 // the last varying one writes A (not run when the top bits and the windows
@@ -308,8 +345,10 @@ struct Pass {
   uint64_t k;
   int p;
   SortCtl* ctl;
-  uint32_t* cnt;  // counts, then offsets, of digit d and block b at d * gridDim.x + b
+  uint32_t* grp;  // this pass's counts of digit d in blocks 32 g .. 32 g + 31, at 256 g + d
+  uint32_t* cnt;  // the blocks' counts, of digit d and block b at 256 b + d
 };
+constexpr uint32_t kGroup = 32;
 struct PassIo {
   const uint64_t* src;
   const uint32_t* vsrc;
@@ -326,11 +365,11 @@ __device__ __forceinline__ bool pass_io(const Pass& a, PassIo& io) {
   }
   if (a.p == kTop0) {
     io = PassIo{a.in, a.vin, a.A, a.VA, (int)c.fshift - 8};
-    return c.msd != 0;
+    return !c.rest;
   }
   if (a.p == kTop1) {
     io = PassIo{a.A, a.VA, a.B, a.VB, (int)c.fshift};
-    return c.msd != 0;
+    return !c.rest;
   }
   if (!c.varying[a.p] || !c.rest) return false;
   const uint32_t left = c.npass - c.rank[a.p];  // passes from this one on
@@ -342,8 +381,35 @@ __device__ __forceinline__ bool pass_io(const Pass& a, PassIo& io) {
   return true;
 }
 
-// Keys per digit of the block's tiles.
-__global__ void __launch_bounds__(kT) k_digit_count(Pass a) {
+// The block's keys [e0, e1), in tiles of at most 256 * ipw.  From kWholeTiles
+// tiles a block on, blocks own whole tiles; below, where one tile more or less
+// counts, equal shares (from a multiple of 32 keys on) in equal tiles: keys with
+// tags 4e6 363 and 287 us, 4e7 the other way round by some 2 %.
+constexpr uint64_t kWholeTiles = 8;
+struct Share {
+  uint64_t e0, e1;
+  uint32_t ipw;
+};
+__device__ __forceinline__ Share share_of(uint64_t k) {
+  Share s;
+  const uint64_t b = blockIdx.x, G = gridDim.x, nt = (k + kTile - 1) / kTile;
+  if (nt >= kWholeTiles * G) {
+    s.e0 = nt * b / G * kTile;
+    s.e1 = min(k, nt * (b + 1) / G * kTile);
+    s.ipw = kItems;
+    return s;
+  }
+  s.e0 = k * b / G & ~31ull;
+  s.e1 = b + 1 == G ? k : k * (b + 1) / G & ~31ull;
+  const uint64_t n = s.e1 - s.e0, step = (uint64_t)kT * ((n + kTile - 1) / kTile);
+  s.ipw = step ? (uint32_t)((n + step - 1) / step) : 0u;
+  return s;
+}
+
+// Keys per digit of the block, and of its group.
+// (three blocks per SM run: with the 32 registers it would take, half of the eight
+// loads wait for the others, 1e8 keys 128 us instead of 116)
+__global__ void __launch_bounds__(kT, 3) k_digit_count(Pass a) {
   constexpr int kCopies = 4;  // histograms per block: fewer lanes on one counter
   __shared__ uint32_t hs[kCopies][256];
   pdl_wait();
@@ -353,53 +419,38 @@ __global__ void __launch_bounds__(kT) k_digit_count(Pass a) {
   for (int i = threadIdx.x; i < kCopies * 256; i += kT) (&hs[0][0])[i] = 0;
   __syncthreads();
   uint32_t* h = hs[(threadIdx.x >> 5) & (kCopies - 1)];
-  const uint64_t ntiles = (a.k + kTile - 1) / kTile;
-  const uint64_t e0 = ntiles * blockIdx.x / gridDim.x * kTile;
-  const uint64_t e1 = min(a.k, ntiles * (blockIdx.x + 1) / gridDim.x * kTile);
-  uint64_t i = e0 + threadIdx.x;
-  for (; i + 7 * kT < e1; i += 8 * kT) {
+  const Share sh = share_of(a.k);
+  uint64_t i = sh.e0 + threadIdx.x;
+  for (; i + 7 * kT < sh.e1; i += 8 * kT) {
     uint64_t x[8];
 #pragma unroll
     for (int j = 0; j < 8; j++) x[j] = io.src[i + j * kT];
 #pragma unroll
     for (int j = 0; j < 8; j++) atomicAdd(&h[(uint32_t)(x[j] >> io.shift) & 255u], 1u);
   }
-  for (; i < e1; i += kT) atomicAdd(&h[(uint32_t)(io.src[i] >> io.shift) & 255u], 1u);
+  for (; i < sh.e1; i += kT) atomicAdd(&h[(uint32_t)(io.src[i] >> io.shift) & 255u], 1u);
   __syncthreads();
   static_assert(kT == 256, "a thread per digit");
   uint32_t n = 0;
 #pragma unroll
   for (int q = 0; q < kCopies; q++) n += hs[q][threadIdx.x];
-  a.cnt[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = n;
+  a.cnt[(size_t)blockIdx.x * 256 + threadIdx.x] = n;
+  if (n) atomicAdd(&a.grp[(blockIdx.x / kGroup) * 256 + threadIdx.x], n);
 }
 
-// Block d: the G blocks' counts of digit d to exclusive offsets among them,
-// and their total.
-__global__ void __launch_bounds__(kT) k_digit_scan(Pass a, uint32_t G) {
-  __shared__ uint32_t ws[kWarps];
-  pdl_wait();
-  pdl_launch();
-  PassIo io;
-  if (!pass_io(a, io)) return;
-  uint32_t* row = a.cnt + (size_t)blockIdx.x * G;
-  const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
-  uint32_t carry = 0;
-  for (uint32_t b0 = 0; b0 < G; b0 += kT) {
-    const uint32_t b = b0 + threadIdx.x;
-    const uint32_t v = b < G ? row[b] : 0u;
-    const uint32_t inc = warp_incl_scan(v);
-    if (lane == 31) ws[warp] = inc;
-    __syncthreads();
-    uint32_t before = carry;
-#pragma unroll
-    for (unsigned w = 0; w < kWarps; w++) {
-      if (w < warp) before += ws[w];
-      carry += ws[w];
-    }
-    if (b < G) row[b] = before + inc - v;
-    __syncthreads();
+// Digit d's keys in all blocks, and in the blocks before this one.
+__device__ __forceinline__ void digit_before(const Pass& a, uint32_t d, uint32_t& all,
+                                             uint32_t& before) {
+  const uint32_t ng = (gridDim.x + kGroup - 1) / kGroup, g0 = blockIdx.x / kGroup;
+  all = before = 0;
+#pragma unroll 8
+  for (uint32_t g = 0; g < ng; g++) {
+    const uint32_t v = a.grp[g * 256 + d];
+    all += v;
+    before += g < g0 ? v : 0u;
   }
-  if (threadIdx.x == 0) a.ctl->tot[blockIdx.x] = carry;
+#pragma unroll 8
+  for (uint32_t b = g0 * kGroup; b < blockIdx.x; b++) before += a.cnt[(size_t)b * 256 + d];
 }
 
 // Partition of the tile by digit with no order among equal digits (keys
@@ -431,8 +482,9 @@ __device__ __forceinline__ void tile_rank_any(const uint64_t (&key)[kItems], uin
 }
 
 // The block's tiles in order, each ranked in shared memory and written behind
-// the block's earlier keys of every digit.
-template <bool VALS, bool STABLE>
+// the block's earlier keys of every digit.  WHOLE: its tiles are whole ones (with
+// the items per thread known, 3e7 keys 182 us, else 195).
+template <bool VALS, bool STABLE, bool WHOLE>
 __global__ void __launch_bounds__(kT, 3) k_digit_scatter(Pass a) {
   static_assert(STABLE || !VALS, "tags move stably");
   extern __shared__ __align__(16) uint8_t smem_raw[];
@@ -447,26 +499,35 @@ __global__ void __launch_bounds__(kT, 3) k_digit_scatter(Pass a) {
   const uint32_t d = threadIdx.x;
   // digit d's next position: the keys of lower digits, then those of d in
   // earlier blocks
-  const uint32_t t = a.ctl->tot[d], inc = warp_incl_scan(t);
+  uint32_t t, before;
+  digit_before(a, d, t, before);
+  if (blockIdx.x == 0) a.ctl->tot[d] = t;
+  const uint32_t inc = warp_incl_scan(t);
   if (lane == 31) s_ws[warp] = inc;
   __syncthreads();
-  uint32_t run = a.cnt[(size_t)d * gridDim.x + blockIdx.x] + inc - t;
+  uint32_t run = before + inc - t;
   for (unsigned w = 0; w < warp; w++) run += s_ws[w];
-  const uint64_t ntiles = (a.k + kTile - 1) / kTile;
-  const uint64_t t0 = ntiles * blockIdx.x / gridDim.x, t1 = ntiles * (blockIdx.x + 1) / gridDim.x;
-  for (uint64_t tile = t0; tile < t1; tile++) {
-    const uint64_t base = tile * kTile;
-    const uint32_t nvalid = (uint32_t)min((uint64_t)kTile, a.k - base);
+  // Equal tiles where the ranks are what a tile costs (a last tile of few keys
+  // would cost the block as many steps as a full one has); whole ones and a rest
+  // where it is one atomic per key.
+  const Share sh = share_of(a.k);
+  const uint32_t ipw = STABLE && !WHOLE ? sh.ipw : (uint32_t)kItems;
+  io.src += sh.e0;
+  if constexpr (VALS) io.vsrc += sh.e0;
+  const uint32_t n = (uint32_t)(sh.e1 - sh.e0);
+  for (uint32_t base = 0; base < n; base += kT * ipw) {
+    const uint32_t nvalid = min(kT * ipw, n - base);
     uint64_t key[kItems];
     uint32_t val[kItems];
 #pragma unroll
     for (int j = 0; j < kItems; j++) {
-      const uint32_t li = warp * 32 * kItems + j * 32 + lane;
-      key[j] = li < nvalid ? io.src[base + li] : 0ull;
-      if constexpr (VALS) val[j] = li < nvalid ? io.vsrc[base + li] : 0u;
+      const uint32_t li = warp * 32 * ipw + j * 32 + lane;
+      const bool in = (uint32_t)j < ipw && li < nvalid;
+      key[j] = in ? io.src[base + li] : 0ull;
+      if constexpr (VALS) val[j] = in ? io.vsrc[base + li] : 0u;
       else val[j] = 0u;
     }
-    if constexpr (STABLE) tile_rank<VALS>(key, val, nvalid, io.shift, sm);
+    if constexpr (STABLE) tile_rank<VALS>(key, val, nvalid, io.shift, sm, ipw);
     else tile_rank_any(key, nvalid, io.shift, sm);
     s_off[d] = run - sm.dstart[d];
     run += (d < 255 ? sm.dstart[d + 1] : nvalid) - sm.dstart[d];
@@ -570,13 +631,15 @@ __global__ void __launch_bounds__(kBT, 2) k_window_sort(const uint64_t* __restri
                                                         SortCtl* ctl) {
   extern __shared__ __align__(16) uint8_t smem_raw[];
   FinishSmem<false>& sm = *reinterpret_cast<FinishSmem<false>*>(smem_raw);
-  __shared__ uint32_t s_at[2];
+  __shared__ uint32_t s_at[2], s_rest;
   pdl_wait();
   pdl_launch();
-  if (!ctl->msd) return;
   const int sh = (int)ctl->fshift - 8;
+  // (other blocks may raise the flag meanwhile: one thread reads it)
+  if (threadIdx.x == 0) s_rest = *((volatile uint32_t*)&ctl->rest);
   if (threadIdx.x < 2) s_at[threadIdx.x] = 0xFFFFFFFFu;
   __syncthreads();
+  if (s_rest) return;
   // the first bucket start at or after either end of the tile, each searched
   // by half of the block
   const uint64_t t0 = (uint64_t)blockIdx.x * kTile;
@@ -814,17 +877,19 @@ void sort_attrs() {
   static bool done = false;  // one per instantiation
   if (done) return;
   const int smem = (int)sizeof(TileSmemT<VALS>);
-  cudaFuncSetAttribute(k_digit_scatter<VALS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       smem);
+  cudaFuncSetAttribute(k_digit_scatter<VALS, true, false>,
+                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaFuncSetAttribute(k_digit_scatter<VALS, true, true>,
+                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if constexpr (!VALS)
-    cudaFuncSetAttribute(k_digit_scatter<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         smem);
+    cudaFuncSetAttribute(k_digit_scatter<false, false, true>,
+                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   cudaFuncSetAttribute(k_bucket_sort<VALS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        (int)sizeof(FinishSmem<VALS>));
   cudaFuncSetAttribute(k_window_sort, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        (int)sizeof(FinishSmem<false>));
   int bps = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_digit_scatter<VALS, true>, kT, smem) ==
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_digit_scatter<VALS, true, false>, kT, smem) ==
           cudaSuccess &&
       bps > 0)
     scatter_blocks_per_sm<VALS>() = bps;
@@ -833,14 +898,44 @@ void sort_attrs() {
 }
 }  // namespace
 
-// Blocks of a digit pass over k keys: as many as run at once (the scatter
-// kernel's limit), and then the fewest that give no block more tiles.
+// Blocks of a digit pass over k keys, at most: one tile each, no more than run at
+// once (the scatter kernel's limit), and that many for a large batch.
+template <bool VALS>
+uint32_t pass_blocks_most(const cpma* h, uint64_t k) {
+  const uint64_t most = (uint64_t)h->num_sms * (uint64_t)scatter_blocks_per_sm<VALS>();
+  return (uint32_t)(k > kBucketMax ? most : std::min<uint64_t>((k + kTile - 1) / kTile, most));
+}
+
+// The blocks it takes: that many, or with whole tiles the fewest that give no
+// block more of them.
 template <bool VALS>
 uint32_t pass_blocks(const cpma* h, uint64_t k) {
-  const uint64_t ntiles = (k + kTile - 1) / kTile;
-  const uint64_t most = (uint64_t)h->num_sms * (uint64_t)scatter_blocks_per_sm<VALS>();
-  const uint64_t per = (ntiles + most - 1) / most;
-  return (uint32_t)((ntiles + per - 1) / per);
+  const uint64_t nt = (k + kTile - 1) / kTile, most = pass_blocks_most<VALS>(h, k);
+  if (nt < kWholeTiles * most) return (uint32_t)most;
+  const uint64_t per = (nt + most - 1) / most;
+  return (uint32_t)((nt + per - 1) / per);
+}
+
+// The sort's words in the scratch: control, group counts per pass (row 0: by the
+// field or kTop0, 1: kTop1, 2 + p: digit p), sample, counts per block.  Sizes
+// grow with k and are largest without tags, so that a reservation covers smaller
+// and untagged batches.
+struct HistLayout {
+  uint32_t G, row;       // blocks, words of a row
+  size_t grp, bins, cnt, bytes;
+};
+template <bool VALS>
+HistLayout hist_layout(const cpma* h, uint64_t k) {
+  HistLayout l;
+  const bool large = k > kBucketMax;
+  l.G = pass_blocks<VALS>(h, k);
+  const uint32_t most = pass_blocks_most<VALS>(h, k);
+  l.row = (most + kGroup - 1) / kGroup * 256;
+  l.grp = ctl_bytes();
+  l.bins = l.grp + (size_t)(large ? 10 : 1) * l.row * 4;
+  l.cnt = l.bins + (large && !VALS ? kSampleBins * 4 : 0);
+  l.bytes = l.cnt + (size_t)most * 256 * 4;
+  return l;
 }
 
 int sort_scratch(cpma* h, uint64_t k, bool vals) {
@@ -852,44 +947,46 @@ int sort_scratch(cpma* h, uint64_t k, bool vals) {
   if (k <= (uint64_t)kTile) return CPMA_OK;
   CPMA_TRY(ensure(h, h->s.keysB, k * 8));
   if (vals) CPMA_TRY(ensure(h, h->s.valsB, k * 4));
-  // (fewer keys may take more blocks, and keys alone more than keys with tags:
-  // room for all that a reservation for k covers)
-  const uint64_t most = std::min<uint64_t>(
-      (k + kTile - 1) / kTile, (uint64_t)h->num_sms * (uint64_t)scatter_blocks_per_sm<false>());
-  return ensure(h, h->s.hist, ctl_bytes() + (size_t)most * 256 * 4);
+  return ensure(h, h->s.hist, hist_layout<false>(h, k).bytes);
 }
 
 template <bool VALS>
 Pass pass_of(cpma* h, const uint64_t* d_in, const uint32_t* v_in, uint64_t k) {
   Scratch& s = h->s;
   uint8_t* ctl = reinterpret_cast<uint8_t*>(s.hist.p);
+  const HistLayout l = hist_layout<VALS>(h, k);
   return Pass{d_in, v_in, (uint64_t*)s.keysA.p, (uint64_t*)s.keysB.p,
               VALS ? (uint32_t*)s.valsA.p : nullptr, VALS ? (uint32_t*)s.valsB.p : nullptr, k, 0,
-              reinterpret_cast<SortCtl*>(ctl), reinterpret_cast<uint32_t*>(ctl + ctl_bytes())};
+              reinterpret_cast<SortCtl*>(ctl), reinterpret_cast<uint32_t*>(ctl + l.grp),
+              reinterpret_cast<uint32_t*>(ctl + l.cnt)};
 }
 
-// The three kernels of a digit pass, each scheduled while the one before it
+// The two kernels of a digit pass, each scheduled while the one before it
 // finishes (programmatic dependent launch; each waits for it first).
 template <bool VALS>
-int digit_pass(cpma* h, Pass a, uint32_t G, int p, bool stable, cudaStream_t st) {
+int digit_pass(cpma* h, Pass a, const HistLayout& l, int p, bool stable, cudaStream_t st) {
   const size_t smem = sizeof(TileSmemT<VALS>);
   a.p = p;
-  CPMA_CUDA(launch_pdl(k_digit_count, G, kT, 0, st, a));
-  CPMA_CUDA(launch_pdl(k_digit_scan, 256, kT, 0, st, a, G));
+  a.grp += (size_t)(p >= 0 ? 2 + p : p == kTop1 ? 1 : 0) * l.row;
+  CPMA_CUDA(launch_pdl(k_digit_count, l.G, kT, 0, st, a));
   if constexpr (VALS) stable = true;
-  CPMA_CUDA(launch_pdl(stable ? k_digit_scatter<VALS, true> : k_digit_scatter<false, false>, G, kT,
-                       smem, st, a));
-  h->launches += 3;
+  const bool whole = (a.k + kTile - 1) / kTile >= kWholeTiles * l.G;  // as share_of
+  CPMA_CUDA(launch_pdl(!stable ? k_digit_scatter<false, false, true>
+                       : whole ? k_digit_scatter<VALS, true, true>
+                               : k_digit_scatter<VALS, true, false>,
+                       l.G, kT, smem, st, a));
+  h->launches += 2;
   return CPMA_OK;
 }
 
 // A large batch by the digits that vary, lowest first: with tags, when few
-// bits vary, or when a window gave up (the kernels return at once otherwise).
+// bits vary, or when a bucket is too large for a window (the kernels return at
+// once otherwise).
 template <bool VALS>
 int sort_digits(cpma* h, const uint64_t* d_in, const uint32_t* v_in, uint64_t k, cudaStream_t st) {
   const Pass a = pass_of<VALS>(h, d_in, v_in, k);
-  const uint32_t G = pass_blocks<VALS>(h, k);
-  for (int p = 0; p < 8; p++) CPMA_TRY(digit_pass<VALS>(h, a, G, p, true, st));
+  const HistLayout l = hist_layout<VALS>(h, k);
+  for (int p = 0; p < 8; p++) CPMA_TRY(digit_pass<VALS>(h, a, l, p, true, st));
   CPMA_CUDA(launch_pdl(k_copy_if_no_pass,
                        (unsigned)std::min<uint64_t>((uint64_t)h->num_sms * 4, (k + kT - 1) / kT),
                        kT, 0, st, d_in, a.A, v_in, a.VA, k, a.ctl));
@@ -931,25 +1028,36 @@ int sort_impl(cpma* h, const uint64_t* d_in, const uint32_t* v_in, uint64_t k, c
   uint64_t* B = (uint64_t*)h->s.keysB.p;
   uint32_t* VB = VALS ? (uint32_t*)h->s.valsB.p : nullptr;
   SortCtl* ctl = reinterpret_cast<SortCtl*>(h->s.hist.p);
-  const uint32_t G = pass_blocks<VALS>(h, k);
+  const HistLayout l = hist_layout<VALS>(h, k);
   const Pass a = pass_of<VALS>(h, d_in, v_in, k);
   if (!cleared) CPMA_CUDA(cudaMemsetAsync(ctl, 0, sizeof(SortCtl), st));
   // about eight keys per thread: one step of the unrolled loop
   const int ogrid = (int)std::max<uint64_t>(
       1, std::min<uint64_t>((uint64_t)h->num_sms * 8, (k + 8 * kT - 1) / (8 * kT)));
-  CPMA_CUDA(launch_pdl(k_orand, ogrid, kT, 0, st, d_in, k, ctl, VALS));
+  // buckets by the 16 highest bits hold k / 65536 keys and more: no window's worth
+  const bool digits = VALS || k > kMsdMax;
+  CPMA_CUDA(launch_pdl(k_orand, ogrid, kT, 0, st, d_in, k, ctl, digits, a.grp,
+                       (uint32_t)((l.cnt - l.grp) / 4)));
   h->launches++;
   if (k <= kBucketMax) {
-    CPMA_TRY(digit_pass<VALS>(h, a, G, kField, VALS, st));
+    CPMA_TRY(digit_pass<VALS>(h, a, l, kField, VALS, st));
     CPMA_CUDA(launch_pdl(k_bucket_sort<VALS>, 256, kBT, sizeof(FinishSmem<VALS>), st, B, VB, A, VA,
                          ctl, d_in, v_in, k));
     h->launches++;
     // OR/AND and count reads, scatter and bucket read + write
     prof_add_bytes(h, PH_SORT, 16ull * k + (VALS ? 24ull : 16ull) * k * 2);
   } else {
-    if (!VALS) {
-      CPMA_TRY(digit_pass<VALS>(h, a, G, kTop0, false, st));
-      CPMA_TRY(digit_pass<VALS>(h, a, G, kTop1, true, st));
+    if (!digits) {
+      // the mean bucket's sample and eight standard deviations, but at least
+      // that of 3700 keys: a bucket of 2048 to 6144 fits its window if it starts
+      // early in it, and the passes over all digits take half as long again
+      const double mean = (double)(k / kSampleEvery) / kSampleBins;
+      const uint32_t many = (uint32_t)std::max(29.0, mean + 8.0 * std::sqrt(mean));
+      uint32_t* bins = reinterpret_cast<uint32_t*>((uint8_t*)h->s.hist.p + l.bins);
+      CPMA_CUDA(launch_pdl(k_sample, (unsigned)h->num_sms * 4u, kT, 0, st, d_in, k, ctl, bins, many));
+      h->launches++;
+      CPMA_TRY(digit_pass<VALS>(h, a, l, kTop0, false, st));
+      CPMA_TRY(digit_pass<VALS>(h, a, l, kTop1, true, st));
       CPMA_CUDA(launch_pdl(k_window_sort, (unsigned)((k + kTile - 1) / kTile), kBT,
                            sizeof(FinishSmem<false>), st, B, A, k, ctl));
       h->launches++;
