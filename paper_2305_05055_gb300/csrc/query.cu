@@ -228,6 +228,7 @@ __global__ void __launch_bounds__(kT) k_range_prep(const uint64_t* __restrict__ 
 
 // Rank of the first key >= x: elements before its leaf plus the leaf's
 // elements below x (the whole warp decodes the leaf).
+template <bool RAW>
 __device__ __forceinline__ uint64_t rank_of(uint64_t x, const uint64_t* __restrict__ heads,
                                             const uint8_t* __restrict__ data,
                                             const uint32_t* __restrict__ used, uint64_t L,
@@ -235,7 +236,7 @@ __device__ __forceinline__ uint64_t rank_of(uint64_t x, const uint64_t* __restri
   const uint64_t j = route_leaf(heads, L, x);
   uint32_t below = 0;
   warp_decode(data + j * LB, min(used[j], LB), [&](uint32_t, uint64_t v) { below += v < x; },
-              true);
+              RAW);
   return P[j] + warp_sum(below);
 }
 
@@ -243,7 +244,8 @@ __device__ __forceinline__ uint64_t rank_of(uint64_t x, const uint64_t* __restri
 // [r0, r1) and the leaves holding it.  KEYS: [a, b) is a key range, r0 =
 // rank(a), r1 = rank(b) (r1 = r0 when a >= b).  Otherwise (map_range_length)
 // a is the start key and b the length: r1 = min(r0 + b, n).
-template <bool KEYS>
+// RAW: the leaves hold cells.
+template <bool KEYS, bool RAW>
 __global__ void __launch_bounds__(kT) k_rank_prep(const uint64_t* __restrict__ A,
                                                   const uint64_t* __restrict__ B, uint64_t q,
                                                   const uint64_t* __restrict__ heads,
@@ -256,14 +258,16 @@ __global__ void __launch_bounds__(kT) k_rank_prep(const uint64_t* __restrict__ A
                                                   uint64_t* __restrict__ items,
                                                   uint64_t* __restrict__ sum,
                                                   uint64_t* __restrict__ count) {
+  pdl_wait();
+  pdl_launch();
   const unsigned lane = lane_id();
   const uint64_t gw = gtid() >> 5, nw = gstride() >> 5;
   const uint64_t n = P[L];
   for (uint64_t i = gw; i < q; i += nw) {
     const uint64_t a = A[i], b = B[i];
-    const uint64_t r0 = rank_of(a, heads, data, used, L, LB, P);
+    const uint64_t r0 = rank_of<RAW>(a, heads, data, used, L, LB, P);
     uint64_t r1;
-    if constexpr (KEYS) r1 = a < b ? rank_of(b, heads, data, used, L, LB, P) : r0;
+    if constexpr (KEYS) r1 = a < b ? rank_of<RAW>(b, heads, data, used, L, LB, P) : r0;
     else r1 = (b >= n - r0) ? n : r0 + b;
     uint64_t f = 0, it = 0;
     if (r1 > r0) {
@@ -300,7 +304,9 @@ struct ExtractArgs {
   const leafwalk::Mark* start = nullptr;  // where each query's first key lies (leaf_below)
 };
 
+template <bool RAW>
 __global__ void __launch_bounds__(kT) k_extract(ExtractArgs a) {
+  pdl_wait();
   const uint64_t gw = gtid() >> 5, nw = gstride() >> 5;
   const uint64_t N = a.item_off[a.q];
   const uint64_t g0 = N * gw / nw, g1 = N * (gw + 1) / nw;
@@ -313,7 +319,7 @@ __global__ void __launch_bounds__(kT) k_extract(ExtractArgs a) {
     warp_decode(a.data + j * a.LB, min(a.used[j], a.LB), [&](uint32_t idx, uint64_t v) {
       const uint64_t r = base + idx;
       if (r >= r0 && r < r1 && o + (r - r0) < a.cap) a.out[o + (r - r0)] = v;
-    }, true);
+    }, RAW);
   }
 }
 
@@ -1447,6 +1453,22 @@ int scratch_address(int dev, uint8_t** out) {
 
 }  // namespace
 
+namespace {
+
+// Few enough queries for range_extract to take a warp per leaf, as for cells: a
+// thread walks and stores a whole leaf in a chain that grows with its size, and
+// with few leaves nothing hides it.  Warps / threads, us, lists of up to 50 and of
+// 100 to 1000 keys: 512-byte leaves, 100 queries 33 / 31 and 37 / 44 (40-bit keys), 35
+// / 41 and 37 / 54 (edges), 1000 41 / 35 and 49 / 46, 41 / 45 and 49 / 59; 2048-byte
+// ones, 1000 47 / 46 and 56 / 92, 46 / 82 and 55 / 139, 9700 114 / 57 and 148 / 108,
+// 116 / 102 and 135 / 165.  256-byte leaves by threads always.
+bool extract_by_warps(const cpma* h, uint64_t q) {
+  const uint64_t LB = h->cfg.leaf_bytes;
+  return LB >= 512 && q <= (uint64_t)h->num_sms * LB / 128;
+}
+
+}  // namespace
+
 int run_has(const cpma* h, const uint64_t* d_keys, uint64_t q, uint8_t* d_out, cudaStream_t st) {
   if (q == 0) return CPMA_OK;
   // (a lookup is half a range: 2048-byte leaves, 4e3 keys 15 us by teams and
@@ -1776,7 +1798,7 @@ int run_range_length(const cpma* h, const uint64_t* start, const uint64_t* lengt
   }
   uint64_t* r0 = (uint64_t*)s.q_lo.p;
   uint64_t* r1 = (uint64_t*)s.q_hi.p;
-  k_rank_prep<false><<<query_grid(h, q * 32, kT, 16), kT, 0, st>>>(
+  k_rank_prep<false, true><<<query_grid(h, q * 32, kT, 16), kT, 0, st>>>(
       start, length, q, h->heads, h->data, h->used, h->L, h->cfg.leaf_bytes, P, r0, r1, r.first,
       r.items, sum, count);
   CPMA_LAUNCHED(h);
@@ -1807,15 +1829,17 @@ int run_range_extract(const cpma* h, const uint64_t* lo, const uint64_t* hi, uin
   uint64_t* r1 = (uint64_t*)s.q_hi.p;
   // where each query's first key lies in its leaf, when there is room
   leafwalk::Mark* start = nullptr;
-  if (!h->cfg.codec && out && cap)
+  const bool warps = h->cfg.codec || extract_by_warps(h, q);
+  if (!warps && out && cap)
     start = (leafwalk::Mark*)prefix_memory(hm, s.q_marks, q * sizeof(leafwalk::Mark), st);
   prof_begin(h, PH_RANGE_PREP, st);
   CPMA_TRY(scan_u32_query(hm, h->cnt, P, h->L, st));
   // the counts (r1 - r0) go to `offsets` first
-  if (h->cfg.codec) {
-    k_rank_prep<true><<<query_grid(h, q * 32, kT, 16), kT, 0, st>>>(
-        lo, hi, q, h->heads, h->data, h->used, h->L, h->cfg.leaf_bytes, P, r0, r1, r.first, r.items,
-        nullptr, offsets);
+  if (warps) {
+    CPMA_CUDA(launch_pdl(h->cfg.codec ? k_rank_prep<true, true> : k_rank_prep<true, false>,
+                         (unsigned)query_grid(h, q * 32, kT, 16), kT, 0, st, lo, hi, q, h->heads,
+                         h->data, h->used, h->L, h->cfg.leaf_bytes, P, r0, r1, r.first, r.items,
+                         nullptr, offsets));
   } else {
     CPMA_CUDA(launch_pdl(k_rank_ends, (unsigned)query_grid(h, 2 * q, kT, 8), kT, 0, st, lo, hi, q,
                          leaves_of(h), P, r0, r1, r.first, r.items, offsets, start));
@@ -1841,8 +1865,8 @@ int run_range_extract(const cpma* h, const uint64_t* lo, const uint64_t* hi, uin
   a.out = out;
   a.cap = cap;
   prof_begin(h, PH_RANGE, st);
-  if (h->cfg.codec) k_extract<<<persistent_grid(h), kT, 0, st>>>(a);
-  else CPMA_CUDA(launch_pdl(k_extract_leaf, (unsigned)persistent_grid(h), kT, 0, st, a));
+  CPMA_CUDA(launch_pdl(h->cfg.codec ? k_extract<true> : warps ? k_extract<false> : k_extract_leaf,
+                       (unsigned)persistent_grid(h), kT, 0, st, a));
   CPMA_LAUNCHED(h);
   prof_end(h, st);
   return check_cuda(cudaGetLastError());
