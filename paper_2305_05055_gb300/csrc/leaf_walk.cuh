@@ -770,8 +770,9 @@ LT_HD uint32_t leaf_below(const uint8_t* leafp, uint32_t u, uint64_t x, Mark& at
 // ---- a leaf walked by a team of lanes ----
 //
 // One lane walks a leaf in some 30 steps that wait for one another; with few
-// queries on the GPU that chain is what a call waits for.  Here each of kTeam
-// lanes takes an equal run of 16-byte chunks: it enters with the code open at
+// queries on the GPU that chain is what a call waits for.  Here each of N lanes
+// (eight, or a warp for leaves of more than 512 bytes) takes an equal run of
+// 16-byte chunks: it enters with the code open at
 // its first byte (found by walking the chunk before from any state: every code
 // has at most 10 bytes, so one ends in it), sums its deltas, learns from a scan
 // over the team the element before its run, and then visits its elements.
@@ -784,9 +785,10 @@ struct Run {
   uint32_t codes = 0;
 };
 
-// Lane tl's run of a leaf of u used bytes (0: no leaf).
+// Lane tl's run (of N) of a leaf of u used bytes (0: no leaf).
+template <uint32_t N = kTeam>
 LT_HD Run team_run(const uint8_t* leafp, uint32_t u, uint32_t tl) {
-  const uint32_t per = 16u * (((u + 15u) / 16u + kTeam - 1u) / kTeam);
+  const uint32_t per = 16u * (((u + 15u) / 16u + N - 1u) / N);
   Run r;
   r.b0 = per * tl;
   r.b1 = r.b0 + per < u ? r.b0 + per : u;

@@ -13,8 +13,8 @@
 //    once however often the queries overlap.
 //    From one query per leaf on, every leaf is walked once with its state kept
 //    at every 32nd byte, and a query looks up its two ends (k_marks,
-//    k_range_marked).  A few thousand queries and fewer take eight lanes per
-//    leaf instead of one.
+//    k_range_marked).  Few queries take eight lanes or a warp per leaf instead of
+//    one.
 //  sum (App. A sum()): every leaf once.
 //  map_range_length (App. A: f on at most `length` elements from the first
 //    key >= start): a prefix sum of the leaves' element counts gives the leaf
@@ -68,20 +68,26 @@ __global__ void __launch_bounds__(kT) k_has(const uint64_t* __restrict__ keys, u
 
 // ---- few queries: a team of lanes per leaf (leafwalk::team_run) ----
 
-constexpr unsigned kTeam = leafwalk::kTeam;
+// Lanes of a team: eight, or a warp where a leaf has more than 512 bytes.
+constexpr unsigned kTeam = leafwalk::kTeam, kTeamLarge = 32;
 static_assert(kTeam == 8, "four teams to a warp");
 
-__device__ __forceinline__ unsigned team_lane() { return lane_id() & (kTeam - 1); }
-__device__ __forceinline__ unsigned team_mask() { return 0xFFu << (lane_id() & ~(kTeam - 1)); }
+template <unsigned N>
+__device__ __forceinline__ unsigned team_lane() { return lane_id() & (N - 1); }
+template <unsigned N>
+__device__ __forceinline__ unsigned team_mask() {
+  return (N < 32 ? (1u << (N & 31u)) - 1u : FULL) << (lane_id() & ~(N - 1));
+}
 
-// upper_count by a team: each step its lanes probe eight entries, so the
-// search waits for 6 loads where one lane would for 18 (2e5 entries).
+// upper_count by a team: each step its lanes probe an entry each, so the
+// search waits for 6 loads where one lane would for 18 (2e5 entries, 8 lanes).
+template <unsigned N>
 __device__ __forceinline__ uint64_t team_upper_count(const uint64_t* __restrict__ a, uint64_t n,
                                                      uint64_t x) {
-  const unsigned tl = team_lane(), m = team_mask();
+  const unsigned tl = team_lane<N>(), m = team_mask<N>();
   uint64_t base = 0, len = n;
   while (len) {
-    const uint64_t step = len / (kTeam + 1) + 1, at = (tl + 1) * step - 1;
+    const uint64_t step = len / (N + 1) + 1, at = (tl + 1) * step - 1;
     const uint64_t c = __popc(__ballot_sync(m, at < len && __ldg(a + base + at) <= x));
     base += c * step;
     len = min(step - 1, len - c * step);
@@ -89,26 +95,28 @@ __device__ __forceinline__ uint64_t team_upper_count(const uint64_t* __restrict_
   return base;
 }
 
+template <unsigned N>
 __device__ __forceinline__ uint64_t team_route(const uint64_t* __restrict__ heads, uint64_t L,
                                                uint64_t x) {
   if (x == KEY_MAX) return heads[L];
-  const uint64_t c = team_upper_count(heads, L, x);
+  const uint64_t c = team_upper_count<N>(heads, L, x);
   return c ? c - 1 : 0;
 }
 
 // The lane's run with the element before it (in k.val) and the number of
 // elements before it (the head included); a whole warp calls.
+template <unsigned N>
 __device__ __forceinline__ leafwalk::Run team_leaf(const uint8_t* leafp, uint32_t u,
                                                    uint32_t& idx) {
-  const unsigned tl = team_lane();
-  leafwalk::Run r = leafwalk::team_run(leafp, u, tl);
+  const unsigned tl = team_lane<N>();
+  leafwalk::Run r = leafwalk::team_run<N>(leafp, u, tl);
   __syncwarp();
   uint64_t d = r.delta;
   uint32_t n = r.codes;
 #pragma unroll
-  for (unsigned o = 1; o < kTeam; o <<= 1) {
-    const uint64_t y = __shfl_up_sync(FULL, d, o, kTeam);
-    const uint32_t z = __shfl_up_sync(FULL, n, o, kTeam);
+  for (unsigned o = 1; o < N; o <<= 1) {
+    const uint64_t y = __shfl_up_sync(FULL, d, o, N);
+    const uint32_t z = __shfl_up_sync(FULL, n, o, N);
     if (tl >= o) { d += y; n += z; }
   }
   r.k.val = (u ? leafwalk::leaf_head(leafp) : 0) + (d - r.delta);
@@ -117,6 +125,7 @@ __device__ __forceinline__ leafwalk::Run team_leaf(const uint8_t* leafp, uint32_
 }
 
 // The thread-per-key kernel's work by a team per key.
+template <unsigned N>
 __global__ void __launch_bounds__(kT) k_has_team(const uint64_t* __restrict__ keys, uint64_t q,
                                                  const uint8_t* __restrict__ data,
                                                  const uint32_t* __restrict__ used,
@@ -124,24 +133,24 @@ __global__ void __launch_bounds__(kT) k_has_team(const uint64_t* __restrict__ ke
                                                  uint32_t LB, uint8_t* __restrict__ out,
                                                  ull* prof) {
   ull nbytes = 0;
-  const unsigned tl = team_lane(), team = lane_id() / kTeam;
-  for (uint64_t i0 = (gtid() >> 5) * (32 / kTeam); i0 < q; i0 += (gstride() >> 5) * (32 / kTeam)) {
+  const unsigned tl = team_lane<N>(), team = lane_id() / N;
+  for (uint64_t i0 = (gtid() >> 5) * (32 / N); i0 < q; i0 += (gstride() >> 5) * (32 / N)) {
     const uint64_t i = i0 + team;
     uint64_t x = 0, j = 0;
     uint32_t u = 0, idx;
     if (i < q) {
       x = keys[i];
-      j = team_route(heads, L, x);
+      j = team_route<N>(heads, L, x);
       u = min(used[j], LB);
     }
     __syncwarp();
     const uint8_t* leafp = data + j * LB;
-    const leafwalk::Run r = team_leaf(leafp, u, idx);
+    const leafwalk::Run r = team_leaf<N>(leafp, u, idx);
     bool found = u && tl == 0 && r.k.val == x;  // the head
     if (r.k.val < x && x - r.k.val <= r.delta)
       leafwalk::run_visit(leafp, u, r, [&](uint64_t v) { found |= v == x; });
     __syncwarp();
-    const unsigned hit = __ballot_sync(FULL, found) & team_mask();
+    const unsigned hit = __ballot_sync(FULL, found) & team_mask<N>();
     if (i < q && tl == 0) {
       out[i] = hit ? 1u : 0u;
       nbytes += u + 9;
@@ -643,17 +652,18 @@ __device__ __forceinline__ void scan_ends(const EndsScan& z, const uint64_t* ite
   if (threadIdx.x == 0) *z.done = 0;
 }
 
-template <int OP>
+template <int OP, unsigned N>
 __device__ __forceinline__ void team_reduce(uint64_t& r, uint64_t& c) {
 #pragma unroll
-  for (unsigned o = kTeam / 2; o; o >>= 1) {
+  for (unsigned o = N / 2; o; o >>= 1) {
     r = op_apply<OP>(r, __shfl_xor_sync(FULL, r, o));
     c += __shfl_xor_sync(FULL, c, o);
   }
 }
 
-// k_range_ends by a team per end: the two teams of a query sit side by side.
-template <int OP, bool PLAIN>
+// k_range_ends by a team per end: the two teams of a query sit side by side, a
+// warp's worth takes one end after the other.
+template <int OP, bool PLAIN, unsigned N>
 __global__ void __launch_bounds__(kT) k_range_ends_team(const uint64_t* __restrict__ lo,
                                                         const uint64_t* __restrict__ hi, uint64_t q,
                                                         Leaves t, Reduce<OP, PLAIN> f,
@@ -663,39 +673,53 @@ __global__ void __launch_bounds__(kT) k_range_ends_team(const uint64_t* __restri
                                                         uint64_t* __restrict__ count, uint32_t* ticket, EndsScan z, ull* prof) {
   if (ticket && gtid() == 0) *ticket = 0;
   ull nbytes = 0;
-  const unsigned tl = team_lane(), team = lane_id() / kTeam;
-  for (uint64_t e0 = (gtid() >> 5) * (32 / kTeam); e0 < 2 * q;
-       e0 += (gstride() >> 5) * (32 / kTeam)) {
-    const uint64_t i = (e0 + team) >> 1;
-    const bool side = (team & 1u) != 0u;
-    uint64_t a = 0, b = 0, j = 0;
+  constexpr unsigned kPer = N < 32 ? 2 * N : 32;  // lanes of a query
+  const unsigned tl = team_lane<N>(), mine = lane_id() / kPer;
+  for (uint64_t i0 = (gtid() >> 5) * (32 / kPer); i0 < q; i0 += (gstride() >> 5) * (32 / kPer)) {
+    const uint64_t i = i0 + mine;
+    uint64_t a = 0, b = 0, fl = 0, ll = 0;
     if (i < q) { a = lo[i]; b = hi[i]; }
-    if (a < b) j = team_route(t.heads, t.L, side ? b - 1 : a);
-    __syncwarp();
-    const uint64_t other = __shfl_xor_sync(FULL, j, kTeam);
-    const uint64_t fl = side ? other : j, ll = side ? j : other;
-    const uint32_t u = a < b && (!side || ll > fl) ? min(t.used[j], t.LB) : 0u;
-    const uint8_t* leafp = t.data + j * t.LB;
-    uint32_t idx;
-    const leafwalk::Run run = team_leaf(leafp, u, idx);
     uint64_t r = op_identity<OP>(), c = 0;
     auto take = [&](uint64_t v) {
       if (v >= a && v < b && (PLAIN || (v & f.mask) == f.value)) { r = op_apply<OP>(r, v); c++; }
     };
-    if (u && tl == 0) take(run.k.val);
-    if (u && run.k.val < b && run.k.val + run.delta >= a) leafwalk::run_visit(leafp, u, run, take);
-    __syncwarp();
-    team_reduce<OP>(r, c);
-    r = op_apply<OP>(r, __shfl_down_sync(FULL, r, kTeam));
-    c += __shfl_down_sync(FULL, c, kTeam);
-    if (tl == 0) {
-      nbytes += u;
-      if (!side && i < q) {
-        first[i] = fl + 1;
-        items[i] = ll > fl ? ll - fl - 1 : 0;
-        out[i] = r;
-        count[i] = c;
+    auto end = [&](uint64_t j, uint32_t u) {
+      const uint8_t* leafp = t.data + j * t.LB;
+      uint32_t idx;
+      const leafwalk::Run run = team_leaf<N>(leafp, u, idx);
+      if (u && tl == 0) take(run.k.val);
+      if (u && run.k.val < b && run.k.val + run.delta >= a)
+        leafwalk::run_visit(leafp, u, run, take);
+      __syncwarp();
+      if (tl == 0) nbytes += u;
+    };
+    if constexpr (N < 32) {
+      const bool side = (lane_id() & N) != 0u;
+      uint64_t j = 0;
+      if (a < b) j = team_route<N>(t.heads, t.L, side ? b - 1 : a);
+      __syncwarp();
+      const uint64_t other = __shfl_xor_sync(FULL, j, N);
+      fl = side ? other : j;
+      ll = side ? j : other;
+      end(j, a < b && (!side || ll > fl) ? min(t.used[j], t.LB) : 0u);
+      team_reduce<OP, N>(r, c);
+      r = op_apply<OP>(r, __shfl_down_sync(FULL, r, N));
+      c += __shfl_down_sync(FULL, c, N);
+    } else {
+      if (a < b) {
+        fl = team_route<N>(t.heads, t.L, a);
+        ll = team_route<N>(t.heads, t.L, b - 1);
+        end(fl, min(t.used[fl], t.LB));
+        if (ll > fl) end(ll, min(t.used[ll], t.LB));
       }
+      __syncwarp();
+      team_reduce<OP, N>(r, c);
+    }
+    if (lane_id() % kPer == 0 && i < q) {
+      first[i] = fl + 1;
+      items[i] = ll > fl ? ll - fl - 1 : 0;
+      out[i] = r;
+      count[i] = c;
     }
   }
   nbytes = warp_sum(nbytes);
@@ -773,6 +797,7 @@ __global__ void __launch_bounds__(kT) k_length_ends(const uint64_t* __restrict__
 }
 
 // k_length_ends by a team per query.
+template <unsigned N>
 __global__ void __launch_bounds__(kT) k_length_ends_team(
     const uint64_t* __restrict__ start, const uint64_t* __restrict__ length, uint64_t q, Leaves t,
     const uint64_t* __restrict__ P, uint64_t* __restrict__ first, uint64_t* __restrict__ items,
@@ -782,21 +807,21 @@ __global__ void __launch_bounds__(kT) k_length_ends_team(
   if (ticket && gtid() == 0) *ticket = 0;
   ull nbytes = 0;
   const uint64_t n = P[t.L];
-  const unsigned tl = team_lane(), team = lane_id() / kTeam;
-  for (uint64_t i0 = (gtid() >> 5) * (32 / kTeam); i0 < q; i0 += (gstride() >> 5) * (32 / kTeam)) {
+  const unsigned tl = team_lane<N>(), team = lane_id() / N;
+  for (uint64_t i0 = (gtid() >> 5) * (32 / N); i0 < q; i0 += (gstride() >> 5) * (32 / N)) {
     const uint64_t i = i0 + team;
     uint64_t x = 0, len = 0, fl = 0, s = 0, c = 0;
     uint32_t u = 0, idx;
     if (i < q) len = length[i];
     if (len) {
       x = start[i];
-      fl = team_route(t.heads, t.L, x);
+      fl = team_route<N>(t.heads, t.L, x);
       u = min(t.used[fl], t.LB);
     }
     __syncwarp();
     const uint8_t* leafp = t.data + fl * t.LB;
-    leafwalk::Run run = team_leaf(leafp, u, idx);
-    const uint64_t head = __shfl_sync(FULL, run.k.val, 0, kTeam);
+    leafwalk::Run run = team_leaf<N>(leafp, u, idx);
+    const uint64_t head = __shfl_sync(FULL, run.k.val, 0, N);
     uint64_t below = u && tl == 0 && head < x ? 1u : 0u;
     // the run's elements below x: none, all or, for one lane, some
     if (u && run.k.val < x) {
@@ -804,7 +829,7 @@ __global__ void __launch_bounds__(kT) k_length_ends_team(
       else leafwalk::run_visit(leafp, u, run, [&](uint64_t v) { below += v < x ? 1u : 0u; });
     }
     __syncwarp();
-    team_reduce<CPMA_OP_SUM>(s, below);
+    team_reduce<CPMA_OP_SUM, N>(s, below);
     const uint64_t r0 = P[fl] + below;  // rank of the first key >= x
     const uint64_t r1 = len >= n - r0 ? n : r0 + len;
     // the elements of ranks [r0, r1) in two leaves: its first, and its last one
@@ -832,9 +857,9 @@ __global__ void __launch_bounds__(kT) k_length_ends_team(
       }
       __syncwarp();
       leafp = t.data + j * t.LB;
-      run = team_leaf(leafp, u, idx);
+      run = team_leaf<N>(leafp, u, idx);
     }
-    team_reduce<CPMA_OP_SUM>(s, c);
+    team_reduce<CPMA_OP_SUM, N>(s, c);
     if (tl == 0 && i < q) {
       first[i] = fl + 1;
       items[i] = ll > fl ? ll - fl - 1 : 0;
@@ -1043,7 +1068,7 @@ __device__ __forceinline__ void lane_share(uint64_t N, uint64_t& g0, uint64_t& g
 // warp, one leaf per lane: a lane keeps its partial while it stays on one
 // query and adds it atomically when it leaves it (the functions commute); a
 // warp whose lanes end on one query adds once.
-template <int OP, bool PLAIN>
+template <int OP, bool PLAIN, unsigned TL>
 __global__ void __launch_bounds__(kT) k_range_inner(Leaves t, Reduce<OP, PLAIN> f, uint64_t q,
                                                     const uint64_t* __restrict__ first,
                                                     const uint64_t* __restrict__ off, LeafPrefix p,
@@ -1070,33 +1095,33 @@ __global__ void __launch_bounds__(kT) k_range_inner(Leaves t, Reduce<OP, PLAIN> 
     return;
   }
   const unsigned lane = lane_id();
-  if (N * kTeam * 4 <= gstride()) {  // few: a team per item
-    const uint64_t e0 = ((uint64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * (32 / kTeam);
+  if (N * kTeam * 4 <= gstride() && N * TL <= gstride()) {  // few: a team per item
+    const uint64_t e0 = ((uint64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * (32 / TL);
     if (e0 >= N) return;
-    const uint64_t e = e0 + lane / kTeam;
+    const uint64_t e = e0 + lane / TL;
     uint64_t qi = 0, j = 0;
     uint32_t u = 0, idx;
     if (e < N) {
-      qi = team_upper_count(off, q + 1, e) - 1;
+      qi = team_upper_count<TL>(off, q + 1, e) - 1;
       j = first[qi] + (e - off[qi]);
       u = min(t.used[j], t.LB);
     }
     __syncwarp();
     const uint8_t* leafp = t.data + j * t.LB;
-    const leafwalk::Run run = team_leaf(leafp, u, idx);
+    const leafwalk::Run run = team_leaf<TL>(leafp, u, idx);
     uint64_t r = op_identity<OP>(), c = 0;
     auto take = [&](uint64_t v) {
       if (PLAIN || (v & f.mask) == f.value) { r = op_apply<OP>(r, v); c++; }
     };
-    if (u && team_lane() == 0) take(run.k.val);
+    if (u && team_lane<TL>() == 0) take(run.k.val);
     leafwalk::run_visit(leafp, u, run, take);
     __syncwarp();
-    team_reduce<OP>(r, c);
-    if (team_lane() == 0 && c) {
+    team_reduce<OP, TL>(r, c);
+    if (team_lane<TL>() == 0 && c) {
       op_atomic<OP>(&out[qi], r);
       atomicAdd((ull*)&count[qi], (ull)c);
     }
-    if (prof && team_lane() == 0 && u) atomicAdd(prof, (ull)u);
+    if (prof && team_lane<TL>() == 0 && u) atomicAdd(prof, (ull)u);
     return;
   }
   uint64_t g0, g1;
@@ -1409,13 +1434,34 @@ __global__ void __launch_bounds__(kT, 4) k_sum(const uint8_t* __restrict__ data,
 
 int persistent_grid(const cpma* h) { return h->num_sms * 8; }
 
-// Few enough queries for a team of lanes per leaf.  A team spends about twice
-// a thread's instructions on a leaf in a third of its time.  Team / thread per
-// leaf, us (about 35 of them the call's own), 1e7 keys: masked ranges of 50
-// elements, 1e3 queries 36 / 52, 1e4 47 / 57, 4e4 74 / 70; plain ones 38 / 42,
-// 45 / 44, 72 / 53; scans by length 33 / 43, 42 / 49, 84 / 66.  With leaves of
-// 2048 bytes masked ones, 1e4 queries, 60 / 63 and 2e4 93 / 69.
-bool few_queries(const cpma* h, uint64_t q) { return q <= (uint64_t)h->num_sms * 64; }
+bool large_leaves(const cpma* h) { return h->cfg.leaf_bytes > 512; }
+
+// Few enough queries for a team of lanes per leaf instead of a thread: a team
+// spends about twice a thread's instructions on a leaf in a fraction of its time.
+// Speed of teams over threads, geometric mean over sets of 300 to 1e7 keys of 1 to
+// 6 bytes and short and wide queries (lowest, highest): ranges with a mask, 512-byte
+// leaves, 9.8e3 queries 1.47 (1.23, 1.66), 1.5e4 1.33, 2.5e4 1.08 (0.90, 1.26), 4e4
+// 0.92; plain ones 1.39, 1.28, 1.02, 0.86; scans by length 1.12, 0.99, 0.81, 0.71;
+// 256-byte leaves within 0.1 of these.  2048-byte leaves, 1.5e4 and 2.5e4 queries:
+// ranges 1.27 and about 1, scans by length 0.9 and 0.7.
+bool few_ranges(const cpma* h, uint64_t q) { return q <= (uint64_t)h->num_sms * 160; }
+bool few_scans(const cpma* h, uint64_t q) {
+  return q <= (uint64_t)h->num_sms * (large_leaves(h) ? 64 : 96);
+}
+// A lookup is half a range.  2048-byte leaves, 4e3 keys 12 to 15 us by teams and 14
+// to 23 by threads, 9e3 21 to 25 and 19 to 83; 512-byte ones, 4e3 keys 8 to 12 and
+// 10 to 27.
+bool few_lookups(const cpma* h, uint64_t q) {
+  return q <= (uint64_t)h->num_sms * (large_leaves(h) ? 48 : 32);
+}
+
+// A team is a warp where a leaf has more than 512 bytes and the queries are few
+// enough for that.  Speed of warps over eight lanes, 1e3, 2.5e3, 5e3, 9.7e3 queries:
+// 2048-byte leaves, ranges 1.15, 1.11, 1.04, 0.94, scans by length 1.51, 1.36, 1.15,
+// 0.96; 1024-byte ones 1.07, 1.02, 0.96, 0.88 and 1.30, 1.21, 1.06, 0.92.
+bool warp_teams(const cpma* h, uint64_t q) {
+  return large_leaves(h) && q <= (uint64_t)h->num_sms * 24;
+}
 
 // Scratch of the allocation-free range_map: per-query first leaf, item count
 // and item offsets, plus the partial sums of the offset scan.  It lives in the
@@ -1471,14 +1517,14 @@ bool extract_by_warps(const cpma* h, uint64_t q) {
 
 int run_has(const cpma* h, const uint64_t* d_keys, uint64_t q, uint8_t* d_out, cudaStream_t st) {
   if (q == 0) return CPMA_OK;
-  // (a lookup is half a range: 2048-byte leaves, 4e3 keys 15 us by teams and
-  // 19 by threads, 9e3 21 and 19)
-  const bool few = !h->cfg.codec && few_queries(h, 2 * q);
-  const uint64_t per = few ? kT / kTeam : kT;  // keys a block
+  const bool few = !h->cfg.codec && few_lookups(h, q);
+  const uint64_t per = few ? kT / (warp_teams(h, q) ? kTeamLarge : kTeam) : kT;  // keys a block
   const int grid = (int)std::max<uint64_t>(
       1, std::min<uint64_t>((q + per - 1) / per, (uint64_t)persistent_grid(h)));
   prof_begin(h, PH_HAS, st);
-  const auto kern = h->cfg.codec ? k_has_cells : few ? k_has_team : k_has;
+  const auto kern = h->cfg.codec ? k_has_cells
+                    : !few       ? k_has
+                    : warp_teams(h, q) ? k_has_team<kTeamLarge> : k_has_team<kTeam>;
   kern<<<grid, kT, 0, st>>>(d_keys, q, h->data, h->used, h->heads, h->L, h->cfg.leaf_bytes, d_out,
                             prof_bytes(h, PH_HAS));
   CPMA_LAUNCHED(h);
@@ -1622,7 +1668,7 @@ int range_scratch(cpma* h, uint64_t q, RangeScratch* r) {
 // carries nothing over from one call to the next.
 EndsScan ends_scan(const cpma* h, const RangeScratch& r, uint64_t q) {
   EndsScan z;
-  if (r.done && few_queries(h, q) && q <= kEndsScan) {
+  if (r.done && few_ranges(h, q) && few_scans(h, q) && q <= kEndsScan) {
     z.off = r.off;
     z.done = r.done;
   }
@@ -1648,8 +1694,10 @@ int range_inner(cpma* h, Reduce<OP, PLAIN> f, uint64_t q, uint64_t* out, uint64_
     CPMA_CUDA(launch_pdl(k_leaf_prefix<OP, PLAIN>, g, kT, 0, st, t, f, total, p, prof));
     h->launches++;
   }
-  CPMA_CUDA(launch_pdl(k_range_inner<OP, PLAIN>, (unsigned)persistent_grid(h), kT, 0, st, t, f, q,
-                       r.first, r.off, p, out, count, prof));
+  CPMA_CUDA(launch_pdl(large_leaves(h) ? k_range_inner<OP, PLAIN, kTeamLarge>
+                                       : k_range_inner<OP, PLAIN, kTeam>,
+                       (unsigned)persistent_grid(h), kT, 0, st, t, f, q, r.first, r.off, p, out,
+                       count, prof));
   CPMA_LAUNCHED(h);
   return check_cuda(cudaGetLastError());
 }
@@ -1659,8 +1707,10 @@ int range_leaves(cpma* h, const uint64_t* lo, const uint64_t* hi, uint64_t q, ui
                  uint64_t value, uint64_t* out, uint64_t* count, const RangeScratch& r,
                  const LeafPrefix& p, cudaStream_t st, ull* prof) {
   const Reduce<OP, PLAIN> f{mask, value};
-  if (few_queries(h, q)) {
-    k_range_ends_team<OP, PLAIN><<<query_grid(h, 2 * q * kTeam, 64, 32), 64, 0, st>>>(
+  if (few_ranges(h, q)) {
+    const auto kern = warp_teams(h, q) ? k_range_ends_team<OP, PLAIN, kTeamLarge>
+                                      : k_range_ends_team<OP, PLAIN, kTeam>;
+    kern<<<query_grid(h, q * (warp_teams(h, q) ? kTeamLarge : 2 * kTeam), 64, 32), 64, 0, st>>>(
         lo, hi, q, leaves_of(h), f, r.first, r.items, out, count, p.ticket, ends_scan(h, r, q),
         prof);
   } else {
@@ -1780,13 +1830,14 @@ int run_range_length(const cpma* h, const uint64_t* start, const uint64_t* lengt
     const LeafPrefix p = leaf_prefix(hm, q, st);
     ull* prof = prof_bytes(h, PH_RANGE);
     prof_begin(h, PH_RANGE, st);
-    const bool few = few_queries(h, q);
+    const bool few = few_scans(h, q);
     const int b = few ? 64 : query_block(h, q);
-    const int g = few ? query_grid(h, q * kTeam, b, 32) : query_grid(h, q, b, 8);
+    const int g = few ? query_grid(h, q * (warp_teams(h, q) ? kTeamLarge : kTeam), b, 32) : query_grid(h, q, b, 8);
     if (few)
-      CPMA_CUDA(launch_pdl(k_length_ends_team, (unsigned)g, (unsigned)b, 0, st, start, length, q,
-                           leaves_of(h), P, r.first, r.items, sum, count, p.ticket,
-                           ends_scan(h, r, q), prof));
+      CPMA_CUDA(launch_pdl(warp_teams(h, q) ? k_length_ends_team<kTeamLarge>
+                                           : k_length_ends_team<kTeam>,
+                           (unsigned)g, (unsigned)b, 0, st, start, length, q, leaves_of(h), P,
+                           r.first, r.items, sum, count, p.ticket, ends_scan(h, r, q), prof));
     else
       CPMA_CUDA(launch_pdl(k_length_ends, (unsigned)g, (unsigned)b, 0, st, start, length, q,
                            leaves_of(h), P, r.first, r.items, sum, count, p.ticket, prof));
