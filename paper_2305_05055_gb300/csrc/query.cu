@@ -1606,12 +1606,18 @@ LeafPrefix leaf_prefix(cpma* h, uint64_t q, cudaStream_t st) {
 // a query per two leaves, per leaf, two and four per leaf: uniform 40-bit keys
 // (1.9e5 leaves, ranges of 32 elements) 73 / 66, 87 / 94, 106 / 160, 151 / 312;
 // edges (1.4e5 leaves, adjacent ranges) 59 / 75, 63 / 118, 78 / 180, 101 / 281.
+// On small sets a few queries are done before the leaves are marked: up to 478
+// leaves of 512 bytes, 100 queries 31 / 23, 1000 31 / 26 short and 32 / 38 wide ones;
+// 117 leaves of 2048 bytes 35 / 25 and 35 / 35 at 2500, 35 / 44 and 35 / 57 at 9700;
+// 9.5e3 of them (edges) 98 / 56 and 101 / 83, at 1.4e4 98 / 74 and 100 / 101.
 // The memory they take is that of the leaves again; without room for it the
 // queries walk.
 uint32_t marks_per_leaf(const cpma* h) {
   return (h->cfg.leaf_bytes + leafwalk::kMark - 1) / leafwalk::kMark;
 }
-bool marks_pay(const cpma* h, uint64_t q) { return q >= 2 && q >= h->L; }
+bool marks_pay(const cpma* h, uint64_t q) {
+  return q >= h->L && q > (uint64_t)h->num_sms * (large_leaves(h) ? 48 : 4);
+}
 size_t marks_bytes(const cpma* h) {
   return h->L * marks_per_leaf(h) * sizeof(leafwalk::Mark) + (h->L + kT - 1) / kT * 16;
 }
