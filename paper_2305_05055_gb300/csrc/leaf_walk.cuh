@@ -782,11 +782,12 @@ struct Run {
   Walk k;               // at byte b0; val 0 until the scan over the team
   uint32_t b0, b1;      // the lane's bytes
   uint64_t delta = 0;   // what its codes add up to
+  uint64_t sum = 0;     // SUM: its elements', less the element before the run
   uint32_t codes = 0;
 };
 
 // Lane tl's run (of N) of a leaf of u used bytes (0: no leaf).
-template <uint32_t N = kTeam>
+template <uint32_t N = kTeam, bool SUM = false>
 LT_HD Run team_run(const uint8_t* leafp, uint32_t u, uint32_t tl) {
   const uint32_t per = 16u * (((u + 15u) / 16u + N - 1u) / N);
   Run r;
@@ -804,12 +805,16 @@ LT_HD Run team_run(const uint8_t* leafp, uint32_t u, uint32_t tl) {
   r.k = k;
   for (uint32_t p0 = r.b0; p0 < r.b1; p0 += 16) {
     load_chunk(leafp, p0, u, w, t);
+    uint64_t v = k.val;
     if (p0) {
       group_sum(w[0], w[1], t[0], t[1], k, T, ss);
       r.codes += T;
+      if (SUM) r.sum += T * v + ss;
     }
+    v = k.val;
     group_sum(w[2], w[3], t[2], t[3], k, T, ss);
     r.codes += T;
+    if (SUM) r.sum += T * v + ss;
   }
   r.delta = k.val;
   return r;

@@ -105,11 +105,11 @@ __device__ __forceinline__ uint64_t team_route(const uint64_t* __restrict__ head
 
 // The lane's run with the element before it (in k.val) and the number of
 // elements before it (the head included); a whole warp calls.
-template <unsigned N>
+template <unsigned N, bool SUM = false>
 __device__ __forceinline__ leafwalk::Run team_leaf(const uint8_t* leafp, uint32_t u,
                                                    uint32_t& idx) {
   const unsigned tl = team_lane<N>();
-  leafwalk::Run r = leafwalk::team_run<N>(leafp, u, tl);
+  leafwalk::Run r = leafwalk::team_run<N, SUM>(leafp, u, tl);
   __syncwarp();
   uint64_t d = r.delta;
   uint32_t n = r.codes;
@@ -994,13 +994,55 @@ __global__ void __launch_bounds__(kT) k_tile_scan(LeafPrefix p, uint64_t nt) {
   tile_scan<CPMA_OP_SUM>(p, nt, s_ws);
 }
 
-// Every leaf reduced once, scanned inside tiles of kT leaves, and the tiles by
-// the last block to finish (when the queries cover more than p.most leaves;
-// otherwise nothing).
+// The reductions and counts of the leaves by eight lanes each, for sets of few
+// leaves (sum_by_teams), to p.val and p.cnt.
+template <int OP, bool PLAIN>
+__global__ void __launch_bounds__(kT) k_leaf_reduce(Leaves t, Reduce<OP, PLAIN> f,
+                                                    const uint64_t* __restrict__ total,
+                                                    LeafPrefix p, ull* prof) {
+  pdl_wait();
+  pdl_launch();
+  if (*total <= p.most) return;
+  const unsigned tl = team_lane<kTeam>();
+  ull nbytes = 0;
+  for (uint64_t j0 = (gtid() >> 5) * (32 / kTeam); j0 < t.L; j0 += (gstride() >> 5) * (32 / kTeam)) {
+    const uint64_t j = j0 + lane_id() / kTeam;
+    const uint32_t u = j < t.L ? min(t.used[j], t.LB) : 0u;
+    const uint8_t* leafp = t.data + (j < t.L ? j : 0) * t.LB;
+    uint32_t idx;
+    const leafwalk::Run run = team_leaf<kTeam, PLAIN>(leafp, u, idx);
+    uint64_t r = op_identity<OP>(), c = 0;
+    if constexpr (PLAIN) {
+      if (u) {
+        r = run.codes * run.k.val + run.sum + (tl == 0 ? run.k.val : 0ull);
+        c = run.codes + (tl == 0 ? 1u : 0u);
+      }
+    } else {
+      auto take = [&](uint64_t v) {
+        if ((v & f.mask) == f.value) { r = op_apply<OP>(r, v); c++; }
+      };
+      if (u && tl == 0) take(run.k.val);
+      leafwalk::run_visit(leafp, u, run, take);
+      __syncwarp();
+    }
+    team_reduce<OP, kTeam>(r, c);
+    if (tl == 0 && j < t.L) {
+      p.val[j] = r;
+      p.cnt[j] = (uint32_t)c;
+      nbytes += u;
+    }
+  }
+  nbytes = warp_sum(nbytes);
+  if (prof && lane_id() == 0 && nbytes) atomicAdd(prof, nbytes);
+}
+
+// Every leaf reduced once (GIVEN: k_leaf_reduce has done it), scanned inside tiles
+// of kT leaves, and the tiles by the last block to finish (when the queries cover
+// more than p.most leaves; otherwise nothing).
 // Four blocks per SM: the lanes' scattered loads are what it waits for (plain,
 // 1e8 keys: 106 us with the registers it would take, 76 us; masked sums, 5e7
 // keys: 157 and 109 us).
-template <int OP, bool PLAIN>
+template <int OP, bool PLAIN, bool GIVEN>
 __global__ void __launch_bounds__(kT, 4) k_leaf_prefix(Leaves t, Reduce<OP, PLAIN> f,
                                                     const uint64_t* __restrict__ total,
                                                     LeafPrefix p, ull* prof) {
@@ -1015,11 +1057,11 @@ __global__ void __launch_bounds__(kT, 4) k_leaf_prefix(Leaves t, Reduce<OP, PLAI
   for (uint64_t tile = blockIdx.x; tile < nt; tile += gridDim.x) {
     const uint64_t j0 = tile * kT, j = j0 + threadIdx.x;
     const uint32_t n = (uint32_t)min((uint64_t)kT, t.L - j0);
-    order_tile(threadIdx.x < n ? min(t.used[j], t.LB) : 0u, n, s_hist, s_order);
-    s_r[threadIdx.x] = op_identity<OP>();
-    s_c[threadIdx.x] = 0;
+    if (!GIVEN) order_tile(threadIdx.x < n ? min(t.used[j], t.LB) : 0u, n, s_hist, s_order);
+    s_r[threadIdx.x] = GIVEN && threadIdx.x < n ? p.val[j] : op_identity<OP>();
+    s_c[threadIdx.x] = GIVEN && threadIdx.x < n ? p.cnt[j] : 0;
     __syncthreads();
-    if (threadIdx.x < n) {
+    if (!GIVEN && threadIdx.x < n) {
       const uint32_t o = s_order[threadIdx.x];
       const uint32_t u = min(t.used[j0 + o], t.LB);
       uint64_t r = op_identity<OP>(), c = 0;
@@ -1432,6 +1474,37 @@ __global__ void __launch_bounds__(kT, 4) k_sum(const uint8_t* __restrict__ data,
   if (prof && lane == 0 && nbytes) atomicAdd(prof, nbytes + (raw ? 8ull * (j1 - j0) : 0ull));
 }
 
+// The same of byte codes by eight lanes per leaf, for sets of few leaves: bound by
+// the walk of the longest run.
+__global__ void __launch_bounds__(kT) k_sum_team(const uint8_t* __restrict__ data,
+                                                 const uint32_t* __restrict__ used,
+                                                 const uint32_t* __restrict__ cnt, uint64_t L,
+                                                 uint32_t LB, uint64_t* sum, uint64_t* count,
+                                                 ull* prof) {
+  const unsigned tl = team_lane<kTeam>();
+  uint64_t s = 0, c = 0;
+  ull nbytes = 0;
+  for (uint64_t j0 = (gtid() >> 5) * (32 / kTeam); j0 < L; j0 += (gstride() >> 5) * (32 / kTeam)) {
+    const uint64_t j = j0 + lane_id() / kTeam;
+    const uint32_t u = j < L ? min(used[j], LB) : 0u;
+    uint32_t idx;
+    const leafwalk::Run r = team_leaf<kTeam, true>(data + (j < L ? j : 0) * LB, u, idx);
+    if (u) s += r.codes * r.k.val + r.sum + (tl == 0 ? r.k.val : 0ull);
+    if (j < L && tl == 0) {
+      nbytes += 8 + u;  // its used and element counts
+      if (u) c += cnt[j];
+    }
+  }
+  s = warp_sum(s);
+  c = warp_sum(c);
+  nbytes = warp_sum(nbytes);
+  if (lane_id() == 0 && (s | c)) {
+    atomicAdd((ull*)sum, (ull)s);
+    if (count) atomicAdd((ull*)count, (ull)c);
+  }
+  if (prof && lane_id() == 0 && nbytes) atomicAdd(prof, nbytes);
+}
+
 int persistent_grid(const cpma* h) { return h->num_sms * 8; }
 
 bool large_leaves(const cpma* h) { return h->cfg.leaf_bytes > 512; }
@@ -1461,6 +1534,15 @@ bool few_lookups(const cpma* h, uint64_t q) {
 // 0.96; 1024-byte ones 1.07, 1.02, 0.96, 0.88 and 1.30, 1.21, 1.06, 0.92.
 bool warp_teams(const cpma* h, uint64_t q) {
   return large_leaves(h) && q <= (uint64_t)h->num_sms * 24;
+}
+
+// Whether a full sum takes eight lanes per leaf: while that many threads run at
+// once (half of them for large leaves, where a lane's own walk is long).  Eight
+// lanes / one, us: 512-byte leaves 4.3e3 of them 16.5 / 22.7, 3.9e4 (edges) 29 / 45,
+// 1.2e5 43 / 28; 2048-byte ones 9.5e3 (edges) 30 / 114, 2.8e4 34 / 57, 1.4e5 100 / 91.
+bool sum_by_teams(const cpma* h) {
+  const uint64_t threads = (uint64_t)persistent_grid(h) * kT;
+  return !h->cfg.codec && h->L * kTeam <= threads * (large_leaves(h) ? 2 : 1);
 }
 
 // Scratch of the allocation-free range_map: per-query first leaf, item count
@@ -1697,7 +1779,14 @@ int range_inner(cpma* h, Reduce<OP, PLAIN> f, uint64_t q, uint64_t* out, uint64_
   if (p.val) {
     const unsigned g = (unsigned)std::min<uint64_t>(nt, (uint64_t)persistent_grid(h));
     const uint64_t* total = r.off + q;
-    CPMA_CUDA(launch_pdl(k_leaf_prefix<OP, PLAIN>, g, kT, 0, st, t, f, total, p, prof));
+    const bool teams = large_leaves(h) && sum_by_teams(h);
+    if (teams) {
+      CPMA_CUDA(launch_pdl(k_leaf_reduce<OP, PLAIN>, (unsigned)query_grid(h, t.L * kTeam, kT, 8),
+                           kT, 0, st, t, f, total, p, prof));
+      h->launches++;
+    }
+    CPMA_CUDA(launch_pdl(teams ? k_leaf_prefix<OP, PLAIN, true> : k_leaf_prefix<OP, PLAIN, false>,
+                         g, kT, 0, st, t, f, total, p, prof));
     h->launches++;
   }
   CPMA_CUDA(launch_pdl(large_leaves(h) ? k_range_inner<OP, PLAIN, kTeamLarge>
@@ -2023,7 +2112,11 @@ int run_sum(const cpma* h, uint64_t* sum, uint64_t* count, cudaStream_t st) {
   CPMA_CUDA(cudaMemsetAsync(sum, 0, 8, st));
   if (count) CPMA_CUDA(cudaMemsetAsync(count, 0, 8, st));
   prof_begin(h, PH_SUM, st);
-  k_sum<<<persistent_grid(h), kT, 0, st>>>(h->data, h->used, h->cnt, h->heads, h->L,
+  if (sum_by_teams(h))
+    k_sum_team<<<query_grid(h, h->L * kTeam, kT, 8), kT, 0, st>>>(
+        h->data, h->used, h->cnt, h->L, h->cfg.leaf_bytes, sum, count, prof_bytes(h, PH_SUM));
+  else
+    k_sum<<<persistent_grid(h), kT, 0, st>>>(h->data, h->used, h->cnt, h->heads, h->L,
                                            h->cfg.leaf_bytes, sum, count, prof_bytes(h, PH_SUM), (int)h->cfg.codec);
   CPMA_LAUNCHED(h);
   prof_end(h, st);

@@ -26,7 +26,7 @@ def lt(tmp_path_factory):
                     os.path.join(HERE, "leaf_team_host.cu")], check=True)
     lib = C.CDLL(out)
     lib.lt_team.restype = C.c_uint32
-    lib.lt_team.argtypes = [C.c_void_p, C.c_uint32, C.c_int, C.POINTER(C.c_uint64)]
+    lib.lt_team.argtypes = [C.c_void_p, C.c_uint32, C.c_int, C.c_int, C.POINTER(C.c_uint64)]
     return lib
 
 
@@ -48,5 +48,6 @@ def test_runs_of_a_team(lt, LB, lanes):
         leaf, u = oracle.leaf_encode(np.array(keys, np.uint64), LB)
         buf = (C.c_uint8 * (LB + 16)).from_buffer_copy(bytes(leaf) + bytes(16))
         out = (C.c_uint64 * (len(keys) + 64))()
-        assert lt.lt_team(buf, u, lanes, out) == len(keys), u
-        assert list(out[:len(keys)]) == keys
+        for s in (0, 1):
+            assert lt.lt_team(buf, u, lanes, s, out) == len(keys), (u, s)
+            assert list(out[:len(keys)]) == keys
