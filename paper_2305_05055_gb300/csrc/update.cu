@@ -422,6 +422,7 @@ struct MergeArgs {
   uint32_t* list_long;   // leaves for k_insert_thread_long (st->n_long)
   int raw;               // leaves hold 8-byte cells (codec 1), not byte codes
   int small;             // a small batch: every slice goes to a warp per leaf
+  int long_warp;         // so does a leaf with a code of more than 4 bytes (long_by_warp)
   Bounds B;              // density bounds and tree height, for the leaves the
   unsigned H;            // thread-granular merge finalises itself
   uint32_t* viol;        // touched leaves over their own bound (count st->nviol)
@@ -1432,7 +1433,12 @@ __global__ void __launch_bounds__(kThrT, 4) k_insert_thread(MergeArgs a) {
                            leafp, y, S, res, R, nbytes, dl, db);
       }
     }
-    warp_append(lng != 0xFFFFFFFFu, lng, a.list_long, &a.st->n_long);
+    if (a.long_warp) {
+      if (lng != 0xFFFFFFFFu) a.T_state[lng] = kFallback;
+      warp_append(lng != 0xFFFFFFFFu, lng, a.list_v1, &a.st->n_v1);
+    } else {
+      warp_append(lng != 0xFFFFFFFFu, lng, a.list_long, &a.st->n_long);
+    }
     dl = warp_sum(dl);
     db = warp_sum(db);
     if (lane_id() == 0) {
@@ -3303,6 +3309,19 @@ void merge_attrs() {
   done = true;
 }
 
+// Whether leaves with a code of more than 4 bytes go to a warp each
+// (k_merge_small) instead of a thread (k_insert_thread_long).  A thread's chain over
+// a leaf of more than 512 bytes is longer than what the warps take for all of them
+// while those are few, and for the few slices of at most four keys of a batch with
+// more keys per leaf.  Insert and delete by warps / threads, us, 2048-byte leaves:
+// edges, 9.5e3 leaves, 1e4 keys 349 / 469, 1e5 556 / 716, 3e5 1026 / 1041; 64-bit
+// keys, 1.9e4 leaves, 2e4 keys 383 / 405, 1e5 531 / 606; 6.4e4 leaves, 2e4 keys 422 /
+// 362, 1e5 968 / 584, 1e6 1589 / 1729.
+bool long_by_warp(const cpma* h, uint64_t k) {
+  return h->cfg.leaf_bytes > 512 &&
+         (std::min<uint64_t>(k, h->L) < (uint64_t)h->num_sms * 128 || k > 4 * h->L);
+}
+
 // The thread-granular insert (or delete) over the touched leaves of a batch
 // of k keys (at most k of them).
 template <bool DEL>
@@ -3310,10 +3329,12 @@ int launch_insert_thread(cpma* h, const MergeArgs& ma, uint64_t k, cudaStream_t 
   const int g = (int)std::max<uint64_t>(
       1, std::min<uint64_t>((k + kThrT - 1) / kThrT, (uint64_t)h->num_sms * 16));
   k_insert_thread<DEL><<<g, kThrT, 0, st>>>(ma);
+  h->launches++;
+  if (ma.long_warp) return check_cuda(cudaGetLastError());
   const unsigned gl = (unsigned)std::max<uint64_t>(
       1, std::min<uint64_t>((k + kLongT - 1) / kLongT, (uint64_t)h->num_sms * 8));
   const cudaError_t e = launch_pdl(k_insert_thread_long<DEL>, gl, kLongT, 0, st, ma);
-  h->launches += 2;
+  h->launches++;
   return check_cuda(e);
 }
 
@@ -3518,6 +3539,7 @@ int run_front(cpma* h, const uint64_t* d_keys, uint64_t k, int sorted, int is_de
   ma.list_long = P<uint32_t>(s.list_long);
   ma.raw = (int)h->cfg.codec;
   ma.small = k <= kSmallBatch ? 1 : 0;
+  ma.long_warp = long_by_warp(h, k) ? 1 : 0;
   ma.B = B;
   ma.H = H;
   ma.viol = P<uint32_t>(s.viol);
@@ -3534,12 +3556,25 @@ int run_front(cpma* h, const uint64_t* d_keys, uint64_t k, int sorted, int is_de
     // few leaves are latency-bound.  Without a thread-granular merge there is
     // nothing to run beside them, and the fork and join cost 3 us each (tagged
     // insert and delete of 1e3 keys 138 us, 131 without).
-    const bool thread = !ma.raw && !ma.small;
-    const cudaStream_t side = thread ? h->side : st;
     const size_t sper = small_warp_bytes(LB);
     const int swarps = (int)std::max<size_t>(1, std::min<size_t>(8, (216 * 1024) / (4 * sper)));
     const int sgrid = (int)std::max<uint64_t>(
         1, std::min<uint64_t>((k + swarps - 1) / swarps, (uint64_t)h->num_sms * 8));
+    const bool thread = !ma.raw && !ma.small;
+    const cudaStream_t side = thread ? h->side : st;
+    // (the leaves that the thread kernel leaves to a warp come after it)
+    const bool late = thread && ma.long_warp;
+    auto others = [&](cudaStream_t on) -> int {
+      prof_begin_side(h, PH_MERGE2, on);
+      ma.prof = prof_bytes(h, PH_MERGE2);
+      k_merge_small<<<sgrid, swarps * 32, sper * swarps, on>>>(ma);
+      ma.prof = nullptr;
+      CPMA_CUDA(launch_pdl(k_merge<false>, (unsigned)mgrid, (unsigned)(mwarps * 32), msmem, on,
+                           ma));
+      h->launches += 2;
+      prof_end_side(h, on);
+      return CPMA_OK;
+    };
     if (thread) {
       CPMA_CUDA(cudaEventRecord(h->ev_fork, st));
       CPMA_CUDA(cudaStreamWaitEvent(side, h->ev_fork, 0));
@@ -3555,14 +3590,8 @@ int run_front(cpma* h, const uint64_t* d_keys, uint64_t k, int sorted, int is_de
       h->launches++;
     }
     prof_end_side(h, side);
-    prof_begin_side(h, PH_MERGE2, side);
-    ma.prof = prof_bytes(h, PH_MERGE2);
-    k_merge_small<<<sgrid, swarps * 32, sper * swarps, side>>>(ma);
     ma.prof = nullptr;
-    CPMA_CUDA(launch_pdl(k_merge<false>, (unsigned)mgrid, (unsigned)(mwarps * 32), msmem, side,
-                         ma));
-    h->launches += 2;
-    prof_end_side(h, side);
+    if (!late) CPMA_TRY(others(side));
     if (thread) {
       CPMA_CUDA(cudaEventRecord(h->ev_join, side));
       prof_begin(h, PH_MERGE, st);
@@ -3572,6 +3601,8 @@ int run_front(cpma* h, const uint64_t* d_keys, uint64_t k, int sorted, int is_de
       ma.prof = nullptr;
       CPMA_CUDA(cudaStreamWaitEvent(st, h->ev_join, 0));
     }
+    prof_end(h, st);
+    if (late) CPMA_TRY(others(st));
   }
   CPMA_CUDA(cudaGetLastError());
   prof_end(h, st);
