@@ -48,6 +48,8 @@ class cpma_config(C.Structure):
 def lib():
     """Load libcpma.so (building it first when the sources are newer)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             path = _build.LIB
@@ -110,8 +112,8 @@ def _check(rc: int, what: str):
 
 
 def _stream(stream=None) -> int:
-    if stream is None:
-        stream = torch.cuda.current_stream()
+    if stream is None:  # (without a Stream object: a small call is bound by its host side)
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
@@ -124,7 +126,7 @@ def _keys(t, name="keys") -> torch.Tensor:
 
 
 def _ptr(t):
-    return C.c_void_p(t.data_ptr()) if t is not None and t.numel() else None
+    return t.data_ptr() if t is not None and t.numel() else None
 
 
 def to_u64(t: torch.Tensor) -> np.ndarray:
