@@ -208,9 +208,10 @@ int cpma_has_batch(const cpma_t* h, const uint64_t* d_keys, uint64_t q,
  * entries).  lo >= hi gives 0 and 0.  The queries' end leaves are
  * decoded, the leaves between them walked in equal shares; when two or more
  * queries together cover more leaves than the set has, every leaf is reduced
- * once instead (12 bytes of scratch per leaf), and from a query per leaf on the
- * walk of every leaf is kept at each 32nd byte (as much scratch as leaves) and
- * a query looks up its two ends.  Without memory for either (budget, less than
+ * once instead (12 bytes of scratch per leaf), and from a query per leaf on, if
+ * that is also more than 4 (48 with leaves over 512 bytes) per SM, the walk
+ * of every leaf is kept at each 32nd byte (as much scratch as leaves) and a
+ * query looks up its two ends.  Without memory for either (budget, less than
  * twice as much free on the device, a stream being captured) the queries walk:
  * same results.  The scratch is held by the handle and given back when another
  * call on it needs the memory, or by cpma_set_mem_budget. */

@@ -46,9 +46,9 @@ __device__ __forceinline__ uint64_t gstride() { return (uint64_t)gridDim.x * blo
 
 // Byte codes: a thread per query key routes it and searches its leaf
 // (leafthr::leaf_has) up to the key.  Bound by instruction issue: a warp runs
-// as long as its deepest search.  1e6 keys against 1e8: 156 us, 195 us when the
-// leaf was decoded code by code.  (A block ordering its 256 keys by how deep
-// each is likely to lie: 154 us, and 1.9 us more on 1e3 keys.)
+// as long as its deepest search.  1e6 keys against 1e8: 136 to 141 us, 195 us when
+// the leaf was decoded code by code.  (At 156 us, a block ordering its 256 keys by
+// how deep each is likely to lie: 154 us, and 1.9 us more on 1e3 keys.)
 __global__ void __launch_bounds__(kT) k_has(const uint64_t* __restrict__ keys, uint64_t q,
                                             const uint8_t* __restrict__ data,
                                             const uint32_t* __restrict__ used,
@@ -1521,9 +1521,13 @@ bool few_ranges(const cpma* h, uint64_t q) { return q <= (uint64_t)h->num_sms * 
 bool few_scans(const cpma* h, uint64_t q) {
   return q <= (uint64_t)h->num_sms * (large_leaves(h) ? 64 : 96);
 }
-// A lookup is half a range.  2048-byte leaves, 4e3 keys 12 to 15 us by teams and 14
-// to 23 by threads, 9e3 21 to 25 and 19 to 83; 512-byte ones, 4e3 keys 8 to 12 and
-// 10 to 27.
+// A lookup is half a range.  Calls in a row over different batches of 1 to 4000 keys,
+// us a call by teams / by threads, sets of 34- and 40-bit keys, of 64-bit ones and of
+// edges: 256-byte leaves 6 to 8 / 6 to 9, 6 to 9 / 10 to 12, 6 to 10 / 8 to 17; 512-byte
+// ones 6 to 8 / 7 to 10, 8 to 10 / 12 to 17, 7 to 12 / 9 to 27; 1024-byte ones 6 to 10 /
+// 8 to 13, 6 to 12 / 17 to 27, 6 to 16 / 17 to 45; 2048-byte ones 6 to 15 / 11 to 19, 7
+// to 17 / 33 to 47, 6 to 24 / 21 to 84.  7000 of them: 2048-byte leaves 20 / 19, 21 /
+// 47, 30 / 83, 1024-byte ones 14 / 13, 14 / 27, 19 / 46.
 bool few_lookups(const cpma* h, uint64_t q) {
   return q <= (uint64_t)h->num_sms * (large_leaves(h) ? 48 : 32);
 }

@@ -1320,11 +1320,11 @@ __device__ __forceinline__ void thread_finish(const MergeArgs& a, uint32_t t, ui
 // DEL: the same for deletes of at most kThrKeys keys from a byte-code leaf
 // (plan_delete, forward rewrite; never over LB bytes).
 // Bound by instruction issue at half the lanes (ncu: 0.63 issued per cycle and
-// scheduler, 14.6 threads each).  1e6 keys into 1e8: 197 us, out of it 189 us
+// scheduler, 16.9 threads each).  1e6 keys into 1e8: 197 us, out of it 189 us
 // (238 and 191 with 16-byte loads in pass A and word loads in the rewrite);
 // with each thread placing its own leaf's keys 254 and 224 us.  (Sorting the
 // block's leaves once more, by chunks to rewrite: 245 and 225 us.)
-// Four blocks per SM (64 registers, a few spilled) ran faster than three with
+// Four blocks per SM (64 registers, none spilled) ran faster than three with
 // 80 (254 against 257 and 219 against 237 us before) and than five (271, 240).
 template <bool DEL>
 __global__ void __launch_bounds__(kThrT, 4) k_insert_thread(MergeArgs a) {
