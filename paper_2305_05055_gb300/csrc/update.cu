@@ -419,10 +419,10 @@ struct MergeArgs {
   uint32_t* list_v1;     // touched leaves for k_merge_small (count st->n_v1)
   uint32_t* list_gen;    // work items for k_merge in count mode (st->n_gen)
   uint32_t* list_pend;   // pending leaves of k_insert_thread / k_insert_lane (st->n_pendl)
-  uint32_t* list_long;   // leaves for k_insert_thread_long (st->n_long)
+  uint32_t* list_long;   // leaves for k_insert_thread_long, or k_merge_small (st->n_long)
   int raw;               // leaves hold 8-byte cells (codec 1), not byte codes
   int small;             // a small batch: every slice goes to a warp per leaf
-  int long_warp;         // so does a leaf with a code of more than 4 bytes (long_by_warp)
+  int long_warp;         // k_merge_small takes list_long (long_by_warp)
   Bounds B;              // density bounds and tree height, for the leaves the
   unsigned H;            // thread-granular merge finalises itself
   uint32_t* viol;        // touched leaves over their own bound (count st->nviol)
@@ -1433,12 +1433,7 @@ __global__ void __launch_bounds__(kThrT, 4) k_insert_thread(MergeArgs a) {
                            leafp, y, S, res, R, nbytes, dl, db);
       }
     }
-    if (a.long_warp) {
-      if (lng != 0xFFFFFFFFu) a.T_state[lng] = kFallback;
-      warp_append(lng != 0xFFFFFFFFu, lng, a.list_v1, &a.st->n_v1);
-    } else {
-      warp_append(lng != 0xFFFFFFFFu, lng, a.list_long, &a.st->n_long);
-    }
+    warp_append(lng != 0xFFFFFFFFu, lng, a.list_long, &a.st->n_long);
     dl = warp_sum(dl);
     db = warp_sum(db);
     if (lane_id() == 0) {
@@ -1548,8 +1543,8 @@ __global__ void __launch_bounds__(kT) k_classify(MergeArgs a) {
 // shifted by the size change of the edits before it, plus the edits' bytes --
 // the same bytes as encoding the merged sequence from scratch, produced
 // without re-encoding the untouched codes.  A result over LB bytes is left
-// pending for the general merge.
-__global__ void __launch_bounds__(kT, 3) k_merge_small(MergeArgs a) {
+// pending for the general merge.  lng: the leaves of list_long, else of list_v1.
+__global__ void __launch_bounds__(kT, 3) k_merge_small(MergeArgs a, int lng) {
   extern __shared__ __align__(16) uint8_t smem[];
   pdl_wait();
   pdl_launch();
@@ -1567,10 +1562,11 @@ __global__ void __launch_bounds__(kT, 3) k_merge_small(MergeArgs a) {
   uint32_t* ee = es + kSmall;
   uint32_t* en = ee + kSmall;
   int32_t* shc = reinterpret_cast<int32_t*>(en + kSmall);
-  const uint64_t nV = a.st->n_v1;
+  const uint64_t nV = lng ? a.st->n_long : a.st->n_v1;
+  const uint32_t* list = lng ? a.list_long : a.list_v1;
   ull nbytes = 0;
   for (uint64_t li = (uint64_t)blockIdx.x * wpb + warp; li < nV; li += (uint64_t)gridDim.x * wpb) {
-    const uint32_t t = a.list_v1[li];
+    const uint32_t t = list[li];
     const uint32_t tb = a.T_begin[t], te = a.T_begin[t + 1];
     const uint32_t uold = a.T_oldused[t];
     const uint32_t s = te - tb;
@@ -1955,6 +1951,7 @@ struct FinArgs {
   uint32_t* chunk_cnt;
   const uint32_t* chunk_tid;
   const uint32_t *list_v1, *list_gen, *list_pend;
+  const uint32_t* list_long;  // nullptr: the thread-granular merge finished these
   uint32_t* viol;
   uint64_t* cand;
   uint32_t* bits;
@@ -1971,10 +1968,11 @@ __global__ void __launch_bounds__(kT) k_finalize(FinArgs a) {
   if (a.st->err) return;
   ull mb = 0, dl = 0, np = 0, db = 0, ov = 0;  // db: change of the byte total, mod 2^64
   // the touched leaves the thread- and lane-granular inserts did not finish
-  // themselves: the element-array splice's list, the general merge's leaves
+  // themselves: the element-array splice's lists, the general merge's leaves
   // (each once, by its first work item) and the pending leaves they left
   const uint64_t nv = a.st->n_v1, ng = a.st->n_gen, npl = a.st->n_pendl;
-  for (uint64_t i = gtid(); i < nv + ng + npl; i += gstride()) {
+  const uint64_t nl = a.list_long ? a.st->n_long : 0;
+  for (uint64_t i = gtid(); i < nv + ng + npl + nl; i += gstride()) {
     uint64_t t;
     if (i < nv) {
       t = a.list_v1[i];
@@ -1982,8 +1980,10 @@ __global__ void __launch_bounds__(kT) k_finalize(FinArgs a) {
       const uint32_t c = a.list_gen[i - nv];
       t = a.chunk_tid[c];
       if (a.T_first_chunk[t] != c) continue;
-    } else {
+    } else if (i < nv + ng + npl) {
       t = a.list_pend[i - nv - ng];
+    } else {
+      t = a.list_long[i - nv - ng - npl];
     }
     const uint32_t state = a.T_state[t];
     const uint32_t oldc = a.T_oldcnt[t], newc = a.T_newcnt[t];
@@ -3323,7 +3323,7 @@ bool long_by_warp(const cpma* h, uint64_t k) {
 }
 
 // The thread-granular insert (or delete) over the touched leaves of a batch
-// of k keys (at most k of them).
+// of k keys (at most k of them), without list_long's when warps take them.
 template <bool DEL>
 int launch_insert_thread(cpma* h, const MergeArgs& ma, uint64_t k, cudaStream_t st) {
   const int g = (int)std::max<uint64_t>(
@@ -3562,19 +3562,6 @@ int run_front(cpma* h, const uint64_t* d_keys, uint64_t k, int sorted, int is_de
         1, std::min<uint64_t>((k + swarps - 1) / swarps, (uint64_t)h->num_sms * 8));
     const bool thread = !ma.raw && !ma.small;
     const cudaStream_t side = thread ? h->side : st;
-    // (the leaves that the thread kernel leaves to a warp come after it)
-    const bool late = thread && ma.long_warp;
-    auto others = [&](cudaStream_t on) -> int {
-      prof_begin_side(h, PH_MERGE2, on);
-      ma.prof = prof_bytes(h, PH_MERGE2);
-      k_merge_small<<<sgrid, swarps * 32, sper * swarps, on>>>(ma);
-      ma.prof = nullptr;
-      CPMA_CUDA(launch_pdl(k_merge<false>, (unsigned)mgrid, (unsigned)(mwarps * 32), msmem, on,
-                           ma));
-      h->launches += 2;
-      prof_end_side(h, on);
-      return CPMA_OK;
-    };
     if (thread) {
       CPMA_CUDA(cudaEventRecord(h->ev_fork, st));
       CPMA_CUDA(cudaStreamWaitEvent(side, h->ev_fork, 0));
@@ -3590,19 +3577,29 @@ int run_front(cpma* h, const uint64_t* d_keys, uint64_t k, int sorted, int is_de
       h->launches++;
     }
     prof_end_side(h, side);
+    prof_begin_side(h, PH_MERGE2, side);
+    ma.prof = prof_bytes(h, PH_MERGE2);
+    k_merge_small<<<sgrid, swarps * 32, sper * swarps, side>>>(ma, 0);
     ma.prof = nullptr;
-    if (!late) CPMA_TRY(others(side));
+    CPMA_CUDA(launch_pdl(k_merge<false>, (unsigned)mgrid, (unsigned)(mwarps * 32), msmem, side,
+                         ma));
+    h->launches += 2;
+    prof_end_side(h, side);
     if (thread) {
       CPMA_CUDA(cudaEventRecord(h->ev_join, side));
       prof_begin(h, PH_MERGE, st);
       ma.prof = prof_bytes(h, PH_MERGE);
       if (is_delete) CPMA_TRY(launch_insert_thread<true>(h, ma, k, st));
       else CPMA_TRY(launch_insert_thread<false>(h, ma, k, st));
+      if (ma.long_warp) {
+        CPMA_CUDA(launch_pdl(k_merge_small, (unsigned)sgrid, (unsigned)(swarps * 32), sper * swarps,
+                             st, ma, 1));
+        h->launches++;
+      }
       ma.prof = nullptr;
       CPMA_CUDA(cudaStreamWaitEvent(st, h->ev_join, 0));
     }
     prof_end(h, st);
-    if (late) CPMA_TRY(others(st));
   }
   CPMA_CUDA(cudaGetLastError());
   prof_end(h, st);
@@ -3625,6 +3622,7 @@ int run_front(cpma* h, const uint64_t* d_keys, uint64_t k, int sorted, int is_de
   fa.list_v1 = ma.list_v1;
   fa.list_gen = ma.list_gen;
   fa.list_pend = ma.list_pend;
+  fa.list_long = ma.long_warp ? ma.list_long : nullptr;
   fa.viol = P<uint32_t>(s.viol);
   fa.cand = P<uint64_t>(s.cand);
   fa.bits = P<uint32_t>(s.bits);

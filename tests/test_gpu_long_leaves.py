@@ -50,3 +50,9 @@ def test_layouts(LB, n, ks, graphs):
         cp.cpma_insert_batch_tagged(g.handle, T(more), tags, 3, counts)
         assert int(counts.sum().item()) == o.insert_batch(more)
         same_layout(g, o, "tagged")
+
+
+@pytest.mark.parametrize("graphs", [False, True])
+def test_some_keys_in_each_leaf(graphs):
+    """Leaves of up to four keys, of five and more, and of none, beside each other."""
+    test_layouts(1024, 400_000, (9_000, 16_000), graphs)
